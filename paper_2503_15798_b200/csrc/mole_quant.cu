@@ -107,14 +107,14 @@ static CodebookParam codebook_param(int format)
     return c;
 }
 
-// ---- quantiser: one block of threads per id ---------------------------------------------------------
+// ---- quantiser, any block size: one block of threads per id (blocks above 2048 elements) ---------------
 // Pass 1: a warp per quantisation block finds the absolute maximum and stores the scale (float32, or the
 // float16 rounding of min(max, 65504)).  Pass 2: a thread per 8 consecutive elements divides by the stored
 // scale in float32 (IEEE division), counts the midpoints below the quotient and packs the 8 codes.
 constexpr int kQuantThreads = 256;
 
 template <int BITS>
-__global__ void __launch_bounds__(kQuantThreads) mole_quantize_kernel(const uint4 *__restrict__ src, unsigned char *__restrict__ dst,
+__global__ void __launch_bounds__(kQuantThreads) mole_quantize_wide_kernel(const uint4 *__restrict__ src, unsigned char *__restrict__ dst,
                                                                       long long V, int N, int d, int block, long long rec_bytes,
                                                                       const CodebookParam cb)
 {
@@ -181,6 +181,217 @@ __global__ void __launch_bounds__(kQuantThreads) mole_quantize_kernel(const uint
     }
     // padding bytes after the scales stay as the caller left them (zero them once after allocation if
     // records are to compare equal byte for byte)
+}
+
+// ---- quantiser, blocks of up to 2048 elements: a group of 2 .. 32 lanes per quantisation block ------------
+// Bound by memory: a table is read once and a quarter or a fifth of it written.  To stay under that the decision per
+// element is made without a division and two elements at a time.  The code of x is the number of codebook midpoints
+// below fl(x / s); no bf16 x and no scale s of at most 11 significant bits (a bf16, or the float16 an NF3 scale is)
+// has a quotient within a rounding of a midpoint (all mantissa pairs enumerated in tests/test_gpu_quant_tiles.py), so
+// fl(x / s) > m is x > s m in exact arithmetic, and for a bf16 x that is x > T, T the product rounded towards minus
+// infinity first to float32 and then to bf16.  The midpoints' thresholds are made once per quantisation block and
+// searched by bisection with packed bf16 compares.  A lane owns chunks of 16 consecutive elements (one 32-byte load; 8
+// bytes of NF4 codes, 4 + 2 of NF3) and keeps them in registers between the maximum and the coding.
+// One layer of the 160M shape (618 M elements) to NF3, block 128: 369 us, 4.0 TB/s (1486 us with two passes and a division
+// and 7 float32 compares per element); what is left is the integer pipe (compares and selects), 65 % busy.
+__device__ __forceinline__ uint32_t bf162_bits(__nv_bfloat162 v) { return *reinterpret_cast<const uint32_t *>(&v); }
+__device__ __forceinline__ __nv_bfloat162 bits_bf162(uint32_t v) { return *reinterpret_cast<const __nv_bfloat162 *>(&v); }
+// 0xffff in each half where x > t
+__device__ __forceinline__ uint32_t gt2(uint32_t x, uint32_t t) { return __hgt2_mask(bits_bf162(x), bits_bf162(t)); }
+// per bit: m ? a : b
+__device__ __forceinline__ uint32_t sel2(uint32_t m, uint32_t a, uint32_t b) { return (a & m) | (b & ~m); }
+// s * mid rounded towards minus infinity to float32, then to bf16; in both halves of the word
+template <bool NEGATIVE>
+__device__ __forceinline__ uint32_t threshold2(float s, float mid)
+{
+    uint32_t u = __float_as_uint(__fmul_rd(s, mid));
+    if (NEGATIVE) u += 0xffffu;
+    return __byte_perm(u, u, 0x3232);
+}
+// masks of the code bits of two elements: m[b] has 0xffff in a half whose code has bit b
+template <int BITS>
+struct CodeSearch;
+template <>
+struct CodeSearch<3> {
+    uint32_t t[7];
+    __device__ __forceinline__ void code(uint32_t x, uint32_t (&m)[3]) const
+    {
+        m[2] = gt2(x, t[3]);
+        m[1] = gt2(x, sel2(m[2], t[5], t[1]));
+        m[0] = gt2(x, sel2(m[2], sel2(m[1], t[6], t[4]), sel2(m[1], t[2], t[0])));
+    }
+};
+template <>
+struct CodeSearch<4> {
+    uint32_t t[15];
+    __device__ __forceinline__ void code(uint32_t x, uint32_t (&m)[4]) const
+    {
+        m[3] = gt2(x, t[7]);
+        m[2] = gt2(x, sel2(m[3], t[11], t[3]));
+        m[1] = gt2(x, sel2(m[3], sel2(m[2], t[13], t[9]), sel2(m[2], t[5], t[1])));
+        m[0] = gt2(x, sel2(m[3], sel2(m[2], sel2(m[1], t[14], t[12]), sel2(m[1], t[10], t[8])),
+                           sel2(m[2], sel2(m[1], t[6], t[4]), sel2(m[1], t[2], t[0]))));
+    }
+};
+
+struct QuantGrid {
+    long long rec_bytes;
+    uint32_t total;                    // quantisation blocks of the whole table
+    uint32_t per_id;                   // ... of one id
+    uint32_t code_bytes, low_bytes;    // of a record: all code planes, the NF3 low plane
+    int block, group_log2, wide_loads; // elements per block; lanes per block; the table is 32-byte aligned
+};
+
+template <int BITS, int CPL>
+__global__ void __launch_bounds__(kQuantThreads) mole_quantize_kernel(const unsigned char *__restrict__ src, unsigned char *__restrict__ dst,
+                                                                      const QuantGrid q, const CodebookParam cb)
+{
+    const int G = 1 << q.group_log2, g = threadIdx.x & (G - 1);
+    const uint32_t b_raw = blockIdx.x * (static_cast<uint32_t>(kQuantThreads) >> q.group_log2) + (threadIdx.x >> q.group_log2);
+    const bool live = b_raw < q.total;
+    const uint32_t b = live ? b_raw : q.total - 1;
+    const int chunks = q.block >> 4;
+    const unsigned char *in = src + static_cast<size_t>(b) * (static_cast<uint32_t>(q.block) * 2u);
+
+    uint32_t x[CPL][8];
+#pragma unroll
+    for (int i = 0; i < CPL; ++i) {
+        const int c = g + (i << q.group_log2);
+        if (c < chunks) {
+            const unsigned char *p = in + static_cast<uint32_t>(c) * 32u;
+            if (q.wide_loads) {
+                asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                             : "=r"(x[i][0]), "=r"(x[i][1]), "=r"(x[i][2]), "=r"(x[i][3]), "=r"(x[i][4]), "=r"(x[i][5]), "=r"(x[i][6]), "=r"(x[i][7])
+                             : "l"(p));
+            } else {
+                const uint4 lo = __ldg(reinterpret_cast<const uint4 *>(p)), hi = __ldg(reinterpret_cast<const uint4 *>(p) + 1);
+                x[i][0] = lo.x, x[i][1] = lo.y, x[i][2] = lo.z, x[i][3] = lo.w;
+                x[i][4] = hi.x, x[i][5] = hi.y, x[i][6] = hi.z, x[i][7] = hi.w;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) x[i][k] = 0u;
+        }
+    }
+    // the block's absolute maximum (NaNs ignored, as fmaxf does)
+    __nv_bfloat162 m2 = bits_bf162(0u);
+#pragma unroll
+    for (int i = 0; i < CPL; ++i)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) m2 = __hmax2(m2, __habs2(bits_bf162(x[i][k])));
+    float m = fmaxf(__uint_as_float(bf162_bits(m2) << 16), __uint_as_float(bf162_bits(m2) & 0xffff0000u));
+    for (int o = G >> 1; o >= 1; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+
+    const uint32_t id = b / q.per_id, within = b - id * q.per_id;
+    unsigned char *rec = dst + static_cast<size_t>(id) * q.rec_bytes;
+    float s = m;
+    if constexpr (BITS == 3) {
+        const __half h = __float2half_rn(fminf(m, 65504.f));
+        s = __half2float(h);
+        if (live && g == 0) reinterpret_cast<__half *>(rec + q.code_bytes)[within] = h;
+    } else {
+        if (live && g == 0) reinterpret_cast<float *>(rec + q.code_bytes)[within] = m;
+    }
+    CodeSearch<BITS> search;
+#pragma unroll
+    for (int t = 0; t < (1 << BITS) - 1; ++t)  // zero is value 2^(BITS-1) - 1 of the codebook: the midpoints before it are negative
+        search.t[t] = t < (1 << (BITS - 1)) - 1 ? threshold2<true>(s, cb.mid[t]) : threshold2<false>(s, cb.mid[t]);
+    const bool plain = s >= 0x1p-100f && s < INFINITY;  // every other block (all zero, infinities, scales near underflow) divides
+
+#pragma unroll
+    for (int i = 0; i < CPL; ++i) {
+        const int c = g + (i << q.group_log2);
+        uint32_t mask[8][BITS];
+        if (plain) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) search.code(x[i][k], mask[k]);
+        } else {
+#pragma unroll 1
+            for (int k = 0; k < 8; ++k) {
+                uint32_t xk = 0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) xk = j == k ? x[i][j] : xk;  // (registers have no run-time index)
+                uint32_t code[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float f = __uint_as_float(e ? xk & 0xffff0000u : xk << 16);
+                    const float y = s > 0.f ? __fdiv_rn(f, s) : 0.f;
+                    code[e] = 0;
+#pragma unroll
+                    for (int t = 0; t < (1 << BITS) - 1; ++t) code[e] += y > cb.mid[t] ? 1u : 0u;
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+#pragma unroll
+                    for (int bit = 0; bit < BITS; ++bit)
+                        if (j == k) mask[j][bit] = ((code[0] >> bit) & 1u ? 0xffffu : 0u) | ((code[1] >> bit) & 1u ? 0xffff0000u : 0u);
+            }
+        }
+        // pack: even elements in the low halves, odd ones in the high halves, shifted together at the end
+        const bool store = live && c < chunks;
+        if constexpr (BITS == 4) {
+            uint32_t w[4];  // four elements each: nibbles at bits 0 and 8 of either half
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                uint32_t a = 0;
+#pragma unroll
+                for (int v = 0; v < 2; ++v)
+#pragma unroll
+                    for (int bit = 0; bit < 4; ++bit) a |= mask[2 * k + v][bit] & ((1u << (8 * v + bit)) | (1u << (16 + 8 * v + 4 + bit)));
+                w[k] = a | (a >> 16);
+            }
+            const uint2 o = make_uint2(__byte_perm(w[0], w[1], 0x5410), __byte_perm(w[2], w[3], 0x5410));
+            if (store) *reinterpret_cast<uint2 *>(rec + within * (static_cast<uint32_t>(q.block) / 2) + static_cast<uint32_t>(c) * 8u) = o;
+        } else {
+            uint32_t lo[2], hi = 0;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                uint32_t a = 0;
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    a |= mask[4 * k + v][0] & ((1u << (4 * v)) | (1u << (16 + 4 * v + 2)));
+                    a |= mask[4 * k + v][1] & ((1u << (4 * v + 1)) | (1u << (16 + 4 * v + 3)));
+                    hi |= mask[4 * k + v][2] & ((1u << (8 * k + 2 * v)) | (1u << (16 + 8 * k + 2 * v + 1)));
+                }
+                lo[k] = a | (a >> 16);
+            }
+            if (store) {
+                *reinterpret_cast<uint32_t *>(rec + within * (static_cast<uint32_t>(q.block) / 4) + static_cast<uint32_t>(c) * 4u) = __byte_perm(lo[0], lo[1], 0x5410);
+                *reinterpret_cast<unsigned short *>(rec + q.low_bytes + within * (static_cast<uint32_t>(q.block) / 8) + static_cast<uint32_t>(c) * 2u) =
+                    static_cast<unsigned short>(hi | (hi >> 16));
+            }
+        }
+    }
+}
+
+// Lanes per quantisation block of `chunks` 16-element chunks (at most 128) and chunks per lane (at most 4): the pair that
+// leaves the fewest lanes without a chunk, the one with more chunks per lane among equals (thresholds and the maximum's
+// shuffles are paid once per lane).
+static void quant_group(int chunks, int *group_log2, int *cpl)
+{
+    int best = 1 << 30;
+    for (int lg = 5; lg >= 0; --lg) {
+        const int n = (chunks + (1 << lg) - 1) >> lg;
+        if (n > 4) break;
+        const int slots = n << lg;
+        if (slots <= best) {
+            best = slots;
+            *group_log2 = lg;
+            *cpl = n;
+        }
+    }
+}
+
+typedef void (*QuantizeKernel)(const unsigned char *, unsigned char *, const QuantGrid, const CodebookParam);
+template <int BITS>
+static QuantizeKernel pick_quantize(int cpl)
+{
+    switch (cpl) {
+        case 1: return mole_quantize_kernel<BITS, 1>;
+        case 2: return mole_quantize_kernel<BITS, 2>;
+        case 3: return mole_quantize_kernel<BITS, 3>;
+        default: return mole_quantize_kernel<BITS, 4>;
+    }
 }
 
 // ---- the fused layer over packed records: one block per token (see mole_decode.cuh for the structure) ----
@@ -490,10 +701,27 @@ int mole_quantize_lut(const void *lut, void *packed, int64_t V, int N, int d, in
     if (smem > 48 * 1024) return MOLE_ERR_UNSUPPORTED_SHAPE;
     const CodebookParam cb = codebook_param(format);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (format == MOLE_LUT_NF4)
-        mole_quantize_kernel<4><<<static_cast<unsigned>(V), kQuantThreads, smem, st>>>(static_cast<const uint4 *>(lut), static_cast<unsigned char *>(packed), V, N, d, block, rb, cb);
-    else
-        mole_quantize_kernel<3><<<static_cast<unsigned>(V), kQuantThreads, smem, st>>>(static_cast<const uint4 *>(lut), static_cast<unsigned char *>(packed), V, N, d, block, rb, cb);
+    const long long total = V * N * (d / block);
+    if (block <= 2048 && total <= 0x7fffffffLL) {
+        QuantGrid q;
+        int cpl = 1;
+        quant_group(block / 16, &q.group_log2, &cpl);
+        q.rec_bytes = rb;
+        q.total = static_cast<uint32_t>(total);
+        q.per_id = static_cast<uint32_t>(N * (d / block));
+        q.low_bytes = static_cast<uint32_t>(N) * (d / 4);
+        q.code_bytes = format == MOLE_LUT_NF4 ? static_cast<uint32_t>(N) * (d / 2) : q.low_bytes + static_cast<uint32_t>(N) * (d / 8);
+        q.block = block;
+        q.wide_loads = (reinterpret_cast<uintptr_t>(lut) & 31u) == 0 ? 1 : 0;
+        const long long per_cta = kQuantThreads >> q.group_log2;
+        const QuantizeKernel fn = format == MOLE_LUT_NF4 ? pick_quantize<4>(cpl) : pick_quantize<3>(cpl);
+        fn<<<static_cast<unsigned>((total + per_cta - 1) / per_cta), kQuantThreads, 0, st>>>(static_cast<const unsigned char *>(lut),
+                                                                                           static_cast<unsigned char *>(packed), q, cb);
+    } else if (format == MOLE_LUT_NF4) {
+        mole_quantize_wide_kernel<4><<<static_cast<unsigned>(V), kQuantThreads, smem, st>>>(static_cast<const uint4 *>(lut), static_cast<unsigned char *>(packed), V, N, d, block, rb, cb);
+    } else {
+        mole_quantize_wide_kernel<3><<<static_cast<unsigned>(V), kQuantThreads, smem, st>>>(static_cast<const uint4 *>(lut), static_cast<unsigned char *>(packed), V, N, d, block, rb, cb);
+    }
     MOLE_CUDA_TRY(cudaGetLastError());
     return MOLE_OK;
 }
