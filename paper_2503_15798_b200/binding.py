@@ -3,7 +3,9 @@
 Argument marshalling only: every function takes torch tensors (used for device memory and
 streams, nothing else), checks shapes and dtypes, and passes raw pointers and sizes to the
 entry point of the same name.  No arithmetic of the layer happens here, and there is no
-fallback: if ``libmole_b200.so`` has not been built, the first call raises.
+fallback: if ``libmole_b200.so`` has not been built, the first call raises.  The calls a decoding
+loop repeats (a layer, a step, the host and offload steps) go through the extension
+``mole_torch.so`` (csrc/binding_torch.cpp), the others through ctypes.
 """
 from __future__ import annotations
 
@@ -15,6 +17,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmole_b200.so")
+EXT_PATH = os.path.join(_HERE, "mole_torch.so")
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED_SHAPE, ERR_CUDA, ERR_NOMEM, ERR_TOO_LARGE, ERR_IO = range(7)
 STATUS_BAD_ID, STATUS_TIMEOUT = 1, 2
@@ -143,6 +146,30 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_ext = None
+
+
+def _calls():
+    """The extension module with the hot calls (it links against the library, which is loaded and checked first)."""
+    global _ext
+    if _ext is None:
+        lib()
+        if not os.path.exists(EXT_PATH):
+            raise RuntimeError(f"{EXT_PATH} is missing: build it with `python -m paper_2503_15798_b200.build`; this package has no fallback path")
+        import importlib.machinery
+        import importlib.util
+
+        loader = importlib.machinery.ExtensionFileLoader("mole_torch", EXT_PATH)
+        _ext = importlib.util.module_from_spec(importlib.util.spec_from_loader("mole_torch", loader))
+        loader.exec_module(_ext)
+    return _ext
+
+
+def _raw_stream(stream):
+    """What the extension takes: None (the current stream) or a raw stream handle."""
+    return stream if stream is None or isinstance(stream, int) else stream.cuda_stream
+
+
 def _check(code: int, where: str):
     if code != OK:
         raise MoleError(code, where)
@@ -184,6 +211,7 @@ class QuantTable:
         if packed.dtype != torch.uint8 or packed.shape[-1] != self.record_bytes:
             raise ValueError("packed must be uint8 [..., V, record_bytes]")
         self.V = packed.shape[-2]
+        self.shape_args = (self.V, N, d, fmt, block)
 
     def layer(self, l: int) -> "QuantTable":
         return QuantTable(self.packed[l], self.N, self.d, self.fmt, self.block)
@@ -225,50 +253,14 @@ def layer_forward(hidden, ids, lut, w_router, out=None, *, residual=None, gates_
     """mole_layer_forward_ex.  hidden [M][d] (or [B][T][d]), ids [M] int32/int64, lut [V][N][d] or a
     QuantTable, w_router [d][N]; returns out (allocated like hidden if not given).  norm_weight [d]: the
     router reads RMSNorm(hidden) with that scale and norm_eps, the residual stays un-normalised."""
-    quant = lut if isinstance(lut, QuantTable) else None
-    lut_t = quant.packed if quant else lut
-    for name, t in (("hidden", hidden), ("ids", ids), ("lut", lut_t), ("w_router", w_router)):
-        _dev(t, name)
-    if quant:
-        V, N, d = quant.V, quant.N, quant.d
-        if quant.packed.dim() != 2:
-            raise ValueError("a single layer takes one table: use QuantTable.layer(l)")
-    else:
-        V, N, d = lut.shape
-    M = hidden.numel() // d if d else 0
-    if hidden.shape[-1] != d or tuple(w_router.shape) != (d, N) or ids.numel() != M:
-        raise ValueError("shape mismatch between hidden, ids, lut and w_router")
-    tag = _dtype_tag(hidden)
-    if not ((quant or lut.dtype == hidden.dtype) and w_router.dtype == hidden.dtype):
-        raise TypeError("hidden, lut and w_router must share one element type")
-    if out is None:
-        out = torch.empty_like(hidden)
-    _dev(out, "out")
-    flags = 0
-    if ids.dtype == torch.int64:
-        flags |= FLAG_IDS_INT64
-    elif ids.dtype != torch.int32:
-        raise TypeError("ids must be int32 or int64")
-    if chain:
-        flags |= FLAG_CHAIN
-    if B is None:
-        B, T = M, 1
-    a = MoleArgs()
-    a.struct_size = ctypes.sizeof(MoleArgs)
-    a.flags = flags
-    a.hidden, a.ids, a.lut, a.w_router, a.out = _ptr(hidden), _ptr(ids), _ptr(lut_t), _ptr(w_router), _ptr(out)
-    a.residual, a.gates_out, a.status = _ptr(residual), _ptr(gates_out), _ptr(status)
-    a.B, a.T, a.N, a.d, a.V = B, T, N, d, V
-    a.dtype, a.kernel, a.d_split = tag, kernel, d_split
-    a.stream = _stream(stream)
-    if norm_weight is not None:
-        _dev(norm_weight, "norm_weight")
-        if norm_weight.dtype != hidden.dtype or norm_weight.numel() != d:
-            raise ValueError("norm_weight must be [d] of the element type of hidden")
-    a.norm_weight, a.norm_eps, a.reserved2 = _ptr(norm_weight), float(norm_eps), 0
-    a.lut_format, a.lut_block = (quant.fmt, quant.block) if quant else (LUT_PLAIN, 0)
-    _check(lib().mole_layer_forward_ex(ctypes.byref(a)), "mole_layer_forward_ex")
-    return out
+    quant = None
+    if isinstance(lut, QuantTable):
+        lut, quant = lut.packed, lut.shape_args
+    r = (_ext or _calls()).layer_forward(hidden, ids, lut, quant, w_router, out, residual, gates_out, status, d_split, chain,
+                                         _raw_stream(stream), B, T, norm_weight, norm_eps, kernel)
+    if type(r) is int:
+        raise MoleError(r, "mole_layer_forward_ex")
+    return r
 
 
 def layer_forward_basic(hidden, ids, lut, w_router, out, stream=None):
@@ -284,13 +276,8 @@ def decode_step(hidden_in, ids, luts, w_routers, out, tmp=None, status=None, str
                 d_split: int = 0):
     """mole_decode_step_ex: luts [L][V][N][d], w_routers [L][d][N]; returns out.  mode: STEP_AUTO,
     STEP_FUSED (one launch over all layers) or STEP_CHAINED (L launches, needs tmp when L > 1)."""
-    L, V, N, d = luts.shape
-    M = ids.numel()
-    tag = _dtype_tag(hidden_in)
-    _check(lib().mole_decode_step_ex(_ptr(hidden_in), _ptr(ids), _ptr(luts), luts.stride(0) * luts.element_size(),
-                                     _ptr(w_routers), w_routers.stride(0) * w_routers.element_size(), _ptr(out),
-                                     _ptr(tmp), _ptr(status), L, M, 1, N, d, V, tag, mode, d_split, _stream(stream)),
-           "mole_decode_step_ex")
+    _check((_ext or _calls()).decode_step(hidden_in, ids, luts, None, w_routers, out, tmp, status, _raw_stream(stream), mode, d_split,
+                                          None, 0.0, KERNEL_AUTO, False), "mole_decode_step_ex")
     return out
 
 
@@ -299,57 +286,26 @@ def decode_step_args(hidden_in, ids, luts, w_routers, out, tmp=None, status=None
                      chain_first: bool = False):
     """mole_decode_step_args: decode_step with every option; luts [L][V][N][d] or a QuantTable with packed
     [L][V][record_bytes]; norm_weights [L][d] puts RMSNorm(hidden) in front of every layer's router."""
-    quant = luts if isinstance(luts, QuantTable) else None
-    if quant:
-        lut_t = quant.packed
-        L, V, N, d = lut_t.shape[0], quant.V, quant.N, quant.d
-    else:
-        lut_t = luts
-        L, V, N, d = luts.shape
-    a = MoleStepArgs()
-    a.struct_size = ctypes.sizeof(MoleStepArgs)
-    a.flags = FLAG_CHAIN if chain_first else 0
-    a.hidden_in, a.ids, a.lut_base = _ptr(hidden_in), _ptr(ids), _ptr(lut_t)
-    a.lut_layer_stride_bytes = lut_t.stride(0) * lut_t.element_size()
-    a.w_router_base, a.wr_layer_stride_bytes = _ptr(w_routers), w_routers.stride(0) * w_routers.element_size()
-    if norm_weights is not None:
-        _dev(norm_weights, "norm_weights")
-        if norm_weights.dtype != hidden_in.dtype or tuple(norm_weights.shape) != (L, d):
-            raise ValueError("norm_weights must be [L][d] of the element type of hidden")
-        a.norm_weight_base, a.norm_layer_stride_bytes = _ptr(norm_weights), norm_weights.stride(0) * norm_weights.element_size()
-    a.out, a.tmp, a.status = _ptr(out), _ptr(tmp), _ptr(status)
-    a.L, a.B, a.T, a.N, a.d, a.V = L, ids.numel(), 1, N, d, V
-    a.dtype, a.mode, a.d_split, a.kernel = _dtype_tag(hidden_in), mode, d_split, kernel
-    a.norm_eps, a.reserved = float(norm_eps), 0
-    a.lut_format, a.lut_block = (quant.fmt, quant.block) if quant else (LUT_PLAIN, 0)
-    a.stream = _stream(stream)
-    _check(lib().mole_decode_step_args(ctypes.byref(a)), "mole_decode_step_args")
+    quant = None
+    if isinstance(luts, QuantTable):
+        luts, quant = luts.packed, luts.shape_args
+    _check((_ext or _calls()).decode_step(hidden_in, ids, luts, quant, w_routers, out, tmp, status, _raw_stream(stream), mode, d_split,
+                                          norm_weights, norm_eps, kernel, chain_first), "mole_decode_step_args")
     return out
 
 
 def decode_step_basic(hidden_in, ids, luts, w_routers, out, tmp=None, status=None, stream=None):
     """mole_decode_step, the plain entry point (mode and split chosen by the library)."""
-    L, V, N, d = luts.shape
-    M = ids.numel()
-    tag = _dtype_tag(hidden_in)
-    _check(lib().mole_decode_step(_ptr(hidden_in), _ptr(ids), _ptr(luts), luts.stride(0) * luts.element_size(),
-                                  _ptr(w_routers), w_routers.stride(0) * w_routers.element_size(), _ptr(out),
-                                  _ptr(tmp), _ptr(status), L, M, 1, N, d, V, tag, _stream(stream)),
-           "mole_decode_step")
+    _check((_ext or _calls()).decode_step(hidden_in, ids, luts, None, w_routers, out, tmp, status, _raw_stream(stream), STEP_AUTO, 0,
+                                          None, 0.0, KERNEL_AUTO, False), "mole_decode_step")
     return out
 
 
 def decode_step_host(hidden_host, ids_host, out_host, dev_hidden, dev_ids, dev_out, dev_tmp, luts, w_routers,
                      status=None, stream=None):
     """mole_decode_step_host: activations in (pinned) host tensors, tables on the device."""
-    L, V, N, d = luts.shape
-    M = ids_host.numel()
-    tag = _dtype_tag(dev_hidden)
-    _check(lib().mole_decode_step_host(_ptr(hidden_host), _ptr(ids_host), _ptr(out_host), _ptr(dev_hidden),
-                                       _ptr(dev_ids), _ptr(dev_out), _ptr(dev_tmp), _ptr(luts),
-                                       luts.stride(0) * luts.element_size(), _ptr(w_routers),
-                                       w_routers.stride(0) * w_routers.element_size(), _ptr(status), L, M, 1, N, d,
-                                       V, tag, _stream(stream)), "mole_decode_step_host")
+    _check((_ext or _calls()).decode_step_host(hidden_host, ids_host, out_host, dev_hidden, dev_ids, dev_out, dev_tmp, luts, w_routers,
+                                               status, _raw_stream(stream)), "mole_decode_step_host")
     return out_host
 
 
@@ -445,13 +401,8 @@ class OffloadContext:
 
     def decode_step(self, hidden_in, ids, luts_host, w_routers, out, tmp=None, status=None, stream=None, side_stream=None):
         """mole_offload_decode_step: luts_host [L][V][N][d] pinned host tensor, w_routers [L][d][N] device."""
-        L = luts_host.shape[0]
-        M = ids.numel()
-        _check(lib().mole_offload_decode_step(self.handle, _ptr(hidden_in), _ptr(ids), _ptr(luts_host),
-                                              luts_host.stride(0) * luts_host.element_size(), _ptr(w_routers),
-                                              w_routers.stride(0) * w_routers.element_size(), _ptr(out), _ptr(tmp),
-                                              _ptr(status), L, M, 1, _stream(stream), _stream(side_stream)),
-               "mole_offload_decode_step")
+        _check((_ext or _calls()).offload_decode_step(self.handle, hidden_in, ids, luts_host, w_routers, out, tmp, status,
+                                                      _raw_stream(stream), _raw_stream(side_stream)), "mole_offload_decode_step")
         return out
 
     def set_hot_rows(self, hot_ids, luts_host):

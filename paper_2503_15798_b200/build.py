@@ -1,8 +1,10 @@
-"""Build the sm_100a C-ABI library in-tree with nvcc (cross-compiles without a GPU).
+"""Build the sm_100a C-ABI library in-tree with nvcc (cross-compiles without a GPU), and the CPython extension
+through which binding.py makes its hot calls.
 
     python -m paper_2503_15798_b200.build [--force] [--verbose]
 
-Output: paper_2503_15798_b200/libmole_b200.so (CUDA runtime linked statically, no torch).
+Output: paper_2503_15798_b200/libmole_b200.so (CUDA runtime linked statically, no torch) and mole_torch.so beside it
+(torch tensors to the C ABI; argument marshalling only).
 """
 from __future__ import annotations
 
@@ -16,6 +18,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(HERE, "libmole_b200.so")
+EXT_SRC = os.path.join(CSRC, "binding_torch.cpp")
+EXT = os.path.join(HERE, "mole_torch.so")
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -31,17 +35,48 @@ def _deps():
     return sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
 
 
-def is_stale() -> bool:
-    if not os.path.exists(LIB):
+def _older(target, deps) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    return any(os.path.getmtime(p) > t for p in _deps())
+    t = os.path.getmtime(target)
+    return any(os.path.getmtime(p) > t for p in deps)
+
+
+def is_stale() -> bool:
+    return _older(LIB, _deps())
+
+
+def _build_extension(verbose: bool):
+    import sysconfig
+
+    import torch
+
+    inc, lib = os.path.join(torch.__path__[0], "include"), os.path.join(torch.__path__[0], "lib")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = EXT + f".tmp{os.getpid()}"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-w", "-o", tmp, EXT_SRC,
+           "-I", INCLUDE, "-I", sysconfig.get_path("include"), "-I", inc, "-I", os.path.join(inc, "torch", "csrc", "api", "include"),
+           "-I", os.path.join(cuda, "include"), "-L", HERE, "-l:libmole_b200.so", "-L", lib, "-ltorch_python", "-ltorch", "-ltorch_cpu",
+           "-lc10_cuda", "-lc10", "-Wl,-rpath,$ORIGIN", f"-Wl,-rpath,{lib}"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("building mole_torch.so failed")
+    if verbose:
+        sys.stderr.write(res.stdout + res.stderr)
+    os.replace(tmp, EXT)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile if the library is missing or older than a source.  Returns the .so path."""
-    if not force and not is_stale():
-        return LIB
+    """Compile what is missing or older than its sources.  Returns the library's path."""
+    if force or is_stale():
+        _build_library(verbose)
+    if force or _older(EXT, [EXT_SRC, LIB] + glob.glob(os.path.join(INCLUDE, "*.h"))):
+        _build_extension(verbose)
+    return LIB
+
+
+def _build_library(verbose: bool):
     nvcc = os.environ.get("NVCC", "nvcc")
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [nvcc, *NVCC_FLAGS, "-I", INCLUDE, "-I", CSRC, "-o", tmp, *sources()]
@@ -55,7 +90,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if verbose:
         sys.stderr.write(log)
     os.replace(tmp, LIB)
-    return LIB
 
 
 if __name__ == "__main__":

@@ -1,0 +1,299 @@
+// The hot calls of binding.py as a CPython extension: torch tensors in, the C ABI of include/mole.h out.
+//
+// A small launch (one token, one layer) keeps the GPU busy for a few microseconds, and marshalling its arguments in Python
+// -- a ctypes struct of two dozen fields, four method calls per tensor -- took longer than that: 10.7 us per call against
+// about 2.3 us for the launch itself.  Here the tensors' fields are read directly.  No arithmetic, no fallback, and the
+// same argument checks with the same exceptions as binding.py documents; the GIL is released around every library call.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <ATen/core/Tensor.h>
+#include <ATen/ops/empty_like.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <cstring>
+#include <exception>
+
+#include "mole.h"
+
+namespace {
+
+struct Failed {};  // a Python exception is set
+
+[[noreturn]] void fail(PyObject *type, const char *text)
+{
+    PyErr_SetString(type, text);
+    throw Failed();
+}
+
+const at::Tensor &tensor(PyObject *o, const char *name)
+{
+    if (!THPVariable_Check(o)) {
+        PyErr_Format(PyExc_TypeError, "%s must be a tensor", name);
+        throw Failed();
+    }
+    return THPVariable_Unpack(o);
+}
+const at::Tensor &device_tensor(PyObject *o, const char *name)
+{
+    const at::Tensor &t = tensor(o, name);
+    if (!t.is_cuda() || !t.is_contiguous()) {
+        PyErr_Format(PyExc_ValueError, "%s must be a contiguous CUDA tensor", name);
+        throw Failed();
+    }
+    return t;
+}
+// data pointer of an optional tensor (None: null)
+void *optional_ptr(PyObject *o, const char *name) { return o == Py_None ? nullptr : tensor(o, name).data_ptr(); }
+
+long long integer(PyObject *o)
+{
+    const long long v = PyLong_AsLongLong(o);
+    if (v == -1 && PyErr_Occurred()) throw Failed();
+    return v;
+}
+int int32(PyObject *o)
+{
+    const long long v = integer(o);
+    if (v < INT32_MIN || v > INT32_MAX) fail(PyExc_OverflowError, "integer argument out of range");
+    return static_cast<int>(v);
+}
+int int32(int64_t v)
+{
+    if (v < INT32_MIN || v > INT32_MAX) fail(PyExc_OverflowError, "tensor dimension out of range");
+    return static_cast<int>(v);
+}
+float number(PyObject *o)
+{
+    const double v = PyFloat_AsDouble(o);
+    if (v == -1.0 && PyErr_Occurred()) throw Failed();
+    return static_cast<float>(v);
+}
+// None: the current stream of the current device; otherwise a raw cudaStream_t as an integer
+void *stream_of(PyObject *o)
+{
+    if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+    void *p = PyLong_AsVoidPtr(o);
+    if (!p && PyErr_Occurred()) throw Failed();
+    return p;
+}
+int dtype_tag(const at::Tensor &t)
+{
+    if (t.scalar_type() == at::kBFloat16) return MOLE_DTYPE_BF16;
+    if (t.scalar_type() == at::kFloat) return MOLE_DTYPE_F32;
+    fail(PyExc_TypeError, "unsupported element type");
+}
+int64_t stride0_bytes(const at::Tensor &t) { return t.stride(0) * static_cast<int64_t>(t.element_size()); }
+
+template <typename F>
+int without_gil(F f)
+{
+    int rc;
+    Py_BEGIN_ALLOW_THREADS;
+    rc = f();
+    Py_END_ALLOW_THREADS;
+    return rc;
+}
+
+// one table or the tables of a step: a plain tensor, or the records of a quantised table with its shape beside it
+// (arguments lut, quant; quant: None or the tuple (V, N, d, format, block))
+struct Table {
+    const at::Tensor *t;
+    int V, N, d, format, block;
+};
+Table table(PyObject *lut, PyObject *quant, int dims, bool contiguous)
+{
+    Table r;
+    r.t = contiguous ? &device_tensor(lut, "lut") : &tensor(lut, "luts");
+    if (quant != Py_None) {
+        if (!PyTuple_Check(quant) || PyTuple_GET_SIZE(quant) != 5) fail(PyExc_TypeError, "quant must be (V, N, d, format, block)");
+        int *f[5] = {&r.V, &r.N, &r.d, &r.format, &r.block};
+        for (int i = 0; i < 5; ++i) *f[i] = int32(PyTuple_GET_ITEM(quant, i));
+        if (r.t->dim() != dims - 1)
+            fail(PyExc_ValueError, dims == 3 ? "a single layer takes one table: use QuantTable.layer(l)" : "a step takes the records of all its layers");
+        return r;
+    }
+    if (r.t->dim() != dims) fail(PyExc_ValueError, dims == 3 ? "lut must be [V][N][d]" : "luts must be [L][V][N][d]");
+    r.V = int32(r.t->size(dims - 3));
+    r.N = int32(r.t->size(dims - 2));
+    r.d = int32(r.t->size(dims - 1));
+    r.format = MOLE_LUT_PLAIN;
+    r.block = 0;
+    return r;
+}
+
+void expect_args(Py_ssize_t got, Py_ssize_t want)
+{
+    if (got != want) {
+        PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, got);
+        throw Failed();
+    }
+}
+
+template <typename F>
+PyObject *guarded(F f)
+{
+    try {
+        return f();
+    } catch (const Failed &) {
+        return nullptr;
+    } catch (const std::exception &e) {
+        if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
+        return nullptr;
+    }
+}
+
+// layer_forward(hidden, ids, lut, quant, w_router, out, residual, gates_out, status, d_split, chain, stream, B, T,
+//               norm_weight, norm_eps, kernel) -> the output tensor, or a non-zero status code
+PyObject *layer_forward(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        expect_args(n, 17);
+        const at::Tensor &hidden = device_tensor(a[0], "hidden"), &ids = device_tensor(a[1], "ids");
+        const Table lut = table(a[2], a[3], 3, true);
+        const at::Tensor &wr = device_tensor(a[4], "w_router");
+        const int64_t M = lut.d ? hidden.numel() / lut.d : 0;
+        if (hidden.dim() < 1 || hidden.size(-1) != lut.d || wr.dim() != 2 || wr.size(0) != lut.d || wr.size(1) != lut.N || ids.numel() != M)
+            fail(PyExc_ValueError, "shape mismatch between hidden, ids, lut and w_router");
+        mole_args m;
+        std::memset(&m, 0, sizeof m);
+        m.struct_size = sizeof m;
+        m.dtype = dtype_tag(hidden);
+        if ((lut.format == MOLE_LUT_PLAIN && lut.t->scalar_type() != hidden.scalar_type()) || wr.scalar_type() != hidden.scalar_type())
+            fail(PyExc_TypeError, "hidden, lut and w_router must share one element type");
+        at::Tensor fresh;
+        PyObject *result = a[5];
+        if (result == Py_None) fresh = at::empty_like(hidden);
+        const at::Tensor &out = result == Py_None ? fresh : device_tensor(result, "out");
+        if (ids.scalar_type() == at::kLong) m.flags |= MOLE_FLAG_IDS_INT64;
+        else if (ids.scalar_type() != at::kInt) fail(PyExc_TypeError, "ids must be int32 or int64");
+        if (PyObject_IsTrue(a[10])) m.flags |= MOLE_FLAG_CHAIN;
+        m.hidden = hidden.data_ptr();
+        m.ids = ids.data_ptr();
+        m.lut = lut.t->data_ptr();
+        m.w_router = wr.data_ptr();
+        m.out = out.data_ptr();
+        m.residual = optional_ptr(a[6], "residual");
+        m.gates_out = static_cast<float *>(optional_ptr(a[7], "gates_out"));
+        m.status = static_cast<uint32_t *>(optional_ptr(a[8], "status"));
+        m.B = a[12] == Py_None ? int32(M) : int32(a[12]);
+        m.T = a[12] == Py_None ? 1 : int32(a[13]);
+        m.N = lut.N;
+        m.d = lut.d;
+        m.V = lut.V;
+        m.d_split = int32(a[9]);
+        m.kernel = int32(a[16]);
+        m.stream = stream_of(a[11]);
+        if (a[14] != Py_None) {
+            const at::Tensor &nw = device_tensor(a[14], "norm_weight");
+            if (nw.scalar_type() != hidden.scalar_type() || nw.numel() != lut.d)
+                fail(PyExc_ValueError, "norm_weight must be [d] of the element type of hidden");
+            m.norm_weight = nw.data_ptr();
+        }
+        m.norm_eps = number(a[15]);
+        m.lut_format = lut.format;
+        m.lut_block = lut.block;
+        const int rc = without_gil([&] { return mole_layer_forward_ex(&m); });
+        if (rc != MOLE_OK) return PyLong_FromLong(rc);
+        if (result == Py_None) return THPVariable_Wrap(std::move(fresh));
+        Py_INCREF(result);
+        return result;
+    });
+}
+
+// decode_step(hidden_in, ids, luts, quant, w_routers, out, tmp, status, stream, mode, d_split, norm_weights, norm_eps, kernel,
+//             chain_first) -> status code
+PyObject *decode_step(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        expect_args(n, 15);
+        const at::Tensor &hidden = tensor(a[0], "hidden_in"), &ids = tensor(a[1], "ids");
+        const Table luts = table(a[2], a[3], 4, false);
+        const at::Tensor &wr = tensor(a[4], "w_routers");
+        mole_step_args m;
+        std::memset(&m, 0, sizeof m);
+        m.struct_size = sizeof m;
+        m.flags = PyObject_IsTrue(a[14]) ? MOLE_FLAG_CHAIN : 0;
+        m.hidden_in = hidden.data_ptr();
+        m.ids = ids.data_ptr();
+        m.lut_base = luts.t->data_ptr();
+        m.lut_layer_stride_bytes = stride0_bytes(*luts.t);
+        m.w_router_base = wr.data_ptr();
+        m.wr_layer_stride_bytes = stride0_bytes(wr);
+        m.L = int32(luts.t->size(0));
+        if (a[11] != Py_None) {
+            const at::Tensor &nw = device_tensor(a[11], "norm_weights");
+            if (nw.scalar_type() != hidden.scalar_type() || nw.dim() != 2 || nw.size(0) != m.L || nw.size(1) != luts.d)
+                fail(PyExc_ValueError, "norm_weights must be [L][d] of the element type of hidden");
+            m.norm_weight_base = nw.data_ptr();
+            m.norm_layer_stride_bytes = stride0_bytes(nw);
+        }
+        m.out = optional_ptr(a[5], "out");
+        m.tmp = optional_ptr(a[6], "tmp");
+        m.status = static_cast<uint32_t *>(optional_ptr(a[7], "status"));
+        m.B = int32(ids.numel());
+        m.T = 1;
+        m.N = luts.N;
+        m.d = luts.d;
+        m.V = luts.V;
+        m.dtype = dtype_tag(hidden);
+        m.mode = int32(a[9]);
+        m.d_split = int32(a[10]);
+        m.kernel = int32(a[13]);
+        m.norm_eps = number(a[12]);
+        m.lut_format = luts.format;
+        m.lut_block = luts.block;
+        m.stream = stream_of(a[8]);
+        return PyLong_FromLong(without_gil([&] { return mole_decode_step_args(&m); }));
+    });
+}
+
+// decode_step_host(hidden_host, ids_host, out_host, dev_hidden, dev_ids, dev_out, dev_tmp, luts, w_routers, status, stream)
+//   -> status code
+PyObject *decode_step_host(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        expect_args(n, 11);
+        const at::Tensor &ids = tensor(a[1], "ids_host"), &wr = tensor(a[8], "w_routers");
+        const Table luts = table(a[7], Py_None, 4, false);
+        const int L = int32(luts.t->size(0)), M = int32(ids.numel()), tag = dtype_tag(tensor(a[3], "dev_hidden"));
+        void *p[7];
+        for (int i = 0; i < 7; ++i) p[i] = optional_ptr(a[i], "a step's buffers");
+        void *status = optional_ptr(a[9], "status"), *stream = stream_of(a[10]);
+        return PyLong_FromLong(without_gil([&] {
+            return mole_decode_step_host(p[0], static_cast<const int32_t *>(p[1]), p[2], p[3], static_cast<int32_t *>(p[4]), p[5], p[6],
+                                         luts.t->data_ptr(), stride0_bytes(*luts.t), wr.data_ptr(), stride0_bytes(wr),
+                                         static_cast<uint32_t *>(status), L, M, 1, luts.N, luts.d, luts.V, tag, stream);
+        }));
+    });
+}
+
+// offload_decode_step(handle, hidden_in, ids, luts_host, w_routers, out, tmp, status, stream, side_stream) -> status code
+PyObject *offload_decode_step(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded([&]() -> PyObject * {
+        expect_args(n, 10);
+        void *ctx = a[0] == Py_None ? nullptr : PyLong_AsVoidPtr(a[0]);
+        if (PyErr_Occurred()) throw Failed();
+        const at::Tensor &hidden = tensor(a[1], "hidden_in"), &ids = tensor(a[2], "ids"), &luts = tensor(a[3], "luts_host"),
+                         &wr = tensor(a[4], "w_routers");
+        const int L = int32(luts.size(0)), M = int32(ids.numel());
+        void *out = optional_ptr(a[5], "out"), *tmp = optional_ptr(a[6], "tmp"), *status = optional_ptr(a[7], "status");
+        void *stream = stream_of(a[8]), *side = stream_of(a[9]);
+        return PyLong_FromLong(without_gil([&] {
+            return mole_offload_decode_step(static_cast<mole_offload_ctx *>(ctx), hidden.data_ptr(), static_cast<const int32_t *>(ids.data_ptr()),
+                                            luts.data_ptr(), stride0_bytes(luts), wr.data_ptr(), stride0_bytes(wr), out, tmp,
+                                            static_cast<uint32_t *>(status), L, M, 1, stream, side);
+        }));
+    });
+}
+
+#define MOLE_FASTCALL(f) {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(f)), METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {MOLE_FASTCALL(layer_forward), MOLE_FASTCALL(decode_step), MOLE_FASTCALL(decode_step_host),
+                         MOLE_FASTCALL(offload_decode_step), {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "mole_torch", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit_mole_torch(void) { return PyModule_Create(&module); }
