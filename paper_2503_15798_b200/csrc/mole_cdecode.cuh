@@ -95,7 +95,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kClusterThreads) mo
     static_assert(CS >= 2 && CS <= kClusterMaxBlocks && CS % 2 == 0, "portable cluster sizes; a hidden row is CS / 2 passes of 16 bytes per thread");
     extern __shared__ __align__(128) unsigned char smem[];
 
-    pdl_launch_dependents();
+    pdl_enter(p.flags);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int d = p.d;  // CS * 512

@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(decode_max_threads(N)) mole_decode_kernel(cons
     constexpr int R = N / 2;                   // sweep vectors per thread: (d * N / 8) / (d / 4)
     extern __shared__ __align__(128) unsigned char smem[];
 
-    pdl_launch_dependents();
+    pdl_enter(p.flags);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int T = blockDim.x, nwarps = T >> 5, d = p.d;

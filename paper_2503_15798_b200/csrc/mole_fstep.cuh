@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(FStepCut<N, DB>::dmax / 4 + 32) mole_fstep_ker
     constexpr int RW = N / 2;           // vectors of a whole matrix per thread
     extern __shared__ __align__(128) unsigned char smem[];
 
-    pdl_launch_dependents();
+    pdl_enter(p.flags);
 
     const int d = p.d, L = p.L, stages = p.stages, T = d / 4;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = T >> 5;

@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(kMaxConsumers + 32) mole_step_kernel(const Ste
     constexpr int EB = static_cast<int>(sizeof(T));
     extern __shared__ __align__(128) unsigned char smem[];
 
-    pdl_launch_dependents();
+    pdl_enter(p.flags);
 
     const int N = NFAST > 0 ? NFAST : p.N;
     const int K = (MODE == 1 || MODE == 2) ? 1 : p.K, L = p.L, stages = p.stages, HR = p.hring;

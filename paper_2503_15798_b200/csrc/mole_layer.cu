@@ -671,6 +671,25 @@ static int cached_launch(const StepLaunch &a, const LaunchChoice **out)
     return MOLE_OK;
 }
 
+int launch_pdl(const void *fn, unsigned grid, unsigned threads, int smem, cudaStream_t stream, void **args, bool chained)
+{
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (!chained) MOLE_CUDA_TRY(cudaStreamIsCapturing(stream, &capturing));
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = capturing == cudaStreamCaptureStatusNone ? 1 : 0;
+    MOLE_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, args));
+    return MOLE_OK;
+}
+
 int launch_step(const StepLaunch &a)
 {
     if (a.M == 0) return MOLE_OK;
@@ -679,22 +698,8 @@ int launch_step(const StepLaunch &a)
     int rc = cached_launch(a, &c);
     if (rc != MOLE_OK) return rc;
 
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3(static_cast<unsigned>(c->grid), 1, 1);
-    cfg.blockDim = dim3(c->threads, 1, 1);
-    cfg.dynamicSmemBytes = c->smem;
-    cfg.stream = a.stream;
-    cudaLaunchAttribute attrs[1];
-    unsigned na = 0;
-    if (a.flags & MOLE_FLAG_CHAIN) {
-        attrs[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attrs[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
-    cfg.attrs = attrs;
-    cfg.numAttrs = na;
-
+    const bool chained = (a.flags & MOLE_FLAG_CHAIN) != 0;
+    const unsigned grid = static_cast<unsigned>(c->grid), threads = static_cast<unsigned>(c->threads);
     if (c->fstep) {
         FStepParams p;
         p.hidden = a.hidden;
@@ -717,8 +722,8 @@ int launch_step(const StepLaunch &a)
         p.norm_eps = a.norm_eps;
         p.flags = a.flags;
         p.wait_polls = c->wait_polls;
-        MOLE_CUDA_TRY(cudaLaunchKernelEx(&cfg, c->fstep_fn, p));
-        return MOLE_OK;
+        void *args[1] = {&p};
+        return launch_pdl(reinterpret_cast<const void *>(c->fstep_fn), grid, threads, c->smem, a.stream, args, chained);
     }
     if (c->decode) {
         DecodeParams p;
@@ -736,8 +741,8 @@ int launch_step(const StepLaunch &a)
         p.norm_eps = a.norm_eps;
         p.flags = a.flags;
         p.wait_polls = c->wait_polls;
-        MOLE_CUDA_TRY(cudaLaunchKernelEx(&cfg, c->decode_fn, p));
-        return MOLE_OK;
+        void *args[1] = {&p};
+        return launch_pdl(reinterpret_cast<const void *>(c->decode_fn), grid, threads, c->smem, a.stream, args, chained);
     }
     const StepPlan &plan = c->plan;
     StepParams p;
@@ -767,8 +772,8 @@ int launch_step(const StepLaunch &a)
     p.consumers = plan.consumers;
     p.flags = a.flags;
     p.wait_polls = c->wait_polls;
-    MOLE_CUDA_TRY(cudaLaunchKernelEx(&cfg, c->step_fn, p));
-    return MOLE_OK;
+    void *args[1] = {&p};
+    return launch_pdl(reinterpret_cast<const void *>(c->step_fn), grid, threads, c->smem, a.stream, args, chained);
 }
 
 // One thread per (token, layer): an L2 prefetch of the token's N rows of that layer's table, in pieces of at most

@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(kDecodeMaxThreads) mole_qdecode_kernel(const Q
     constexpr int R = N / 2;
     extern __shared__ __align__(128) unsigned char smem[];
 
-    pdl_launch_dependents();
+    pdl_enter(p.flags);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int T = blockDim.x, nwarps = T >> 5, d = p.d;
@@ -645,23 +645,9 @@ int launch_quant_layer(const StepLaunch &a, int format, int block, uint32_t wait
     const int smem = static_cast<int>(qdecode_smem_bytes(a.N, a.d, p.rec_bytes));
     int rc = ensure_smem_opt_in(reinterpret_cast<const void *>(v.fn), smem);
     if (rc != MOLE_OK) return rc;
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3(static_cast<unsigned>(a.M), 1, 1);
-    cfg.blockDim = dim3(a.d / 4, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = a.stream;
-    cudaLaunchAttribute attrs[1];
-    unsigned na = 0;
-    if (a.flags & MOLE_FLAG_CHAIN) {
-        attrs[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attrs[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
-    cfg.attrs = attrs;
-    cfg.numAttrs = na;
-    MOLE_CUDA_TRY(cudaLaunchKernelEx(&cfg, v.fn, p));
-    return MOLE_OK;
+    void *args[1] = {&p};
+    return launch_pdl(reinterpret_cast<const void *>(v.fn), static_cast<unsigned>(a.M), static_cast<unsigned>(a.d / 4), smem, a.stream, args,
+                      (a.flags & MOLE_FLAG_CHAIN) != 0);
 }
 
 }  // namespace mole
