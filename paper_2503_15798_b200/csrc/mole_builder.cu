@@ -388,11 +388,7 @@ __global__ void mole_rmsnorm_rows_kernel(const __nv_bfloat16 *__restrict__ x, co
 
 #endif  // __CUDACC__
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
-                                  const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn encode_tiled()
+EncodeTiledFn encode_tiled()
 {
     static EncodeTiledFn fn = nullptr;
     static std::once_flag once;

@@ -1,6 +1,7 @@
 // Shared device helpers and host-side error plumbing of the MoLE sm_100a library.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -70,6 +71,21 @@ struct StepLaunch {
     int kernel = 0;  // MOLE_KERNEL_*: which kernel family runs the launch (0: the library's choice)
 };
 int launch_step(const StepLaunch &a);
+
+// The tensor-core kernel (mole_mma.cu): the shapes it covers, one launch's geometry.  launch_mma leaves `taken` false, and launches
+// nothing, where the tables' strides do not make tensor maps.
+struct MmaPlan {
+    const void *fn;
+    int cs, tb, threads, smem, groups, grid, w_slots, r_slots;
+};
+bool mma_shape_ok(int dtype, int N, int d);
+int plan_mma(long long M, int L, int N, int d, bool norm, int sms, bool prepare, MmaPlan *w);
+int launch_mma(const StepLaunch &a, const MmaPlan &w, uint32_t wait_polls, bool *taken);
+
+// cuTensorMapEncodeTiled, looked up once (mole_builder.cu); nullptr if the driver has none
+typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
+                                  const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiledFn encode_tiled();
 
 // Every layer kernel is launched with programmatic stream serialization: its blocks may be set up while the kernel before it
 // on the stream still runs, and it waits for that kernel itself -- first thing (pdl_enter), or, with MOLE_FLAG_CHAIN, before

@@ -516,6 +516,8 @@ struct ShapeKey {
 struct LaunchChoice {
     bool decode;        // the one-block-per-token kernel; otherwise the ring kernel with `plan`
     bool fstep;         // the fused step with the decode arithmetic, with `fplan`
+    bool mma;           // the tensor-core kernel, with `mplan` (the ring kernel where it does not take the launch)
+    MmaPlan mplan;
     FStepPlan fplan;
     FStepKernel fstep_fn;
     StepPlan plan;
@@ -540,7 +542,7 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
     int rc = plan_step(M, L, N, d, dtype, d_split, &plan, false, sms, norm);  // also validates the shape
     if (rc != MOLE_OK) return rc;
     const bool decode_ok = L == 1 && d_split == 0 && decode_shape_ok(dtype, N, d);
-    c->decode = c->fstep = false;
+    c->decode = c->fstep = c->mma = false;
     FStepPlan fplan;
     const bool fstep_ok = L > 1 && d_split == 0 && plan_fstep(M, L, N, d, dtype, norm, sms, &fplan);
     const bool cdecode_ok = L == 1 && d_split == 0 && cdecode_shape_ok(dtype, N, d);
@@ -573,6 +575,12 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
         c->grid = static_cast<long long>(per_sm) * sms;
         if (c->grid > M) c->grid = M;
         return MOLE_OK;
+    }
+    const bool mma_ok = kernel != MOLE_KERNEL_DECODE && mma_shape_ok(dtype, N, d) && !getenv("NOMMA");
+    if (mma_ok) {
+        c->mma = true;
+        rc = plan_mma(M, L, N, d, norm, sms, prepare, &c->mplan);
+        if (rc != MOLE_OK) return rc;
     }
     if (cdecode_ok && (kernel == MOLE_KERNEL_DECODE || (kernel == MOLE_KERNEL_AUTO && cdecode_preferred(M, N, sms)))) {
         const DecodeVariant v = pick_cdecode(N, norm);
@@ -698,6 +706,11 @@ int launch_step(const StepLaunch &a)
     int rc = cached_launch(a, &c);
     if (rc != MOLE_OK) return rc;
 
+    if (c->mma) {
+        bool taken = false;
+        rc = launch_mma(a, c->mplan, c->wait_polls, &taken);
+        if (rc != MOLE_OK || taken) return rc;
+    }
     const bool chained = (a.flags & MOLE_FLAG_CHAIN) != 0;
     const unsigned grid = static_cast<unsigned>(c->grid), threads = static_cast<unsigned>(c->threads);
     if (c->fstep) {

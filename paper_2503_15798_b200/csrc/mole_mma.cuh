@@ -1,0 +1,717 @@
+// The tensor-core form of the fused MoLE layer and of the fused L-layer step for sm_100a (Eq. 4 and Eq. 8 of arXiv
+// 2503.15798): bf16, N of 8, 16 or 32 experts, d a multiple of 128.
+//
+// What bounds the layer.  At decode sizes one token's layer is a dependent chain -- router product, a sum over the block, a
+// softmax, a weighted sum -- and with one token per SM each link costs its latency plus its instructions; at prefill sizes it is
+// instructions and the shared-memory port.  On CUDA cores the weighted sum alone is three instructions per two elements (two
+// unpacks and half a packed fma each): clock stamps gave 930 of 2 450 cycles per layer of the 410M shape to it and 700 to
+// the router sweep.  Both are products with a small matrix, so both run on mma.m16n8k16 here:
+//   - Router: A = W_r^T (16 experts x 16 columns per step), B = the hidden state of 1 .. 8 tokens: bf16 products, fp32 sums.
+//   - Weighted sum: A = rows^T (16 columns x 16 experts), B = the softmax numerators.  A numerator is an fp32 number and is
+//     never rounded: it is cut into three bf16 parts of 8 bits each (exactly), and the three products are chained into one
+//     fp32 accumulator.  The sum of the numerators is the same product with A = ones.
+// Split.  Warp w owns the 128 columns 128w .. of everything: of the hidden state, of every row, of the output, and those
+// columns are also its share of the router product.  So what a layer's router needs from the layer before is what the same
+// warp has just computed, and warps exchange nothing but N partial logits per token: one meeting per layer.  (RMSNorm in front
+// of the router adds one for the sum of squares.)  Where a token's rows exceed 64 KB a cluster of CS blocks shares the token;
+// the partial logits then travel through distributed shared memory (st.async) and the meeting is an mbarrier.
+// Data.  One producer warp streams router matrices and rows, whole boxes by tensor copy with the 128-byte swizzle, so that
+// ldmatrix reads either without bank conflicts; a warp loads the next layer's router fragments and its rows while it waits for
+// the logits of the others.  A single layer keeps its router in registers.
+// Groups.  TB = 1 for decode batches: a block per token, every warp forms the softmax itself.  TB = 8 for many tokens: one
+// router product for eight tokens, the softmaxes dealt out over the warps (a second meeting per group).
+// The order of every sum is fixed by N and d: a token gets the same bits with any TB, in any batch, in a single layer and in a
+// fused step.
+#pragma once
+
+#include <cuda.h>
+
+#include "mole_cdecode.cuh"
+
+namespace mole {
+
+constexpr int kMmaCols = 128;      // columns of a warp
+constexpr int kMmaHidStride = 272; // bytes between two tokens' hidden slices: 256 + 16, eight rows of an ldmatrix on different banks
+constexpr int kMmaMaxSlots = 8;
+constexpr int kMmaMaxSlices = 32;
+
+struct MmaParams {
+    const void *hidden, *residual, *row_index, *norm_weight;
+    void *out;
+    float *gates_out;
+    uint32_t *status;
+    long long norm_stride;  // bytes between the scale vectors of consecutive layers
+    long long M, rows;
+    int d, L;
+    int groups;             // groups of TB tokens
+    int w_slots, r_slots;   // router matrices and token rows in flight
+    float norm_eps;
+    uint32_t flags, wait_polls;
+};
+
+// Shared memory of a block: router matrices, rows, hidden slices (two sets with TB > 1), normalised slices, partial logits of
+// the whole token (two sets), split numerators, sums of squares (two sets), per-slot flags, barriers.
+struct MmaSmem {
+    uint32_t matrix;  // bytes of this block's part of a router matrix = of a token's rows
+    uint32_t off_r, off_hid, off_norm, off_partial, off_gates, off_ssq, off_meta, off_bars, total;
+};
+__host__ __device__ inline uint32_t mma_gate_bytes(int N) { return static_cast<uint32_t>(3 * N * 2 + 16); }
+__host__ __device__ inline MmaSmem mma_smem(int N, int d, int cs, int TB, int w_slots, int r_slots, int norm)
+{
+    MmaSmem m;
+    const int dl = d / cs, nw = dl / kMmaCols, slices = d / kMmaCols;
+    m.matrix = static_cast<uint32_t>(N) * dl * 2;
+    m.off_r = static_cast<uint32_t>(w_slots) * m.matrix;
+    m.off_hid = m.off_r + static_cast<uint32_t>(r_slots) * m.matrix;
+    m.off_norm = m.off_hid + static_cast<uint32_t>((TB > 1 ? 2 : 1) * nw * TB * kMmaHidStride);
+    m.off_partial = m.off_norm + (norm ? static_cast<uint32_t>(nw * TB * kMmaHidStride) : 0u);
+    m.off_gates = m.off_partial + static_cast<uint32_t>(2 * TB * slices * N * 4);
+    m.off_ssq = m.off_gates + (TB > 1 ? static_cast<uint32_t>(TB) * mma_gate_bytes(N) : 0u);
+    m.off_meta = m.off_ssq + (norm ? static_cast<uint32_t>(2 * TB * slices * 4) : 0u);
+    m.off_bars = (m.off_meta + (kMmaMaxSlots + 3) * 4 + 7u) & ~7u;
+    m.total = m.off_bars + (4 * kMmaMaxSlots + 4) * 8;
+    return m;
+}
+
+#ifdef __CUDACC__
+
+__device__ __forceinline__ void tensor_load_3d(uint32_t smem_dst, const CUtensorMap *map, int c0, int c1, int c2, uint64_t *bar)
+{
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 ::"r"(smem_dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
+                 : "memory");
+}
+__device__ __forceinline__ void tensor_load_5d(uint32_t smem_dst, const CUtensorMap *map, int c0, int c1, int c2, int c3, int c4, uint64_t *bar)
+{
+    asm volatile("cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+                 ::"r"(smem_dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(smem_u32(bar))
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm_x4_trans(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+// c += a b: A 16 x 16, B 16 x 8, bf16 products, fp32 sums
+__device__ __forceinline__ void mma16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// ... A 16 x 8, B 8 x 8
+__device__ __forceinline__ void mma8(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t b0)
+{
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(b0));
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void sts16(uint32_t a, unsigned short v) { asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(v) : "memory"); }
+__device__ __forceinline__ void stsf(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+__device__ __forceinline__ float ldsf(uint32_t a) { return __uint_as_float(lds32(a)); }
+
+// 1 / sqrt(mean + eps): the hardware's reciprocal root and one Newton step
+__device__ __forceinline__ float rms_scale(float total, int d, float eps)
+{
+    const float x = total / static_cast<float>(d) + eps;
+    const float r = rsqrtf(x);
+    return x > 0.f ? fmaf(r * 0.5f, fmaf(-x * r, r, 1.0f), r) : r;
+}
+
+// The three bf16 parts of two fp32 numbers, packed in pairs: a == hi + mid + lo exactly (8 bits each)
+struct Split2 {
+    uint32_t hi, mid, lo;
+};
+__device__ __forceinline__ Split2 split_pair(float a, float b)
+{
+    const uint32_t ah = __float_as_uint(a) & 0xffff0000u, bh = __float_as_uint(b) & 0xffff0000u;
+    const float ar = a - __uint_as_float(ah), br = b - __uint_as_float(bh);
+    const uint32_t am = __float_as_uint(ar) & 0xffff0000u, bm = __float_as_uint(br) & 0xffff0000u;
+    const float al = ar - __uint_as_float(am), bl = br - __uint_as_float(bm);
+    Split2 s;
+    s.hi = __byte_perm(ah, bh, 0x7632);
+    s.mid = __byte_perm(am, bm, 0x7632);
+    s.lo = __byte_perm(__float_as_uint(al), __float_as_uint(bl), 0x7632);
+    return s;
+}
+
+// This warp's 128 columns of the router matrix as A fragments (experts x columns).  A matrix [columns][N] lies in rows of 128
+// bytes -- 64 / N columns each -- whose 16-byte pieces are swizzled by the row number.
+template <int N>
+struct RouterA {
+    static constexpr int ET = N == 32 ? 2 : 1;  // tiles of 16 experts
+    uint32_t a[8][ET][N == 8 ? 2 : 4];          // N = 8: rows 8 .. 15 of A are zero
+    uint32_t off;                               // this lane's first address inside the slice
+    __device__ __forceinline__ void init(int lane)
+    {
+        const int i = lane & 7, m = lane >> 3;
+        if constexpr (N == 8) off = static_cast<uint32_t>(m * 128 + ((i ^ m) << 4));                                               // column 8 m + i
+        else if constexpr (N == 16) off = static_cast<uint32_t>((2 * (m >> 1) + (i >> 2)) * 128 + ((((i & 3) * 2 + (m & 1)) ^ (2 * (m >> 1) + (i >> 2))) << 4));
+        else off = static_cast<uint32_t>((4 * (m >> 1) + (i >> 1)) * 128 + ((((i & 1) * 4 + (m & 1)) ^ (4 * (m >> 1) + (i >> 1))) << 4));
+    }
+    __device__ __forceinline__ void load(uint32_t slice)
+    {
+        if constexpr (N == 8) {
+#pragma unroll
+            for (int s = 0; s < 8; s += 2) {  // two steps of 16 columns per load
+                uint32_t r[4];
+                ldsm_x4_trans(r, (slice + off + static_cast<uint32_t>(s) * 256u) ^ ((s & 2) ? 64u : 0u));
+                a[s][0][0] = r[0], a[s][0][1] = r[1], a[s + 1][0][0] = r[2], a[s + 1][0][1] = r[3];
+            }
+        } else if constexpr (N == 16) {
+#pragma unroll
+            for (int s = 0; s < 8; ++s) ldsm_x4_trans(a[s][0], (slice + off + static_cast<uint32_t>(s) * 512u) ^ ((s & 1) ? 64u : 0u));
+        } else {
+#pragma unroll
+            for (int s = 0; s < 8; ++s)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) ldsm_x4_trans(a[s][e], (slice + off + static_cast<uint32_t>(s) * 1024u) ^ (e ? 32u : 0u));
+        }
+    }
+    // z[e]: fragment of expert tile e over the slice; steps in four chains.  h: this lane's ldmatrix address in the hidden slice(s)
+    __device__ __forceinline__ void product(uint32_t h, float (&z)[ET][4]) const
+    {
+        uint32_t b[4][4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) ldsm_x4(b[s], h + 64u * s);
+        float c[ET][4][4];
+#pragma unroll
+        for (int e = 0; e < ET; ++e)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) c[e][k][i] = 0.f;
+#pragma unroll
+        for (int s = 0; s < 8; ++s)
+#pragma unroll
+            for (int e = 0; e < ET; ++e) {
+                const uint32_t b0 = b[s >> 1][2 * (s & 1)], b1 = b[s >> 1][2 * (s & 1) + 1];
+                if constexpr (N == 8) mma16(c[e][s & 3], a[s][0][0], 0u, a[s][0][1], 0u, b0, b1);
+                else mma16(c[e][s & 3], a[s][e][0], a[s][e][1], a[s][e][2], a[s][e][3], b0, b1);
+            }
+#pragma unroll
+        for (int e = 0; e < ET; ++e)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) z[e][i] = (c[e][0][i] + c[e][1][i]) + (c[e][2][i] + c[e][3][i]);
+    }
+};
+
+// A token's softmax numerators as B fragments (experts x 8 equal columns), in three parts
+template <int N>
+struct GateB {
+    static constexpr int KS = N == 32 ? 2 : 1;  // steps of 16 experts
+    static constexpr int W = N == 8 ? 1 : 2;    // words per step
+    uint32_t part[3][KS][W];
+    __device__ __forceinline__ void set(int k, int w, const Split2 &s) { part[0][k][w] = s.hi, part[1][k][w] = s.mid, part[2][k][w] = s.lo; }
+    // e: lane j holds the numerator of expert j % N
+    __device__ __forceinline__ void from_lanes(float e, int lane)
+    {
+        const int q = lane & 3;
+#pragma unroll
+        for (int k = 0; k < KS; ++k)
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                const int j = 16 * k + 8 * w + 2 * q;
+                set(k, w, split_pair(__shfl_sync(0xffffffffu, e, j), __shfl_sync(0xffffffffu, e, j + 1)));
+            }
+    }
+    __device__ __forceinline__ void mac(float (&c)[4], const uint32_t (&a)[KS][2 * W]) const
+    {
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int k = 0; k < KS; ++k) {
+                if constexpr (N == 8) mma8(c, a[k][0], a[k][1], part[p][k][0]);
+                else mma16(c, a[k][0], a[k][1], a[k][2], a[k][3], part[p][k][0], part[p][k][1]);
+            }
+    }
+    __device__ __forceinline__ float sum() const  // of the numerators
+    {
+        float c[4] = {0.f, 0.f, 0.f, 0.f};
+        uint32_t ones[KS][2 * W];
+#pragma unroll
+        for (int k = 0; k < KS; ++k)
+#pragma unroll
+            for (int w = 0; w < 2 * W; ++w) ones[k][w] = 0x3f803f80u;
+        mac(c, ones);
+        return c[0];
+    }
+};
+
+// This warp's 128 columns of a token's rows as A fragments (columns x experts): eight tiles of 16 columns.  The rows lie as
+// [64-column chunk][expert][128 bytes], 16-byte pieces swizzled by the expert.
+template <int N>
+struct RowsA {
+    static constexpr int KS = GateB<N>::KS, W = GateB<N>::W;
+    uint32_t a[8][KS][2 * W];
+    static __device__ __forceinline__ uint32_t lane_offset(int lane)
+    {
+        const int i = lane & 7, m = lane >> 3;
+        if constexpr (N == 8) return static_cast<uint32_t>(i * 128 + ((i ^ m) << 4));  // piece m of four: two tiles per load
+        else return static_cast<uint32_t>((i + 8 * (m >> 1)) * 128 + ((i ^ (m & 1)) << 4));
+    }
+    __device__ __forceinline__ void load(uint32_t addr)  // slot + this warp's chunks + lane offset
+    {
+        if constexpr (N == 8) {
+#pragma unroll
+            for (int t = 0; t < 8; t += 2) {
+                uint32_t r[4];
+                ldsm_x4_trans(r, (addr + static_cast<uint32_t>(t >> 2) * (N * 128u)) ^ ((t & 2) ? 64u : 0u));
+                a[t][0][0] = r[0], a[t][0][1] = r[1], a[t + 1][0][0] = r[2], a[t + 1][0][1] = r[3];
+            }
+        } else {
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+#pragma unroll
+                for (int k = 0; k < KS; ++k)
+                    ldsm_x4_trans(a[t][k], (addr + static_cast<uint32_t>(t >> 2) * (N * 128u) + static_cast<uint32_t>(k) * 2048u) ^ (static_cast<uint32_t>(t & 3) << 5));
+        }
+    }
+    // v[i]: the sums of this lane's four columns: 16 q + r, 16 q + 8 + r, 64 + 16 q + r, 64 + 16 q + 8 + r  (lane = 4 r + q)
+    __device__ __forceinline__ void product(const GateB<N> &g, int lane, float (&v)[4]) const
+    {
+        float c[8][4];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) c[t][i] = 0.f;
+        }
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int k = 0; k < KS; ++k)
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    if constexpr (N == 8) mma8(c[t], a[t][k][0], a[t][k][1], g.part[p][k][0]);
+                    else mma16(c[t], a[t][k][0], a[t][k][1], a[t][k][2], a[t][k][3], g.part[p][k][0], g.part[p][k][1]);
+                }
+        const bool q0 = (lane & 1) != 0, q1 = (lane & 2) != 0;  // all columns of the product are equal: lane q takes tiles q and 4 + q
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int base = (i >> 1) * 4, w = (i & 1) * 2;
+            const float x = q0 ? c[base + 1][w] : c[base][w], y = q0 ? c[base + 3][w] : c[base + 2][w];
+            v[i] = q1 ? y : x;
+        }
+    }
+};
+
+// Softmax numerator of a logit; `group`: lanes (a power of two) that hold one token's logits.  The maximum is subtracted only
+// where a token has a logit beyond +-60 (exp and the parts of its result then leave the normal range): any shift gives the same gates.
+__device__ __forceinline__ float softmax_part(float z, int group)
+{
+    float shift = 0.f;
+    if (__any_sync(0xffffffffu, !(fabsf(z) < 60.f))) {
+        float zm = z;
+        int big = !(fabsf(z) < 60.f) ? 1 : 0;
+        for (int o = group / 2; o >= 1; o >>= 1) {
+            zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
+            big |= __shfl_xor_sync(0xffffffffu, big, o);
+        }
+        if (big) shift = zm;
+    }
+    return expf(z - shift);
+}
+
+// N: experts.  TB: tokens per group (1 or 8).  NORM: the router reads RMSNorm(hidden).  CS: blocks per token.
+// Launch: d / CS / 4 + 32 threads, mma_smem(..).total bytes, a multiple of CS blocks.
+template <int N, int TB, int NORM, int CS>
+__global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 32 ? 1 : 2)
+    mole_mma_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap r_map, const MmaParams p)
+{
+    constexpr int ET = RouterA<N>::ET;
+    extern __shared__ __align__(1024) unsigned char smem[];
+
+    pdl_enter(p.flags);
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = static_cast<int>(blockDim.x >> 5) - 1;
+    const int d = p.d, L = p.L, WS = p.w_slots, RS = p.r_slots, slices = nw * CS;
+    const uint32_t rank = CS > 1 ? cluster_ctarank() : 0u;
+    const MmaSmem m = mma_smem(N, d, CS, TB, WS, RS, NORM);
+    const uint32_t base = smem_u32(smem);
+    volatile int *meta = reinterpret_cast<volatile int *>(smem + m.off_meta);  // [r_slots] the slot's id is inside the table
+    volatile int *dead = meta + kMmaMaxSlots;                                  // somebody gave up waiting
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + m.off_bars);
+    uint64_t *wfull = bars, *wempty = bars + kMmaMaxSlots, *rfull = bars + 2 * kMmaMaxSlots, *rempty = bars + 3 * kMmaMaxSlots;
+    uint64_t *xbar = bars + 4 * kMmaMaxSlots, *sbar = xbar + 2;  // the cluster's exchanges: logits, sums of squares
+    const int G = static_cast<int>(gridDim.x) / CS, g0 = static_cast<int>(blockIdx.x) / CS;
+    const int ng = (p.groups - g0 + G - 1) / G;  // groups of this block: g0, g0 + G, ...
+    auto token_of = [&](int gi, int tok) -> long long { return (static_cast<long long>(g0) + static_cast<long long>(gi) * G) * TB + tok; };
+
+    if (tid == 0) {
+        for (int s = 0; s < WS; ++s) {
+            mbar_init(wfull + s, 1);
+            mbar_init(wempty + s, nw);
+        }
+        for (int s = 0; s < RS; ++s) {
+            mbar_init(rfull + s, 1);
+            mbar_init(rempty + s, nw);
+        }
+        for (int s = 0; s < 4; ++s) mbar_init(xbar + s, 1);
+        dead[0] = 0;
+        dead[2] = 0;  // raised by nobody: the drain waits run their (short) course
+        mbar_init_fence();
+    }
+    __syncthreads();
+    if constexpr (CS > 1) cluster_arrive();  // waited for before the first push
+
+    if (warp == nw) {
+        // ================= producer warp: copies in the order they are consumed -- the first router matrix, then per (group,
+        // layer) the rows of the first token, the router matrix of the item after, the rows of the other tokens =================
+        const bool ids64 = (p.flags & MOLE_FLAG_IDS_INT64) != 0;
+        auto load_ids = [&](int window) -> long long {  // ids of 32 consecutive tokens of this block, one per lane; -1: none
+            const int n = window * 32 + lane;
+            const long long t = token_of(n / TB, n % TB);
+            if (n / TB >= ng || t >= p.M) return -1;
+            return ids64 ? __ldg(static_cast<const long long *>(p.row_index) + t) : static_cast<long long>(__ldg(static_cast<const int *>(p.row_index) + t));
+        };
+        int ws = 0, rs = 0, issued_w = 0, issued_r = 0, w_layer = 0;
+        uint32_t wph = 1, rph = 1;  // parity of the `empty` phase that frees the slot
+        bool ok = true;
+        const int matrices = ng > 0 ? (L > 1 ? ng * L : 1) : 0;
+        const int w_rows = nw * (2 * N);  // 128-byte rows of this block's part of a router matrix
+        const int w_box = w_rows <= 256 ? w_rows : w_rows / 2;
+        auto wait_slot = [&](uint64_t *bar, uint32_t parity) {
+            int got = 1;
+            if (lane == 0) {
+                got = wait_or_give_up(bar, parity, dead, p.wait_polls, true);
+                if (!got) report_timeout(dead, p.status);
+            }
+            ok = __shfl_sync(0xffffffffu, got, 0) != 0;
+        };
+        auto issue_router = [&]() {
+            if (issued_w >= matrices) return;
+            if (issued_w >= WS) wait_slot(wempty + ws, wph);
+            if (!ok) return;
+            if (lane == 0) {
+                mbar_expect_tx(wfull + ws, m.matrix);
+                for (int r = 0; r < w_rows; r += w_box)
+                    tensor_load_3d(base + static_cast<uint32_t>(ws) * m.matrix + static_cast<uint32_t>(r) * 128u, &w_map, 0, static_cast<int>(rank) * w_rows + r, w_layer, wfull + ws);
+            }
+            ++issued_w;
+            if (++w_layer == L) w_layer = 0;
+            if (++ws == WS) ws = 0, wph ^= 1u;
+        };
+        issue_router();
+        long long id_now = load_ids(0), id_next = load_ids(1);
+#pragma unroll 1
+        for (int gi = 0; gi < ng && ok; ++gi) {
+#pragma unroll 1
+            for (int l = 0; l < L && ok; ++l) {
+#pragma unroll 1
+                for (int k = 0; k < TB; ++k) {
+                    if (k == 1) issue_router();
+                    const int n = gi * TB + k;
+                    if (l == 0 && (n & 31) == 0 && n > 0) {
+                        id_now = id_next;
+                        id_next = load_ids((n >> 5) + 1);
+                    }
+                    const long long id = __shfl_sync(0xffffffffu, id_now, n & 31);
+                    const bool valid = id >= 0 && id < p.rows;
+                    if (!ok) break;
+                    if (issued_r >= RS) wait_slot(rempty + rs, rph);
+                    if (!ok) break;
+                    if (lane == 0) {
+                        meta[rs] = valid ? 1 : 0;
+                        if (valid) {
+                            mbar_expect_tx(rfull + rs, m.matrix);
+                            tensor_load_5d(base + m.off_r + static_cast<uint32_t>(rs) * m.matrix, &r_map, 0, 0, static_cast<int>(rank) * nw * 2, static_cast<int>(id), l, rfull + rs);
+                        } else {
+                            mbar_arrive(rfull + rs);  // nothing to copy: the routed term is dropped
+                            if (l == 0 && rank == 0 && p.status && token_of(gi, k) < p.M) atomicOr(p.status, MOLE_STATUS_BAD_ID);
+                        }
+                    }
+                    ++issued_r;
+                    if (++rs == RS) rs = 0, rph ^= 1u;
+                }
+                if (TB == 1 && ok) issue_router();
+            }
+        }
+        if (!ok) {
+            // copies already issued land in this block's shared memory: give them a (short) time to, before the block can exit
+            for (int i = issued_w > WS ? issued_w - WS : 0; i < issued_w; ++i) (void)wait_or_give_up(wfull + i % WS, (i / WS) & 1, dead + 2, kDrainPolls);
+            for (int i = issued_r > RS ? issued_r - RS : 0; i < issued_r; ++i) (void)wait_or_give_up(rfull + i % RS, (i / RS) & 1, dead + 2, kDrainPolls);
+        }
+        __syncwarp();
+        if constexpr (CS > 1) cluster_wait();
+    } else {
+        // ================= compute warps ======================================================================================
+        const int nc = nw * 32;
+        const int slice = static_cast<int>(rank) * nw + warp;  // of the whole token
+        const int r8 = lane >> 2, q = lane & 3;
+        const uint32_t hid_set = static_cast<uint32_t>(nw * TB * kMmaHidStride);
+        const uint32_t hid0 = base + m.off_hid + static_cast<uint32_t>(warp * TB * kMmaHidStride);
+        const uint32_t norm0 = base + m.off_norm + static_cast<uint32_t>(warp * TB * kMmaHidStride);
+        const uint32_t frag_off = static_cast<uint32_t>((TB > 1 ? (lane & 7) * kMmaHidStride : 0) + (lane >> 3) * 16);
+        const uint32_t own_off = static_cast<uint32_t>(2 * (16 * q + r8));  // this lane's columns: + 0, 16, 128, 144 bytes
+        const uint32_t part_set = static_cast<uint32_t>(TB * slices * N * 4);
+        const uint32_t w_off = static_cast<uint32_t>(warp) * (256u * N);
+        const uint32_t r_off = m.off_r + static_cast<uint32_t>(warp) * (256u * N) + RowsA<N>::lane_offset(lane);
+        const size_t slice_bytes = static_cast<size_t>(slice) * (kMmaCols * 2);
+        bool alive = true;  // false after a wait ran out: no more waiting, whatever is there is computed on (the status says so)
+        auto acquire = [&](uint64_t *bar, uint32_t parity) {
+            if (alive && mbar_try_wait(bar, parity)) return;
+            alive = acquire_slow(bar, parity, dead, alive, true, p.status, lane, p.wait_polls);
+        };
+        auto acquire_cluster = [&](uint64_t *bar, uint32_t parity) {
+            for (uint32_t i = 0; alive; ++i) {
+                if (mbar_try_wait_cluster(bar, parity)) return;
+                if (i >= p.wait_polls) {
+                    if (lane == 0) report_timeout(dead, p.status);
+                    alive = false;
+                }
+                if (i > 64) __nanosleep(32);
+                if ((i & 127u) == 127u && *dead) alive = false;
+            }
+        };
+        int ws = 0, rs = 0;
+        uint32_t wph = 0, rph = 0;
+        RouterA<N> wf;
+        wf.init(lane);
+        auto load_router = [&]() {
+            acquire(wfull + ws, wph);
+            wf.load(base + static_cast<uint32_t>(ws) * m.matrix + w_off);
+        };
+        auto release_router = [&]() {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(wempty + ws);
+            if (++ws == WS) ws = 0, wph ^= 1u;
+        };
+        auto release_rows = [&]() {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(rempty + rs);
+            if (++rs == RS) rs = 0, rph ^= 1u;
+        };
+        if (ng > 0) load_router();
+        if constexpr (CS > 1) cluster_wait();
+
+        pdl_wait();
+        fence_proxy_async_global();
+
+        const unsigned char *hid_g = static_cast<const unsigned char *>(p.hidden) + slice_bytes + (lane & 15) * 16;
+        const unsigned char *norm_g = static_cast<const unsigned char *>(p.norm_weight) + slice_bytes + own_off;
+        unsigned short nw_next[4] = {0, 0, 0, 0};
+        auto load_norm = [&](int l) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) nw_next[i] = __ldg(reinterpret_cast<const unsigned short *>(norm_g + static_cast<size_t>(l) * p.norm_stride + (i >> 1) * 128 + (i & 1) * 16));
+        };
+        // hidden slices of group gi into set s
+        auto fetch_hidden = [&](int gi, int s) {
+            if (gi < ng) {
+#pragma unroll
+                for (int kk = 0; kk < (TB + 1) / 2; ++kk) {
+                    const int k = 2 * kk + (lane >> 4);
+                    if (k >= TB) break;
+                    long long t = token_of(gi, k);
+                    if (t >= p.M) t = p.M - 1;  // rows past the last token repeat it; nothing of them is used
+                    cp_async16(hid0 + static_cast<uint32_t>(s) * hid_set + static_cast<uint32_t>(k * kMmaHidStride + (lane & 15) * 16), hid_g + static_cast<size_t>(t) * d * 2);
+                }
+            }
+            cp_async_commit();
+        };
+        fetch_hidden(0, 0);
+        if constexpr (NORM) load_norm(0);
+
+        uint32_t buf = 0, xph = 0, hs = 0;  // exchange buffer, its barrier's parity; hidden set
+#pragma unroll 1
+        for (int gi = 0; gi < ng; ++gi) {
+            cp_async_wait_all();
+            __syncwarp();
+            const uint32_t hid = hid0 + hs * hid_set;
+            if constexpr (TB > 1) fetch_hidden(gi + 1, static_cast<int>(hs ^ 1u));
+#pragma unroll 1
+            for (int l = 0; l < L; ++l) {
+                const bool last = l == L - 1;
+                if (CS > 1 && tid == 0) {
+                    mbar_expect_tx(xbar + buf, part_set);
+                    if (NORM) mbar_expect_tx(sbar + buf, static_cast<uint32_t>(TB * slices * 4));
+                }
+                // ---- what the router reads ----
+                uint32_t router_in = hid;
+                if constexpr (NORM) {
+                    router_in = norm0;
+                    const uint32_t sq = base + m.off_ssq + buf * static_cast<uint32_t>(TB * slices * 4);
+                    float wgt[4], ss[TB];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) wgt[i] = bf16_bits_to_float(nw_next[i]);
+                    if (L > 1) load_norm(last ? 0 : l + 1);
+#pragma unroll
+                    for (int k = 0; k < TB; ++k) {
+                        float s = 0.f;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float x = bf16_bits_to_float(lds16(hid + own_off + static_cast<uint32_t>(k * kMmaHidStride + (i >> 1) * 128 + (i & 1) * 16)));
+                            s = fmaf(x, x, s);
+                        }
+                        ss[k] = s;
+                    }
+                    int first = 0;
+                    if constexpr (TB > 1) lane_reduce_scatter<TB, TB, 16, 1>(ss, lane, first);
+                    else ss[0] = warp_sum(ss[0]);
+                    if ((lane & (TB > 1 ? 3 : 31)) == 0) {
+                        const uint32_t at = sq + static_cast<uint32_t>(first * slices + slice) * 4u;
+                        if constexpr (CS == 1) stsf(at, ss[0]);
+                        else
+#pragma unroll
+                            for (int c = 0; c < CS; ++c) cluster_push_f32(cluster_map(at, c), ss[0], cluster_map(smem_u32(sbar + buf), c));
+                    }
+                    if constexpr (CS == 1) named_bar_sync(3, nc);
+                    else acquire_cluster(sbar + buf, xph);
+                    float total = 0.f;
+                    for (int w = 0; w < slices; ++w) total += ldsf(sq + static_cast<uint32_t>((lane & (TB - 1)) * slices + w) * 4u);  // slices in ascending order
+                    const float rinv = rms_scale(total, d, p.norm_eps);
+#pragma unroll
+                    for (int k = 0; k < TB; ++k) {
+                        const float r = TB > 1 ? __shfl_sync(0xffffffffu, rinv, k) : rinv;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const uint32_t o = own_off + static_cast<uint32_t>(k * kMmaHidStride + (i >> 1) * 128 + (i & 1) * 16);
+                            sts16(norm0 + o, float_to_bf16_bits((bf16_bits_to_float(lds16(hid + o)) * r) * wgt[i]));
+                        }
+                    }
+                    __syncwarp();
+                }
+
+                // ---- router: this warp's partial logits: lane (r, q): experts r, r + 8 of tokens 2q, 2q + 1 ----
+                float z[ET][4];
+                wf.product(router_in + frag_off, z);
+                const uint32_t part = base + m.off_partial + buf * part_set;
+#pragma unroll
+                for (int e = 0; e < ET; ++e)
+#pragma unroll
+                    for (int i = 0; i < (N == 8 ? 2 : 4); ++i) {
+                        const int tok = TB > 1 ? 2 * q + (i & 1) : 0;
+                        const uint32_t at = part + static_cast<uint32_t>((tok * slices + slice) * N + 16 * e + r8 + 8 * (i >> 1)) * 4u;
+                        if (TB > 1 || (q == 0 && (i & 1) == 0)) {
+                            if constexpr (CS == 1) stsf(at, z[e][i]);
+                            else
+#pragma unroll
+                                for (int c = 0; c < CS; ++c) cluster_push_f32(cluster_map(at, c), z[e][i], cluster_map(smem_u32(xbar + buf), c));
+                        }
+                    }
+                if (L > 1) release_router();
+                if constexpr (CS == 1) named_bar_arrive(1, 2 * nc);
+                // under the others' products: the first token's rows, the next router matrix
+                acquire(rfull + rs, rph);
+                bool valid = meta[rs] != 0;
+                RowsA<N> rows;
+                rows.load(base + static_cast<uint32_t>(rs) * m.matrix + r_off);
+                if (L > 1 && !(last && gi + 1 == ng)) load_router();
+                if constexpr (CS == 1) named_bar_sync(1, 2 * nc);
+                else acquire_cluster(xbar + buf, xph);
+
+                // ---- softmax numerators (Eq. 4): even slices and odd slices, then the two ----
+                auto numerator_of = [&](int tok) -> float {
+                    const uint32_t z_in = part + static_cast<uint32_t>(tok * slices * N + (lane & (N - 1))) * 4u;
+                    float ze = 0.f, zo = 0.f;
+#pragma unroll 4
+                    for (int w = 0; w + 1 < slices; w += 2) {
+                        ze += ldsf(z_in + static_cast<uint32_t>(w * N) * 4u);
+                        zo += ldsf(z_in + static_cast<uint32_t>((w + 1) * N) * 4u);
+                    }
+                    if (slices & 1) ze += ldsf(z_in + static_cast<uint32_t>((slices - 1) * N) * 4u);
+                    return softmax_part(ze + zo, N);
+                };
+                GateB<N> g;
+                float inv = 0.f;
+                if constexpr (TB == 1) {
+                    const float e = numerator_of(0);
+                    g.from_lanes(e, lane);
+                    const float esum = g.sum();
+                    inv = __frcp_rn(esum);
+                    if (p.gates_out && slice == 0 && lane < N) p.gates_out[token_of(gi, 0) * N + lane] = e / esum;
+                } else {
+                    for (int tok = warp; tok < TB; tok += nw) {
+                        const uint32_t gs = base + m.off_gates + static_cast<uint32_t>(tok) * mma_gate_bytes(N);
+                        const float e = numerator_of(tok);
+                        g.from_lanes(e, lane);
+                        const float esum = g.sum();
+                        if (lane < 4) {
+#pragma unroll
+                            for (int pt = 0; pt < 3; ++pt)
+#pragma unroll
+                                for (int k = 0; k < GateB<N>::KS; ++k)
+#pragma unroll
+                                    for (int w = 0; w < GateB<N>::W; ++w) sts32(gs + static_cast<uint32_t>(pt * N + 16 * k + 8 * w + 2 * lane) * 2u, g.part[pt][k][w]);
+                        }
+                        if (lane == 0) stsf(gs + 3 * N * 2, __frcp_rn(esum));
+                        const long long t = token_of(gi, tok);
+                        if (p.gates_out && rank == 0 && t < p.M && lane < N) p.gates_out[t * N + lane] = e / esum;
+                    }
+                    named_bar_sync(2, nc);
+                }
+
+                // ---- weighted sum of the rows (Eq. 8), residual, one rounding ----
+#pragma unroll 1
+                for (int k = 0; k < TB; ++k) {
+                    if constexpr (TB > 1) {
+                        if (k > 0) {
+                            acquire(rfull + rs, rph);
+                            valid = meta[rs] != 0;
+                            rows.load(base + static_cast<uint32_t>(rs) * m.matrix + r_off);
+                        }
+                        const uint32_t gs = base + m.off_gates + static_cast<uint32_t>(k) * mma_gate_bytes(N);
+#pragma unroll
+                        for (int pt = 0; pt < 3; ++pt)
+#pragma unroll
+                            for (int kk = 0; kk < GateB<N>::KS; ++kk)
+#pragma unroll
+                                for (int w = 0; w < GateB<N>::W; ++w) g.part[pt][kk][w] = lds32(gs + static_cast<uint32_t>(pt * N + 16 * kk + 8 * w + 2 * q) * 2u);
+                        inv = ldsf(gs + 3 * N * 2);
+                    }
+                    float v[4];
+                    rows.product(g, lane, v);
+                    release_rows();
+                    const uint32_t own = hid + own_off + static_cast<uint32_t>(k * kMmaHidStride);
+                    uint32_t res[4];
+                    if (p.residual && last) {
+                        const long long t = token_of(gi, k);
+                        const unsigned char *src = static_cast<const unsigned char *>(p.residual) + static_cast<size_t>(t < p.M ? t : p.M - 1) * d * 2 + slice_bytes + own_off;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) res[i] = ldcg_u16(src + (i >> 1) * 128 + (i & 1) * 16);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) res[i] = lds16(own + static_cast<uint32_t>((i >> 1) * 128 + (i & 1) * 16));
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        sts16(own + static_cast<uint32_t>((i >> 1) * 128 + (i & 1) * 16),
+                              valid ? float_to_bf16_bits(fmaf(v[i], inv, bf16_bits_to_float(res[i]))) : static_cast<unsigned short>(res[i]));
+                }
+                __syncwarp();
+                buf ^= 1u;
+                if (buf == 0) xph ^= 1u;
+            }
+            // ---- the group's outputs ----
+            {
+                unsigned char *out = static_cast<unsigned char *>(p.out) + slice_bytes + (lane & 15) * 16;
+#pragma unroll
+                for (int kk = 0; kk < (TB + 1) / 2; ++kk) {
+                    const int k = 2 * kk + (lane >> 4);
+                    if (k >= TB) break;
+                    const long long t = token_of(gi, k);
+                    if (t < p.M) *reinterpret_cast<uint4 *>(out + static_cast<size_t>(t) * d * 2) = lds128(hid + static_cast<uint32_t>(k * kMmaHidStride + (lane & 15) * 16));
+                }
+            }
+            __syncwarp();
+            if constexpr (TB > 1) hs ^= 1u;
+            else fetch_hidden(gi + 1, 0);
+        }
+    }
+    if constexpr (CS > 1) {  // pushes to this block may still be on their way: nobody leaves before everybody is done
+        cluster_arrive();
+        cluster_wait();
+    }
+}
+
+#endif  // __CUDACC__
+
+}  // namespace mole
