@@ -34,7 +34,9 @@
  *  - An id outside [0, V) never reads out of bounds: that token gets out_t = res_t and, if a
  *    status word was supplied, MOLE_STATUS_BAD_ID is OR-ed into it.
  *  - Results are deterministic: no atomics in the arithmetic, fixed summation order, and a
- *    token's result does not depend on the batch it is in.
+ *    token's result does not depend on the batch it is in (within a kernel family, see MOLE_KERNEL_AUTO).
+ *  - Launches use programmatic stream serialization: a kernel may be set up, but reads nothing, before the
+ *    one before it on the stream has finished (MOLE_FLAG_CHAIN lets it read ids, tables and routers early).
  */
 #ifndef MOLE_H
 #define MOLE_H
@@ -82,7 +84,10 @@ extern "C" {
 
 /* which kernel family runs a single-layer launch (mole_args.kernel, mole_step_args.kernel) */
 #define MOLE_KERNEL_AUTO 0   /* the library's choice: the ring kernel, except d = 2048 with N = 32 at up to 128 tokens (on \
-                                148 SMs), where the one-token-per-cluster kernel of MOLE_KERNEL_DECODE runs */
+                                148 SMs), where the one-token-per-cluster kernel of MOLE_KERNEL_DECODE runs, and except \
+                                single bf16 layers of many tokens (above 2, 6 or 8 per SM, by row size) with N of 8, 16 \
+                                or 32, d a multiple of 128 up to 2048 and d_split 0, where the prefill kernel runs.  \
+                                mole_variant names that by the ring instantiation of the launch's shape. */
 #define MOLE_KERNEL_RING 1   /* persistent blocks, rows and router chunks streamed through a shared-memory ring: any shape */
 #define MOLE_KERNEL_DECODE 2 /* one block per token (single layer: rows held in registers; fused step: rows through a ring, \
                                 router matrix through registers): bf16, N of 4, 8, 16 or 32, d a multiple of 128 up to   \

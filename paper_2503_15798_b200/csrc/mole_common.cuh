@@ -72,6 +72,15 @@ struct StepLaunch {
 };
 int launch_step(const StepLaunch &a);
 
+// The prefill kernel (mole_tile.cu): the shapes it covers, one launch's geometry.
+struct TilePlan {
+    void *fn;
+    int tb, threads, smem, groups, grid;
+};
+bool tile_shape_ok(int dtype, int N, int d);
+int plan_tile(long long M, int N, int d, bool norm, int sms, bool prepare, TilePlan *t);
+int launch_tile(const StepLaunch &a, const TilePlan &t);
+
 // The tensor-core kernel (mole_mma.cu): the shapes it covers, one launch's geometry.  launch_mma leaves `taken` false, and launches
 // nothing, where the tables' strides do not make tensor maps.
 struct MmaPlan {
@@ -233,6 +242,43 @@ __device__ __forceinline__ void sts64(uint32_t a, const uint2 &v)
 __device__ __forceinline__ void sts32(uint32_t a, uint32_t v)
 {
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
+// Warp-wide matrix loads and products, 16-byte asynchronous copies.
+__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm_x4_trans(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+// c += a b: A 16 x 16, B 16 x 8, bf16 products, fp32 sums
+__device__ __forceinline__ void mma16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// ... A 16 x 8, B 8 x 8
+__device__ __forceinline__ void mma8(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t b0)
+{
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(b0));
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+// 1 / sqrt(mean + eps): the hardware's reciprocal root and one Newton step
+__device__ __forceinline__ float rms_scale(float total, int d, float eps)
+{
+    const float x = total / static_cast<float>(d) + eps;
+    const float r = rsqrtf(x);
+    return x > 0.f ? fmaf(r * 0.5f, fmaf(-x * r, r, 1.0f), r) : r;
 }
 
 // 16-byte vectors of the two storage types

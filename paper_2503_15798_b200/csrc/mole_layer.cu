@@ -373,6 +373,16 @@ static DecodeVariant pick_cdecode(int N, bool norm)
     return DecodeVariant{nullptr, "none"};
 }
 
+// Tokens from which a single layer runs on the prefill kernel (mole_tile.cuh).  Measured against the ring kernel, us per layer:
+// rows of more than 32 KB, which the ring cuts into chunks, from two tokens per SM on (1B shape: 11.3 against 10.4 at 200 tokens,
+// 12.1 against 14.7 at 300); rows of up to 32 KB from six (410M shape: 8.3 / 8.3 at 600, 8.4 / 10.4 at 900; 160M: 8.7 / 10.3 at
+// 900); small rows, of which the ring kernel keeps more blocks resident, from eight (N = 16, d = 384: even at 1 200).
+static long long tile_from(int N, int d, int sms)
+{
+    const long long row = static_cast<long long>(N) * d * 2;
+    return (row > 32 * 1024 ? 2LL : (row > 16 * 1024 ? 6LL : 8LL)) * sms;
+}
+
 // The fused step with the decode arithmetic (mole_fstep.cuh): bf16, N of 4, 8, 16 or 32, d a multiple of
 // 128 with d / 4 <= 512 compute threads, router matrix in 1, 2 or 4 column chunks of at most 32 KB, rows in
 // chunks of whole experts of at most 32 KB.
@@ -516,6 +526,8 @@ struct ShapeKey {
 struct LaunchChoice {
     bool decode;        // the one-block-per-token kernel; otherwise the ring kernel with `plan`
     bool fstep;         // the fused step with the decode arithmetic, with `fplan`
+    bool tile;          // the prefill kernel, with `tplan`
+    TilePlan tplan;
     bool mma;           // the tensor-core kernel, with `mplan` (the ring kernel where it does not take the launch)
     MmaPlan mplan;
     FStepPlan fplan;
@@ -542,7 +554,7 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
     int rc = plan_step(M, L, N, d, dtype, d_split, &plan, false, sms, norm);  // also validates the shape
     if (rc != MOLE_OK) return rc;
     const bool decode_ok = L == 1 && d_split == 0 && decode_shape_ok(dtype, N, d);
-    c->decode = c->fstep = c->mma = false;
+    c->decode = c->fstep = c->mma = c->tile = false;
     FStepPlan fplan;
     const bool fstep_ok = L > 1 && d_split == 0 && plan_fstep(M, L, N, d, dtype, norm, sms, &fplan);
     const bool cdecode_ok = L == 1 && d_split == 0 && cdecode_shape_ok(dtype, N, d);
@@ -576,7 +588,7 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
         if (c->grid > M) c->grid = M;
         return MOLE_OK;
     }
-    const bool mma_ok = kernel != MOLE_KERNEL_DECODE && mma_shape_ok(dtype, N, d) && !getenv("NOMMA");
+    const bool mma_ok = getenv("MMA") && L > 1 && kernel == MOLE_KERNEL_AUTO && d_split == 0 && mma_shape_ok(dtype, N, d) && !getenv("NOMMA");
     if (mma_ok) {
         c->mma = true;
         rc = plan_mma(M, L, N, d, norm, sms, prepare, &c->mplan);
@@ -624,6 +636,15 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
                         direct);
     }
     if (!v.fn) return MOLE_ERR_UNSUPPORTED_SHAPE;
+    if (L == 1 && kernel == MOLE_KERNEL_AUTO && d_split == 0 && tile_shape_ok(dtype, N, d) && M > tile_from(N, d, sms)) {
+        c->tile = true;
+        rc = plan_tile(M, N, d, norm, sms, prepare, &c->tplan);
+        if (rc != MOLE_OK) return rc;
+        c->name = v.name;
+        c->threads = c->tplan.threads;
+        c->smem = c->tplan.smem;
+        return MOLE_OK;
+    }
     c->decode = false;
     c->plan = plan;
     c->step_fn = v.fn;
@@ -706,6 +727,7 @@ int launch_step(const StepLaunch &a)
     int rc = cached_launch(a, &c);
     if (rc != MOLE_OK) return rc;
 
+    if (c->tile) return launch_tile(a, c->tplan);
     if (c->mma) {
         bool taken = false;
         rc = launch_mma(a, c->mplan, c->wait_polls, &taken);
