@@ -101,8 +101,7 @@ extern "C" {
 #define MOLE_LUT_NF3 2 /* 3-bit NormalFloat codes, one float16 absmax scale per block (paper: block 128 -> 19.5 % of FP16) */
 
 /* mole_decode_step_ex mode: how the L layers of a step are launched */
-#define MOLE_STEP_AUTO 0    /* fused unless the batch is large (then chained); also chained at up to 16 tokens where \
-                               MOLE_KERNEL_AUTO runs the cluster kernel and a tmp buffer was given */
+#define MOLE_STEP_AUTO 0    /* fused unless the batch is large (then chained) */
 #define MOLE_STEP_FUSED 1   /* ONE launch: every block walks its tokens through all L layers */
 #define MOLE_STEP_CHAINED 2 /* L launches chained with programmatic dependent launch */
 

@@ -81,14 +81,14 @@ bool tile_shape_ok(int dtype, int N, int d);
 int plan_tile(long long M, int N, int d, bool norm, int sms, bool prepare, TilePlan *t);
 int launch_tile(const StepLaunch &a, const TilePlan &t);
 
-// The tensor-core kernel (mole_mma.cu): the shapes it covers, one launch's geometry.  launch_mma leaves `taken` false, and launches
-// nothing, where the tables' strides do not make tensor maps.
+// The tensor-core step kernel (mole_mma.cu): whether a fused step runs on it, one launch's geometry.  launch_mma leaves `taken`
+// false, and launches nothing, where the tables' strides do not make tensor maps.
 struct MmaPlan {
     const void *fn;
-    int cs, tb, threads, smem, groups, grid, w_slots, r_slots;
+    int cs, threads, smem, grid, w_slots, r_slots;
 };
-bool mma_shape_ok(int dtype, int N, int d);
-int plan_mma(long long M, int L, int N, int d, bool norm, int sms, bool prepare, MmaPlan *w);
+bool mma_preferred(long long M, int dtype, int N, int d, int sms);
+int plan_mma(long long M, int N, int d, bool norm, int sms, bool prepare, MmaPlan *w);
 int launch_mma(const StepLaunch &a, const MmaPlan &w, uint32_t wait_polls, bool *taken);
 
 // cuTensorMapEncodeTiled, looked up once (mole_builder.cu); nullptr if the driver has none

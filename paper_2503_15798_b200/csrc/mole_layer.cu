@@ -588,11 +588,11 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
         if (c->grid > M) c->grid = M;
         return MOLE_OK;
     }
-    const bool mma_ok = getenv("MMA") && L > 1 && kernel == MOLE_KERNEL_AUTO && d_split == 0 && mma_shape_ok(dtype, N, d) && !getenv("NOMMA");
-    if (mma_ok) {
+    if (L > 1 && kernel == MOLE_KERNEL_AUTO && d_split == 0 && mma_preferred(M, dtype, N, d, sms)) {
         c->mma = true;
-        rc = plan_mma(M, L, N, d, norm, sms, prepare, &c->mplan);
+        rc = plan_mma(M, N, d, norm, sms, prepare, &c->mplan);
         if (rc != MOLE_OK) return rc;
+        if (c->mplan.grid < M * c->mplan.cs) c->mma = false;  // not all tokens resident at once (clusters leave SMs unused)
     }
     if (cdecode_ok && (kernel == MOLE_KERNEL_DECODE || (kernel == MOLE_KERNEL_AUTO && cdecode_preferred(M, N, sms)))) {
         const DecodeVariant v = pick_cdecode(N, norm);
@@ -936,13 +936,6 @@ int mole_decode_step_args(const mole_step_args *a)
         return MOLE_ERR_INVALID_ARG;
     if (mode == MOLE_STEP_AUTO) {
         mode = (quant || (L > 1 && M > kFusedMaxTokens)) ? MOLE_STEP_CHAINED : MOLE_STEP_FUSED;
-        // the widest layers at up to 16 tokens: L chained launches of the cluster kernel are ahead of the fused launch
-        // (measured: 2.7 - 3.3 us against 3.5 - 3.65 us per layer); they need the caller's second buffer
-        int sms = kNumSMs;
-        if (mode == MOLE_STEP_FUSED && L > 1 && M <= 16 && a->d_split == 0 && a->kernel == MOLE_KERNEL_AUTO && debug_env(nullptr).kernel <= 0 &&
-            cdecode_shape_ok(a->dtype, a->N, a->d) && sm_count(&sms) == MOLE_OK &&
-            cdecode_preferred(M, a->N, sms) && a->tmp && aligned16(a->tmp) && a->out != a->hidden_in && a->tmp != a->hidden_in && a->tmp != a->out)
-            mode = MOLE_STEP_CHAINED;
     }
     if (quant) {
         // quantised tables run layer by layer (one block per token de-quantising inside the weighted sum)

@@ -1,6 +1,4 @@
 // Host side of the tensor-core kernel (mole_mma.cuh): the shapes it covers, a launch's geometry, its tensor maps.
-#include <stdio.h>
-#include <stdlib.h>
 #include <string.h>
 
 #include "mole_mma.cuh"
@@ -12,26 +10,25 @@ constexpr int kSmemBlock = 227 * 1024, kSmemSM = 228 * 1024;
 typedef void (*MmaKernel)(const CUtensorMap, const CUtensorMap, const MmaParams);
 
 template <int N, int CS>
-static MmaKernel pick_mma_tb(int tb, bool norm)
+static MmaKernel pick_mma_norm(bool norm)
 {
-    if (tb == 1) return norm ? mole_mma_kernel<N, 1, 1, CS> : mole_mma_kernel<N, 1, 0, CS>;
-    return norm ? mole_mma_kernel<N, 8, 1, CS> : mole_mma_kernel<N, 8, 0, CS>;
+    return norm ? mole_mma_kernel<N, 1, CS> : mole_mma_kernel<N, 0, CS>;
 }
-static MmaKernel pick_mma(int N, int cs, int tb, bool norm)
+static MmaKernel pick_mma(int N, int cs, bool norm)
 {
     switch (N * 8 + cs) {
-        case 8 * 8 + 1: return pick_mma_tb<8, 1>(tb, norm);
-        case 8 * 8 + 2: return pick_mma_tb<8, 2>(tb, norm);
-        case 16 * 8 + 1: return pick_mma_tb<16, 1>(tb, norm);
-        case 16 * 8 + 2: return pick_mma_tb<16, 2>(tb, norm);
-        case 32 * 8 + 1: return pick_mma_tb<32, 1>(tb, norm);
-        case 32 * 8 + 2: return pick_mma_tb<32, 2>(tb, norm);
-        case 32 * 8 + 4: return pick_mma_tb<32, 4>(tb, norm);
+        case 8 * 8 + 1: return pick_mma_norm<8, 1>(norm);
+        case 8 * 8 + 2: return pick_mma_norm<8, 2>(norm);
+        case 16 * 8 + 1: return pick_mma_norm<16, 1>(norm);
+        case 16 * 8 + 2: return pick_mma_norm<16, 2>(norm);
+        case 32 * 8 + 1: return pick_mma_norm<32, 1>(norm);
+        case 32 * 8 + 2: return pick_mma_norm<32, 2>(norm);
+        case 32 * 8 + 4: return pick_mma_norm<32, 4>(norm);
         default: return nullptr;
     }
 }
 
-static int smem_of(int N, int d, int cs, int tb, int ws, int rs, bool norm) { return static_cast<int>(mma_smem(N, d, cs, tb, ws, rs, norm ? 1 : 0).total); }
+static int smem_of(int N, int d, int cs, int ws, int rs, bool norm) { return static_cast<int>(mma_smem(N, d, cs, ws, rs, norm ? 1 : 0).total); }
 
 // Blocks per token: as few as keep a block's part of a token's rows at 32 KB and its compute warps at eight; 0: not covered.
 static int mma_blocks(int N, int d)
@@ -40,63 +37,69 @@ static int mma_blocks(int N, int d)
         if (d % (kMmaCols * cs) != 0) return 0;
         const int dl = d / cs;
         if (dl > 8 * kMmaCols || N * dl * 2 > 32 * 1024) continue;
-        return pick_mma(N, cs, 1, false) ? cs : 0;
+        return pick_mma(N, cs, false) ? cs : 0;
     }
     return 0;
 }
 
-bool mma_shape_ok(int dtype, int N, int d)
+// Whether a fused step of M tokens runs here.  Up to one block per SM: every shape but d = 768 and 1024 with N = 16, for which
+// the ring kernel is compiled to size (16.4 against 17.8 us for 12 layers of 768).  Up to two blocks per SM: where a block's part
+// is small (N = 8, d = 1024, 250 tokens, 10 layers: 17.0 against 19.5 us; N = 32, d = 512: 27.3 against 22.2) or the rows are so
+// wide that the ring kernel cuts them finely (1B shape, 64 tokens: 44.0 against 55.9).  Beyond that a second wave starts where
+// the ring kernel has the next token's rows in flight already.
+bool mma_preferred(long long M, int dtype, int N, int d, int sms)
 {
-    return dtype == MOLE_DTYPE_BF16 && (N == 8 || N == 16 || N == 32) && d % kMmaCols == 0 && d <= 2048 && mma_blocks(N, d) > 0;
+    if (dtype != MOLE_DTYPE_BF16 || (N != 8 && N != 16 && N != 32) || d % kMmaCols != 0 || d > kMmaMaxSlices * kMmaCols) return false;
+    if (N == 16 && (d == 768 || d == 1024)) return false;
+    const int cs = mma_blocks(N, d);
+    if (!cs) return false;
+    if (M * cs <= sms) return true;
+    return M * cs <= 2LL * sms && (N * (d / cs) * 2 <= 24 * 1024 || N * d * 2 >= 128 * 1024);
 }
 
-int plan_mma(long long M, int L, int N, int d, bool norm, int sms, bool prepare, MmaPlan *w)
+int plan_mma(long long M, int N, int d, bool norm, int sms, bool prepare, MmaPlan *w)
 {
     const int cs = mma_blocks(N, d);
     if (!cs) return MOLE_ERR_UNSUPPORTED_SHAPE;
-    const long long per_sm_tokens = (M * cs + sms - 1) / sms;
-    int tb = per_sm_tokens > 4 ? 8 : 1;
-    if (const char *e = getenv("WTB")) tb = atoi(e);
-    const long long groups = (M + tb - 1) / tb;
-    if (groups > 0x1fffffff) return MOLE_ERR_TOO_LARGE;
-    // blocks per SM aimed at
-    const long long per_sm_blocks = (groups * cs + sms - 1) / sms;
-    int want = static_cast<int>(per_sm_blocks < 1 ? 1 : (per_sm_blocks > (tb == 1 ? 4 : 2) ? (tb == 1 ? 4 : 2) : per_sm_blocks));
-    if (const char *e = getenv("WBPS")) want = atoi(e);
-    int ws = L > 1 ? 2 : 1, rs = 0;
-    for (; want >= 1 && rs == 0; --want) {
-        const int budget = kSmemSM / want - 1024 < kSmemBlock ? kSmemSM / want - 1024 : kSmemBlock;
-        for (ws = L > 1 ? 2 : 1; ws >= 1 && rs == 0; --ws)
-            for (int r = L > 1 || tb > 1 ? kMmaMaxSlots : 2; r >= (L > 1 ? 2 : 1); --r)
-                if (smem_of(N, d, cs, tb, ws, r, norm) <= budget) {
-                    rs = r;
-                    break;
-                }
-        ++ws;
-    }
-    if (rs == 0) return MOLE_ERR_UNSUPPORTED_SHAPE;
-    if (const char *e = getenv("WRS")) rs = atoi(e);
-    if (const char *e = getenv("WWS")) ws = L > 1 ? atoi(e) : 1;
-    w->w_slots = ws;
-    w->r_slots = rs;
-    w->smem = smem_of(N, d, cs, tb, ws, rs, norm);
-    if (w->smem > kSmemBlock) return MOLE_ERR_UNSUPPORTED_SHAPE;
-    const MmaKernel fn = pick_mma(N, cs, tb, norm);
+    const MmaKernel fn = pick_mma(N, cs, norm);
     w->fn = reinterpret_cast<const void *>(fn);
     w->cs = cs;
-    w->tb = tb;
     w->threads = d / cs / 4 + 32;
-    w->groups = static_cast<int>(groups);
-    int per_sm = 1;
-    if (prepare) {
-        int rc = ensure_smem_opt_in(w->fn, w->smem);
-        if (rc != MOLE_OK) return rc;
-        MOLE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, w->threads, w->smem));
-        if (per_sm < 1) per_sm = 1;
+    // one block per SM with deep rings, or two with shallower ones if that is what it takes to have all tokens resident
+    // (clusters do not always fill the last SMs, so the driver is asked)
+    for (int want = 1; want <= 2; ++want) {
+        const int budget = kSmemSM / want - 1024 < kSmemBlock ? kSmemSM / want - 1024 : kSmemBlock;
+        int ws = 2, rs = kMmaMaxSlots;
+        while (rs > 2 && smem_of(N, d, cs, ws, rs, norm) > budget) --rs;
+        if (smem_of(N, d, cs, ws, rs, norm) > budget) ws = 1;
+        if (smem_of(N, d, cs, ws, rs, norm) > budget) {
+            if (want == 1) return MOLE_ERR_UNSUPPORTED_SHAPE;
+            break;
+        }
+        w->w_slots = ws;
+        w->r_slots = rs;
+        w->smem = smem_of(N, d, cs, ws, rs, norm);
+        long long resident = static_cast<long long>(want) * sms / cs;
+        if (prepare) {
+            int rc = ensure_smem_opt_in(w->fn, w->smem);
+            if (rc != MOLE_OK) return rc;
+            cudaLaunchConfig_t cfg;
+            memset(&cfg, 0, sizeof cfg);
+            cfg.gridDim = dim3(static_cast<unsigned>(cs), 1, 1);
+            cfg.blockDim = dim3(static_cast<unsigned>(w->threads), 1, 1);
+            cfg.dynamicSmemBytes = w->smem;
+            int n = 0;
+            if (cs > 1) {
+                MOLE_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, w->fn, &cfg));
+            } else {
+                MOLE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, w->threads, w->smem));
+                n *= sms;
+            }
+            resident = n > 0 ? n : 1;
+        }
+        w->grid = static_cast<int>(M < resident ? M : resident) * cs;
+        if (M <= resident) break;
     }
-    const long long resident = static_cast<long long>(per_sm) * sms / cs;
-    w->grid = static_cast<int>(groups < resident ? groups : resident) * cs;
-    if (getenv("WDBG")) fprintf(stderr, "mma M %lld L %d N %d d %d: cs %d tb %d ws %d rs %d smem %d per_sm %d grid %d\n", M, L, N, d, cs, tb, ws, rs, w->smem, per_sm, w->grid);
     return MOLE_OK;
 }
 
@@ -156,6 +159,7 @@ static const CUtensorMap *map_for(const MapKey &k)
     return &e.map;
 }
 
+// (a fused step has neither gates to write nor a residual of its own)
 int launch_mma(const StepLaunch &a, const MmaPlan &w, uint32_t wait_polls, bool *taken)
 {
     *taken = false;
@@ -169,18 +173,15 @@ int launch_mma(const StepLaunch &a, const MmaPlan &w, uint32_t wait_polls, bool 
     *taken = true;
     MmaParams p;
     p.hidden = a.hidden;
-    p.residual = a.residual;
     p.row_index = a.row_index;
     p.norm_weight = a.norm_weight;
     p.out = a.out;
-    p.gates_out = a.gates_out;
     p.status = a.status;
     p.norm_stride = a.norm_stride;
     p.M = a.M;
     p.rows = a.rows;
     p.d = a.d;
     p.L = a.L;
-    p.groups = w.groups;
     p.w_slots = w.w_slots;
     p.r_slots = w.r_slots;
     p.norm_eps = a.norm_eps;

@@ -1,27 +1,28 @@
-// The tensor-core form of the fused MoLE layer and of the fused L-layer step for sm_100a (Eq. 4 and Eq. 8 of arXiv
-// 2503.15798): bf16, N of 8, 16 or 32 experts, d a multiple of 128.
+// The tensor-core form of the fused L-layer step for sm_100a (Eq. 8 of arXiv 2503.15798 applied layer after layer): one launch,
+// bf16, N of 8, 16 or 32 experts, d a multiple of 128, a token per block or per cluster of blocks.
 //
-// What bounds the layer.  At decode sizes one token's layer is a dependent chain -- router product, a sum over the block, a
-// softmax, a weighted sum -- and with one token per SM each link costs its latency plus its instructions; at prefill sizes it is
-// instructions and the shared-memory port.  On CUDA cores the weighted sum alone is three instructions per two elements (two
-// unpacks and half a packed fma each): clock stamps gave 930 of 2 450 cycles per layer of the 410M shape to it and 700 to
-// the router sweep.  Both are products with a small matrix, so both run on mma.m16n8k16 here:
-//   - Router: A = W_r^T (16 experts x 16 columns per step), B = the hidden state of 1 .. 8 tokens: bf16 products, fp32 sums.
+// What bounds a step.  One token's layer is a dependent chain -- router product, a sum over the block, a softmax, a weighted sum --
+// and with one token per SM each link costs its latency plus its instructions.  On CUDA cores the weighted sum alone is three
+// instructions per two elements (two unpacks and half a packed fma each).  Both products are with a small matrix, so both run on
+// mma.m16n8k16 here:
+//   - Router: A = W_r^T (16 experts x 16 columns per step), B = the hidden state: bf16 products, fp32 sums.
 //   - Weighted sum: A = rows^T (16 columns x 16 experts), B = the softmax numerators.  A numerator is an fp32 number and is
 //     never rounded: it is cut into three bf16 parts of 8 bits each (exactly), and the three products are chained into one
 //     fp32 accumulator.  The sum of the numerators is the same product with A = ones.
 // Split.  Warp w owns the 128 columns 128w .. of everything: of the hidden state, of every row, of the output, and those
 // columns are also its share of the router product.  So what a layer's router needs from the layer before is what the same
 // warp has just computed, and warps exchange nothing but N partial logits per token: one meeting per layer.  (RMSNorm in front
-// of the router adds one for the sum of squares.)  Where a token's rows exceed 64 KB a cluster of CS blocks shares the token;
+// of the router adds one for the sum of squares.)  Where a token's rows exceed 32 KB a cluster of CS blocks shares the token;
 // the partial logits then travel through distributed shared memory (st.async) and the meeting is an mbarrier.
 // Data.  One producer warp streams router matrices and rows, whole boxes by tensor copy with the 128-byte swizzle, so that
 // ldmatrix reads either without bank conflicts; a warp loads the next layer's router fragments and its rows while it waits for
-// the logits of the others.  A single layer keeps its router in registers.
-// Groups.  TB = 1 for decode batches: a block per token, every warp forms the softmax itself.  TB = 8 for many tokens: one
-// router product for eight tokens, the softmaxes dealt out over the warps (a second meeting per group).
-// The order of every sum is fixed by N and d: a token gets the same bits with any TB, in any batch, in a single layer and in a
-// fused step.
+// the logits of the others.
+// Measured against the ring kernel, us per step: 16 layers of the 1B shape, 16 tokens 55.2 -> 28.6 (46.4 for chained launches of
+// the cluster kernel), 64 tokens 55.9 -> 44.0; 10 layers of N = 8, d = 1024, 40 tokens 17.8 -> 12.7; N = 32, d = 1024
+// 27.3 -> 18.7; N = 16, d = 384 with the norm 26.0 -> 19.7.  At d = 768 and 1024 with N = 16, for which the ring kernel is compiled to size,
+// there is nothing in it (17.8 against 16.4 for 12 layers of 768): clock stamps give 1 300 cycles per layer to the chain itself
+// and the rest to the shared-memory port, through which matrix and rows pass twice.
+// The order of every sum is fixed by N and d: a token gets the same bits in any batch.
 #pragma once
 
 #include <cuda.h>
@@ -31,43 +32,38 @@
 namespace mole {
 
 constexpr int kMmaCols = 128;      // columns of a warp
-constexpr int kMmaHidStride = 272; // bytes between two tokens' hidden slices: 256 + 16, eight rows of an ldmatrix on different banks
 constexpr int kMmaMaxSlots = 8;
-constexpr int kMmaMaxSlices = 32;
+constexpr int kMmaMaxSlices = 16;  // of a token: d <= 2048
 
 struct MmaParams {
-    const void *hidden, *residual, *row_index, *norm_weight;
+    const void *hidden, *row_index, *norm_weight;
     void *out;
-    float *gates_out;
     uint32_t *status;
     long long norm_stride;  // bytes between the scale vectors of consecutive layers
     long long M, rows;
     int d, L;
-    int groups;             // groups of TB tokens
     int w_slots, r_slots;   // router matrices and token rows in flight
     float norm_eps;
     uint32_t flags, wait_polls;
 };
 
-// Shared memory of a block: router matrices, rows, hidden slices (two sets with TB > 1), normalised slices, partial logits of
-// the whole token (two sets), split numerators, sums of squares (two sets), per-slot flags, barriers.
+// Shared memory of a block: router matrices, rows, hidden slices, normalised slices, partial logits of the whole token (two
+// sets), sums of squares (two sets), per-slot flags, barriers.
 struct MmaSmem {
     uint32_t matrix;  // bytes of this block's part of a router matrix = of a token's rows
-    uint32_t off_r, off_hid, off_norm, off_partial, off_gates, off_ssq, off_meta, off_bars, total;
+    uint32_t off_r, off_hid, off_norm, off_partial, off_ssq, off_meta, off_bars, total;
 };
-__host__ __device__ inline uint32_t mma_gate_bytes(int N) { return static_cast<uint32_t>(3 * N * 2 + 16); }
-__host__ __device__ inline MmaSmem mma_smem(int N, int d, int cs, int TB, int w_slots, int r_slots, int norm)
+__host__ __device__ inline MmaSmem mma_smem(int N, int d, int cs, int w_slots, int r_slots, int norm)
 {
     MmaSmem m;
-    const int dl = d / cs, nw = dl / kMmaCols, slices = d / kMmaCols;
+    const int dl = d / cs, slices = d / kMmaCols;
     m.matrix = static_cast<uint32_t>(N) * dl * 2;
     m.off_r = static_cast<uint32_t>(w_slots) * m.matrix;
     m.off_hid = m.off_r + static_cast<uint32_t>(r_slots) * m.matrix;
-    m.off_norm = m.off_hid + static_cast<uint32_t>((TB > 1 ? 2 : 1) * nw * TB * kMmaHidStride);
-    m.off_partial = m.off_norm + (norm ? static_cast<uint32_t>(nw * TB * kMmaHidStride) : 0u);
-    m.off_gates = m.off_partial + static_cast<uint32_t>(2 * TB * slices * N * 4);
-    m.off_ssq = m.off_gates + (TB > 1 ? static_cast<uint32_t>(TB) * mma_gate_bytes(N) : 0u);
-    m.off_meta = m.off_ssq + (norm ? static_cast<uint32_t>(2 * TB * slices * 4) : 0u);
+    m.off_norm = m.off_hid + static_cast<uint32_t>(dl * 2);
+    m.off_partial = m.off_norm + (norm ? static_cast<uint32_t>(dl * 2) : 0u);
+    m.off_ssq = m.off_partial + static_cast<uint32_t>(2 * slices * N * 4);
+    m.off_meta = m.off_ssq + (norm ? static_cast<uint32_t>(2 * slices * 4) : 0u);
     m.off_bars = (m.off_meta + (kMmaMaxSlots + 3) * 4 + 7u) & ~7u;
     m.total = m.off_bars + (4 * kMmaMaxSlots + 4) * 8;
     return m;
@@ -285,9 +281,9 @@ __device__ __forceinline__ float softmax_part(float z, int group)
     return expf(z - shift);
 }
 
-// N: experts.  TB: tokens per group (1 or 8).  NORM: the router reads RMSNorm(hidden).  CS: blocks per token.
+// N: experts.  NORM: the router reads RMSNorm(hidden).  CS: blocks per token.
 // Launch: d / CS / 4 + 32 threads, mma_smem(..).total bytes, a multiple of CS blocks.
-template <int N, int TB, int NORM, int CS>
+template <int N, int NORM, int CS>
 __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 32 ? 1 : 2)
     mole_mma_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap r_map, const MmaParams p)
 {
@@ -299,16 +295,15 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 3
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = static_cast<int>(blockDim.x >> 5) - 1;
     const int d = p.d, L = p.L, WS = p.w_slots, RS = p.r_slots, slices = nw * CS;
     const uint32_t rank = CS > 1 ? cluster_ctarank() : 0u;
-    const MmaSmem m = mma_smem(N, d, CS, TB, WS, RS, NORM);
+    const MmaSmem m = mma_smem(N, d, CS, WS, RS, NORM);
     const uint32_t base = smem_u32(smem);
     volatile int *meta = reinterpret_cast<volatile int *>(smem + m.off_meta);  // [r_slots] the slot's id is inside the table
     volatile int *dead = meta + kMmaMaxSlots;                                  // somebody gave up waiting
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + m.off_bars);
     uint64_t *wfull = bars, *wempty = bars + kMmaMaxSlots, *rfull = bars + 2 * kMmaMaxSlots, *rempty = bars + 3 * kMmaMaxSlots;
     uint64_t *xbar = bars + 4 * kMmaMaxSlots, *sbar = xbar + 2;  // the cluster's exchanges: logits, sums of squares
-    const int G = static_cast<int>(gridDim.x) / CS, g0 = static_cast<int>(blockIdx.x) / CS;
-    const int ng = (p.groups - g0 + G - 1) / G;  // groups of this block: g0, g0 + G, ...
-    auto token_of = [&](int gi, int tok) -> long long { return (static_cast<long long>(g0) + static_cast<long long>(gi) * G) * TB + tok; };
+    const long long G = gridDim.x / CS, t0 = blockIdx.x / CS;    // this block's tokens: t0, t0 + G, ...
+    const int ntok = t0 < p.M ? static_cast<int>((p.M - t0 + G - 1) / G) : 0;
 
     if (tid == 0) {
         for (int s = 0; s < WS; ++s) {
@@ -328,19 +323,19 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 3
     if constexpr (CS > 1) cluster_arrive();  // waited for before the first push
 
     if (warp == nw) {
-        // ================= producer warp: copies in the order they are consumed -- the first router matrix, then per (group,
-        // layer) the rows of the first token, the router matrix of the item after, the rows of the other tokens =================
+        // ================= producer warp: copies in the order they are consumed -- the first router matrix, then per item
+        // (token, layer) its rows and the router matrix of the item after =================
         const bool ids64 = (p.flags & MOLE_FLAG_IDS_INT64) != 0;
         auto load_ids = [&](int window) -> long long {  // ids of 32 consecutive tokens of this block, one per lane; -1: none
             const int n = window * 32 + lane;
-            const long long t = token_of(n / TB, n % TB);
-            if (n / TB >= ng || t >= p.M) return -1;
+            if (n >= ntok) return -1;
+            const long long t = t0 + static_cast<long long>(n) * G;
             return ids64 ? __ldg(static_cast<const long long *>(p.row_index) + t) : static_cast<long long>(__ldg(static_cast<const int *>(p.row_index) + t));
         };
         int ws = 0, rs = 0, issued_w = 0, issued_r = 0, w_layer = 0;
         uint32_t wph = 1, rph = 1;  // parity of the `empty` phase that frees the slot
         bool ok = true;
-        const int matrices = ng > 0 ? (L > 1 ? ng * L : 1) : 0;
+        const int items = ntok * L;
         const int w_rows = nw * (2 * N);  // 128-byte rows of this block's part of a router matrix
         const int w_box = w_rows <= 256 ? w_rows : w_rows / 2;
         auto wait_slot = [&](uint64_t *bar, uint32_t parity) {
@@ -352,7 +347,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 3
             ok = __shfl_sync(0xffffffffu, got, 0) != 0;
         };
         auto issue_router = [&]() {
-            if (issued_w >= matrices) return;
+            if (issued_w >= items) return;
             if (issued_w >= WS) wait_slot(wempty + ws, wph);
             if (!ok) return;
             if (lane == 0) {
@@ -367,36 +362,30 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 3
         issue_router();
         long long id_now = load_ids(0), id_next = load_ids(1);
 #pragma unroll 1
-        for (int gi = 0; gi < ng && ok; ++gi) {
+        for (int k = 0; k < ntok && ok; ++k) {
+            if ((k & 31) == 0 && k > 0) {
+                id_now = id_next;
+                id_next = load_ids((k >> 5) + 1);
+            }
+            const long long id = __shfl_sync(0xffffffffu, id_now, k & 31);
+            const bool valid = id >= 0 && id < p.rows;
+            if (!valid && lane == 0 && rank == 0 && p.status) atomicOr(p.status, MOLE_STATUS_BAD_ID);
 #pragma unroll 1
             for (int l = 0; l < L && ok; ++l) {
-#pragma unroll 1
-                for (int k = 0; k < TB; ++k) {
-                    if (k == 1) issue_router();
-                    const int n = gi * TB + k;
-                    if (l == 0 && (n & 31) == 0 && n > 0) {
-                        id_now = id_next;
-                        id_next = load_ids((n >> 5) + 1);
+                if (issued_r >= RS) wait_slot(rempty + rs, rph);
+                if (!ok) break;
+                if (lane == 0) {
+                    meta[rs] = valid ? 1 : 0;
+                    if (valid) {
+                        mbar_expect_tx(rfull + rs, m.matrix);
+                        tensor_load_5d(base + m.off_r + static_cast<uint32_t>(rs) * m.matrix, &r_map, 0, 0, static_cast<int>(rank) * nw * 2, static_cast<int>(id), l, rfull + rs);
+                    } else {
+                        mbar_arrive(rfull + rs);  // nothing to copy: the routed term is dropped
                     }
-                    const long long id = __shfl_sync(0xffffffffu, id_now, n & 31);
-                    const bool valid = id >= 0 && id < p.rows;
-                    if (!ok) break;
-                    if (issued_r >= RS) wait_slot(rempty + rs, rph);
-                    if (!ok) break;
-                    if (lane == 0) {
-                        meta[rs] = valid ? 1 : 0;
-                        if (valid) {
-                            mbar_expect_tx(rfull + rs, m.matrix);
-                            tensor_load_5d(base + m.off_r + static_cast<uint32_t>(rs) * m.matrix, &r_map, 0, 0, static_cast<int>(rank) * nw * 2, static_cast<int>(id), l, rfull + rs);
-                        } else {
-                            mbar_arrive(rfull + rs);  // nothing to copy: the routed term is dropped
-                            if (l == 0 && rank == 0 && p.status && token_of(gi, k) < p.M) atomicOr(p.status, MOLE_STATUS_BAD_ID);
-                        }
-                    }
-                    ++issued_r;
-                    if (++rs == RS) rs = 0, rph ^= 1u;
                 }
-                if (TB == 1 && ok) issue_router();
+                ++issued_r;
+                if (++rs == RS) rs = 0, rph ^= 1u;
+                issue_router();
             }
         }
         if (!ok) {
@@ -411,12 +400,11 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 3
         const int nc = nw * 32;
         const int slice = static_cast<int>(rank) * nw + warp;  // of the whole token
         const int r8 = lane >> 2, q = lane & 3;
-        const uint32_t hid_set = static_cast<uint32_t>(nw * TB * kMmaHidStride);
-        const uint32_t hid0 = base + m.off_hid + static_cast<uint32_t>(warp * TB * kMmaHidStride);
-        const uint32_t norm0 = base + m.off_norm + static_cast<uint32_t>(warp * TB * kMmaHidStride);
-        const uint32_t frag_off = static_cast<uint32_t>((TB > 1 ? (lane & 7) * kMmaHidStride : 0) + (lane >> 3) * 16);
+        const uint32_t hid = base + m.off_hid + static_cast<uint32_t>(warp) * (kMmaCols * 2);
+        const uint32_t router_in = (NORM ? base + m.off_norm + static_cast<uint32_t>(warp) * (kMmaCols * 2) : hid);
         const uint32_t own_off = static_cast<uint32_t>(2 * (16 * q + r8));  // this lane's columns: + 0, 16, 128, 144 bytes
-        const uint32_t part_set = static_cast<uint32_t>(TB * slices * N * 4);
+        auto col = [](int i) -> uint32_t { return static_cast<uint32_t>((i >> 1) * 128 + (i & 1) * 16); };
+        const uint32_t part_set = static_cast<uint32_t>(slices * N * 4);
         const uint32_t w_off = static_cast<uint32_t>(warp) * (256u * N);
         const uint32_t r_off = m.off_r + static_cast<uint32_t>(warp) * (256u * N) + RowsA<N>::lane_offset(lane);
         const size_t slice_bytes = static_cast<size_t>(slice) * (kMmaCols * 2);
@@ -444,230 +432,127 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 3
             acquire(wfull + ws, wph);
             wf.load(base + static_cast<uint32_t>(ws) * m.matrix + w_off);
         };
-        auto release_router = [&]() {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(wempty + ws);
-            if (++ws == WS) ws = 0, wph ^= 1u;
-        };
-        auto release_rows = [&]() {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(rempty + rs);
-            if (++rs == RS) rs = 0, rph ^= 1u;
-        };
-        if (ng > 0) load_router();
+        if (ntok > 0) load_router();
         if constexpr (CS > 1) cluster_wait();
 
         pdl_wait();
-        fence_proxy_async_global();
 
         const unsigned char *hid_g = static_cast<const unsigned char *>(p.hidden) + slice_bytes + (lane & 15) * 16;
         const unsigned char *norm_g = static_cast<const unsigned char *>(p.norm_weight) + slice_bytes + own_off;
-        unsigned short nw_next[4] = {0, 0, 0, 0};
+        float wgt_next[4] = {0.f, 0.f, 0.f, 0.f};
         auto load_norm = [&](int l) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) nw_next[i] = __ldg(reinterpret_cast<const unsigned short *>(norm_g + static_cast<size_t>(l) * p.norm_stride + (i >> 1) * 128 + (i & 1) * 16));
+            for (int i = 0; i < 4; ++i) wgt_next[i] = bf16_bits_to_float(__ldg(reinterpret_cast<const unsigned short *>(norm_g + static_cast<size_t>(l) * p.norm_stride + col(i))));
         };
-        // hidden slices of group gi into set s
-        auto fetch_hidden = [&](int gi, int s) {
-            if (gi < ng) {
-#pragma unroll
-                for (int kk = 0; kk < (TB + 1) / 2; ++kk) {
-                    const int k = 2 * kk + (lane >> 4);
-                    if (k >= TB) break;
-                    long long t = token_of(gi, k);
-                    if (t >= p.M) t = p.M - 1;  // rows past the last token repeat it; nothing of them is used
-                    cp_async16(hid0 + static_cast<uint32_t>(s) * hid_set + static_cast<uint32_t>(k * kMmaHidStride + (lane & 15) * 16), hid_g + static_cast<size_t>(t) * d * 2);
-                }
-            }
+        auto fetch_hidden = [&](int k) {
+            if (k < ntok && lane < 16) cp_async16(hid + lane * 16, hid_g + static_cast<size_t>(t0 + static_cast<long long>(k) * G) * d * 2);
             cp_async_commit();
         };
-        fetch_hidden(0, 0);
+        fetch_hidden(0);
         if constexpr (NORM) load_norm(0);
 
-        uint32_t buf = 0, xph = 0, hs = 0;  // exchange buffer, its barrier's parity; hidden set
+        uint32_t buf = 0, xph = 0;  // exchange buffer, its barrier's parity
 #pragma unroll 1
-        for (int gi = 0; gi < ng; ++gi) {
+        for (int k = 0; k < ntok; ++k) {
             cp_async_wait_all();
             __syncwarp();
-            const uint32_t hid = hid0 + hs * hid_set;
-            if constexpr (TB > 1) fetch_hidden(gi + 1, static_cast<int>(hs ^ 1u));
+            float h[4];  // this lane's columns of the running hidden state
+#pragma unroll
+            for (int i = 0; i < 4; ++i) h[i] = bf16_bits_to_float(lds16(hid + own_off + col(i)));
 #pragma unroll 1
             for (int l = 0; l < L; ++l) {
                 const bool last = l == L - 1;
                 if (CS > 1 && tid == 0) {
                     mbar_expect_tx(xbar + buf, part_set);
-                    if (NORM) mbar_expect_tx(sbar + buf, static_cast<uint32_t>(TB * slices * 4));
+                    if (NORM) mbar_expect_tx(sbar + buf, static_cast<uint32_t>(slices * 4));
                 }
-                // ---- what the router reads ----
-                uint32_t router_in = hid;
                 if constexpr (NORM) {
-                    router_in = norm0;
-                    const uint32_t sq = base + m.off_ssq + buf * static_cast<uint32_t>(TB * slices * 4);
-                    float wgt[4], ss[TB];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) wgt[i] = bf16_bits_to_float(nw_next[i]);
-                    if (L > 1) load_norm(last ? 0 : l + 1);
-#pragma unroll
-                    for (int k = 0; k < TB; ++k) {
-                        float s = 0.f;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const float x = bf16_bits_to_float(lds16(hid + own_off + static_cast<uint32_t>(k * kMmaHidStride + (i >> 1) * 128 + (i & 1) * 16)));
-                            s = fmaf(x, x, s);
-                        }
-                        ss[k] = s;
-                    }
-                    int first = 0;
-                    if constexpr (TB > 1) lane_reduce_scatter<TB, TB, 16, 1>(ss, lane, first);
-                    else ss[0] = warp_sum(ss[0]);
-                    if ((lane & (TB > 1 ? 3 : 31)) == 0) {
-                        const uint32_t at = sq + static_cast<uint32_t>(first * slices + slice) * 4u;
-                        if constexpr (CS == 1) stsf(at, ss[0]);
-                        else
-#pragma unroll
-                            for (int c = 0; c < CS; ++c) cluster_push_f32(cluster_map(at, c), ss[0], cluster_map(smem_u32(sbar + buf), c));
+                    // y = (x / sqrt(mean(x^2) + eps)) * w, rounded once to bf16: what the router reads
+                    const uint32_t sq = base + m.off_ssq + buf * static_cast<uint32_t>(slices * 4);
+                    const float ss = warp_sum(fmaf(h[3], h[3], fmaf(h[2], h[2], fmaf(h[1], h[1], h[0] * h[0]))));
+                    if (lane < CS) {
+                        const uint32_t at = sq + static_cast<uint32_t>(slice) * 4u;
+                        if constexpr (CS == 1) stsf(at, ss);
+                        else cluster_push_f32(cluster_map(at, lane), ss, cluster_map(smem_u32(sbar + buf), lane));
                     }
                     if constexpr (CS == 1) named_bar_sync(3, nc);
                     else acquire_cluster(sbar + buf, xph);
-                    float total = 0.f;
-                    for (int w = 0; w < slices; ++w) total += ldsf(sq + static_cast<uint32_t>((lane & (TB - 1)) * slices + w) * 4u);  // slices in ascending order
+                    float v[kMmaMaxSlices], total = 0.f;
+#pragma unroll
+                    for (int w = 0; w < kMmaMaxSlices; ++w) v[w] = w < slices ? ldsf(sq + static_cast<uint32_t>(w) * 4u) : 0.f;
+#pragma unroll
+                    for (int w = 0; w < kMmaMaxSlices; ++w) total += v[w];  // slices in ascending order
                     const float rinv = rms_scale(total, d, p.norm_eps);
 #pragma unroll
-                    for (int k = 0; k < TB; ++k) {
-                        const float r = TB > 1 ? __shfl_sync(0xffffffffu, rinv, k) : rinv;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const uint32_t o = own_off + static_cast<uint32_t>(k * kMmaHidStride + (i >> 1) * 128 + (i & 1) * 16);
-                            sts16(norm0 + o, float_to_bf16_bits((bf16_bits_to_float(lds16(hid + o)) * r) * wgt[i]));
-                        }
-                    }
+                    for (int i = 0; i < 4; ++i) sts16(router_in + own_off + col(i), float_to_bf16_bits((h[i] * rinv) * wgt_next[i]));
+                    load_norm(last ? 0 : l + 1);
                     __syncwarp();
                 }
 
-                // ---- router: this warp's partial logits: lane (r, q): experts r, r + 8 of tokens 2q, 2q + 1 ----
+                // ---- router: this warp's partial logits: lane 4 r holds experts r, r + 8 ----
                 float z[ET][4];
-                wf.product(router_in + frag_off, z);
+                wf.product(router_in + static_cast<uint32_t>(lane >> 3) * 16u, z);
                 const uint32_t part = base + m.off_partial + buf * part_set;
+                if (q == 0) {
 #pragma unroll
-                for (int e = 0; e < ET; ++e)
+                    for (int e = 0; e < ET; ++e)
 #pragma unroll
-                    for (int i = 0; i < (N == 8 ? 2 : 4); ++i) {
-                        const int tok = TB > 1 ? 2 * q + (i & 1) : 0;
-                        const uint32_t at = part + static_cast<uint32_t>((tok * slices + slice) * N + 16 * e + r8 + 8 * (i >> 1)) * 4u;
-                        if (TB > 1 || (q == 0 && (i & 1) == 0)) {
-                            if constexpr (CS == 1) stsf(at, z[e][i]);
+                        for (int i = 0; i < (N == 8 ? 1 : 2); ++i) {
+                            const uint32_t at = part + static_cast<uint32_t>(slice * N + 16 * e + r8 + 8 * i) * 4u;
+                            if constexpr (CS == 1) stsf(at, z[e][2 * i]);
                             else
 #pragma unroll
-                                for (int c = 0; c < CS; ++c) cluster_push_f32(cluster_map(at, c), z[e][i], cluster_map(smem_u32(xbar + buf), c));
+                                for (int c = 0; c < CS; ++c) cluster_push_f32(cluster_map(at, c), z[e][2 * i], cluster_map(smem_u32(xbar + buf), c));
                         }
-                    }
-                if (L > 1) release_router();
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(wempty + ws);  // the matrix has been multiplied: its slot goes back
+                if (++ws == WS) ws = 0, wph ^= 1u;
                 if constexpr (CS == 1) named_bar_arrive(1, 2 * nc);
-                // under the others' products: the first token's rows, the next router matrix
+                // under the others' products: this token's rows, the next router matrix
                 acquire(rfull + rs, rph);
-                bool valid = meta[rs] != 0;
+                const bool valid = meta[rs] != 0;
                 RowsA<N> rows;
                 rows.load(base + static_cast<uint32_t>(rs) * m.matrix + r_off);
-                if (L > 1 && !(last && gi + 1 == ng)) load_router();
+                if (!(last && k + 1 == ntok)) load_router();
                 if constexpr (CS == 1) named_bar_sync(1, 2 * nc);
                 else acquire_cluster(xbar + buf, xph);
 
-                // ---- softmax numerators (Eq. 4): even slices and odd slices, then the two ----
-                auto numerator_of = [&](int tok) -> float {
-                    const uint32_t z_in = part + static_cast<uint32_t>(tok * slices * N + (lane & (N - 1))) * 4u;
-                    float ze = 0.f, zo = 0.f;
-#pragma unroll 4
-                    for (int w = 0; w + 1 < slices; w += 2) {
-                        ze += ldsf(z_in + static_cast<uint32_t>(w * N) * 4u);
-                        zo += ldsf(z_in + static_cast<uint32_t>((w + 1) * N) * 4u);
-                    }
-                    if (slices & 1) ze += ldsf(z_in + static_cast<uint32_t>((slices - 1) * N) * 4u);
-                    return softmax_part(ze + zo, N);
-                };
-                GateB<N> g;
-                float inv = 0.f;
-                if constexpr (TB == 1) {
-                    const float e = numerator_of(0);
-                    g.from_lanes(e, lane);
-                    const float esum = g.sum();
-                    inv = __frcp_rn(esum);
-                    if (p.gates_out && slice == 0 && lane < N) p.gates_out[token_of(gi, 0) * N + lane] = e / esum;
-                } else {
-                    for (int tok = warp; tok < TB; tok += nw) {
-                        const uint32_t gs = base + m.off_gates + static_cast<uint32_t>(tok) * mma_gate_bytes(N);
-                        const float e = numerator_of(tok);
-                        g.from_lanes(e, lane);
-                        const float esum = g.sum();
-                        if (lane < 4) {
+                // ---- softmax numerators (Eq. 4), by every warp for itself: even slices and odd slices, then the two ----
+                float e;
+                {
+                    const uint32_t z_in = part + static_cast<uint32_t>(lane & (N - 1)) * 4u;
+                    float v[kMmaMaxSlices], ze = 0.f, zo = 0.f;
 #pragma unroll
-                            for (int pt = 0; pt < 3; ++pt)
+                    for (int w = 0; w < kMmaMaxSlices; ++w) v[w] = w < slices ? ldsf(z_in + static_cast<uint32_t>(w * N) * 4u) : 0.f;
 #pragma unroll
-                                for (int k = 0; k < GateB<N>::KS; ++k)
-#pragma unroll
-                                    for (int w = 0; w < GateB<N>::W; ++w) sts32(gs + static_cast<uint32_t>(pt * N + 16 * k + 8 * w + 2 * lane) * 2u, g.part[pt][k][w]);
-                        }
-                        if (lane == 0) stsf(gs + 3 * N * 2, __frcp_rn(esum));
-                        const long long t = token_of(gi, tok);
-                        if (p.gates_out && rank == 0 && t < p.M && lane < N) p.gates_out[t * N + lane] = e / esum;
-                    }
-                    named_bar_sync(2, nc);
+                    for (int w = 0; w < kMmaMaxSlices; w += 2) ze += v[w], zo += v[w + 1];
+                    e = softmax_part(ze + zo, N);
                 }
+                GateB<N> g;
+                g.from_lanes(e, lane);
+                const float inv = __frcp_rn(g.sum());
 
                 // ---- weighted sum of the rows (Eq. 8), residual, one rounding ----
-#pragma unroll 1
-                for (int k = 0; k < TB; ++k) {
-                    if constexpr (TB > 1) {
-                        if (k > 0) {
-                            acquire(rfull + rs, rph);
-                            valid = meta[rs] != 0;
-                            rows.load(base + static_cast<uint32_t>(rs) * m.matrix + r_off);
-                        }
-                        const uint32_t gs = base + m.off_gates + static_cast<uint32_t>(k) * mma_gate_bytes(N);
+                float v[4];
+                rows.product(g, lane, v);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(rempty + rs);
+                if (++rs == RS) rs = 0, rph ^= 1u;
 #pragma unroll
-                        for (int pt = 0; pt < 3; ++pt)
-#pragma unroll
-                            for (int kk = 0; kk < GateB<N>::KS; ++kk)
-#pragma unroll
-                                for (int w = 0; w < GateB<N>::W; ++w) g.part[pt][kk][w] = lds32(gs + static_cast<uint32_t>(pt * N + 16 * kk + 8 * w + 2 * q) * 2u);
-                        inv = ldsf(gs + 3 * N * 2);
-                    }
-                    float v[4];
-                    rows.product(g, lane, v);
-                    release_rows();
-                    const uint32_t own = hid + own_off + static_cast<uint32_t>(k * kMmaHidStride);
-                    uint32_t res[4];
-                    if (p.residual && last) {
-                        const long long t = token_of(gi, k);
-                        const unsigned char *src = static_cast<const unsigned char *>(p.residual) + static_cast<size_t>(t < p.M ? t : p.M - 1) * d * 2 + slice_bytes + own_off;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) res[i] = ldcg_u16(src + (i >> 1) * 128 + (i & 1) * 16);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) res[i] = lds16(own + static_cast<uint32_t>((i >> 1) * 128 + (i & 1) * 16));
-                    }
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        sts16(own + static_cast<uint32_t>((i >> 1) * 128 + (i & 1) * 16),
-                              valid ? float_to_bf16_bits(fmaf(v[i], inv, bf16_bits_to_float(res[i]))) : static_cast<unsigned short>(res[i]));
+                for (int i = 0; i < 4; ++i) {
+                    const unsigned short o = float_to_bf16_bits(valid ? fmaf(v[i], inv, h[i]) : h[i]);
+                    h[i] = bf16_bits_to_float(o);
+                    if (!NORM || last) sts16(hid + own_off + col(i), o);
                 }
                 __syncwarp();
                 buf ^= 1u;
                 if (buf == 0) xph ^= 1u;
             }
-            // ---- the group's outputs ----
-            {
-                unsigned char *out = static_cast<unsigned char *>(p.out) + slice_bytes + (lane & 15) * 16;
-#pragma unroll
-                for (int kk = 0; kk < (TB + 1) / 2; ++kk) {
-                    const int k = 2 * kk + (lane >> 4);
-                    if (k >= TB) break;
-                    const long long t = token_of(gi, k);
-                    if (t < p.M) *reinterpret_cast<uint4 *>(out + static_cast<size_t>(t) * d * 2) = lds128(hid + static_cast<uint32_t>(k * kMmaHidStride + (lane & 15) * 16));
-                }
-            }
+            if (lane < 16)
+                *reinterpret_cast<uint4 *>(static_cast<unsigned char *>(p.out) + static_cast<size_t>(t0 + static_cast<long long>(k) * G) * d * 2 + slice_bytes + lane * 16) = lds128(hid + lane * 16);
             __syncwarp();
-            if constexpr (TB > 1) hs ^= 1u;
-            else fetch_hidden(gi + 1, 0);
+            fetch_hidden(k + 1);
         }
     }
     if constexpr (CS > 1) {  // pushes to this block may still be on their way: nobody leaves before everybody is done

@@ -1,0 +1,93 @@
+"""The tensor-core step kernel (the library's choice for fused steps of one or two blocks per SM) against the oracle's
+chain: one, two and four blocks per token, one to eight warps, every expert count, tokens at and beyond one block per
+SM, RMSNorm, ids outside the table, output in place; and its bounded waits."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import as_f64, rand_case
+from paper_2503_15798_b200 import binding as mole
+from test_gpu_variants import _oracle_chain
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+# N, d, M, L
+CASES = [(8, 128, 1, 3), (8, 256, 290, 2), (8, 1024, 37, 3), (8, 2048, 74, 2), (8, 2048, 5, 4), (16, 128, 148, 3), (16, 640, 9, 5), (16, 1280, 74, 2),
+         (16, 2048, 3, 3), (32, 128, 64, 2), (32, 512, 148, 2), (32, 768, 20, 3), (32, 1024, 74, 2), (32, 1536, 11, 3), (32, 2048, 1, 4), (32, 2048, 30, 2),
+         (32, 2048, 60, 2)]
+
+
+@pytest.mark.parametrize("N,d,M,L", CASES)
+@pytest.mark.parametrize("norm", [False, True])
+def test_fused_step_against_the_oracles_chain(N, d, M, L, norm):
+    V = 83
+    g = torch.Generator().manual_seed(N * d + M + L)
+    luts = torch.empty(L, V, N, d).normal_(0, 0.05, generator=g).to(torch.bfloat16)
+    wrs = torch.empty(L, d, N).normal_(0, 0.02, generator=g).to(torch.bfloat16)
+    hidden = (1.5 * torch.empty(M, d).normal_(0, 1, generator=g)).to(torch.bfloat16)
+    ids = torch.randint(0, V, (M,), generator=g, dtype=torch.int32)
+    if M > 1:
+        ids[M - 1] = V  # outside the table: its routed term is dropped in every layer
+    gammas = (1.0 + 0.2 * torch.empty(L, d).normal_(0, 1, generator=g)).to(torch.bfloat16) if norm else None
+    ref, _, _ = _oracle_chain(hidden, ids, luts, wrs, gammas, 1e-5)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    h = hidden.to(DEV)
+    gd = None if gammas is None else gammas.to(DEV)
+    out = mole.decode_step_args(h, ids.to(DEV), luts.to(DEV), wrs.to(DEV), torch.empty_like(h), None, status=status, mode=mole.STEP_FUSED,
+                                norm_weights=gd, norm_eps=1e-5)
+    again = mole.decode_step_args(h, ids.to(DEV), luts.to(DEV), wrs.to(DEV), h, None, status=status, mode=mole.STEP_FUSED, norm_weights=gd,
+                                  norm_eps=1e-5)  # in place
+    torch.cuda.synchronize()
+    assert int(status.item()) == (mole.STATUS_BAD_ID if M > 1 else 0)
+    assert torch.equal(out, again)
+    err = np.abs(as_f64(out) - ref)
+    slack = L * 1e-3 * float(luts.abs().max()) * N if norm else 0.0  # a rounding tie in a normalised element moves a gate
+    assert (err <= L * 2.0 ** -7 * np.maximum(1.0, np.abs(ref)) + slack).all(), float(err.max())
+    if M > 1:
+        assert torch.equal(out[M - 1].cpu(), hidden[M - 1])
+
+
+def test_a_tokens_bits_do_not_depend_on_its_batch_and_large_logits():
+    """Logits far beyond the range where the maximum has to be subtracted; tokens alone and in a batch."""
+    N, d, M, L, V = 16, 512, 40, 3, 50
+    _, ids, _, _ = rand_case(M, N, d, V, seed=3)
+    g = torch.Generator().manual_seed(8)
+    luts = torch.empty(L, V, N, d).normal_(0, 0.05, generator=g).to(torch.bfloat16)
+    wrs = torch.empty(L, d, N).normal_(0, 4.0, generator=g).to(torch.bfloat16)
+    hidden = torch.empty(M, d).normal_(0, 1, generator=g).to(torch.bfloat16)
+    ref, gref, _ = _oracle_chain(hidden, ids, luts, wrs, None, 0.0)
+    assert gref.max() > 0.999
+    h, i, lu, w = hidden.to(DEV), ids.to(DEV), luts.to(DEV), wrs.to(DEV)
+    out = mole.decode_step(h, i, lu, w, torch.empty_like(h))
+    # a gate near 1/2 can turn over when a state's rounding moves a logit of ~90 by an ulp of the state: such tokens are few
+    bad = (np.abs(as_f64(out) - ref) > L * 2.0 ** -7 * np.maximum(1.0, np.abs(ref)) + 0.02).any(axis=1)
+    assert bad.mean() <= 0.1
+    for t in (0, 7, M - 1):
+        one = mole.decode_step(h[t:t + 1].contiguous(), i[t:t + 1].contiguous(), lu, w, torch.empty(1, d, dtype=torch.bfloat16, device=DEV))
+        assert torch.equal(one[0], out[t])
+
+
+@pytest.mark.parametrize("N,d,M", [(8, 256, 6), (32, 2048, 5), (16, 2048, 4)])
+def test_waits_that_run_out_are_reported(N, d, M):
+    """No polls allowed: every wait that is not satisfied at once gives up -- for slots, for copies, for the other blocks of the
+    cluster.  The launch returns, reports it, writes nothing beyond its rows, and the next launch is right."""
+    L, V, guard = 6, 20, 3
+    g = torch.Generator().manual_seed(3)
+    luts = torch.empty(L, V, N, d).normal_(0, 0.05, generator=g).to(torch.bfloat16).to(DEV)
+    wrs = torch.empty(L, d, N).normal_(0, 0.02, generator=g).to(torch.bfloat16).to(DEV)
+    hidden = torch.empty(M, d).normal_(0, 1, generator=g).to(torch.bfloat16).to(DEV)
+    ids = torch.randint(0, V, (M,), generator=g, dtype=torch.int32).to(DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    buf = torch.full((M + 2 * guard, d), 12345.0, dtype=torch.bfloat16, device=DEV)
+    out = buf[guard:guard + M]
+    want = mole.decode_step(hidden, ids, luts, wrs, torch.empty_like(hidden)).clone()
+    with mole.debug_env(MOLE_DEBUG_WAIT_LIMIT=-1):
+        mole.decode_step(hidden, ids, luts, wrs, out, status=status)
+        torch.cuda.synchronize()
+    assert int(status.item()) & mole.STATUS_TIMEOUT
+    assert (buf[:guard] == 12345.0).all() and (buf[guard + M:] == 12345.0).all()
+    status.zero_()
+    mole.decode_step(hidden, ids, luts, wrs, out, status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and torch.equal(out, want)
