@@ -235,7 +235,8 @@ typedef struct mole_step_args {
     int32_t kernel;        /* as mole_args.kernel: the family of the single-layer launches of CHAINED mode and of the
                               one launch of FUSED mode */
     float norm_eps;        /* >= 0; read only with norm_weight_base */
-    int32_t lut_format;    /* as mole_args.lut_format; quantised tables run as CHAINED steps (AUTO picks that) */
+    int32_t lut_format;    /* as mole_args.lut_format; AUTO runs a quantised step in one launch or layer by layer (the same
+                              bits), CHAINED layer by layer; FUSED is not supported for L > 1 */
     int32_t lut_block;     /* as mole_args.lut_block */
     int32_t reserved;      /* must be 0 */
     void *stream;          /* cudaStream_t */

@@ -105,6 +105,8 @@ int launch_pdl(const void *fn, unsigned grid, unsigned threads, int smem, cudaSt
 // kernels that need more than 48 KB of dynamic shared memory opt in once per device
 int ensure_smem_opt_in(const void *fn, int smem);
 int sm_count(int *out, int *dev_out = nullptr);  // SM count of the current device, asked once per device
+// resident blocks per SM of a launch, asked once per (kernel, threads, shared memory) and thread
+int blocks_per_sm(const void *fn, int threads, int smem, int *out);
 // poll limit of the bounded device-side waits (the default unless a debugging variable shortens it)
 uint32_t current_wait_polls();
 
@@ -112,6 +114,9 @@ uint32_t current_wait_polls();
 bool quant_layer_shape_ok(int N, int d, int format, int block);
 const char *quant_variant_name(int N, int format, bool norm);
 int launch_quant_layer(const StepLaunch &a, int format, int block, uint32_t wait_polls);
+// ... and the fused step over L quantised tables, the same bits as L single layers
+bool quant_step_preferred(long long M, int N, int d, int format, int block);
+int launch_quant_step(const StepLaunch &a, int format, int block, uint32_t wait_polls);
 
 #ifdef __CUDACC__
 // ---- device side ---------------------------------------------------------------------------

@@ -82,7 +82,7 @@ __host__ __device__ inline SmemMap smem_map(int N, int d, int dcc, int eb, int s
     m.off_hid = m.off_hring + hring * up128(m.hid_bytes);                                 // running hidden state between layers
     m.off_norm = m.off_hid + up128(m.hid_bytes);                                          // RMSNorm(hidden), what a normalised router reads
     m.off_partial = m.off_norm + (norm ? up128(m.hid_bytes) : 0u);
-    m.off_gates = m.off_partial + up128((warps > static_cast<uint32_t>(d) / 128 ? warps : static_cast<uint32_t>(d) / 128) * N * 4);  // per warp or per 128 columns
+    m.off_gates = m.off_partial + up128((N == 16 && d == 1024 ? 8u : warps) * N * 4);  // per warp, or per 128 columns (router_mma16)
     m.off_meta = m.off_gates + up128(N * 4);
     m.off_bars = m.off_meta + up128((kMaxStages + 3) * 4);
     m.total = m.off_bars + (2 * kMaxStages + 1) * 8;

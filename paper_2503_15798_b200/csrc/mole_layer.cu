@@ -513,6 +513,31 @@ int sm_count(int *out, int *dev_out)
     return MOLE_OK;
 }
 
+int blocks_per_sm(const void *fn, int threads, int smem, int *out)
+{
+    struct Entry {
+        const void *fn = nullptr;
+        int threads = 0, smem = 0, dev = -1, n = 0;
+    };
+    thread_local Entry cache[16];
+    thread_local int next = 0;
+    int dev = 0;
+    MOLE_CUDA_TRY(cudaGetDevice(&dev));
+    for (const Entry &e : cache)
+        if (e.fn == fn && e.threads == threads && e.smem == smem && e.dev == dev) {
+            *out = e.n;
+            return MOLE_OK;
+        }
+    int n = 0;
+    MOLE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem));
+    if (n < 1) n = 1;
+    Entry &e = cache[next];
+    next = (next + 1) % 16;
+    e.fn = fn, e.threads = threads, e.smem = smem, e.dev = dev, e.n = n;
+    *out = n;
+    return MOLE_OK;
+}
+
 // Everything about a launch that depends only on its shape: found once, then looked up.
 struct ShapeKey {
     long long M;
@@ -937,12 +962,14 @@ int mole_decode_step_args(const mole_step_args *a)
     if (mode == MOLE_STEP_AUTO) {
         mode = (quant || (L > 1 && M > kFusedMaxTokens)) ? MOLE_STEP_CHAINED : MOLE_STEP_FUSED;
     }
+    bool quant_fused = false;
     if (quant) {
-        // quantised tables run layer by layer (one block per token de-quantising inside the weighted sum)
+        // quantised tables: MOLE_STEP_AUTO may take the fused step kernel, MOLE_STEP_CHAINED runs layer by layer
         if (mode == MOLE_STEP_FUSED && L > 1) return MOLE_ERR_UNSUPPORTED_SHAPE;
         mode = MOLE_STEP_CHAINED;
         if (a->dtype != MOLE_DTYPE_BF16 || a->d_split != 0 || a->kernel == MOLE_KERNEL_RING) return MOLE_ERR_UNSUPPORTED_SHAPE;
         if (!quant_layer_shape_ok(a->N, a->d, a->lut_format, a->lut_block)) return MOLE_ERR_UNSUPPORTED_SHAPE;
+        quant_fused = a->mode == MOLE_STEP_AUTO && L > 1 && quant_step_preferred(M, a->N, a->d, a->lut_format, a->lut_block);
     }
 
     StepLaunch s;
@@ -962,7 +989,7 @@ int mole_decode_step_args(const mole_step_args *a)
     s.d_split = a->d_split;
     s.kernel = a->kernel;
     s.stream = static_cast<cudaStream_t>(a->stream);
-    if (mode == MOLE_STEP_FUSED) {
+    if (mode == MOLE_STEP_FUSED || quant_fused) {
         // one launch: every block walks its tokens through all L layers
         s.hidden = a->hidden_in;
         s.lut = a->lut_base;
@@ -971,6 +998,7 @@ int mole_decode_step_args(const mole_step_args *a)
         s.out = a->out;
         s.L = L;
         s.flags = a->flags & MOLE_FLAG_CHAIN;
+        if (quant_fused) return launch_quant_step(s, a->lut_format, a->lut_block, current_wait_polls());
         return launch_step(s);
     }
     if (L > 1 && (!a->tmp || !aligned16(a->tmp) || a->out == a->hidden_in || a->tmp == a->hidden_in || a->tmp == a->out))

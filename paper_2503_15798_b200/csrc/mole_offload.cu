@@ -583,8 +583,9 @@ int mole_offload_decode_step(mole_offload_ctx *c, const void *hidden_in, const i
         a.dtype = c->dtype;
         a.d_split = 0;
         a.stream = st;
-        if (c->lut_format != MOLE_LUT_PLAIN) {
-            // quantised records: layer by layer from the staging area (the layers of a group chained to one
+        const bool quant = c->lut_format != MOLE_LUT_PLAIN;
+        if (quant && !(n > 1 && quant_step_preferred(M, c->N, c->d, c->lut_format, c->lut_block))) {
+            // quantised records, many tokens: layer by layer from the staging area (the layers of a group chained to one
             // another with programmatic dependent launch), ping-pong so that the last layer writes `out`
             for (int i = 0; i < n; ++i) {
                 const int l = l0 + i;
@@ -611,7 +612,7 @@ int mole_offload_decode_step(mole_offload_ctx *c, const void *hidden_in, const i
             a.L = n;
             a.flags = 0;
             a.kernel = MOLE_KERNEL_RING;  // every group on one kernel family: the step's bits do not depend on how it is grouped
-            rc = launch_step(a);
+            rc = quant ? launch_quant_step(a, c->lut_format, c->lut_block, current_wait_polls()) : launch_step(a);
             if (rc != MOLE_OK) return rc;
             src = dst;
         }

@@ -1,0 +1,57 @@
+"""The fused step over quantised tables: the bits of the same layers one after the other, at every expert count, with and
+without norm, odd blocks, several tokens per block, ids outside the table; its bounded waits."""
+import pytest
+import torch
+
+from paper_2503_15798_b200 import binding as mole
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+# format, block, N, d, M, L
+CASES = [(1, 32, 4, 128, 1, 5), (2, 128, 4, 2048, 148, 2), (1, 384, 8, 384, 700, 3), (2, 32, 8, 128, 2368, 2), (1, 768, 16, 768, 394, 3), (2, 64, 16, 1024, 65, 4),
+         (1, 2048, 16, 2048, 3, 3), (2, 128, 32, 256, 40, 3), (1, 1024, 32, 1024, 296, 2), (2, 96, 16, 384, 9, 7)]
+
+
+def _case(fmt, block, N, d, M, L, V=60):
+    g = torch.Generator(device=DEV).manual_seed(N * d + M)
+    luts = torch.empty(L, V, N, d, device=DEV).normal_(0, 0.05, generator=g).to(torch.bfloat16)
+    wrs = torch.empty(L, d, N, device=DEV).normal_(0, 0.02, generator=g).to(torch.bfloat16)
+    gam = (1.0 + 0.2 * torch.empty(L, d, device=DEV).normal_(0, 1, generator=g)).to(torch.bfloat16)
+    hidden = torch.empty(M, d, device=DEV).normal_(0, 1, generator=g).to(torch.bfloat16)
+    ids = torch.randint(0, V, (M,), generator=g, dtype=torch.int32, device=DEV)
+    return mole.QuantTable.quantize(luts, fmt, block), wrs, gam, hidden, ids
+
+
+@pytest.mark.parametrize("fmt,block,N,d,M,L", CASES)
+@pytest.mark.parametrize("norm", [False, True])
+def test_fused_quantised_step_is_its_layers_one_after_the_other(fmt, block, N, d, M, L, norm):
+    q, wrs, gam, hidden, ids = _case(fmt, block, N, d, M, L)
+    if M > 1:
+        ids[0], ids[M - 1] = -1, 60
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    out = mole.decode_step_args(hidden, ids, q, wrs, torch.empty_like(hidden), None, status=status, norm_weights=gam if norm else None, norm_eps=1e-5)
+    h = hidden
+    for l in range(L):
+        h = mole.layer_forward(h, ids, q.layer(l), wrs[l], norm_weight=gam[l] if norm else None, norm_eps=1e-5)
+    chained = mole.decode_step_args(hidden, ids, q, wrs, torch.empty_like(hidden), torch.empty_like(hidden), mode=mole.STEP_CHAINED,
+                                    norm_weights=gam if norm else None, norm_eps=1e-5)
+    torch.cuda.synchronize()
+    assert int(status.item()) == (mole.STATUS_BAD_ID if M > 1 else 0)
+    assert torch.equal(out, h) and torch.equal(out, chained) and not torch.equal(out, hidden)
+    if M > 1:
+        assert torch.equal(out[0], hidden[0]) and torch.equal(out[M - 1], hidden[M - 1])
+
+
+def test_waits_that_run_out_are_reported():
+    q, wrs, _, hidden, ids = _case(1, 768, 16, 768, 6, 12)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    want = mole.decode_step_args(hidden, ids, q, wrs, torch.empty_like(hidden), None).clone()
+    buf = torch.full((12, 768), 12345.0, dtype=torch.bfloat16, device=DEV)
+    with mole.debug_env(MOLE_DEBUG_WAIT_LIMIT=-1):
+        mole.decode_step_args(hidden, ids, q, wrs, buf[3:9], None, status=status)
+        torch.cuda.synchronize()
+    assert int(status.item()) & mole.STATUS_TIMEOUT and (buf[:3] == 12345.0).all() and (buf[9:] == 12345.0).all()
+    status.zero_()
+    mole.decode_step_args(hidden, ids, q, wrs, buf[3:9], None, status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and torch.equal(buf[3:9], want)
