@@ -14,33 +14,43 @@
 // tcgen05.mma 128 x 256 x 16 on the staged tiles and hands stages back with tcgen05.commit; the accumulator
 // is double-buffered in tensor memory (2 x 256 of the 512 columns), so that warps 2-9 read tile i back with
 // tcgen05.ld, apply the epilogue (GELU for the first GEMM) and store bf16 while the tensor cores already
-// work on tile i + 1.  Every wait is bounded; a wait that runs out sets MOLE_STATUS_TIMEOUT and the block
+// work on tile i + 1.
+// Pairs (PAIR = 1): two blocks of a cluster work on a 256 x 256 tile with tcgen05.mma.cta_group::2, 256 x 256 x 16 issued by
+// the first of them; each stages its own 128 rows of A and only half of B (32 KB per stage instead of 48, six stages instead
+// of four), both copies counted on the first block's barrier, and reads its own 128 accumulator rows back.  A third less operand
+// traffic per flop, which is what bounds the main loop (about 53 bytes a clock and SM out of L2 at 1.65 GHz, whatever the tile
+// order) and, as power, a long build.  The first GEMM is bound by its epilogue on top: without the GELU its tiles of
+// K = 512 take 71 instead of 94 us (5000 x 8 x 2048 outputs).  Sixteen epilogue warps, stores straight from registers, halves or
+// both of the staging tile per store, and one reciprocal for two elements all measured the same or slower: what they take
+// from the ring's six stages costs the main loop 5 %.  Every wait is bounded; a wait that runs out sets MOLE_STATUS_TIMEOUT and the block
 // winds down: copies and MMAs in flight are waited for (again bounded) and tensor memory is freed on every path.
 #include <cuda.h>
 #include <math.h>
 #include <mutex>
 #include <string.h>
 
-#include "mole_kernel.cuh"
+#include "mole_cdecode.cuh"
 
 namespace mole {
 
 constexpr int kBM = 128, kBN = 256, kBK = 64;          // tile; kBK bf16 = one 128-byte swizzle span
-constexpr int kGemmStages = 4;                         // 192 KB of operand tiles in flight per SM
 constexpr int kTileBytesA = kBM * kBK * 2;             // 16 KB
-constexpr int kTileBytesB = kBN * kBK * 2;             // 32 KB
-constexpr int kStageBytes = kTileBytesA + kTileBytesB;
+__host__ __device__ constexpr int gemm_stages(int pair) { return pair ? 6 : 4; }  // 192 KB of operand tiles in flight per SM
+__host__ __device__ constexpr int gemm_rows_b(int pair) { return pair ? kBN / 2 : kBN; }
+__host__ __device__ constexpr int gemm_stage_bytes(int pair) { return kTileBytesA + gemm_rows_b(pair) * kBK * 2; }
+constexpr int kGemmRingBytes = 192 * 1024;
+static_assert(gemm_stages(0) * gemm_stage_bytes(0) == kGemmRingBytes && gemm_stages(1) * gemm_stage_bytes(1) == kGemmRingBytes, "the ring's size");
 constexpr int kAccBuffers = 2;                         // accumulators in tensor memory: 2 x kBN of the 512 columns
 constexpr int kTmemCols = kAccBuffers * kBN;
 constexpr int kEpiWarps = 8;
 constexpr int kGemmThreads = (2 + kEpiWarps) * 32;     // producer warp, MMA warp, eight epilogue warps
 constexpr int kRasterRows = 8;                         // tile rows walked together
-constexpr int kGemmBarriers = 2 * kGemmStages + 2 * kAccBuffers + 1;
+constexpr int kGemmBarriers = 2 * 6 + 2 * kAccBuffers + 1;
 constexpr int kStoreBytes = 32 * 128;                  // an epilogue warp's staging tile: 32 rows x 64 bf16, 128-byte swizzle
-constexpr uint32_t kGemmSmem = kGemmStages * kStageBytes + kEpiWarps * kStoreBytes + 1024 /* alignment slack */ + 256 /* barriers */;
+constexpr uint32_t kGemmSmem = kGemmRingBytes + kEpiWarps * kStoreBytes + 1024 /* alignment slack */ + 256 /* barriers */;
 static_assert(kGemmSmem <= 232448, "one block's shared memory");
 constexpr uint32_t kGemmWaitPolls = 1u << 22;
-static_assert(kTmemCols == 512 && kGemmBarriers * 8 <= 128 && kEpiWarps % 4 == 0 && kBN % (8 * kEpiWarps) == 0, "tensor-memory columns are a power of two; barriers fit their block");
+static_assert(kTmemCols == 512 && kGemmBarriers * 8 <= 144 && kEpiWarps % 4 == 0 && kBN % (8 * kEpiWarps) == 0, "tensor-memory columns are a power of two; barriers fit their block");
 
 struct GemmParams {
     int M, N, K;            // per z slice
@@ -107,10 +117,35 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t smem_addr)
     d |= static_cast<uint64_t>(2) << 61;                      // 128-byte swizzle
     return d;
 }
-// instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = kBM, N = kBN
-__device__ __forceinline__ uint32_t umma_idesc()
+// instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = kBM (2 kBM for a pair), N = kBN
+__device__ __forceinline__ uint32_t umma_idesc(int pair)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(kBN >> 3) << 17) | (static_cast<uint32_t>(kBM >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(kBN >> 3) << 17) | (static_cast<uint32_t>((kBM << pair) >> 4) << 24);
+}
+// a pair's copy: into this block's own shared memory, counted at a barrier of either block
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t smem_dst, const CUtensorMap *map, int c0, int c1, int c2, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 ::"r"(smem_dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// when the pair's MMAs issued so far are done: one arrival at this barrier in both blocks
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar)
+{
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"(static_cast<unsigned short>(3)) : "memory");
+}
+__device__ __forceinline__ void bar_arrive_cluster(uint32_t cluster_bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
 {
@@ -182,7 +217,7 @@ struct TileCoord {
     int m0, n0, z;
 };
 // tiles in the order the blocks walk them: z slice by z slice, kRasterRows tile rows at a time, down the rows first
-__device__ __forceinline__ TileCoord tile_coord(int tile, const GemmParams &p)
+__device__ __forceinline__ TileCoord tile_coord(int tile, const GemmParams &p, int tile_rows)
 {
     const int per_z = p.m_tiles * p.n_tiles;
     const int z = tile / per_z, r = tile - z * per_z;
@@ -191,13 +226,13 @@ __device__ __forceinline__ TileCoord tile_coord(int tile, const GemmParams &p)
     const int rows = min(kRasterRows, p.m_tiles - first);
     const int w = r - band * kRasterRows * p.n_tiles;
     TileCoord t;
-    t.m0 = (first + w % rows) * kBM;
+    t.m0 = (first + w % rows) * tile_rows;
     t.n0 = (w / rows) * kBN;
     t.z = z;
     return t;
 }
 
-template <int GELU>
+template <int GELU, int PAIR>
 __global__ void __launch_bounds__(kGemmThreads, 1) mole_gemm_tn_kernel(const __grid_constant__ CUtensorMap map_a,
                                                                     const __grid_constant__ CUtensorMap map_b,
                                                                     const __grid_constant__ CUtensorMap map_c, const GemmParams p)
@@ -205,69 +240,94 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mole_gemm_tn_kernel(const __g
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t tiles = (raw + 1023u) & ~1023u;  // swizzled tiles want 1024-byte alignment
-    const uint32_t staging = tiles + kGemmStages * kStageBytes;
-    unsigned char *ctl = smem_raw + (tiles - raw) + kGemmStages * kStageBytes + kEpiWarps * kStoreBytes;
+    constexpr int STAGES = gemm_stages(PAIR), STAGE = gemm_stage_bytes(PAIR);
+    const uint32_t staging = tiles + kGemmRingBytes;
+    unsigned char *ctl = smem_raw + (tiles - raw) + kGemmRingBytes + kEpiWarps * kStoreBytes;
     uint64_t *bars = reinterpret_cast<uint64_t *>(ctl);  // full[stages], empty[stages], acc_full[2], acc_empty[2], drain
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ctl + 128);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ctl + 144);
+    // a pair shares its tiles; the first block of it issues the MMAs and holds the barriers that start them
+    const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
+    const int first_tile = PAIR ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
+    const int tile_step = PAIR ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
+    constexpr int TILE_ROWS = kBM << PAIR;
     volatile int *dead = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    const uint32_t full0 = smem_u32(bars), empty0 = full0 + kGemmStages * 8, acc_full0 = empty0 + kGemmStages * 8,
+    const uint32_t full0 = smem_u32(bars), empty0 = full0 + STAGES * 8, acc_full0 = empty0 + STAGES * 8,
                    acc_empty0 = acc_full0 + kAccBuffers * 8, drain_bar = acc_empty0 + kAccBuffers * 8;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ktiles = (p.K + kBK - 1) / kBK;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kGemmBarriers; ++s) {
-            const bool acc_empty = s >= 2 * kGemmStages + kAccBuffers && s < 2 * kGemmStages + 2 * kAccBuffers;
-            mbar_init(bars + s, acc_empty ? kEpiWarps : 1);  // every epilogue warp hands an accumulator back
+        for (int s = 0; s < 2 * STAGES + 2 * kAccBuffers + 1; ++s) {
+            const bool acc_empty = s >= 2 * STAGES + kAccBuffers && s < 2 * STAGES + 2 * kAccBuffers;
+            mbar_init(bars + s, acc_empty ? kEpiWarps << PAIR : 1);  // every epilogue warp (of both blocks) hands an accumulator back
         }
         dead[0] = 0;
         dead[1] = 0;  // stays 0: the flag the draining waits look at
         mbar_init_fence();
     }
     if (warp == 1) {  // all of this SM's tensor memory: two 128 x kBN fp32 accumulators (one block per SM)
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if constexpr (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if constexpr (PAIR) {  // the other block's barriers and tensor memory are ready, too
+        cluster_arrive();
+        cluster_wait();
+    }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_acc = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {  // ---- producer: tiles of A and B, kGemmStages ahead, across output tiles ----
+        if (lane == 0) {  // ---- producer: tiles of A and B, STAGES ahead, across output tiles ----
             uint32_t it = 0;  // k-tiles issued by this block so far
             bool ok = true;
-            for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += gridDim.x) {
-                const TileCoord tc = tile_coord(tile, p);
+            for (int tile = first_tile; tile < p.total_tiles && ok; tile += tile_step) {
+                const TileCoord tc = tile_coord(tile, p, TILE_ROWS);
                 for (int kt = 0; kt < ktiles; ++kt, ++it) {
-                    const uint32_t s = it % kGemmStages;
-                    const uint32_t par = ((it / kGemmStages) & 1u) ^ 1u;  // first pass: the stage has never been used
+                    const uint32_t s = it % STAGES;
+                    const uint32_t par = ((it / STAGES) & 1u) ^ 1u;  // first pass: the stage has never been used
                     if (!bar_wait_bounded(empty0 + s * 8, par, dead)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t a_dst = tiles + s * kStageBytes, b_dst = a_dst + kTileBytesA;
-                    mbar_expect_tx(bars + s, kStageBytes);
-                    tma_load_3d(a_dst, &map_a, kt * kBK, tc.m0, tc.z, full0 + s * 8);
-                    tma_load_3d(b_dst, &map_b, kt * kBK, tc.n0, tc.z, full0 + s * 8);
+                    const uint32_t a_dst = tiles + s * STAGE, b_dst = a_dst + kTileBytesA;
+                    if constexpr (PAIR) {
+                        // the first block's barrier counts both blocks' copies (those of the second may come in first)
+                        const uint32_t bar = cluster_map(full0 + s * 8, 0);
+                        if (rank == 0) mbar_expect_tx(bars + s, 2 * STAGE);
+                        tma_load_3d_pair(a_dst, &map_a, kt * kBK, tc.m0 + static_cast<int>(rank) * kBM, tc.z, bar);
+                        tma_load_3d_pair(b_dst, &map_b, kt * kBK, tc.n0 + static_cast<int>(rank) * (kBN / 2), tc.z, bar);
+                    } else {
+                        mbar_expect_tx(bars + s, STAGE);
+                        tma_load_3d(a_dst, &map_a, kt * kBK, tc.m0, tc.z, full0 + s * 8);
+                        tma_load_3d(b_dst, &map_b, kt * kBK, tc.n0, tc.z, full0 + s * 8);
+                    }
                 }
             }
             if (!ok) {
                 if (!*dead && p.status) atomicOr(p.status, MOLE_STATUS_TIMEOUT);
                 *dead = 1;
                 // the copies already issued land in this block's shared memory: let them, before the block can exit
-                const uint32_t first = it > static_cast<uint32_t>(kGemmStages) ? it - kGemmStages : 0u;
+                const uint32_t first = it > static_cast<uint32_t>(STAGES) ? it - STAGES : 0u;
                 for (uint32_t j = first; j < it; ++j)
-                    (void)bar_wait_bounded(full0 + (j % kGemmStages) * 8, (j / kGemmStages) & 1u, dead + 1, kDrainPolls);
+                    // (the second block of a pair cannot see its copies counted: its own barrier stays in phase 0, and the wait
+                    // is simply that long)
+                    (void)bar_wait_bounded(full0 + (j % STAGES) * 8, rank ? 0u : (j / STAGES) & 1u, dead + 1, kDrainPolls);
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {  // ---- tensor-core issue ----
-            const uint32_t idesc = umma_idesc();
+        if (lane == 0 && rank == 0) {  // ---- tensor-core issue ----
+            const uint32_t idesc = umma_idesc(PAIR);
             uint32_t it = 0, t = 0;  // k-tiles and output tiles consumed by this block so far
             bool ok = true;
-            for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += gridDim.x, ++t) {
+            for (int tile = first_tile; tile < p.total_tiles && ok; tile += tile_step, ++t) {
                 const uint32_t b = t & 1u;
                 // the epilogue warps have read this accumulator's previous tile out
                 ok = bar_wait_bounded(acc_empty0 + b * 8, ((t >> 1) & 1u) ^ 1u, dead);
@@ -275,23 +335,30 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mole_gemm_tn_kernel(const __g
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t acc = tmem_acc + b * kBN;
                 for (int kt = 0; kt < ktiles; ++kt, ++it) {
-                    const uint32_t s = it % kGemmStages;
-                    ok = bar_wait_bounded(full0 + s * 8, (it / kGemmStages) & 1u, dead);
+                    const uint32_t s = it % STAGES;
+                    ok = bar_wait_bounded(full0 + s * 8, (it / STAGES) & 1u, dead);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t a_src = tiles + s * kStageBytes, b_src = a_src + kTileBytesA;
+                    const uint32_t a_src = tiles + s * STAGE, b_src = a_src + kTileBytesA;
                     const uint64_t adesc = umma_desc(a_src), bdesc = umma_desc(b_src);
 #pragma unroll
                     for (int k = 0; k < kBK / 16; ++k)  // 16 bf16 = 32 bytes along K inside the swizzle span: +2 in 16-byte units
-                        umma_bf16(acc, adesc + 2 * k, bdesc + 2 * k, idesc, (kt > 0 || k > 0) ? 1u : 0u);
-                    umma_commit(empty0 + s * 8);  // the stage is free once these have read it
+                        if constexpr (PAIR) umma_bf16_pair(acc, adesc + 2 * k, bdesc + 2 * k, idesc, (kt > 0 || k > 0) ? 1u : 0u);
+                        else umma_bf16(acc, adesc + 2 * k, bdesc + 2 * k, idesc, (kt > 0 || k > 0) ? 1u : 0u);
+                    // the stage is free once these have read it
+                    if constexpr (PAIR) umma_commit_pair(empty0 + s * 8);
+                    else umma_commit(empty0 + s * 8);
                 }
-                if (ok) umma_commit(acc_full0 + b * 8);
+                if (ok) {
+                    if constexpr (PAIR) umma_commit_pair(acc_full0 + b * 8);
+                    else umma_commit(acc_full0 + b * 8);
+                }
             }
             if (!ok) {
                 if (!*dead && p.status) atomicOr(p.status, MOLE_STATUS_TIMEOUT);
                 *dead = 1;
-                umma_commit(drain_bar);  // whatever was issued finishes reading shared memory before the block exits
+                if constexpr (PAIR) umma_commit_pair(drain_bar);
+                else umma_commit(drain_bar);  // whatever was issued finishes reading shared memory before the block exits
                 (void)bar_wait_bounded(drain_bar, 0, dead + 1, kDrainPolls);
             }
         }
@@ -309,13 +376,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mole_gemm_tn_kernel(const __g
         const uint32_t stage_row = staging + static_cast<uint32_t>((warp - 2) * kStoreBytes + lane * 128);
         uint32_t t = 0;
         bool ok = true;
-        for (int tile = blockIdx.x; tile < p.total_tiles && ok; tile += gridDim.x, ++t) {
+        for (int tile = first_tile; tile < p.total_tiles && ok; tile += tile_step, ++t) {
             const uint32_t b = t & 1u;
             ok = bar_wait_bounded(acc_full0 + b * 8, (t >> 1) & 1u, dead);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const TileCoord tc = tile_coord(tile, p);
-            const int row0 = tc.m0 + quarter * 32;
+            const TileCoord tc = tile_coord(tile, p, TILE_ROWS);
+            const int row0 = tc.m0 + static_cast<int>(rank) * kBM + quarter * 32;
             const int ncol0 = tc.n0 + part * kColsPerWarp;
             const uint32_t tsrc = tmem_acc + (static_cast<uint32_t>(quarter * 32) << 16) + b * kBN + static_cast<uint32_t>(part * kColsPerWarp);
             uint32_t r[2][32];
@@ -329,7 +396,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mole_gemm_tn_kernel(const __g
                     // this warp's part of the accumulator is in registers: hand the buffer back to the tensor cores
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) bar_arrive(acc_empty0 + b * 8);
+                    if (lane == 0) {
+                        if constexpr (PAIR) bar_arrive_cluster(cluster_map(acc_empty0 + b * 8, 0));
+                        else bar_arrive(acc_empty0 + b * 8);
+                    }
                 }
                 uint32_t packed[16];  // 32 consecutive columns of this thread's row, rounded in pairs
 #pragma unroll
@@ -361,9 +431,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) mole_gemm_tn_kernel(const __g
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if constexpr (PAIR) {  // neither block leaves, or gives tensor memory back, while the other's MMAs or arrivals may reach it
+        cluster_arrive();
+        cluster_wait();
+    }
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "r"(kTmemCols) : "memory");
+        if constexpr (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "r"(kTmemCols) : "memory");
+        else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "r"(kTmemCols) : "memory");
     }
 }
 
@@ -428,32 +503,49 @@ static int launch_gemm(const void *a, long long a_row_stride, long long a_z_stri
     CUtensorMap map_a, map_b, map_c;
     int rc = make_matrix_map(&map_a, a, K, M, Z, a_row_stride, a_z_stride, kBM);
     if (rc != MOLE_OK) return rc;
-    rc = make_matrix_map(&map_b, b, K, N, Z, b_row_stride, b_z_stride, kBN);
+    int sms = 0;
+    rc = sm_count(&sms);
+    if (rc != MOLE_OK) return rc;
+    // Pairs of blocks (50304 rows, 16 x 768 -> 3072: 6.26 -> 5.75 ms alone, 7.23 -> 6.67 ms back to back under the power
+    // limit; 2000 rows 286 -> 267 us), unless half of a pair's last tile row would be padding and the rows are so few
+    // (under nine tiles of 128) that this is over a tenth of the work.
+    const int tile_rows1 = (M + kBM - 1) / kBM;
+    const int pair = sms >= 2 && (tile_rows1 % 2 == 0 || tile_rows1 >= 9) ? 1 : 0;
+    rc = make_matrix_map(&map_b, b, K, N, Z, b_row_stride, b_z_stride, gemm_rows_b(pair));
     if (rc != MOLE_OK) return rc;
     rc = make_matrix_map(&map_c, c, N, M, Z, c_row_stride, c_z_stride, 32);
     if (rc != MOLE_OK) return rc;
-    const void *fn = gelu ? reinterpret_cast<const void *>(mole_gemm_tn_kernel<1>) : reinterpret_cast<const void *>(mole_gemm_tn_kernel<0>);
-    rc = ensure_smem_opt_in(fn, static_cast<int>(kGemmSmem));
-    if (rc != MOLE_OK) return rc;
-    int sms = 0;
-    rc = sm_count(&sms);
+    typedef void (*GemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmParams);
+    const GemmKernel fn = pair ? (gelu ? mole_gemm_tn_kernel<1, 1> : mole_gemm_tn_kernel<0, 1>) : (gelu ? mole_gemm_tn_kernel<1, 0> : mole_gemm_tn_kernel<0, 0>);
+    rc = ensure_smem_opt_in(reinterpret_cast<const void *>(fn), static_cast<int>(kGemmSmem));
     if (rc != MOLE_OK) return rc;
     GemmParams p;
     p.M = M;
     p.N = N;
     p.K = K;
-    p.m_tiles = (M + kBM - 1) / kBM;
+    p.m_tiles = (tile_rows1 + pair) >> pair;
     p.n_tiles = (N + kBN - 1) / kBN;
     const long long total = static_cast<long long>(p.m_tiles) * p.n_tiles * Z;
     if (total > 0x7fffffffLL) return MOLE_ERR_TOO_LARGE;
     p.total_tiles = static_cast<int>(total);
     p.status = status;
-    const unsigned grid = static_cast<unsigned>(total < sms ? total : sms);  // persistent: one block per SM
-    if (gelu)
-        mole_gemm_tn_kernel<1><<<grid, kGemmThreads, kGemmSmem, st>>>(map_a, map_b, map_c, p);
-    else
-        mole_gemm_tn_kernel<0><<<grid, kGemmThreads, kGemmSmem, st>>>(map_a, map_b, map_c, p);
-    MOLE_CUDA_TRY(cudaGetLastError());
+    const long long workers = sms >> pair;  // persistent: one block per SM
+    const unsigned grid = static_cast<unsigned>(total < workers ? total : workers) << pair;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(kGemmThreads, 1, 1);
+    cfg.dynamicSmemBytes = kGemmSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    if (pair) {
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 2;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+    }
+    MOLE_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, map_a, map_b, map_c, p));
     return MOLE_OK;
 }
 

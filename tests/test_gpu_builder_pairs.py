@@ -1,0 +1,27 @@
+"""The table builder's two tilings at the row counts where the choice between them, or a pair's halves, can go wrong:
+one row in the second block of a pair, an odd number of tile rows just below and from the size where pairs take it,
+columns that end inside the first and the second half of a pair's B tile."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_util import as_f64
+from paper_2503_15798_b200 import binding as mole
+from test_gpu_builder import _bound, _weights
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("V,N,d,D", [(129, 2, 72, 136), (256, 3, 264, 64), (896, 2, 64, 128), (1025, 2, 40, 200), (1152, 1, 128, 392)])
+def test_pairs_and_single_blocks_against_the_oracle_builder(V, N, d, D):
+    E, W1, W2 = _weights(V, N, d, D, seed=V)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    lut = mole.build_lut(E.cuda(), W1.cuda(), W2.cuda(), status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    E64 = as_f64(E)
+    ref = oracle.build_lut(E64, as_f64(W1), as_f64(W2))
+    err, bound = np.abs(as_f64(lut) - ref), _bound(E64, W1, W2, ref)  # the bound of the builder's own test
+    assert (err <= bound).all(), float((err / bound).max())
+    assert np.abs(as_f64(lut)).max() > 0.05
