@@ -107,14 +107,77 @@ struct HotRows {
     int layer0;                 // cache layer of this launch's z = 0
     unsigned long long *hits;   // rows served from the cache (one count per row and layer), or NULL
 };
+struct DistinctIds {
+    int32_t *uniq, *count;  // read, or written with SCAN
+    // SCAN only
+    const int32_t *ids;
+    int32_t *slot;
+    uint32_t *status;
+    int M, V;
+};
+// A few tokens (SCAN, at most one per thread): every block works the distinct ids out for itself, by comparing each token
+// with those before it, and the first block publishes them for the later fetches and the layers.  A whole step then starts
+// with its first fetch instead of with the dedup kernel and the wait for it: 4 us of the step, at most a microsecond back in
+// the scan.  The same numbering (first occurrence) as the dedup kernel's.
+template <int SCAN>
 __global__ void __launch_bounds__(kFetchThreads) mole_fetch_kernel(const unsigned char *__restrict__ table_host,
-                                                                   const int32_t *__restrict__ uniq,
-                                                                   const int32_t *__restrict__ count, long long row_bytes,
+                                                                   const DistinctIds q, long long row_bytes,
                                                                    unsigned char *__restrict__ staging, long long table_stride,
                                                                    long long staging_stride, const HotRows hot)
 {
+    int rows;  // distinct ids
+    const int32_t *uniq = q.uniq;
+    __shared__ int32_t list[SCAN ? kFetchThreads : 1];  // SCAN: the distinct ids, in order
+    if constexpr (SCAN) {
+        __shared__ __align__(16) int32_t sid[kFetchThreads];
+        __shared__ int32_t pos[kFetchThreads];
+        __shared__ int warp_reps[kFetchThreads / 32];
+        const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+        const int raw = t < q.M ? q.ids[t] : -1;
+        const bool valid = raw >= 0 && raw < q.V;
+        const int id = valid ? raw : -1;
+        sid[t] = id;
+        __syncthreads();
+        int rep = t;  // the first token with this id
+        if (valid) {
+            const int4 *s4 = reinterpret_cast<const int4 *>(sid);
+            for (int j = 0; j < t; j += 4) {
+                const int4 v = s4[j >> 2];
+                const int hit = v.x == id ? j : v.y == id ? j + 1 : v.z == id ? j + 2 : v.w == id ? j + 3 : t;
+                if (hit < t) {
+                    rep = hit;
+                    break;
+                }
+            }
+        }
+        const bool first = valid && rep == t;
+        const unsigned reps = __ballot_sync(0xffffffffu, first);
+        if (lane == 0) warp_reps[warp] = __popc(reps);
+        __syncthreads();
+        int mine = __popc(reps & ((1u << lane) - 1u));
+        rows = 0;
+#pragma unroll
+        for (int w = 0; w < kFetchThreads / 32; ++w) {
+            if (w < warp) mine += warp_reps[w];
+            rows += warp_reps[w];
+        }
+        if (first) list[mine] = id;
+        pos[t] = mine;
+        __syncthreads();
+        if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
+            if (t < q.M) {
+                q.slot[t] = valid ? pos[rep] : -1;
+                if (first) q.uniq[mine] = id;
+                if (!valid && q.status) atomicOr(q.status, MOLE_STATUS_BAD_ID);
+            }
+            if (t == 0) *q.count = rows;
+        }
+        uniq = list;
+    } else {
+        rows = *q.count;
+    }
     const int u = blockIdx.y;
-    if (u >= *count) return;
+    if (u >= rows) return;
     const long long row = uniq[u];
     const long long chunk0 = static_cast<long long>(blockIdx.x) * kFetchChunk;
     const long long z = blockIdx.z;
@@ -174,21 +237,44 @@ static int device_alias(const void *host, const unsigned char **out)
 
 // `layers` tables, table_stride bytes apart from lut_host on (one pinned allocation), into staging areas
 // staging_stride bytes apart
-static int launch_fetch(const void *lut_host, const int32_t *uniq, const int32_t *count, int max_rows, long long row_bytes,
-                        void *staging, cudaStream_t st, int layers = 1, long long table_stride = 0, long long staging_stride = 0,
-                        const HotRows *hot = nullptr)
+static int launch_fetch(const void *lut_host, const DistinctIds &q, int max_rows, long long row_bytes, void *staging, cudaStream_t st,
+                        int layers = 1, long long table_stride = 0, long long staging_stride = 0, const HotRows *hot = nullptr)
 {
     const unsigned char *dev_alias = nullptr;
     int rc = device_alias(lut_host, &dev_alias);
     if (rc != MOLE_OK) return rc;
-    dim3 grid(static_cast<unsigned>((row_bytes + kFetchChunk - 1) / kFetchChunk), static_cast<unsigned>(max_rows),
-              static_cast<unsigned>(layers));
     HotRows none;
     memset(&none, 0, sizeof none);
-    mole_fetch_kernel<<<grid, kFetchThreads, 0, st>>>(dev_alias, uniq, count, row_bytes, static_cast<unsigned char *>(staging),
-                                                      table_stride, staging_stride, hot ? *hot : none);
+    const dim3 grid(static_cast<unsigned>((row_bytes + kFetchChunk - 1) / kFetchChunk), static_cast<unsigned>(max_rows),
+                    static_cast<unsigned>(layers));
+    unsigned char *to = static_cast<unsigned char *>(staging);
+    if (q.ids) mole_fetch_kernel<1><<<grid, kFetchThreads, 0, st>>>(dev_alias, q, row_bytes, to, table_stride, staging_stride, hot ? *hot : none);
+    else mole_fetch_kernel<0><<<grid, kFetchThreads, 0, st>>>(dev_alias, q, row_bytes, to, table_stride, staging_stride, hot ? *hot : none);
     MOLE_CUDA_TRY(cudaGetLastError());
     return MOLE_OK;
+}
+static DistinctIds distinct(int32_t *uniq, int32_t *count)
+{
+    DistinctIds q;
+    memset(&q, 0, sizeof q);
+    q.uniq = uniq;
+    q.count = count;
+    return q;
+}
+// Layers of a whole step's next group, `left` of L still to come and at most g to a group.  The step takes the first group's
+// fetch, then the slower of the fetches and the layers, then the last group's layers, and 4 to 5 us of link for every
+// group more.  A layer takes 1.5 to 2.2 us, its rows 1 us for every 50 KB.  So three groups; where the link is the slower by
+// about two, 5/8, 1/4 and 1/8 of the layers (few run after the last byte, and those before still end under the next fetch),
+// unless g is too small for that; two groups, a third and the rest, where the layers are the slower; equal ones in between.
+// (24 layers of 16 x 1024, 8 tokens: 157 -> 147 us with this and the ids scanned in the fetch; 1 token: 62 -> 53.)
+static int next_group(int left, int L, int g, long long layer_bytes)
+{
+    const int last = L / 8 > 2 ? L / 8 : 2;
+    int n = (L + 2) / 3;
+    if (layer_bytes >= (192LL << 10) && 2 * g + last >= L) n = left == L ? (5 * L + 4) / 8 : left > last ? left - last : left;
+    else if (layer_bytes <= (48LL << 10) && left < L) n = left;
+    n = n > g ? g : n;
+    return n > left ? left : n;
 }
 
 }  // namespace mole
@@ -235,7 +321,8 @@ int mole_fetch_rows(const void *lut_host, const int32_t *uniq, const int32_t *co
     if (max_rows == 0) return MOLE_OK;
     if (max_rows > 65535) return MOLE_ERR_TOO_LARGE;
     if (!lut_host || !uniq || !count || !staging || !aligned16(lut_host) || !aligned16(staging)) return MOLE_ERR_INVALID_ARG;
-    return launch_fetch(lut_host, uniq, count, max_rows, row_bytes, staging, static_cast<cudaStream_t>(stream));
+    return launch_fetch(lut_host, distinct(const_cast<int32_t *>(uniq), const_cast<int32_t *>(count)), max_rows, row_bytes, staging,
+                        static_cast<cudaStream_t>(stream));
 }
 
 int mole_host_alloc(void **ptr, size_t bytes)
@@ -456,7 +543,7 @@ int mole_offload_prefetch(mole_offload_ctx *c, int b, const int32_t *ids, int M,
     if (rc != MOLE_OK) return rc;
     HotRows hot;
     const bool use_hot = hot_for(c, lut_host_layer, 0, 1, &hot);
-    rc = launch_fetch(lut_host_layer, B.uniq, B.count, M, c->row_bytes, B.staging, st, 1, 0, 0, use_hot ? &hot : nullptr);
+    rc = launch_fetch(lut_host_layer, distinct(B.uniq, B.count), M, c->row_bytes, B.staging, st, 1, 0, 0, use_hot ? &hot : nullptr);
     if (rc != MOLE_OK) return rc;
     MOLE_CUDA_TRY(cudaEventRecord(B.ready, st));
     return MOLE_OK;
@@ -530,8 +617,9 @@ int mole_offload_decode_step(mole_offload_ctx *c, const void *hidden_in, const i
         MOLE_CUDA_TRY(cudaStreamWaitEvent(side, B1.consumed, 0));
     }
     // one dedup for the whole step: every layer looks up the same ids (slot map and distinct ids in buffer 0)
-    int rc = launch_dedup(ids, static_cast<int>(M), c->V, c->table, B0.uniq, B0.slot, B0.count, status, side);
-    if (rc != MOLE_OK) return rc;
+    int rc = MOLE_OK;
+    const bool scan = M <= kFetchThreads;  // ... by the first fetch itself, when a block can
+    if (!scan && (rc = launch_dedup(ids, static_cast<int>(M), c->V, c->table, B0.uniq, B0.slot, B0.count, status, side)) != MOLE_OK) return rc;
     B0.M = B1.M = static_cast<int>(M);
 
     // A staging area holds max_tokens rows; a step of M tokens needs at most M per layer, so one area
@@ -541,34 +629,43 @@ int mole_offload_decode_step(mole_offload_ctx *c, const void *hidden_in, const i
     // bound by the launch + PCIe round trip of every fetch, not by the link.
     int g = static_cast<int>(c->max_tokens / M);
     g = g < 1 ? 1 : (g > L ? L : g);
-    // ... but unless the whole step's rows are a small transfer, keep at least three groups so that all fetches
-    // but the first run under the previous group's layers.  Small: 256 KB (measured, one token of the 410M shape,
+    // ... but unless the whole step's rows are a small transfer, make two or three groups so that all fetches
+    // but the first run under the previous group's layers (next_group).  Small: 256 KB (measured, one token of the 410M shape,
     // 786 KB per step: 54.9 -> 49.8 us with three groups); 1 MB when a hot-row cache is set, since most of a
     // small step's rows then do not cross the link at all (42 us in one group against 45 us in three).
     const long long small_step = c->hot_rows > 0 ? (1LL << 20) : (1LL << 18);
-    if (M * c->row_bytes * L > small_step && g > (L + 2) / 3) g = (L + 2) / 3;
-    const int groups = (L + g - 1) / g;
+    const bool split = M * c->row_bytes * L > small_step;
     const long long area = M * c->row_bytes;  // one layer's rows inside a staging area
-    auto fetch = [&](int k) -> int {
+    auto size_of = [&](int first) { return split ? next_group(L - first, L, g, area) : (g < L - first ? g : L - first); };
+    int groups = 0;
+    for (int l = 0; l < L; l += size_of(l)) ++groups;
+    auto fetch = [&](int k, int l0, int n) -> int {
         mole_offload_ctx::Buffer &Bk = c->buf[k & 1];
-        const int l0 = k * g, n = (l0 + g <= L) ? g : L - l0;
         if (k >= 2) MOLE_CUDA_TRY(cudaStreamWaitEvent(side, Bk.consumed, 0));
         const unsigned char *tables = static_cast<const unsigned char *>(lut_host_base) + static_cast<int64_t>(l0) * lut_layer_stride_bytes;
+        DistinctIds q = distinct(B0.uniq, B0.count);
+        if (scan && k == 0) {
+            q.ids = ids;
+            q.slot = B0.slot;
+            q.status = status;
+            q.M = static_cast<int>(M);
+            q.V = c->V;
+        }
         HotRows hot;
         const bool use_hot = hot_for(c, tables, lut_layer_stride_bytes, n, &hot);
-        int r = launch_fetch(tables, B0.uniq, B0.count, static_cast<int>(M), c->row_bytes, Bk.staging, side, n, lut_layer_stride_bytes,
+        int r = launch_fetch(tables, q, static_cast<int>(M), c->row_bytes, Bk.staging, side, n, lut_layer_stride_bytes,
                              area, use_hot ? &hot : nullptr);
         if (r != MOLE_OK) return r;
         MOLE_CUDA_TRY(cudaEventRecord(Bk.ready, side));
         return MOLE_OK;
     };
     const void *src = hidden_in;
-    if ((rc = fetch(0)) != MOLE_OK) return rc;
-    for (int k = 0; k < groups; ++k) {
-        if (k + 1 < groups && (rc = fetch(k + 1)) != MOLE_OK) return rc;  // queued before group k's layers: they overlap
+    if ((rc = fetch(0, 0, size_of(0))) != MOLE_OK) return rc;
+    for (int k = 0, l0 = 0; k < groups; ++k) {
+        const int n = size_of(l0), next = l0 + n;
+        if (k + 1 < groups && (rc = fetch(k + 1, next, size_of(next))) != MOLE_OK) return rc;  // queued before group k's layers: they overlap
         mole_offload_ctx::Buffer &Bk = c->buf[k & 1];
         MOLE_CUDA_TRY(cudaStreamWaitEvent(st, Bk.ready, 0));
-        const int l0 = k * g, n = (l0 + g <= L) ? g : L - l0;
         StepLaunch a;
         a.residual = nullptr;
         a.row_index = B0.slot;  // gather from staging[slot[t]]; slot is -1 for an id outside [0, V)
@@ -617,6 +714,7 @@ int mole_offload_decode_step(mole_offload_ctx *c, const void *hidden_in, const i
             src = dst;
         }
         MOLE_CUDA_TRY(cudaEventRecord(Bk.consumed, st));
+        l0 = next;
     }
     return MOLE_OK;
 }
