@@ -584,11 +584,11 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
     const bool fstep_ok = L > 1 && d_split == 0 && plan_fstep(M, L, N, d, dtype, norm, sms, &fplan);
     const bool cdecode_ok = L == 1 && d_split == 0 && cdecode_shape_ok(dtype, N, d);
     if (kernel == MOLE_KERNEL_DECODE && !(decode_ok || fstep_ok || cdecode_ok)) return MOLE_ERR_UNSUPPORTED_SHAPE;
-    // MOLE_KERNEL_AUTO takes the ring kernel for plain tables, except for the widest layers at up to 128 tokens (the
-    // cluster kernel, see cdecode_preferred): measured on B200, neither the one-block-per-token kernel (chained steps)
-    // nor the fused step built on it beats it -- a decode batch is bound by the latency of one token's dependent
-    // instruction stream, which the two families execute at about the same length.  They run on request
-    // (MOLE_KERNEL_DECODE), and their structure carries the quantised tables.
+    // MOLE_KERNEL_AUTO, plain tables: the prefill kernel for one layer of many tokens (tile_from), the cluster kernel for the widest
+    // layers at up to 128 tokens (cdecode_preferred), the tensor-core step for fused steps of the shapes where it is ahead
+    // (mma_preferred), the ring kernel for the rest.  The one-block-per-token kernel and the fused step built on it run on
+    // request (MOLE_KERNEL_DECODE): a decode batch is bound by the latency of one token's dependent instruction stream, which they
+    // and the ring kernel execute at about the same length.
     if (fstep_ok && kernel == MOLE_KERNEL_DECODE) {
         const FStepVariant v = pick_fstep(N, fplan.db, norm);
         if (!v.fn) return MOLE_ERR_UNSUPPORTED_SHAPE;
