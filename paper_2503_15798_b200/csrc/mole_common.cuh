@@ -99,8 +99,8 @@ EncodeTiledFn encode_tiled();
 // Every layer kernel is launched with programmatic stream serialization: its blocks may be set up while the kernel before it
 // on the stream still runs, and it waits for that kernel itself -- first thing (pdl_enter), or, with MOLE_FLAG_CHAIN, before
 // it reads the hidden state.  Back-to-back launches of one token of a 160M-shaped layer: 4.9 -> 3.4 us.
-// (Not inside a stream capture unless chained: there the attribute costs a graph of one kernel 2 us.)
-int launch_pdl(const void *fn, unsigned grid, unsigned threads, int smem, cudaStream_t stream, void **args, bool chained);
+// (Not inside a stream capture unless chained: there the attribute costs a graph of one kernel 2 us.  `alone`: not at all.)
+int launch_pdl(const void *fn, unsigned grid, unsigned threads, int smem, cudaStream_t stream, void **args, bool chained, bool alone = false);
 
 // kernels that need more than 48 KB of dynamic shared memory opt in once per device
 int ensure_smem_opt_in(const void *fn, int smem);

@@ -725,10 +725,10 @@ static int cached_launch(const StepLaunch &a, const LaunchChoice **out)
     return MOLE_OK;
 }
 
-int launch_pdl(const void *fn, unsigned grid, unsigned threads, int smem, cudaStream_t stream, void **args, bool chained)
+int launch_pdl(const void *fn, unsigned grid, unsigned threads, int smem, cudaStream_t stream, void **args, bool chained, bool alone)
 {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    if (!chained) MOLE_CUDA_TRY(cudaStreamIsCapturing(stream, &capturing));
+    if (!chained && !alone) MOLE_CUDA_TRY(cudaStreamIsCapturing(stream, &capturing));
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = dim3(grid, 1, 1);
@@ -739,7 +739,7 @@ int launch_pdl(const void *fn, unsigned grid, unsigned threads, int smem, cudaSt
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = capturing == cudaStreamCaptureStatusNone ? 1 : 0;
+    cfg.numAttrs = !alone && capturing == cudaStreamCaptureStatusNone ? 1 : 0;
     MOLE_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, args));
     return MOLE_OK;
 }
@@ -833,7 +833,11 @@ int launch_step(const StepLaunch &a)
     p.flags = a.flags;
     p.wait_polls = c->wait_polls;
     void *args[1] = {&p};
-    return launch_pdl(reinterpret_cast<const void *>(c->step_fn), grid, threads, c->smem, a.stream, args, chained);
+    // A fused step with the loops over any N, with more tokens than blocks, starts on an empty machine: set up under the kernel before,
+    // consecutive blocks -- the ones with a token more -- land on the same SM as it gets free (6 layers of 24 x 640, 600 tokens
+    // 90 against 86 us).  Shorter items lose more by the launch than by that (16 x 504: 23.9 against 26.7).
+    const bool alone = !chained && a.L > 1 && a.M > c->grid && plan.n_fast == 0;
+    return launch_pdl(reinterpret_cast<const void *>(c->step_fn), grid, threads, c->smem, a.stream, args, chained, alone);
 }
 
 // One thread per (token, layer): an L2 prefetch of the token's N rows of that layer's table, in pieces of at most
