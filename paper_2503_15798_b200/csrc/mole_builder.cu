@@ -508,9 +508,11 @@ static int launch_gemm(const void *a, long long a_row_stride, long long a_z_stri
     if (rc != MOLE_OK) return rc;
     // Pairs of blocks (50304 rows, 16 x 768 -> 3072: 6.26 -> 5.75 ms alone, 7.23 -> 6.67 ms back to back under the power
     // limit; 2000 rows 286 -> 267 us), unless half of a pair's last tile row would be padding and the rows are so few
-    // (under nine tiles of 128) that this is over a tenth of the work.
+    // (under nine tiles of 128) that this is over a tenth of the work.  Short products with the GELU are bound by the
+    // epilogue, and the two blocks of a pair wait for each other's: single blocks below K = 640 (both GEMMs together, first one
+    // in pairs / single: K = 128 887 / 822 us, 512 316 / 300, 640 907 / 909, 768 180 / 186).
     const int tile_rows1 = (M + kBM - 1) / kBM;
-    const int pair = sms >= 2 && (tile_rows1 % 2 == 0 || tile_rows1 >= 9) ? 1 : 0;
+    const int pair = sms >= 2 && (tile_rows1 % 2 == 0 || tile_rows1 >= 9) && (!gelu || K >= 640) ? 1 : 0;
     rc = make_matrix_map(&map_b, b, K, N, Z, b_row_stride, b_z_stride, gemm_rows_b(pair));
     if (rc != MOLE_OK) return rc;
     rc = make_matrix_map(&map_c, c, N, M, Z, c_row_stride, c_z_stride, 32);
