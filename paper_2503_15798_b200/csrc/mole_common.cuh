@@ -69,6 +69,7 @@ struct StepLaunch {
     long long norm_stride = 0;          // bytes between the scale vectors of consecutive layers
     float norm_eps = 0.f;
     int kernel = 0;  // MOLE_KERNEL_*: which kernel family runs the launch (0: the library's choice)
+    bool first = false;  // the first of a step's chained layers
 };
 int launch_step(const StepLaunch &a);
 

@@ -613,14 +613,18 @@ struct ShapeOf {
 // Blocks per SM to leave registers for.  Left to itself the compiler aims at four and keeps nearly every instantiation to 56
 // registers, which puts the loads of a sweep and of a weighted sum behind one another -- in the one chain that bounds a step.
 // The compiled widths have one or two blocks per SM (their rings fill the shared memory): all the registers they
-// want, 104 for most.  Any other width may be small enough for three: 72.  Rows cut by experts are large: two.  The loops over
-// any N keep nothing in registers.  Measured, us: 12 chained layers of 16 x 768, 256 tokens 39.3 -> 37.1; 24 fused layers of 16 x 1024 with
+// want, 104 for most.  Any other width may be small enough for three: 72.  Rows cut by experts are large: two.  Up to 8
+// experts, and 16 at narrow widths (several lanes to a column group), there is little to load at once and blocks count for more (four
+// chained layers of 8 x 512 at 1000 tokens: 17.5 us, 21.4 at 72 registers), and the loops over any N keep nothing in registers: the compiler's choice.  Measured, us: 12 chained layers of 16 x 768, 256 tokens 39.3 -> 37.1; 24 fused layers of 16 x 1024 with
 // the norm, 64 tokens 37.8 -> 35.4; 3 of 64 x 768, 128 tokens 17.7 -> 13.2; 6 of 32 x 1000, 600 tokens 81 -> 69; one fp32 layer of
-// 16 x 832, 4380 tokens 83 -> 75 (73 at two blocks, with which 4 x 1000 at 700 tokens is 7.8 -> 10.0).
-constexpr int step_min_blocks(int nfast, int mode, int shape) { return nfast == 0 ? 0 : shape ? 1 : mode == 3 ? 2 : 3; }
+// 16 x 832, 4380 tokens 83 -> 75.
+constexpr int step_min_blocks(int nfast, int lanes, int mode, int shape)
+{
+    return nfast < 16 ? 0 : shape ? 1 : mode == 3 ? 2 : nfast == 16 && lanes > 1 ? 0 : 3;
+}
 
 template <typename T, int NFAST, int P, int MODE, int SHAPE, int DIRECT = 0, int NORM = 0>
-__global__ void __launch_bounds__(kMaxConsumers + 32, step_min_blocks(NFAST, MODE, SHAPE)) mole_step_kernel(const StepParams p)
+__global__ void __launch_bounds__(kMaxConsumers + 32, step_min_blocks(NFAST, P, MODE, SHAPE)) mole_step_kernel(const StepParams p)
 {
     using E = Elem<T>;
     constexpr int VEC = E::VEC;

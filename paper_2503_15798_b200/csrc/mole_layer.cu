@@ -1023,6 +1023,7 @@ int mole_decode_step_args(const mole_step_args *a)
         s.out = dst;
         s.L = 1;
         s.flags = l > 0 ? MOLE_FLAG_CHAIN : (a->flags & MOLE_FLAG_CHAIN);
+        s.first = l == 0 && L > 1;
         rc = quant ? launch_quant_layer(s, a->lut_format, a->lut_block, current_wait_polls()) : launch_step(s);
         if (rc != MOLE_OK) return rc;
         src = dst;

@@ -860,8 +860,20 @@ int launch_quant_layer(const StepLaunch &a, int format, int block, uint32_t wait
     int rc = ensure_smem_opt_in(reinterpret_cast<const void *>(v.fn), smem);
     if (rc != MOLE_OK) return rc;
     void *args[1] = {&p};
+    // The first of a step's layers starts on an empty machine while its blocks fill part of it only: with the launches of step after
+    // step set up under one another, the blocks of a layer end up unevenly over the SMs, and stay so (8 layers of the 410M shape,
+    // 256 tokens, 40 against 51 us; 12 of the 160M shape, 300 tokens, 51 against 62).  Not where an SM holds one or two blocks, or
+    // so many that a few more do not matter: there the 2 us of launch count for more.
+    bool alone = false;
+    int sms = 0, resident = 0;
+    if (a.first && !(a.flags & MOLE_FLAG_CHAIN)) {
+        rc = sm_count(&sms);
+        if (rc == MOLE_OK) rc = blocks_per_sm(reinterpret_cast<const void *>(v.fn), a.d / 4, smem, &resident);
+        if (rc != MOLE_OK) return rc;
+        alone = resident >= 3 && resident <= 8 && a.M * 2 > sms && a.M <= static_cast<long long>(resident - 1) * sms;
+    }
     return launch_pdl(reinterpret_cast<const void *>(v.fn), static_cast<unsigned>(a.M), static_cast<unsigned>(a.d / 4), smem, a.stream, args,
-                      (a.flags & MOLE_FLAG_CHAIN) != 0);
+                      (a.flags & MOLE_FLAG_CHAIN) != 0, alone);
 }
 
 // Whether a fused step over quantised tables exists for a shape (the router matrix goes through registers) and is ahead of L
