@@ -19,8 +19,7 @@
 // N/K experts in one contiguous copy, which the copy engine moves three times as fast.  The rows
 // depend only on the id, so they run ahead of the arithmetic and, in a chained launch, ahead of
 // the previous kernel.  A token's hidden state arrives with its first chunk in a small ring of
-// its own (in DIRECT kernels the block's first token excepted: the compute warps load it
-// themselves).  Completion is counted on one mbarrier per slot ("full"); the consumer warps hand
+// its own.  Completion is counted on one mbarrier per slot ("full"); the consumer warps hand
 // a slot back through a second one ("empty").  Otherwise (L == 1, small matrix) the router matrix
 // is loaded once per block and stays.
 //
@@ -569,35 +568,31 @@ __device__ __forceinline__ void drain_ring(uint64_t *full, int stages, int issue
 // measured 10 % faster), 0 = any: 1 = router chunks in the ring, one chunk per item; 2 = router
 // resident, one chunk per item; 3 = router chunks in the ring, several chunks per item, the rows
 // cut by experts (K divides N) instead of by columns.
-// SHAPE: the layer widths of the paper's Table 2 with d, the chunk width and the number of compute
-// threads as constants (0 = any): 1: d = 768; 2: d = 1024; 3: d = 2048 in chunks of 512; 4: d = 2048 in
-// chunks of 1024 (fused steps of at most one token per SM).
-// DIRECT: the compute warps load the hidden state of the block's first token themselves, with plain
-// 16-byte loads, instead of waiting for the producer's bulk copy (a variant of its own because any
-// growth of the loop body costs the other launches 2 - 6 %).
+// SHAPE: the widest layer of the paper's Table 2 with d, the chunk width and the number of compute
+// threads as constants (0 = any): 3: d = 2048 in chunks of 512; 4: d = 2048 in chunks of 1024 (fused
+// steps of at most one token per SM).  (1 and 2, d = 768 and 1024, are the kernels of mole_slice.cuh.)
 // NORM: the router reads RMSNorm(hidden) -- normalised into a buffer of its own in shared memory
 // after the hidden state has landed (layer l of a fused step with the l-th scale vector) -- while
 // the residual stays the hidden state itself (App. A.2 listing).
 template <int SHAPE>
 struct ShapeOf {
-    static constexpr int d = SHAPE == 1 ? 768 : (SHAPE == 2 ? 1024 : 2048);
-    static constexpr int dcc = SHAPE == 1 ? 768 : (SHAPE == 2 ? 1024 : (SHAPE == 3 ? 512 : 1024));
-    static constexpr int consumers = SHAPE == 1 ? 96 : 128;
+    static constexpr int d = 2048;
+    static constexpr int dcc = SHAPE == 3 ? 512 : 1024;
+    static constexpr int consumers = 128;
 };
 // Blocks per SM to leave registers for.  Left to itself the compiler aims at four and keeps nearly every instantiation to 56
 // registers, which puts the loads of a sweep and of a weighted sum behind one another -- in the one chain that bounds a step.
-// The compiled widths have one or two blocks per SM (their rings fill the shared memory): all the registers they
-// want, 104 for most.  Any other width may be small enough for three: 72.  Rows cut by experts are large: two.  Up to 8
+// The compiled width has one or two blocks per SM (its ring fills the shared memory): all the registers it
+// wants.  Any other width may be small enough for three: 72.  Rows cut by experts are large: two.  Up to 8
 // experts, and 16 at narrow widths (several lanes to a column group), there is little to load at once and blocks count for more (four
-// chained layers of 8 x 512 at 1000 tokens: 17.5 us, 21.4 at 72 registers), and the loops over any N keep nothing in registers: the compiler's choice.  Measured, us: 12 chained layers of 16 x 768, 256 tokens 39.3 -> 37.1; 24 fused layers of 16 x 1024 with
-// the norm, 64 tokens 37.8 -> 35.4; 3 of 64 x 768, 128 tokens 17.7 -> 13.2; 6 of 32 x 1000, 600 tokens 81 -> 69; one fp32 layer of
+// chained layers of 8 x 512 at 1000 tokens: 17.5 us, 21.4 at 72 registers), and the loops over any N keep nothing in registers: the compiler's choice.  Measured, us: 3 layers of 64 x 768, 128 tokens 17.7 -> 13.2; 6 of 32 x 1000, 600 tokens 81 -> 69; one fp32 layer of
 // 16 x 832, 4380 tokens 83 -> 75.
 constexpr int step_min_blocks(int nfast, int lanes, int mode, int shape)
 {
     return nfast < 16 ? 0 : shape ? 1 : mode == 3 ? 2 : nfast == 16 && lanes > 1 ? 0 : 3;
 }
 
-template <typename T, int NFAST, int P, int MODE, int SHAPE, int DIRECT = 0, int NORM = 0>
+template <typename T, int NFAST, int P, int MODE, int SHAPE, int NORM = 0>
 __global__ void __launch_bounds__(kMaxConsumers + 32, step_min_blocks(NFAST, P, MODE, SHAPE)) mole_step_kernel(const StepParams p)
 {
     using E = Elem<T>;
@@ -657,10 +652,7 @@ __global__ void __launch_bounds__(kMaxConsumers + 32, step_min_blocks(NFAST, P, 
             bulk_g2s(smem + m.off_hring + static_cast<size_t>(entry) * hid_stride,
                      static_cast<const unsigned char *>(p.hidden) + static_cast<size_t>(t) * d * EB, m.hid_bytes, full + st);
         };
-        // Issue the next chunk; the hidden state (first chunk of a token) only if with_hidden.  With
-        // DIRECT the block's first token is the exception: the compute warps fetch its hidden state
-        // themselves.
-        constexpr int k_first_copied = DIRECT ? 1 : 0;
+        // Issue the next chunk; the hidden state (first chunk of a token) only if with_hidden.
         auto issue = [&](long long ci, bool with_hidden) {
             if (l == 0 && q == 0) {
                 if ((k & 31) == 0) {  // ids of the next 32 tokens of this block, one per lane
@@ -681,7 +673,7 @@ __global__ void __launch_bounds__(kMaxConsumers + 32, step_min_blocks(NFAST, P, 
             if (lane == 0) {
                 meta[st] = valid ? 1 : 0;
                 if (!valid && first && p.status) atomicOr(p.status, MOLE_STATUS_BAD_ID);
-                mbar_expect_tx(full + st, m.chunk_bytes + (first && k >= k_first_copied ? m.hid_bytes : 0u));
+                mbar_expect_tx(full + st, m.chunk_bytes + (first ? m.hid_bytes : 0u));
                 *issued = static_cast<int>(ci + 1 < 0x7fffffff ? ci + 1 : 0x7fffffff);
             }
             __syncwarp();
@@ -711,7 +703,7 @@ __global__ void __launch_bounds__(kMaxConsumers + 32, step_min_blocks(NFAST, P, 
                         bulk_g2s(slot + static_cast<size_t>(j) * piece, src + static_cast<size_t>(j) * d * EB, piece, full + st);
                 }
             }
-            if (with_hidden && first && k >= k_first_copied && lane == 31) hidden_copy(k, he, st);
+            if (with_hidden && first && lane == 31) hidden_copy(k, he, st);
             if (++q == cpi) {
                 q = 0;
                 if (++l == L) {
@@ -734,7 +726,7 @@ __global__ void __launch_bounds__(kMaxConsumers + 32, step_min_blocks(NFAST, P, 
         fence_proxy_async_global();
         if (lane == 31) {
             const int per_tok = L * cpi;  // chunk tok*per_tok is the first chunk of token tok
-            for (int tok = k_first_copied; static_cast<long long>(tok) * per_tok < pre; ++tok)
+            for (int tok = 0; static_cast<long long>(tok) * per_tok < pre; ++tok)
                 hidden_copy(tok, tok % HR, static_cast<int>((static_cast<long long>(tok) * per_tok) % stages));
         }
         for (long long ci = pre; ci < total; ++ci) {
@@ -762,7 +754,6 @@ __global__ void __launch_bounds__(kMaxConsumers + 32, step_min_blocks(NFAST, P, 
         // memory and the block's own rows of `out` -- so that no other warp is left at a barrier; the
         // status word says that the outputs are meaningless.
         bool alive = true;
-        constexpr bool direct = DIRECT != 0;
 
         auto give_up = [&]() {
             if (lane == 0) report_timeout(dead, p.status);
@@ -803,15 +794,6 @@ __global__ void __launch_bounds__(kMaxConsumers + 32, step_min_blocks(NFAST, P, 
                 // the item's hidden state: as loaded (first layer) or as left by the previous layer
                 const uint32_t haddr = (l == 0) ? smem_base + m.off_hring + static_cast<uint32_t>(he) * hid_stride : hid_s;
 
-                if (k == 0 && l == 0 && direct) {
-                    // first token of the block: plain 16-byte loads straight after the grid dependency
-                    // (measured faster than the bulk copy for chained one-token blocks once a launch has
-                    // more than about a hundred of them, slower below)
-                    const uint4 *src = reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(p.hidden) + tbyte);
-                    for (int g = tid; g < d / VEC; g += nc) sts128(haddr + 16u * g, __ldcg(src + g));
-                    named_bar_sync(kBarHidden, nc);
-                }
-
                 // ---- router: partial logits over all d columns ----
                 const uint32_t raddr = NORM ? norm_s : haddr;  // what the router reads: RMSNorm(hidden) or hidden itself
                 const void *norm_w = static_cast<const unsigned char *>(p.norm_weight) + static_cast<size_t>(l) * p.norm_stride;
@@ -833,7 +815,7 @@ __global__ void __launch_bounds__(kMaxConsumers + 32, step_min_blocks(NFAST, P, 
                         release();
                     }
                 } else {
-                    if (k > 0 || !direct) acquire(st, ph);  // the first rows chunk brings the hidden state with it
+                    acquire(st, ph);  // the first rows chunk brings the hidden state with it
                     if constexpr (NORM)
                         rmsnorm_to_shared<T>(haddr, norm_s, norm_w, p.norm_eps, d, partial, kBarHidden, tid, nc, lane, warp,
                                              nwarps);
@@ -905,7 +887,7 @@ __global__ void __launch_bounds__(kMaxConsumers + 32, step_min_blocks(NFAST, P, 
                 } else {
 #pragma unroll 1
                     for (int kk = 0; kk < K; ++kk) {
-                        if (ring || kk > 0 || direct) acquire(st, ph);
+                        if (ring || kk > 0) acquire(st, ph);
                         {
                             const bool valid = meta[st] != 0;
                             const uint32_t off = kk * chunk_cols_bytes;

@@ -11,6 +11,7 @@
 #include "mole_decode.cuh"
 #include "mole_fstep.cuh"
 #include "mole_kernel.cuh"
+#include "mole_slice.cuh"
 
 namespace mole {
 
@@ -217,37 +218,42 @@ int plan_step(long long M, int L, int N, int d, int dtype, int d_split, StepPlan
 }
 
 // A kernel instantiation and its name ("step<storage,NFAST,P,MODE,SHAPE,DIRECT,NORM>" for the ring
-// kernel, "decode<N,NORM>" for the one-block-per-token kernel): what mole_variant() reports, so that a
+// kernel -- SHAPE 1 and 2: the kernels of mole_slice.cuh, MODE 2 a single layer and MODE 1 a fused step, DIRECT 1 from 128 tokens up to
+// four per SM, which once was a kernel of its own and is a part of the name only -- "decode<N,NORM>" for the one-block-per-token kernel): what mole_variant() reports, so that a
 // test can tell which instantiations a workload reaches.
 typedef void (*StepKernel)(const StepParams);
 typedef void (*DecodeKernel)(const DecodeParams);
 struct Variant {
     StepKernel fn;
     const char *name;
+    bool slice = false;  // the kernels of mole_slice.cuh, chosen by slice_kernel()
 };
-#define MOLE_V(T, TN, NF, P, MODE, SHAPE, DIRECT, NORM) \
-    Variant { mole_step_kernel<T, NF, P, MODE, SHAPE, DIRECT, NORM>, "step<" TN "," #NF "," #P "," #MODE "," #SHAPE "," #DIRECT "," #NORM ">" }
-#define MOLE_VB(NF, P, MODE, SHAPE, DIRECT, NORM) MOLE_V(__nv_bfloat16, "bf16", NF, P, MODE, SHAPE, DIRECT, NORM)
-#define MOLE_VF(NF, P, MODE, SHAPE, DIRECT, NORM) MOLE_V(float, "f32", NF, P, MODE, SHAPE, DIRECT, NORM)
+// N = 16, d = 768 and 1024 (SHAPE 1 and 2): mole_slice.cuh
+#define MOLE_VS(MODE, SHAPE, DIRECT, NORM) \
+    Variant { nullptr, "step<bf16,16,1," #MODE "," #SHAPE "," #DIRECT "," #NORM ">", true }
+#define MOLE_V(T, TN, NF, P, MODE, SHAPE, NORM) \
+    Variant { mole_step_kernel<T, NF, P, MODE, SHAPE, NORM>, "step<" TN "," #NF "," #P "," #MODE "," #SHAPE ",0," #NORM ">" }
+#define MOLE_VB(NF, P, MODE, SHAPE, NORM) MOLE_V(__nv_bfloat16, "bf16", NF, P, MODE, SHAPE, NORM)
+#define MOLE_VF(NF, P, MODE, SHAPE, NORM) MOLE_V(float, "f32", NF, P, MODE, SHAPE, NORM)
 static const Variant kNoVariant = {nullptr, "none"};
 
 // bf16, compile-time launch flags (MODE 1, 2, 3), any of the unrolled N
 #define MOLE_PICK_N_BF16(P, MODE, NORM)                      \
     switch (n_fast) {                                        \
-        case 4: return MOLE_VB(4, P, MODE, 0, 0, NORM);      \
-        case 8: return MOLE_VB(8, P, MODE, 0, 0, NORM);      \
-        case 16: return MOLE_VB(16, P, MODE, 0, 0, NORM);    \
-        case 32: return MOLE_VB(32, P, MODE, 0, 0, NORM);    \
-        case 64: return MOLE_VB(64, P, MODE, 0, 0, NORM);    \
+        case 4: return MOLE_VB(4, P, MODE, 0, NORM);      \
+        case 8: return MOLE_VB(8, P, MODE, 0, NORM);      \
+        case 16: return MOLE_VB(16, P, MODE, 0, NORM);    \
+        case 32: return MOLE_VB(32, P, MODE, 0, NORM);    \
+        case 64: return MOLE_VB(64, P, MODE, 0, NORM);    \
         default: return kNoVariant;                          \
     }
 #define MOLE_PICK_N_F32(P, MODE, NORM)                       \
     switch (n_fast) {                                        \
-        case 4: return MOLE_VF(4, P, MODE, 0, 0, NORM);      \
-        case 8: return MOLE_VF(8, P, MODE, 0, 0, NORM);      \
-        case 16: return MOLE_VF(16, P, MODE, 0, 0, NORM);    \
-        case 32: return MOLE_VF(32, P, MODE, 0, 0, NORM);    \
-        case 64: return MOLE_VF(64, P, MODE, 0, 0, NORM);    \
+        case 4: return MOLE_VF(4, P, MODE, 0, NORM);      \
+        case 8: return MOLE_VF(8, P, MODE, 0, NORM);      \
+        case 16: return MOLE_VF(16, P, MODE, 0, NORM);    \
+        case 32: return MOLE_VF(32, P, MODE, 0, NORM);    \
+        case 64: return MOLE_VF(64, P, MODE, 0, NORM);    \
         default: return kNoVariant;                          \
     }
 #define MOLE_PICK_BF16(MODE)                               \
@@ -273,24 +279,22 @@ static Variant pick_f32(int n_fast, int lanes)
 static Variant pick_kernel(int dtype, int n_fast, int lanes, int chunks, int in_ring, int d, int dcc, int consumers,
                            int by_expert, bool direct)
 {
-    // the layer widths of the paper's Table 2 (160M, 410M and 1B models) with their sizes compiled in;
-    // `direct`: single-layer launches of 128 tokens up to one token per resident block, where the compute
-    // warps loading the hidden state themselves measured 6 % faster per chained layer (slower below)
+    // the layer widths of the paper's Table 2 (160M, 410M and 1B models) with their sizes compiled in
     if (dtype == MOLE_DTYPE_BF16) {
         if (n_fast == 16 && lanes == 1 && chunks == 1 && d == 768 && consumers == 96)
-            return in_ring ? MOLE_VB(16, 1, 1, 1, 0, 0) : (direct ? MOLE_VB(16, 1, 2, 1, 1, 0) : MOLE_VB(16, 1, 2, 1, 0, 0));
+            return in_ring ? MOLE_VS(1, 1, 0, 0) : (direct ? MOLE_VS(2, 1, 1, 0) : MOLE_VS(2, 1, 0, 0));
         if (n_fast == 16 && lanes == 1 && chunks == 1 && d == 1024 && consumers == 128)
-            return in_ring ? MOLE_VB(16, 1, 1, 2, 0, 0) : (direct ? MOLE_VB(16, 1, 2, 2, 1, 0) : MOLE_VB(16, 1, 2, 2, 0, 0));
+            return in_ring ? MOLE_VS(1, 2, 0, 0) : (direct ? MOLE_VS(2, 2, 1, 0) : MOLE_VS(2, 2, 0, 0));
         if (n_fast == 32 && lanes == 2 && chunks == 4 && d == 2048 && dcc == 512 && consumers == 128 && by_expert)
-            return MOLE_VB(32, 2, 3, 3, 0, 0);
+            return MOLE_VB(32, 2, 3, 3, 0);
         if (n_fast == 32 && lanes == 2 && chunks == 2 && d == 2048 && dcc == 1024 && consumers == 128 && by_expert)
-            return MOLE_VB(32, 2, 3, 4, 0, 0);
+            return MOLE_VB(32, 2, 3, 4, 0);
         if (by_expert) return pick_bf16_3(n_fast, lanes);
     }
     if (n_fast == 0) {
         if (dtype == MOLE_DTYPE_BF16)
-            return lanes == 4 ? MOLE_VB(0, 4, 0, 0, 0, 0) : (lanes == 2 ? MOLE_VB(0, 2, 0, 0, 0, 0) : MOLE_VB(0, 1, 0, 0, 0, 0));
-        return lanes == 4 ? MOLE_VF(0, 4, 0, 0, 0, 0) : (lanes == 2 ? MOLE_VF(0, 2, 0, 0, 0, 0) : MOLE_VF(0, 1, 0, 0, 0, 0));
+            return lanes == 4 ? MOLE_VB(0, 4, 0, 0, 0) : (lanes == 2 ? MOLE_VB(0, 2, 0, 0, 0) : MOLE_VB(0, 1, 0, 0, 0));
+        return lanes == 4 ? MOLE_VF(0, 4, 0, 0, 0) : (lanes == 2 ? MOLE_VF(0, 2, 0, 0, 0) : MOLE_VF(0, 1, 0, 0, 0));
     }
     if (dtype != MOLE_DTYPE_BF16) return pick_f32(n_fast, lanes);
     if (chunks == 1) return in_ring ? pick_bf16_1(n_fast, lanes) : pick_bf16_2(n_fast, lanes);
@@ -301,12 +305,12 @@ static Variant pick_kernel(int dtype, int n_fast, int lanes, int chunks, int in_
 static Variant pick_norm_kernel(int dtype, int n_fast, int lanes)
 {
     if (dtype == MOLE_DTYPE_BF16) {
-        if (n_fast == 0) return lanes == 4 ? MOLE_VB(0, 4, 0, 0, 0, 1) : (lanes == 2 ? MOLE_VB(0, 2, 0, 0, 0, 1) : MOLE_VB(0, 1, 0, 0, 0, 1));
+        if (n_fast == 0) return lanes == 4 ? MOLE_VB(0, 4, 0, 0, 1) : (lanes == 2 ? MOLE_VB(0, 2, 0, 0, 1) : MOLE_VB(0, 1, 0, 0, 1));
         if (lanes == 4) { MOLE_PICK_N_BF16(4, 0, 1) }
         if (lanes == 2) { MOLE_PICK_N_BF16(2, 0, 1) }
         MOLE_PICK_N_BF16(1, 0, 1)
     }
-    if (n_fast == 0) return lanes == 4 ? MOLE_VF(0, 4, 0, 0, 0, 1) : (lanes == 2 ? MOLE_VF(0, 2, 0, 0, 0, 1) : MOLE_VF(0, 1, 0, 0, 0, 1));
+    if (n_fast == 0) return lanes == 4 ? MOLE_VF(0, 4, 0, 0, 1) : (lanes == 2 ? MOLE_VF(0, 2, 0, 0, 1) : MOLE_VF(0, 1, 0, 0, 1));
     if (lanes == 4) { MOLE_PICK_N_F32(4, 0, 1) }
     if (lanes == 2) { MOLE_PICK_N_F32(2, 0, 1) }
     MOLE_PICK_N_F32(1, 0, 1)
@@ -317,18 +321,42 @@ static Variant pick_norm_shape_kernel(const StepPlan &plan, int dtype, int d, bo
     if (dtype != MOLE_DTYPE_BF16) return kNoVariant;
     if (plan.n_fast == 16 && plan.lanes == 1 && plan.d_split == 1) {
         if (!plan.wr_in_ring) {
-            if (d == 768 && plan.consumers == 96) return direct ? MOLE_VB(16, 1, 2, 1, 1, 1) : MOLE_VB(16, 1, 2, 1, 0, 1);
-            if (d == 1024 && plan.consumers == 128) return direct ? MOLE_VB(16, 1, 2, 2, 1, 1) : MOLE_VB(16, 1, 2, 2, 0, 1);
+            if (d == 768 && plan.consumers == 96) return direct ? MOLE_VS(2, 1, 1, 1) : MOLE_VS(2, 1, 0, 1);
+            if (d == 1024 && plan.consumers == 128) return direct ? MOLE_VS(2, 2, 1, 1) : MOLE_VS(2, 2, 0, 1);
         } else {
-            if (d == 768 && plan.consumers == 96) return MOLE_VB(16, 1, 1, 1, 0, 1);
-            if (d == 1024 && plan.consumers == 128) return MOLE_VB(16, 1, 1, 2, 0, 1);
+            if (d == 768 && plan.consumers == 96) return MOLE_VS(1, 1, 0, 1);
+            if (d == 1024 && plan.consumers == 128) return MOLE_VS(1, 2, 0, 1);
         }
     }
     if (plan.n_fast == 32 && plan.lanes == 2 && d == 2048 && plan.consumers == 128 && plan.rows_by_expert) {
-        if (plan.d_split == 4 && plan.dc == 512) return MOLE_VB(32, 2, 3, 3, 0, 1);
-        if (plan.d_split == 2 && plan.dc == 1024) return MOLE_VB(32, 2, 3, 4, 0, 1);
+        if (plan.d_split == 4 && plan.dc == 512) return MOLE_VB(32, 2, 3, 3, 1);
+        if (plan.d_split == 2 && plan.dc == 1024) return MOLE_VB(32, 2, 3, 4, 1);
     }
     return kNoVariant;
+}
+
+// The kernels of mole_slice.cuh: T tokens per block.  One up to one token per SM, two beyond.
+struct SlicePlan {
+    StepKernel fn;
+    int threads, smem;
+    long long grid;
+};
+template <int D, int T, int NORM, int CS>
+static SlicePlan slice_plan(long long M, int L, int sms)
+{
+    constexpr int NW = D / kMmaCols;
+    const long long groups = (M + T - 1) / T;
+    if (L == 1) return {mole_slice_layer_kernel<D, T, NORM>, NW * 32, static_cast<int>(slice_smem(NW, T, 1, NORM).total), groups};
+    constexpr int NB = NW / CS;
+    return {mole_slice_step_kernel<D, T, NORM, CS>, (NB + kCopyWarps) * 32, static_cast<int>(slice_smem(NB, T, slice_slots(NB, T, CS), NORM, CS).total),
+            (groups < sms / CS ? groups : sms / CS) * CS};
+}
+template <int D>
+static SlicePlan slice_plan_d(long long M, int L, bool norm, int sms)
+{
+    if (L > 1 && M * 2 <= sms) return norm ? slice_plan<D, 1, 1, 2>(M, L, sms) : slice_plan<D, 1, 0, 2>(M, L, sms);
+    if (M <= sms) return norm ? slice_plan<D, 1, 1, 1>(M, L, sms) : slice_plan<D, 1, 0, 1>(M, L, sms);
+    return norm ? slice_plan<D, 2, 1, 1>(M, L, sms) : slice_plan<D, 2, 0, 1>(M, L, sms);
 }
 
 // The one-block-per-token kernel (mole_decode.cuh): bf16, N of 4, 8, 16 or 32, d a multiple of 128
@@ -657,7 +685,7 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
     Variant v = kNoVariant;
     if (norm) {
         v = pick_norm_shape_kernel(plan, dtype, d, direct && L == 1);
-        if (!v.fn) {
+        if (!v.fn && !v.slice) {
             rc = plan_step(M, L, N, d, dtype, d_split, &plan, true, sms, true);  // the general kernels cut the rows by columns
             if (rc != MOLE_OK) return rc;
             v = pick_norm_kernel(dtype, plan.n_fast, plan.lanes);
@@ -666,7 +694,7 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
         v = pick_kernel(dtype, plan.n_fast, plan.lanes, plan.d_split, plan.wr_in_ring, d, plan.dc, plan.consumers, plan.rows_by_expert,
                         direct);
     }
-    if (!v.fn) return MOLE_ERR_UNSUPPORTED_SHAPE;
+    if (!v.fn && !v.slice) return MOLE_ERR_UNSUPPORTED_SHAPE;
     if (L == 1 && kernel == MOLE_KERNEL_AUTO && d_split == 0 && tile_shape_ok(dtype, N, d) && M > tile_from(N, d, sms)) {
         c->tile = true;
         rc = plan_tile(M, N, d, norm, sms, prepare, &c->tplan);
@@ -680,6 +708,14 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
     c->name = v.name;
     c->threads = plan.threads;
     c->smem = plan.smem;
+    if (v.slice) {
+        const SlicePlan sp = d == 768 ? slice_plan_d<768>(M, L, norm, sms) : slice_plan_d<1024>(M, L, norm, sms);
+        c->step_fn = sp.fn;
+        c->threads = sp.threads;
+        c->smem = sp.smem;
+        c->grid = sp.grid;
+        return prepare ? ensure_smem_opt_in(reinterpret_cast<const void *>(sp.fn), sp.smem) : MOLE_OK;
+    }
     int per_sm = plan.blocks_per_sm;
     if (prepare) {
         rc = ensure_smem_opt_in(reinterpret_cast<const void *>(v.fn), plan.smem);

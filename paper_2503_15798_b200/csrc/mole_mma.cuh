@@ -178,15 +178,15 @@ struct GateB {
     static constexpr int W = N == 8 ? 1 : 2;    // words per step
     uint32_t part[3][KS][W];
     __device__ __forceinline__ void set(int k, int w, const Split2 &s) { part[0][k][w] = s.hi, part[1][k][w] = s.mid, part[2][k][w] = s.lo; }
-    // e: lane j holds the numerator of expert j % N
-    __device__ __forceinline__ void from_lanes(float e, int lane)
+    // e: lane first + j holds the numerator of expert j
+    __device__ __forceinline__ void from_lanes(float e, int lane, int first = 0)
     {
         const int q = lane & 3;
 #pragma unroll
         for (int k = 0; k < KS; ++k)
 #pragma unroll
             for (int w = 0; w < W; ++w) {
-                const int j = 16 * k + 8 * w + 2 * q;
+                const int j = first + 16 * k + 8 * w + 2 * q;
                 set(k, w, split_pair(__shfl_sync(0xffffffffu, e, j), __shfl_sync(0xffffffffu, e, j + 1)));
             }
     }
@@ -210,6 +210,41 @@ struct GateB {
             for (int w = 0; w < 2 * W; ++w) ones[k][w] = 0x3f803f80u;
         mac(c, ones);
         return c[0];
+    }
+};
+
+// The numerators as B fragments whose columns 0 - 3 are the three parts and their smallest number (split_pair), columns 4 - 7 the
+// same again: one product per tile and step instead of three.  A lane with even q then has the sums of hi and mid, its neighbour
+// that of lo: PartSums adds them.  N = 16.
+struct GateColumns {
+    uint32_t b[2];
+    float esum;  // of this lane's numerators; summed over q: of all
+    // e: lane first + j holds the numerator of expert j
+    __device__ __forceinline__ void from_lanes(float e, int lane, int first)
+    {
+        const int q = lane & 3, part = (lane >> 2) & 3;
+        const bool p0 = part == 0, p1 = part == 1, p2 = part == 2;
+        float v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = __shfl_sync(0xffffffffu, e, first + 8 * (i >> 1) + 2 * q + (i & 1));
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+            float x[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float a = v[2 * w + i], ar = a - __uint_as_float(__float_as_uint(a) & 0xffff0000u);
+                const float al = ar - __uint_as_float(__float_as_uint(ar) & 0xffff0000u);
+                x[i] = p0 ? a : (p1 ? ar : (p2 ? al : 0.f));
+            }
+            const uint32_t hi = __byte_perm(__float_as_uint(v[2 * w]), __float_as_uint(v[2 * w + 1]), 0x7632);
+            b[w] = __vmaxu2(__byte_perm(__float_as_uint(x[0]), __float_as_uint(x[1]), 0x7632), __vminu2(hi, 0x00800080u));
+        }
+        esum = (v[0] + v[1]) + (v[2] + v[3]);
+    }
+    __device__ __forceinline__ float sum() const
+    {
+        const float s = esum + __shfl_xor_sync(0xffffffffu, esum, 1);
+        return s + __shfl_xor_sync(0xffffffffu, s, 2);
     }
 };
 
@@ -268,7 +303,40 @@ struct RowsA {
             v[i] = q1 ? y : x;
         }
     }
+    // ..., `under` while the products are on their way
+    template <typename F>
+    __device__ __forceinline__ void product(const GateColumns &g, int lane, float (&v)[4], F &&under) const
+    {
+        static_assert(KS == 1 && W == 2, "16 experts");
+        float c[8][4];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) c[t][i] = 0.f;
+            mma16(c[t], a[t][0][0], a[t][0][1], a[t][0][2], a[t][0][3], g.b[0], g.b[1]);
+        }
+        under();
+        const bool q0 = (lane & 1) != 0, q1 = (lane & 2) != 0;  // lane q takes tiles q and 4 + q, the rest of their sums from its neighbour
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int base = (i >> 1) * 4, w = (i & 1) * 2;
+            float s[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) s[t] = c[base + t][w] + c[base + t][w + 1];
+            const float even = q1 ? s[2] : s[0], odd = q1 ? s[3] : s[1];
+            v[i] = (q0 ? odd : even) + __shfl_xor_sync(0xffffffffu, q0 ? even : odd, 1);
+        }
+    }
 };
+
+// 1 / sqrt(x) to within an ulp for x >= 0, infinities included: the hardware's reciprocal root and a Newton step whose residual
+// 1 - x r^2 is taken without a rounding of x r (two roundings of the correctly rounded root and division are no closer).
+__device__ __forceinline__ float rsqrt_refined(float x)
+{
+    const float r = rsqrtf(x), s = x * r;
+    const float e = fmaf(-fmaf(x, r, -s), r, fmaf(-s, r, 1.0f));
+    return x > 0.f && x < INFINITY ? fmaf(0.5f * r, e, r) : r;
+}
 
 // RMSNorm's factor 1 / sqrt(mean + eps) on a layer's critical path: the hardware's reciprocal root and one Newton step, within two ulps;
 // where the sum of squares overflows the root is 0 and stays 0.  Against the correctly rounded root and division of the other

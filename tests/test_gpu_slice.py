@@ -1,0 +1,93 @@
+"""The kernels of the two narrow widths (16 experts, d = 768 and 1024): a cluster of two blocks, a block and half a block per token, on
+both sides of each line, against the oracle's chain; a token's bits in every batch and in single, chained and fused launches; ids
+outside the table beside a valid one; bounded waits."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import as_f64, check_gates, check_out, oracle_layer
+from paper_2503_15798_b200 import binding as mole
+from test_gpu_variants import _oracle_chain
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+N, V, SMS = 16, 61, 148
+COUNTS = [1, SMS // 2, SMS // 2 + 1, SMS, SMS + 1, 2 * SMS + 1, 4 * SMS + 3]
+
+
+def _case(d, M, L, norm):
+    g = torch.Generator().manual_seed(d + M + L)
+    luts = torch.empty(L, V, N, d).normal_(0, 0.05, generator=g).to(torch.bfloat16)
+    wrs = torch.empty(L, d, N).normal_(0, 0.02, generator=g).to(torch.bfloat16)
+    hidden = (1.5 * torch.empty(M, d).normal_(0, 1, generator=g)).to(torch.bfloat16)
+    ids = torch.randint(0, V, (M,), generator=g, dtype=torch.int32)
+    gammas = (1.0 + 0.2 * torch.empty(L, d).normal_(0, 1, generator=g)).to(torch.bfloat16) if norm else None
+    return luts, wrs, hidden, ids, gammas
+
+
+@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("d", [768, 1024])
+def test_steps_against_the_oracles_chain_and_bits_in_every_batch(d, norm):
+    L, M = 3, COUNTS[-1]
+    luts, wrs, hidden, ids, gammas = _case(d, M, L, norm)
+    ids[0] = -1      # the first of a pair, and
+    ids[3] = V       # the second, beside valid ones
+    ids[M - 1] = V   # and one that is alone in its block
+    ref, _, _ = _oracle_chain(hidden, ids, luts, wrs, gammas, 1e-5)
+    h, i, lu, w = hidden.to(DEV), ids.to(DEV), luts.to(DEV), wrs.to(DEV)
+    gam = None if gammas is None else gammas.to(DEV)
+    outs = {}
+    for M in COUNTS:
+        for mode in (mole.STEP_FUSED, mole.STEP_CHAINED):
+            x, status = h[:M].contiguous(), torch.zeros(1, dtype=torch.int32, device=DEV)
+            out = mole.decode_step_args(x, i[:M].contiguous(), lu, w, torch.empty_like(x), torch.empty_like(x), status=status, mode=mode, norm_weights=gam, norm_eps=1e-5)
+            assert int(status.item()) == mole.STATUS_BAD_ID
+            outs[M, mode] = out
+    last = outs[COUNTS[-1], mole.STEP_FUSED]
+    err = np.abs(as_f64(last) - ref)
+    slack = L * 1e-3 * float(luts.abs().max()) * N if norm else 0.0  # a rounding tie in a normalised element moves a gate
+    assert (err <= L * 2.0 ** -7 * np.maximum(1.0, np.abs(ref)) + slack).all(), float(err.max())
+    for (M, mode), out in outs.items():
+        assert torch.equal(out, last[:M]), (M, mode)
+    for t in (0, 3, COUNTS[-1] - 1):
+        assert torch.equal(last[t], h[t])
+
+
+@pytest.mark.parametrize("M", [1, SMS, SMS + 2, 301])
+@pytest.mark.parametrize("d", [768, 1024])
+def test_single_layer_with_gates_residual_and_wide_ids(d, M):
+    luts, wrs, hidden, ids, _ = _case(d, M, 1, False)
+    res = torch.empty(M, d).normal_(0, 1, generator=torch.Generator().manual_seed(M)).to(torch.bfloat16)
+    ref, gref, _ = oracle_layer(hidden, ids, luts[0], wrs[0], residual=res)
+    gates = torch.zeros(M, N, dtype=torch.float32, device=DEV)
+    out = mole.layer_forward(hidden.to(DEV), ids.long().to(DEV), luts[0].to(DEV), wrs[0].to(DEV), residual=res.to(DEV), gates_out=gates)
+    check_out(out, ref)
+    check_gates(gates, gref)
+
+
+@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("d", [768, 1024])
+def test_waits_of_the_cluster_that_run_out_are_reported(d, norm):
+    """No polls allowed: the waits for the other block's logits give up.  The launch returns, reports it, writes nothing beyond its
+    rows, and the next launch is right."""
+    M, L, guard = 5, 6, 3
+    luts, wrs, hidden, ids, gammas = _case(d, M, L, norm)
+    x, i, lu, w = hidden.to(DEV), ids.to(DEV), luts.to(DEV), wrs.to(DEV)
+    gam = None if gammas is None else gammas.to(DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    buf = torch.full((M + 2 * guard, d), 12345.0, dtype=torch.bfloat16, device=DEV)
+    out = buf[guard:guard + M]
+
+    def step(o):
+        return mole.decode_step_args(x, i, lu, w, o, None, status=status, mode=mole.STEP_FUSED, norm_weights=gam, norm_eps=1e-5)
+
+    want = step(torch.empty_like(x)).clone()
+    with mole.debug_env(MOLE_DEBUG_WAIT_LIMIT=-1):
+        step(out)
+        torch.cuda.synchronize()
+    assert int(status.item()) & mole.STATUS_TIMEOUT
+    assert (buf[:guard] == 12345.0).all() and (buf[guard + M:] == 12345.0).all()
+    status.zero_()
+    step(out)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and torch.equal(out, want)
