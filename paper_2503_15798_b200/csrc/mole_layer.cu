@@ -346,9 +346,9 @@ static SlicePlan slice_plan(long long M, int L, int sms)
 {
     constexpr int NW = D / kMmaCols;
     const long long groups = (M + T - 1) / T;
-    if (L == 1) return {mole_slice_layer_kernel<D, T, NORM>, NW * 32, static_cast<int>(slice_smem(NW, T, 1, NORM).total), groups};
+    if (L == 1) return {mole_slice_layer_kernel<D, T, NORM>, NW * 32, static_cast<int>(slice_smem(16, NW, T, 1, NORM).total), groups};
     constexpr int NB = NW / CS;
-    return {mole_slice_step_kernel<D, T, NORM, CS>, (NB + kCopyWarps) * 32, static_cast<int>(slice_smem(NB, T, slice_slots(NB, T, CS), NORM, CS).total),
+    return {mole_slice_step_kernel<16, D, T, NORM, CS>, (NB + slice_copy_warps(16)) * 32, static_cast<int>(slice_smem(16, NB, T, slice_slots(16, NB, T, CS), NORM, CS).total),
             (groups < sms / CS ? groups : sms / CS) * CS};
 }
 template <int D>
@@ -357,6 +357,28 @@ static SlicePlan slice_plan_d(long long M, int L, bool norm, int sms)
     if (L > 1 && M * 2 <= sms) return norm ? slice_plan<D, 1, 1, 2>(M, L, sms) : slice_plan<D, 1, 0, 2>(M, L, sms);
     if (M <= sms) return norm ? slice_plan<D, 1, 1, 1>(M, L, sms) : slice_plan<D, 1, 0, 1>(M, L, sms);
     return norm ? slice_plan<D, 2, 1, 1>(M, L, sms) : slice_plan<D, 2, 0, 1>(M, L, sms);
+}
+
+// ... the fused step of 32 x 2048, a token per cluster of four blocks: as many clusters as are resident at once, or one per token
+template <int NORM>
+static int slice_plan_1b(long long M, int sms, bool prepare, SlicePlan *sp)
+{
+    constexpr int CS = 4, NB = 2048 / kMmaCols / CS;
+    *sp = {mole_slice_step_kernel<32, 2048, 1, NORM, CS>, (NB + slice_copy_warps(32)) * 32, static_cast<int>(slice_smem(32, NB, 1, slice_slots(32, NB, 1, CS), NORM, CS).total), 0};
+    int clusters = sms / CS;
+    if (prepare) {
+        int rc = ensure_smem_opt_in(reinterpret_cast<const void *>(sp->fn), sp->smem);
+        if (rc != MOLE_OK) return rc;
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof cfg);
+        cfg.gridDim = dim3(CS, 1, 1);
+        cfg.blockDim = dim3(static_cast<unsigned>(sp->threads), 1, 1);
+        cfg.dynamicSmemBytes = sp->smem;
+        MOLE_CUDA_TRY(cudaOccupancyMaxActiveClusters(&clusters, reinterpret_cast<const void *>(sp->fn), &cfg));
+        if (clusters < 1) clusters = 1;
+    }
+    sp->grid = (M < clusters ? M : clusters) * CS;
+    return MOLE_OK;
 }
 
 // The one-block-per-token kernel (mole_decode.cuh): bf16, N of 4, 8, 16 or 32, d a multiple of 128
@@ -652,6 +674,20 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
         rc = plan_mma(M, N, d, norm, sms, prepare, &c->mplan);
         if (rc != MOLE_OK) return rc;
         if (!c->mplan.fits) c->mma = false;  // not all tokens resident at once (clusters leave SMs unused)
+        if (c->mma && N == 32 && d == 2048 && M * 4 <= sms) {  // the width of Table 2: the kernel with the sizes compiled in (mole_slice.cuh)
+            SlicePlan sp;
+            rc = norm ? slice_plan_1b<1>(M, sms, prepare, &sp) : slice_plan_1b<0>(M, sms, prepare, &sp);
+            if (rc != MOLE_OK) return rc;
+            c->mma = false;
+            c->plan = plan;
+            c->step_fn = sp.fn;
+            c->decode_fn = nullptr;
+            c->name = c->mplan.name;
+            c->threads = sp.threads;
+            c->smem = sp.smem;
+            c->grid = sp.grid;
+            return MOLE_OK;
+        }
     }
     if (cdecode_ok && (kernel == MOLE_KERNEL_DECODE || (kernel == MOLE_KERNEL_AUTO && cdecode_preferred(M, N, sms)))) {
         const DecodeVariant v = pick_cdecode(N, norm);

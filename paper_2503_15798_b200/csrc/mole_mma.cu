@@ -184,6 +184,7 @@ int launch_mma(const StepLaunch &a, const MmaPlan &w, uint32_t wait_polls, bool 
     p.w_slots = w.w_slots;
     p.r_slots = w.r_slots;
     p.norm_eps = a.norm_eps;
+    p.inv_d = 1.0f / static_cast<float>(a.d);
     p.flags = a.flags;
     p.wait_polls = wait_polls;
     void *args[3] = {&w_map, &r_map, &p};

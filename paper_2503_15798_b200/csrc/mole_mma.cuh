@@ -7,8 +7,9 @@
 // mma.m16n8k16 here:
 //   - Router: A = W_r^T (16 experts x 16 columns per step), B = the hidden state: bf16 products, fp32 sums.
 //   - Weighted sum: A = rows^T (16 columns x 16 experts), B = the softmax numerators.  A numerator is an fp32 number and is
-//     never rounded: it is cut into three bf16 parts of 8 bits each (split_pair), and the three products are chained into one
-//     fp32 accumulator.  The sum of the numerators is the same product with A = ones.
+//     never rounded: its three bf16 parts of 8 bits each are columns of the product (GateColumns).  An mma takes 8.2 cycles of a
+//     quarter of an SM (measured), so that a product per part was the longest link of the chain: 16 layers of the 1B shape, 64 tokens
+//     40.8 -> 36.5 us, 12 of 16 x 2048 16.1 -> 14.8, of 32 x 1024 with the norm 27.0 -> 23.9.
 // Split.  Warp w owns the 128 columns 128w .. of everything: of the hidden state, of every row, of the output, and those
 // columns are also its share of the router product.  So what a layer's router needs from the layer before is what the same
 // warp has just computed, and warps exchange nothing but N partial logits per token: one meeting per layer.  (RMSNorm in front
@@ -17,12 +18,11 @@
 // Data.  One producer warp streams router matrices and rows, whole boxes by tensor copy with the 128-byte swizzle, so that
 // ldmatrix reads either without bank conflicts; a warp loads the next layer's router fragments and its rows while it waits for
 // the logits of the others.
-// Measured, ring kernel / here, us per step: 16 layers of the 1B shape, 1 token 47.6 / 23.9, 16 tokens 48.2 / 25.2 (46.4 for chained
-// launches of the cluster kernel), 64 tokens 53.2 / 39.8; 10 layers of 8 x 1024, 40 tokens 17.6 / 10.8, 250 tokens 19.1 / 15.4; 12 layers
-// of 32 x 1024, 64 tokens 24.7 / 18.9, of 32 x 512, 140 tokens 19.9 / 15.4, of 16 x 384 with the norm, 64 tokens 30.2 / 15.2, of 16 x 2048
-// 24.0 / 16.1.  At d = 768 and 1024 with N = 16, for which the ring kernel is compiled to size, there is nothing in it (17.8 against
-// 16.4 for 12 layers of 768): clock stamps give 1 300 cycles per layer to the chain itself and the rest to the shared-memory port,
-// through which matrix and rows pass twice.
+// Measured, ring kernel / here, us per step: 16 layers of the 1B shape, 64 tokens 53.2 / 36.5 (up to one block per SM: mole_slice.cuh); 10
+// layers of 8 x 1024, 250 tokens 19.1 / 15.4; 12 layers with the norm, 64 tokens, of 16 x 384 30.2 / 14.8, of 16 x 2048 - / 20.4.
+// The norm: a lane adds up one slice and forms one root, and the scales of the layer after stay as they were loaded until they are
+// used (widened at once they were waited for at once, 300 cycles of every layer): 1B shape, 64 tokens 55.9 -> 45.7, of 16 x 2048 24.0 -> 20.4,
+// of 8 x 2048 23.2 -> 21.1.
 // The order of every sum is fixed by N and d: a token gets the same bits in any batch.
 #pragma once
 
@@ -44,7 +44,7 @@ struct MmaParams {
     long long rows;
     int d, L;
     int w_slots, r_slots;   // router matrices and rows of the token in flight
-    float norm_eps;
+    float norm_eps, inv_d;
     uint32_t flags, wait_polls;
 };
 
@@ -63,8 +63,8 @@ __host__ __device__ inline MmaSmem mma_smem(int N, int d, int cs, int w_slots, i
     m.off_hid = m.off_r + static_cast<uint32_t>(r_slots) * m.matrix;
     m.off_norm = m.off_hid + static_cast<uint32_t>(dl * 2);
     m.off_partial = m.off_norm + (norm ? static_cast<uint32_t>(dl * 2) : 0u);
-    m.off_ssq = m.off_partial + static_cast<uint32_t>(2 * slices * N * 4);
-    m.off_dead = m.off_ssq + (norm ? static_cast<uint32_t>(2 * slices * 4) : 0u);
+    m.off_ssq = (m.off_partial + static_cast<uint32_t>(2 * slices * N * 4) + 15u) & ~15u;
+    m.off_dead = m.off_ssq + (norm ? static_cast<uint32_t>(2 * slices * 16) : 0u);
     m.off_bars = (m.off_dead + 3 * 4 + 7u) & ~7u;
     m.total = m.off_bars + (4 * kMmaMaxSlots + 4) * 8;
     return m;
@@ -87,28 +87,6 @@ __device__ __forceinline__ void tensor_load_5d(uint32_t smem_dst, const CUtensor
 __device__ __forceinline__ void sts16(uint32_t a, unsigned short v) { asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(v) : "memory"); }
 __device__ __forceinline__ void stsf(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
 __device__ __forceinline__ float ldsf(uint32_t a) { return __uint_as_float(lds32(a)); }
-
-// The three bf16 parts of two fp32 numbers >= 0, packed in pairs: a == hi + mid + lo exactly (8 bits each), but that a mid or lo of
-// zero beside a hi that is not becomes 2^-126, the smallest normal number: zero times an infinite table entry would be NaN
-// where the number times it is infinite, and the sums of finite entries, whose largest numerator is 2^-87 at least, do not see it.
-struct Split2 {
-    uint32_t hi, mid, lo;
-};
-__device__ __forceinline__ Split2 split_pair(float a, float b)
-{
-    const uint32_t ah = __float_as_uint(a) & 0xffff0000u, bh = __float_as_uint(b) & 0xffff0000u;
-    const float ar = a - __uint_as_float(ah), br = b - __uint_as_float(bh);
-    const uint32_t am = __float_as_uint(ar) & 0xffff0000u, bm = __float_as_uint(br) & 0xffff0000u;
-    const float al = ar - __uint_as_float(am), bl = br - __uint_as_float(bm);
-    Split2 s;
-    s.hi = __byte_perm(ah, bh, 0x7632);
-    s.mid = __byte_perm(am, bm, 0x7632);
-    s.lo = __byte_perm(__float_as_uint(al), __float_as_uint(bl), 0x7632);
-    const uint32_t least = __vminu2(s.hi, 0x00800080u);
-    s.mid = __vmaxu2(s.mid, least);
-    s.lo = __vmaxu2(s.lo, least);
-    return s;
-}
 
 // This warp's 128 columns of the router matrix as A fragments (experts x columns).  A matrix [columns][N] lies in rows of 128
 // bytes -- 64 / N columns each -- whose 16-byte pieces are swizzled by the row number.
@@ -171,64 +149,29 @@ struct RouterA {
     }
 };
 
-// A token's softmax numerators as B fragments (experts x 8 equal columns), in three parts
+// A token's softmax numerators as B fragments (experts x 8 columns).  A numerator is an fp32 number >= 0 and is not rounded: it is
+// hi + mid + lo, three bf16 parts of 8 bits each.  Columns 0 - 2 of the product are the parts, columns 4 - 6 the same again: one
+// product per tile and step, of which a lane with even q has the sums of hi and mid and its neighbour that of lo (RowsA).
+// A mid or lo of zero beside a hi that is not becomes 2^-126, the smallest normal number (and so is column 3): zero times an infinite
+// table entry would be NaN where the number times it is infinite, and the sums of finite entries, whose largest numerator is
+// 2^-87 at least, do not see it.
 template <int N>
-struct GateB {
+struct GateColumns {
     static constexpr int KS = N == 32 ? 2 : 1;  // steps of 16 experts
     static constexpr int W = N == 8 ? 1 : 2;    // words per step
-    uint32_t part[3][KS][W];
-    __device__ __forceinline__ void set(int k, int w, const Split2 &s) { part[0][k][w] = s.hi, part[1][k][w] = s.mid, part[2][k][w] = s.lo; }
-    // e: lane first + j holds the numerator of expert j
-    __device__ __forceinline__ void from_lanes(float e, int lane, int first = 0)
-    {
-        const int q = lane & 3;
-#pragma unroll
-        for (int k = 0; k < KS; ++k)
-#pragma unroll
-            for (int w = 0; w < W; ++w) {
-                const int j = first + 16 * k + 8 * w + 2 * q;
-                set(k, w, split_pair(__shfl_sync(0xffffffffu, e, j), __shfl_sync(0xffffffffu, e, j + 1)));
-            }
-    }
-    __device__ __forceinline__ void mac(float (&c)[4], const uint32_t (&a)[KS][2 * W]) const
-    {
-#pragma unroll
-        for (int p = 0; p < 3; ++p)
-#pragma unroll
-            for (int k = 0; k < KS; ++k) {
-                if constexpr (N == 8) mma8(c, a[k][0], a[k][1], part[p][k][0]);
-                else mma16(c, a[k][0], a[k][1], a[k][2], a[k][3], part[p][k][0], part[p][k][1]);
-            }
-    }
-    __device__ __forceinline__ float sum() const  // of the numerators
-    {
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-        uint32_t ones[KS][2 * W];
-#pragma unroll
-        for (int k = 0; k < KS; ++k)
-#pragma unroll
-            for (int w = 0; w < 2 * W; ++w) ones[k][w] = 0x3f803f80u;
-        mac(c, ones);
-        return c[0];
-    }
-};
-
-// The numerators as B fragments whose columns 0 - 3 are the three parts and their smallest number (split_pair), columns 4 - 7 the
-// same again: one product per tile and step instead of three.  A lane with even q then has the sums of hi and mid, its neighbour
-// that of lo: PartSums adds them.  N = 16.
-struct GateColumns {
-    uint32_t b[2];
+    uint32_t b[KS][W];
     float esum;  // of this lane's numerators; summed over q: of all
     // e: lane first + j holds the numerator of expert j
     __device__ __forceinline__ void from_lanes(float e, int lane, int first)
     {
         const int q = lane & 3, part = (lane >> 2) & 3;
         const bool p0 = part == 0, p1 = part == 1, p2 = part == 2;
-        float v[4];
+        float v[2 * W * KS];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = __shfl_sync(0xffffffffu, e, first + 8 * (i >> 1) + 2 * q + (i & 1));
+        for (int i = 0; i < 2 * W * KS; ++i) v[i] = __shfl_sync(0xffffffffu, e, first + 8 * (i >> 1) + 2 * q + (i & 1));
+        esum = 0.f;
 #pragma unroll
-        for (int w = 0; w < 2; ++w) {
+        for (int w = 0; w < W * KS; ++w) {
             float x[2];
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
@@ -237,9 +180,9 @@ struct GateColumns {
                 x[i] = p0 ? a : (p1 ? ar : (p2 ? al : 0.f));
             }
             const uint32_t hi = __byte_perm(__float_as_uint(v[2 * w]), __float_as_uint(v[2 * w + 1]), 0x7632);
-            b[w] = __vmaxu2(__byte_perm(__float_as_uint(x[0]), __float_as_uint(x[1]), 0x7632), __vminu2(hi, 0x00800080u));
+            b[w / W][w % W] = __vmaxu2(__byte_perm(__float_as_uint(x[0]), __float_as_uint(x[1]), 0x7632), __vminu2(hi, 0x00800080u));
+            esum += v[2 * w] + v[2 * w + 1];
         }
-        esum = (v[0] + v[1]) + (v[2] + v[3]);
     }
     __device__ __forceinline__ float sum() const
     {
@@ -252,7 +195,7 @@ struct GateColumns {
 // [64-column chunk][expert][128 bytes], 16-byte pieces swizzled by the expert.
 template <int N>
 struct RowsA {
-    static constexpr int KS = GateB<N>::KS, W = GateB<N>::W;
+    static constexpr int KS = GateColumns<N>::KS, W = GateColumns<N>::W;
     uint32_t a[8][KS][2 * W];
     static __device__ __forceinline__ uint32_t lane_offset(int lane)
     {
@@ -277,44 +220,23 @@ struct RowsA {
                     ldsm_x4_trans(a[t][k], (addr + static_cast<uint32_t>(t >> 2) * (N * 128u) + static_cast<uint32_t>(k) * 2048u) ^ (static_cast<uint32_t>(t & 3) << 5));
         }
     }
-    // v[i]: the sums of this lane's four columns: 16 q + r, 16 q + 8 + r, 64 + 16 q + r, 64 + 16 q + 8 + r  (lane = 4 r + q)
-    __device__ __forceinline__ void product(const GateB<N> &g, int lane, float (&v)[4]) const
-    {
-        float c[8][4];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) c[t][i] = 0.f;
-        }
-#pragma unroll
-        for (int p = 0; p < 3; ++p)
-#pragma unroll
-            for (int k = 0; k < KS; ++k)
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    if constexpr (N == 8) mma8(c[t], a[t][k][0], a[t][k][1], g.part[p][k][0]);
-                    else mma16(c[t], a[t][k][0], a[t][k][1], a[t][k][2], a[t][k][3], g.part[p][k][0], g.part[p][k][1]);
-                }
-        const bool q0 = (lane & 1) != 0, q1 = (lane & 2) != 0;  // all columns of the product are equal: lane q takes tiles q and 4 + q
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int base = (i >> 1) * 4, w = (i & 1) * 2;
-            const float x = q0 ? c[base + 1][w] : c[base][w], y = q0 ? c[base + 3][w] : c[base + 2][w];
-            v[i] = q1 ? y : x;
-        }
-    }
-    // ..., `under` while the products are on their way
+    // v[i]: the sums of this lane's four columns: 16 q + r, 16 q + 8 + r, 64 + 16 q + r, 64 + 16 q + 8 + r  (lane = 4 r + q); `under` is
+    // done while the products are on their way
     template <typename F>
-    __device__ __forceinline__ void product(const GateColumns &g, int lane, float (&v)[4], F &&under) const
+    __device__ __forceinline__ void product(const GateColumns<N> &g, int lane, float (&v)[4], F &&under) const
     {
-        static_assert(KS == 1 && W == 2, "16 experts");
         float c[8][4];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) {
+        for (int t = 0; t < 8; ++t)
 #pragma unroll
             for (int i = 0; i < 4; ++i) c[t][i] = 0.f;
-            mma16(c[t], a[t][0][0], a[t][0][1], a[t][0][2], a[t][0][3], g.b[0], g.b[1]);
-        }
+#pragma unroll
+        for (int k = 0; k < KS; ++k)
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                if constexpr (N == 8) mma8(c[t], a[t][k][0], a[t][k][1], g.b[k][0]);
+                else mma16(c[t], a[t][k][0], a[t][k][1], a[t][k][2], a[t][k][3], g.b[k][0], g.b[k][1]);
+            }
         under();
         const bool q0 = (lane & 1) != 0, q1 = (lane & 2) != 0;  // lane q takes tiles q and 4 + q, the rest of their sums from its neighbour
 #pragma unroll
@@ -336,16 +258,6 @@ __device__ __forceinline__ float rsqrt_refined(float x)
     const float r = rsqrtf(x), s = x * r;
     const float e = fmaf(-fmaf(x, r, -s), r, fmaf(-s, r, 1.0f));
     return x > 0.f && x < INFINITY ? fmaf(0.5f * r, e, r) : r;
-}
-
-// RMSNorm's factor 1 / sqrt(mean + eps) on a layer's critical path: the hardware's reciprocal root and one Newton step, within two ulps;
-// where the sum of squares overflows the root is 0 and stays 0.  Against the correctly rounded root and division of the other
-// kernels, us per step: 12 layers of 16 x 1280, 64 tokens 30.7 -> 27.2, of 16 x 2048 34.7 -> 30.9; 16 of the 1B shape, 16 tokens 37.4 -> 35.1.
-__device__ __forceinline__ float rms_scale_newton(float total, int d, float eps)
-{
-    const float x = total / static_cast<float>(d) + eps;
-    const float r = rsqrtf(x);
-    return x > 0.f && x < INFINITY ? fmaf(r * 0.5f, fmaf(-x * r, r, 1.0f), r) : r;
 }
 
 // Softmax numerator of a logit; `group`: lanes (a power of two) that hold one token's logits.  The maximum is subtracted only
@@ -506,10 +418,10 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 3
         if (lane < 16) cp_async16(hid + lane * 16, static_cast<const unsigned char *>(p.hidden) + token_bytes);
         cp_async_commit();
         const unsigned char *norm_g = static_cast<const unsigned char *>(p.norm_weight) + slice_bytes + own_off;
-        float wgt_next[4] = {0.f, 0.f, 0.f, 0.f};
+        unsigned short wgt_next[4] = {0, 0, 0, 0};  // as loaded: widened here they would be waited for here
         auto load_norm = [&](int l) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) wgt_next[i] = bf16_bits_to_float(__ldg(reinterpret_cast<const unsigned short *>(norm_g + static_cast<size_t>(l) * p.norm_stride + col(i))));
+            for (int i = 0; i < 4; ++i) wgt_next[i] = __ldg(reinterpret_cast<const unsigned short *>(norm_g + static_cast<size_t>(l) * p.norm_stride + col(i)));
         };
         if constexpr (NORM) load_norm(0);
 
@@ -524,27 +436,34 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 3
             const bool last = l == L - 1;
             if (CS > 1 && tid == 0) {
                 mbar_expect_tx(xbar + buf, part_set);
-                if (NORM) mbar_expect_tx(sbar + buf, static_cast<uint32_t>(slices * 4));
+                if (NORM) mbar_expect_tx(sbar + buf, static_cast<uint32_t>(slices * 16));
             }
             if constexpr (NORM) {
                 // y = (x / sqrt(mean(x^2) + eps)) * w, rounded once to bf16: what the router reads
-                const uint32_t sq = base + m.off_ssq + buf * static_cast<uint32_t>(slices * 4);
-                const float ss = warp_sum(fmaf(h[3], h[3], fmaf(h[2], h[2], fmaf(h[1], h[1], h[0] * h[0]))));
-                if (lane < CS) {
-                    const uint32_t at = sq + static_cast<uint32_t>(slice) * 4u;
+                const uint32_t sq = base + m.off_ssq + buf * static_cast<uint32_t>(slices * 16);
+                float ss = fmaf(h[1], h[1], h[0] * h[0]) + fmaf(h[3], h[3], h[2] * h[2]);
+#pragma unroll
+                for (int o = 16; o >= 4; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                if (lane < 4 * CS) {  // (the sums are the same in all lanes with the same last two bits)
+                    const uint32_t at = sq + static_cast<uint32_t>(slice * 4 + (lane & 3)) * 4u, to = static_cast<uint32_t>(lane) >> 2;
                     if constexpr (CS == 1) stsf(at, ss);
-                    else cluster_push_f32(cluster_map(at, lane), ss, cluster_map(smem_u32(sbar + buf), lane));
+                    else cluster_push_f32(cluster_map(at, to), ss, cluster_map(smem_u32(sbar + buf), to));
                 }
                 if constexpr (CS == 1) named_bar_sync(3, nc);
                 else acquire_cluster(sbar + buf, xph);
-                float v[kMmaMaxSlices], total = 0.f;
+                // lane l adds up slice l % 16, then they add up each other's: one load and one root per lane
+                const int from = lane & 15;
+                const uint4 part = lds128(sq + static_cast<uint32_t>(from < slices ? from : 0) * 16u);
+                float total = (__uint_as_float(part.x) + __uint_as_float(part.y)) + (__uint_as_float(part.z) + __uint_as_float(part.w));
+                if (from >= slices) total = 0.f;
 #pragma unroll
-                for (int w = 0; w < kMmaMaxSlices; ++w) v[w] = w < slices ? ldsf(sq + static_cast<uint32_t>(w) * 4u) : 0.f;
+                for (int o = 8; o >= 1; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+                // total / d, correctly rounded (an infinite total would make the correction NaN)
+                float mean = total * p.inv_d;
+                mean = total < INFINITY ? fmaf(fmaf(-mean, static_cast<float>(d), total), p.inv_d, mean) : total;
+                const float rinv = rsqrt_refined(mean + p.norm_eps);
 #pragma unroll
-                for (int w = 0; w < kMmaMaxSlices; ++w) total += v[w];  // slices in ascending order
-                const float rinv = rms_scale_newton(total, d, p.norm_eps);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) sts16(router_in + own_off + col(i), float_to_bf16_bits((h[i] * rinv) * wgt_next[i]));
+                for (int i = 0; i < 4; ++i) sts16(router_in + own_off + col(i), float_to_bf16_bits((h[i] * rinv) * bf16_bits_to_float(wgt_next[i])));
                 if (!last) load_norm(l + 1);
                 __syncwarp();
             }
@@ -588,13 +507,11 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 3
                 for (int w = 0; w < kMmaMaxSlices; w += 2) ze += v[w], zo += v[w + 1];
                 e = softmax_part(ze + zo, N);
             }
-            GateB<N> g;
-            g.from_lanes(e, lane);
-            const float inv = __frcp_rn(g.sum());
-
             // ---- weighted sum of the rows (Eq. 8), residual, one rounding ----
-            float v[4];
-            rows.product(g, lane, v);
+            float v[4], inv;
+            GateColumns<N> g;
+            g.from_lanes(e, lane, 0);
+            rows.product(g, lane, v, [&]() { inv = __frcp_rn(g.sum()); });
             __syncwarp();
             if (lane == 0) mbar_arrive(rempty + rs);
             if (++rs == RS) rs = 0, rph ^= 1u;

@@ -1,5 +1,6 @@
 // The layer and the fused L-layer step of the two narrow widths of the paper's Table 2 (N = 16 experts, d = 768 and 1024, bf16) for
-// sm_100a: what mole_variant calls the step kernels of SHAPE 1 and 2.  (Eq. 4 and Eq. 8 of arXiv 2503.15798.)
+// sm_100a -- what mole_variant calls the step kernels of SHAPE 1 and 2 -- and the fused step of its widest (N = 32, d = 2048) while every
+// token has four SMs to itself, the bits of mma<32,..,4>.  (Eq. 4 and Eq. 8 of arXiv 2503.15798.)
 //
 // What bounds them.  A token's layer is a dependent chain -- router product, a sum over the block, a softmax, a weighted sum -- and a
 // decode batch has one or two tokens per SM, so a layer costs the length of the chain, and what it shares the chip's queues with: the
@@ -21,6 +22,8 @@
 // the norm 44.7 / 40.3; 1000 tokens 173 / 129.  Chained, 256 tokens: 12 of 768 35.8 / 31.4, 24 of 1024 73.6 / 72.0 (up to 148 tokens
 // the host's launches are what is left: 2.2 us each).  Of a layer's 1 300 cycles at 64 tokens of d = 1024: router product 125, exchange and loads 370, logits
 // and exp 200, parts of the numerators 95, weighted sum and output 300.
+// The widest layer, 16 layers, 16 tokens, mole_mma.cuh / here: 25.2 / 20.0, with the norm 35.7 / 28.4.  Beyond one block per SM a second
+// round of clusters is no faster than two blocks per SM there (64 tokens 43.7 against 36.5, with the norm 54.9 against 45.7).
 // Tried: rows straight from L2 to registers, packed with byte permutes (no slots, half the port's bytes, but one layer of lead is too
 // little for L2's latency: 256 tokens 14.5 -> 25.8 us); slots freed by a barrier of their own, half a layer earlier (14.5 -> 15.8).
 // The order of every sum is that of one token and fixed by d: single layers, chained and fused steps and any batch give the same bits.
@@ -30,33 +33,34 @@
 
 namespace mole {
 
-constexpr int kSliceN = 16;
-constexpr int kCopyWarps = 4;  // of a fused step: one per quarter of the SM
-constexpr uint32_t kSliceBytes = kMmaCols * kSliceN * 2;  // of a warp: its columns of a router matrix, or of a token's rows
+// copying warps of a fused step: one per quarter of the SM; one in all beside a cluster's four warps
+__host__ __device__ constexpr int slice_copy_warps(int N) { return N == 16 ? 4 : 1; }
+// of a warp: its columns of a router matrix, or of a token's rows
+__host__ __device__ constexpr uint32_t slice_bytes(int N) { return static_cast<uint32_t>(kMmaCols * N * 2); }
 
 // Shared memory of a block of NW warps and T tokens with S slots: [slot][router | token rows][warp] slices, hidden and normalised
 // slices [warp][token], partial logits [2][warp][token][expert], sums of squares [2][token][warp][4], a barrier and a flag.
 struct SliceSmem {
     uint32_t slot, off_hid, off_norm, off_partial, off_ssq, off_bar, total;
 };
-__host__ __device__ constexpr SliceSmem slice_smem(int nw, int tokens, int slots, int norm, int cs = 1)
+__host__ __device__ constexpr SliceSmem slice_smem(int N, int nw, int tokens, int slots, int norm, int cs = 1)
 {
     SliceSmem m{};
-    m.slot = static_cast<uint32_t>(nw) * kSliceBytes * static_cast<uint32_t>(1 + tokens);
+    m.slot = static_cast<uint32_t>(nw) * slice_bytes(N) * static_cast<uint32_t>(1 + tokens);
     m.off_hid = m.slot * static_cast<uint32_t>(slots);
     const uint32_t state = static_cast<uint32_t>(nw * tokens * kMmaCols * 2);
     m.off_norm = m.off_hid + state;
     m.off_partial = m.off_norm + (norm ? state : 0u);
-    m.off_ssq = m.off_partial + static_cast<uint32_t>(2 * cs * nw * tokens * kSliceN * 4);
+    m.off_ssq = m.off_partial + static_cast<uint32_t>(2 * cs * nw * tokens * N * 4);
     m.off_bar = m.off_ssq + (norm ? static_cast<uint32_t>(2 * cs * nw * tokens * 16) : 0u);
     m.total = m.off_bar + 48u;
     return m;
 }
 // slots of a fused step: as many as fit (a block has the SM to itself)
-__host__ __device__ constexpr int slice_slots(int nw, int tokens, int cs = 1)
+__host__ __device__ constexpr int slice_slots(int N, int nw, int tokens, int cs = 1)
 {
     int s = 4;
-    while (s > 2 && slice_smem(nw, tokens, s, 1, cs).total > 227u * 1024u) --s;
+    while (s > 2 && slice_smem(N, nw, tokens, s, 1, cs).total > 227u * 1024u) --s;
     return s;
 }
 
@@ -66,33 +70,34 @@ template <int PENDING>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// This warp's 16 x 128 slice of a token's rows (row: the first expert's row, at the warp's columns) into a slot: [64-column
+// This warp's N x 128 slice of a token's rows (row: the first expert's row, at the warp's columns) into a slot: [64-column
 // half][expert][128 bytes], 16-byte pieces swizzled by the expert (RowsA).
-template <int D>
+template <int N, int D>
 __device__ __forceinline__ void slice_copy_rows(uint32_t slot, const unsigned char *row, int lane)
 {
     const uint32_t e = static_cast<uint32_t>(lane) >> 4, piece = static_cast<uint32_t>(lane) & 15u;
-    const uint32_t dst = slot + (piece >> 3) * 2048u + e * 128u + (((piece & 7u) ^ e) << 4);
+    const uint32_t dst = slot + (piece >> 3) * (N * 128u) + e * 128u + (((piece & 7u) ^ e) << 4);
     const unsigned char *src = row + e * (D * 2u) + piece * 16u;
 #pragma unroll
-    for (uint32_t i = 0; i < 8; ++i) cp_async16((dst ^ ((2u * i & 6u) << 4)) + i * 256u, src + i * (D * 4u));
+    for (uint32_t i = 0; i < N / 2; ++i) cp_async16((dst ^ ((2u * i & 6u) << 4)) + i * 256u, src + i * (D * 4u));
 }
-// ... its 128 x 16 slice of a router matrix (4 KB in one piece): rows of 128 bytes, four columns each, 16-byte pieces swizzled by
+// ... its 128 x N slice of a router matrix (one piece): rows of 128 bytes, 64 / N columns each, 16-byte pieces swizzled by
 // the row (RouterA)
+template <int N>
 __device__ __forceinline__ void slice_copy_router(uint32_t slot, const unsigned char *w, int lane)
 {
     const uint32_t row = static_cast<uint32_t>(lane) >> 3, within = static_cast<uint32_t>(lane) & 7u;
     const uint32_t dst = slot + row * 128u + ((within ^ row) << 4);
     const unsigned char *src = w + lane * 16;
 #pragma unroll
-    for (uint32_t i = 0; i < 8; ++i) cp_async16((dst ^ ((i & 1u) << 6)) + i * 512u, src + i * 512u);
+    for (uint32_t i = 0; i < N / 2; ++i) cp_async16((dst ^ ((i & 1u) << 6)) + i * 512u, src + i * 512u);
 }
 
 // One layer of a block's T tokens from the fragments on: what single layers and fused steps have in common.
 // COUNT: threads at the layer's barrier.  CS: blocks of a cluster that share the token, each NB of its slices: the barrier is then an
 // mbarrier of each block (mbar + 0, 1 by turns), at which the partial logits pushed into it are counted in, and likewise for the
 // sums of squares (mbar + 2, 3).
-template <int D, int T, int NORM, int COUNT_, int CS = 1>
+template <int N, int D, int T, int NORM, int COUNT_, int CS = 1>
 struct SliceLayer {
     static constexpr int NW = D / kMmaCols, NB = NW / CS, NC = NB * 32, COUNT = COUNT_;
     static_assert(CS == 1 || T == 1, "a cluster owns one token");
@@ -143,7 +148,7 @@ struct SliceLayer {
     {
         if constexpr (CS > 1) {
             if (threadIdx.x == 0 && alive) {  // (a barrier whose phase was not waited for takes no arrivals of the next)
-                mbar_expect_tx(mbar + buf, NW * kSliceN * 4);
+                mbar_expect_tx(mbar + buf, NW * N * 4);
                 if (NORM) mbar_expect_tx(mbar + 2 + buf, NW * 16);
             }
         }
@@ -187,13 +192,14 @@ struct SliceLayer {
         }
         if constexpr (CS == 1) named_bar_sync(kBarSquares, NC);
         else wait_cluster(mbar + 2 + buf);
-        // lane l adds up slice l % 8 of token l / 16 (of two), then eight lanes each other's: one load and one root per lane for all tokens
-        const int from = lane & 7;
+        // lane l adds up slice l % 8 of token l / 16 (of two), or slice l % 16, then they add up each other's: one load and one root per lane
+        constexpr int R = NW > 8 ? 16 : 8;
+        const int from = lane & (R - 1);
         const uint4 part = lds128(sq + static_cast<uint32_t>((T == 2 ? lane >> 4 : 0) * NW + (from < NW ? from : 0)) * 16u);
         float total = (__uint_as_float(part.x) + __uint_as_float(part.y)) + (__uint_as_float(part.z) + __uint_as_float(part.w));
         if (from >= NW) total = 0.f;
 #pragma unroll
-        for (int o = 4; o >= 1; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+        for (int o = R / 2; o >= 1; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
         float mean = total * (1.0f / D);
         if constexpr ((D & (D - 1)) != 0)  // the correctly rounded quotient (an infinite total would make the correction NaN)
             mean = total < INFINITY ? fmaf(fmaf(-mean, static_cast<float>(D), total), 1.0f / D, mean) : total;
@@ -207,24 +213,30 @@ struct SliceLayer {
         __syncwarp();
     }
     // this warp's partial logits
-    __device__ __forceinline__ void logits(const RouterA<kSliceN> &w, uint32_t buf)
+    __device__ __forceinline__ void logits(const RouterA<N> &w, uint32_t buf)
     {
-        float z[1][4];
+        float z[N / 16][4];
         w.product((NORM ? normed : hid) + b_off, z);
         const int r = lane >> 2, q = lane & 3;  // columns 2q, 2q + 1 of the product; token 0's are 0 - 3
         if constexpr (CS == 1) {
             if (q == 0 || (T == 2 && q == 2)) {
-                const uint32_t at = partial + (buf * NW + static_cast<uint32_t>(warp)) * (T * kSliceN * 4u) + static_cast<uint32_t>((T == 2 ? q >> 1 : 0) * kSliceN + r) * 4u;
+                const uint32_t at = partial + (buf * NW + static_cast<uint32_t>(warp)) * (T * N * 4u) + static_cast<uint32_t>((T == 2 ? q >> 1 : 0) * N + r) * 4u;
                 stsf(at, z[0][0]);
                 stsf(at + 32u, z[0][2]);
             }
-        } else {  // all columns are equal: lane q pushes to block q / 2, experts r or 8 + r
-            static_assert(CS <= 2, "four lanes have an expert's logit");
-            const uint32_t at = partial + (buf * NW + static_cast<uint32_t>(slice)) * (kSliceN * 4u) + static_cast<uint32_t>(r + 8 * (q & 1)) * 4u, to = static_cast<uint32_t>(q) >> 1;
+        } else if constexpr (CS == 2) {  // all columns are equal: lane q pushes to block q / 2, experts r or 8 + r
+            static_assert(N == 16, "four lanes have an expert's logit");
+            const uint32_t at = partial + (buf * NW + static_cast<uint32_t>(slice)) * (N * 4u) + static_cast<uint32_t>(r + 8 * (q & 1)) * 4u, to = static_cast<uint32_t>(q) >> 1;
             cluster_push_f32(cluster_map(at, to), (q & 1) ? z[0][2] : z[0][0], cluster_map(smem_u32(mbar + buf), to));
+        } else {  // ... to block q, every expert it has
+            static_assert(CS == 4, "four lanes have an expert's logit");
+            const uint32_t at = cluster_map(partial + (buf * NW + static_cast<uint32_t>(slice)) * (N * 4u) + static_cast<uint32_t>(r) * 4u, q);
+            const uint32_t bar = cluster_map(smem_u32(mbar + buf), q);
+#pragma unroll
+            for (int i = 0; i < N / 8; ++i) cluster_push_f32(at + 32u * i, z[i >> 1][2 * (i & 1)], bar);
         }
     }
-    // softmax numerators (Eq. 4): lane 16 j + e has token j's expert e (one token: both halves have it).  `loads`: what is to be
+    // softmax numerators (Eq. 4): lane 16 j + e has token j's expert e (one token of 16: both halves have it).  `loads`: what is to be
     // asked of shared memory while the numerators and the weighted sum are computed -- not before, where the partial logits and
     // the state would queue behind it
     template <typename F>
@@ -232,22 +244,22 @@ struct SliceLayer {
     {
         if constexpr (CS == 1) named_bar_sync(kBarLogits, COUNT);
         else wait_cluster(mbar + buf);
-        const uint32_t at = partial + buf * static_cast<uint32_t>(NW * T * kSliceN * 4) + static_cast<uint32_t>(T == 2 ? lane : lane & 15) * 4u;
+        const uint32_t at = partial + buf * static_cast<uint32_t>(NW * T * N * 4) + static_cast<uint32_t>(T == 2 || N == 32 ? lane : lane & 15) * 4u;
         float v[NW];
 #pragma unroll
-        for (int i = 0; i < NW; ++i) v[i] = ldsf(at + static_cast<uint32_t>(i) * (T * kSliceN * 4u));
+        for (int i = 0; i < NW; ++i) v[i] = ldsf(at + static_cast<uint32_t>(i) * (T * N * 4u));
         loads();
         float even = v[0], odd = v[1];
 #pragma unroll
         for (int i = 2; i < NW; i += 2) even += v[i], odd += v[i + 1];
-        return softmax_part(even + odd, kSliceN);
+        return softmax_part(even + odd, N);
     }
     // weighted sum (Eq. 8), residual, one rounding: the new state, in registers and in the hidden slices.  after(j): token j's rows
     // have been given to the product
     template <typename F>
-    __device__ __forceinline__ void weighted(const RowsA<kSliceN> (&rows)[T], float e, const bool (&valid)[T], F &&after)
+    __device__ __forceinline__ void weighted(const RowsA<N> (&rows)[T], float e, const bool (&valid)[T], F &&after)
     {
-        GateColumns g[T];
+        GateColumns<N> g[T];
 #pragma unroll
         for (int j = 0; j < T; ++j) g[j].from_lanes(e, lane, 16 * j);
 #pragma unroll
@@ -278,14 +290,14 @@ __device__ __forceinline__ long long slice_id(const StepParams &p, long long t)
 // i % S holds item i's rows and router matrix.  The copying warp arrives at item i's barrier when the rows of item i + 1 and the
 // router matrix of item i + 2 have landed; ahead of it the compute warps have taken item i's rows and router matrix into registers,
 // behind it they take item i + 1's.  So it frees the slot of item i for item i + S.
-template <int D, int T, int NORM, int CS>
-__global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS + kCopyWarps) * 32, 1) mole_slice_step_kernel(const StepParams p)
+template <int N, int D, int T, int NORM, int CS>
+__global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS + slice_copy_warps(N)) * 32, 1) mole_slice_step_kernel(const StepParams p)
 {
-    constexpr int NW = D / kMmaCols / CS, S = slice_slots(NW, T, CS);  // warps of this block
+    constexpr int NW = D / kMmaCols / CS, S = slice_slots(N, NW, T, CS), kCopyWarps = slice_copy_warps(N);  // warps of this block
     constexpr int AHEAD = CS > 1 ? 2 : 1;  // items landed before an item's barrier, beside its own
     static_assert(S > AHEAD, "slots");
-    using Layer = SliceLayer<D, T, NORM, (NW + kCopyWarps) * 32, CS>;
-    constexpr SliceSmem m = slice_smem(NW, T, S, NORM, CS);
+    using Layer = SliceLayer<N, D, T, NORM, (NW + kCopyWarps) * 32, CS>;
+    constexpr SliceSmem m = slice_smem(N, NW, T, S, NORM, CS);
     extern __shared__ __align__(1024) unsigned char smem[];
 
     pdl_enter(p.flags);
@@ -309,7 +321,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
     if (warp >= NW) {
         // ================= copying warps: warp NW + k copies the slices k, k + kCopyWarps, .. =================
         const int first = warp - NW;
-        const unsigned char *w0 = static_cast<const unsigned char *>(p.w_router) + rank * (NW * kSliceBytes), *w = w0;
+        const unsigned char *w0 = static_cast<const unsigned char *>(p.w_router) + rank * (NW * slice_bytes(N)), *w = w0;
         const unsigned char *row[T];
         long long g = g0, next_id[T];  // the group whose rows are issued next; ids of the group after
         int l = 0, s = 0;
@@ -321,7 +333,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
 #pragma unroll
             for (int j = 0; j < T; ++j) {
                 const bool ok = next_id[j] >= 0 && next_id[j] < p.rows;  // otherwise row 0 is fetched and its term dropped
-                row[j] = static_cast<const unsigned char *>(p.lut) + static_cast<size_t>(ok ? next_id[j] : 0) * (kSliceN * D * 2) + rank * (NW * 256u);
+                row[j] = static_cast<const unsigned char *>(p.lut) + static_cast<size_t>(ok ? next_id[j] : 0) * (N * D * 2) + rank * (NW * 256u);
             }
             fetch_ids(g + G);
         };
@@ -329,7 +341,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
 #pragma unroll
             for (int c0 = 0; c0 < NW; c0 += kCopyWarps) {
                 const int c = c0 + first;
-                if (NW % kCopyWarps == 0 || c < NW) slice_copy_router(base + static_cast<uint32_t>(s) * m.slot + static_cast<uint32_t>(c) * kSliceBytes, w + c * kSliceBytes, lane);
+                if (NW % kCopyWarps == 0 || c < NW) slice_copy_router<N>(base + static_cast<uint32_t>(s) * m.slot + static_cast<uint32_t>(c) * slice_bytes(N), w + c * slice_bytes(N), lane);
             }
         };
         auto issue = [&]() {  // rows and router matrix of the next item: one group of copies (an empty one behind the last item)
@@ -341,9 +353,16 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
                     for (int c0 = 0; c0 < NW; c0 += kCopyWarps) {
                         const int c = c0 + first;
                         if (NW % kCopyWarps == 0 || c < NW)
-                            slice_copy_rows<D>(base + static_cast<uint32_t>(s) * m.slot + static_cast<uint32_t>((1 + j) * NW + c) * kSliceBytes, row[j] + c * 256, lane);
+                            slice_copy_rows<N, D>(base + static_cast<uint32_t>(s) * m.slot + static_cast<uint32_t>((1 + j) * NW + c) * slice_bytes(N), row[j] + c * 256, lane);
                     }
                     row[j] += p.lut_stride;
+                    if constexpr (N == 32) {  // few slots: the next layer's rows are asked of L2
+                        constexpr int kLines = NW * 2;  // 128-byte lines of an expert's row
+                        if (l + 1 < L) {
+#pragma unroll
+                            for (int i = lane; i < N * kLines; i += 32) prefetch_l2(row[j] + (i / kLines) * (D * 2) + (i % kLines) * 128);
+                        }
+                    }
                 }
                 w += p.wr_stride;
                 if (++l == L) {
@@ -403,12 +422,12 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
         for (int i = 0; i < 4; ++i) wgt[i] = __ldg(reinterpret_cast<const unsigned short *>(norm_g + static_cast<size_t>(l) * p.norm_stride + Layer::col(i)));
     };
     if constexpr (NORM) load_norm(0);
-    RouterA<kSliceN> wf;
+    RouterA<N> wf;
     wf.init(lane);
-    const uint32_t w_lane = static_cast<uint32_t>(warp) * kSliceBytes, r_lane = w_lane + RowsA<kSliceN>::lane_offset(lane);
-    RowsA<kSliceN> rows[T];
+    const uint32_t w_lane = static_cast<uint32_t>(warp) * slice_bytes(N), r_lane = w_lane + RowsA<N>::lane_offset(lane);
+    RowsA<N> rows[T];
     uint32_t slot = base, buf = 0;
-    auto load_rows = [&](RowsA<kSliceN> &r, int j) { r.load(slot + static_cast<uint32_t>((1 + j) * NW) * kSliceBytes + r_lane); };
+    auto load_rows = [&](RowsA<N> &r, int j) { r.load(slot + static_cast<uint32_t>((1 + j) * NW) * slice_bytes(N) + r_lane); };
     __syncthreads();
     wf.load(base + w_lane);
 #pragma unroll
@@ -427,7 +446,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
             if (!valid[j] && g * T + j < p.M && threadIdx.x == 0 && rank == 0 && p.status) atomicOr(p.status, MOLE_STATUS_BAD_ID);
         }
         y.load_hidden(static_cast<const unsigned char *>(p.hidden), g * T, p.M);
-#pragma unroll(T == 1 ? 2 : 1)
+#pragma unroll(T == 1 && N == 16 ? 2 : 1)
         for (int l = 0; l < L; ++l) {
             y.arm(buf);
             if constexpr (NORM) {
@@ -437,18 +456,18 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
             y.logits(wf, buf);
             slot = slot == base + static_cast<uint32_t>(S - 1) * m.slot ? base : slot + m.slot;
             // one token: the next rows go to registers of their own; two tokens: to those of the rows just multiplied
-            RowsA<kSliceN> next;
-            if constexpr (CS > 1) {  // the exchange is long enough to hide both
+            RowsA<N> next;
+            if constexpr (CS > 1) {  // the exchange is long enough to hide both (32 experts: to hide one, and the registers for one)
                 wf.load(slot + w_lane);
-                load_rows(next, 0);
+                if constexpr (N == 16) load_rows(next, 0);
             }
             const float e = y.numerators(buf, [&]() {
                 if constexpr (CS == 1) wf.load(slot + w_lane);
             });
             y.weighted(rows, e, valid, [&](int j) {
-                if constexpr (CS == 1) load_rows(T == 1 ? next : rows[j], j);
+                if constexpr (CS == 1 || N == 32) load_rows(T == 1 && N == 16 ? next : rows[j], j);
             });
-            if constexpr (T == 1) rows[0] = next;
+            if constexpr (T == 1 && N == 16) rows[0] = next;
             buf ^= 1u;
             if (CS > 1 && buf == 0) y.phase ^= 1u;
         }
@@ -468,10 +487,10 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
 template <int D, int T, int NORM>
 __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(const StepParams p)
 {
-    constexpr int NW = D / kMmaCols;
-    using Layer = SliceLayer<D, T, NORM, NW * 32>;
-    constexpr SliceSmem m = slice_smem(NW, T, 1, NORM);
-    constexpr uint32_t kRouterBytes = D * kSliceN * 2;
+    constexpr int N = 16, NW = D / kMmaCols;
+    using Layer = SliceLayer<N, D, T, NORM, NW * 32>;
+    constexpr SliceSmem m = slice_smem(N, NW, T, 1, NORM);
+    constexpr uint32_t kRouterBytes = D * N * 2;
     extern __shared__ __align__(1024) unsigned char smem[];
 
     pdl_enter(p.flags);
@@ -498,8 +517,8 @@ __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(
 #pragma unroll
     for (int j = 0; j < T; ++j) {
         valid[j] = id[j] >= 0 && id[j] < p.rows;  // otherwise row 0 is fetched and its term dropped
-        const unsigned char *row = static_cast<const unsigned char *>(p.lut) + static_cast<size_t>(valid[j] ? id[j] : 0) * (kSliceN * D * 2) + warp * 256;
-        slice_copy_rows<D>(base + static_cast<uint32_t>(1 + j) * (NW * kSliceBytes) + static_cast<uint32_t>(warp) * kSliceBytes, row, lane);
+        const unsigned char *row = static_cast<const unsigned char *>(p.lut) + static_cast<size_t>(valid[j] ? id[j] : 0) * (N * D * 2) + warp * 256;
+        slice_copy_rows<N, D>(base + static_cast<uint32_t>(1 + j) * (NW * slice_bytes(N)) + static_cast<uint32_t>(warp) * slice_bytes(N), row, lane);
         if (!valid[j] && t0 + j < p.M && threadIdx.x == 0 && p.status) atomicOr(p.status, MOLE_STATUS_BAD_ID);
     }
     cp_async_commit();
@@ -515,18 +534,18 @@ __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(
         (void)wait_or_give_up(bar, 0, dead + 1, kDrainPolls);
     }
     // the matrix lies as it does in memory, 32 bytes a column: two-way bank conflicts, but ahead of the wait for the kernel before
-    RouterA<kSliceN> wf;
+    RouterA<N> wf;
     {
-        const uint32_t w = base + static_cast<uint32_t>(warp) * kSliceBytes + static_cast<uint32_t>(8 * (lane >> 4) + (lane & 7)) * 32u + static_cast<uint32_t>((lane >> 3) & 1) * 16u;
+        const uint32_t w = base + static_cast<uint32_t>(warp) * slice_bytes(N) + static_cast<uint32_t>(8 * (lane >> 4) + (lane & 7)) * 32u + static_cast<uint32_t>((lane >> 3) & 1) * 16u;
 #pragma unroll
         for (int k = 0; k < 8; ++k) ldsm_x4_trans(wf.a[k][0], w + static_cast<uint32_t>(k) * 512u);
     }
 
     cp_async_wait<0>();
     __syncwarp();
-    RowsA<kSliceN> rows[T];
+    RowsA<N> rows[T];
 #pragma unroll
-    for (int j = 0; j < T; ++j) rows[j].load(base + static_cast<uint32_t>(1 + j) * (NW * kSliceBytes) + static_cast<uint32_t>(warp) * kSliceBytes + RowsA<kSliceN>::lane_offset(lane));
+    for (int j = 0; j < T; ++j) rows[j].load(base + static_cast<uint32_t>(1 + j) * (NW * slice_bytes(N)) + static_cast<uint32_t>(warp) * slice_bytes(N) + RowsA<N>::lane_offset(lane));
 
     pdl_wait();
 
@@ -554,7 +573,7 @@ __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(
 #pragma unroll
         for (int o = 8; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         const long long t = t0 + (T == 2 ? lane >> 4 : 0);
-        if ((T == 2 || lane < 16) && t < p.M) p.gates_out[t * kSliceN + (lane & 15)] = e / sum;
+        if ((T == 2 || lane < 16) && t < p.M) p.gates_out[t * N + (lane & 15)] = e / sum;
     }
     y.weighted(rows, e, valid, [](int) {});
     y.store_out(static_cast<unsigned char *>(p.out), t0, p.M);
