@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kQuantThreads) mole_quantize_wide_kernel(const
 // infinity first to float32 and then to bf16.  The midpoints' thresholds are made once per quantisation block and
 // searched by bisection with packed bf16 compares.  A lane owns chunks of 16 consecutive elements (one 32-byte load; 8
 // bytes of NF4 codes, 4 + 2 of NF3) and keeps them in registers between the maximum and the coding.
-// One layer of the 160M shape (618 M elements) to NF3, block 128: 369 us, 4.0 TB/s (1486 us with two passes and a division
+// One layer of the 160M shape (618 M elements) to NF3, block 128: 369 us before the bounds below, 345 with them (1486 us with two passes and a division
 // and 7 float32 compares per element); what is left is the integer pipe (compares and selects), 65 % busy.
 __device__ __forceinline__ uint32_t bf162_bits(__nv_bfloat162 v) { return *reinterpret_cast<const uint32_t *>(&v); }
 __device__ __forceinline__ __nv_bfloat162 bits_bf162(uint32_t v) { return *reinterpret_cast<const __nv_bfloat162 *>(&v); }
@@ -242,12 +242,17 @@ struct QuantGrid {
     int block, group_log2, wide_loads; // elements per block; lanes per block; the table is 32-byte aligned
 };
 
+// Six blocks of 128 threads per SM (80 registers; left to itself the compiler takes 93 to 98 and four blocks' worth fit): 24 warps hide
+// more of the loads than 16, though a few values of the dividing branch are spilled.  20 000 ids, us: NF3 16 x 768 in blocks of 128 151.0 -> 126.6,
+// NF4 16 x 768 in blocks of 768 236.8 -> 196.2, 16 x 2048 in blocks of 1024 564.6 -> 501.0; seven blocks 128.5, 196.4, 499.2, three of 256
+// threads 128.6, 202.2, 510.
+constexpr int kQuantTileThreads = 128;
 template <int BITS, int CPL>
-__global__ void __launch_bounds__(kQuantThreads) mole_quantize_kernel(const unsigned char *__restrict__ src, unsigned char *__restrict__ dst,
+__global__ void __launch_bounds__(kQuantTileThreads, 6) mole_quantize_kernel(const unsigned char *__restrict__ src, unsigned char *__restrict__ dst,
                                                                       const QuantGrid q, const CodebookParam cb)
 {
     const int G = 1 << q.group_log2, g = threadIdx.x & (G - 1);
-    const uint32_t b_raw = blockIdx.x * (static_cast<uint32_t>(kQuantThreads) >> q.group_log2) + (threadIdx.x >> q.group_log2);
+    const uint32_t b_raw = blockIdx.x * (static_cast<uint32_t>(kQuantTileThreads) >> q.group_log2) + (threadIdx.x >> q.group_log2);
     const bool live = b_raw < q.total;
     const uint32_t b = live ? b_raw : q.total - 1;
     const int chunks = q.block >> 4;
@@ -993,9 +998,9 @@ int mole_quantize_lut(const void *lut, void *packed, int64_t V, int N, int d, in
         q.code_bytes = format == MOLE_LUT_NF4 ? static_cast<uint32_t>(N) * (d / 2) : q.low_bytes + static_cast<uint32_t>(N) * (d / 8);
         q.block = block;
         q.wide_loads = (reinterpret_cast<uintptr_t>(lut) & 31u) == 0 ? 1 : 0;
-        const long long per_cta = kQuantThreads >> q.group_log2;
+        const long long per_cta = kQuantTileThreads >> q.group_log2;
         const QuantizeKernel fn = format == MOLE_LUT_NF4 ? pick_quantize<4>(cpl) : pick_quantize<3>(cpl);
-        fn<<<static_cast<unsigned>((total + per_cta - 1) / per_cta), kQuantThreads, 0, st>>>(static_cast<const unsigned char *>(lut),
+        fn<<<static_cast<unsigned>((total + per_cta - 1) / per_cta), kQuantTileThreads, 0, st>>>(static_cast<const unsigned char *>(lut),
                                                                                            static_cast<unsigned char *>(packed), q, cb);
     } else if (format == MOLE_LUT_NF4) {
         mole_quantize_wide_kernel<4><<<static_cast<unsigned>(V), kQuantThreads, smem, st>>>(static_cast<const uint4 *>(lut), static_cast<unsigned char *>(packed), V, N, d, block, rb, cb);
