@@ -22,7 +22,7 @@
 // the norm 44.7 / 40.3; 1000 tokens 173 / 129.  Chained, 256 tokens: 12 of 768 35.8 / 31.4, 24 of 1024 73.6 / 72.0 (up to 148 tokens
 // the host's launches are what is left: 2.2 us each).  Of a layer's 1 300 cycles at 64 tokens of d = 1024: router product 125, exchange and loads 370, logits
 // and exp 200, parts of the numerators 95, weighted sum and output 300.
-// The widest layer, 16 layers, 16 tokens, mole_mma.cuh / here: 25.2 / 20.0, with the norm 35.7 / 28.4.  Beyond one block per SM a second
+// The widest layer, 16 layers, 16 tokens, mole_mma.cuh / here: 25.7 / 20.2, with the norm (rows in L2) 35.7 / 28.4.  Beyond one block per SM a second
 // round of clusters is no faster than two blocks per SM there (64 tokens 43.7 against 36.5, with the norm 54.9 against 45.7).
 // Tried: rows straight from L2 to registers, packed with byte permutes (no slots, half the port's bytes, but one layer of lead is too
 // little for L2's latency: 256 tokens 14.5 -> 25.8 us); slots freed by a barrier of their own, half a layer earlier (14.5 -> 15.8).
@@ -298,6 +298,15 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
     static_assert(S > AHEAD, "slots");
     using Layer = SliceLayer<N, D, T, NORM, (NW + kCopyWarps) * 32, CS>;
     constexpr SliceSmem m = slice_smem(N, NW, T, S, NORM, CS);
+    // Slots of 32 experts are large: two of router matrices and four of rows, copied in groups of their own, since it is the rows that come
+    // from DRAM and need the lead.  Behind item i's barrier the router matrix of item i + 3 is issued and the rows of item i + 4; ahead
+    // of it the router matrix of item i + 2 has landed and, issued before that, the rows of item i + 2.  (16 tokens, rows not in L2: 23.2 -> 20.2 us.)
+    constexpr bool SPLIT = N == 32;
+    constexpr int SW = SPLIT ? 2 : S, SR = SPLIT ? 4 : S;
+    constexpr uint32_t kStep = SPLIT ? NW * slice_bytes(N) : m.slot, kRows = NW * slice_bytes(N) * (SPLIT ? SW : 1);
+    auto w_slot = [](int i) { return static_cast<uint32_t>(i) * kStep; };
+    auto r_slot = [](int i) { return kRows + static_cast<uint32_t>(i) * kStep; };
+    static_assert(!SPLIT || (T == 1 && SW + SR == 2 * S), "the slots' bytes");
     extern __shared__ __align__(1024) unsigned char smem[];
 
     pdl_enter(p.flags);
@@ -323,8 +332,8 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
         const int first = warp - NW;
         const unsigned char *w0 = static_cast<const unsigned char *>(p.w_router) + rank * (NW * slice_bytes(N)), *w = w0;
         const unsigned char *row[T];
-        long long g = g0, next_id[T];  // the group whose rows are issued next; ids of the group after
-        int l = 0, s = 0;
+        long long g = g0, next_id[T], gw = g0;  // the group whose rows are issued next; ids of the group after; the routers' group
+        int l = 0, s = 0, lw = 0, sw = 0;
         auto fetch_ids = [&](long long gg) {
 #pragma unroll
             for (int j = 0; j < T; ++j) next_id[j] = gg < groups && gg * T + j < p.M ? slice_id(p, gg * T + j) : -1;
@@ -337,50 +346,59 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
             }
             fetch_ids(g + G);
         };
-        auto router = [&]() {
+        auto router = [&]() {  // the next router matrix
+            if (gw >= groups) return;
 #pragma unroll
             for (int c0 = 0; c0 < NW; c0 += kCopyWarps) {
                 const int c = c0 + first;
-                if (NW % kCopyWarps == 0 || c < NW) slice_copy_router<N>(base + static_cast<uint32_t>(s) * m.slot + static_cast<uint32_t>(c) * slice_bytes(N), w + c * slice_bytes(N), lane);
+                if (NW % kCopyWarps == 0 || c < NW) slice_copy_router<N>(base + w_slot(sw) + static_cast<uint32_t>(c) * slice_bytes(N), w + c * slice_bytes(N), lane);
             }
+            w += p.wr_stride;
+            if (++lw == L) lw = 0, gw += G, w = w0;
+            if (++sw == SW) sw = 0;
         };
-        auto issue = [&]() {  // rows and router matrix of the next item: one group of copies (an empty one behind the last item)
-            if (g < groups) {
-                router();
+        auto token_rows = [&]() {  // the next item's rows
+            if (g >= groups) return;
 #pragma unroll
-                for (int j = 0; j < T; ++j) {
+            for (int j = 0; j < T; ++j) {
 #pragma unroll
-                    for (int c0 = 0; c0 < NW; c0 += kCopyWarps) {
-                        const int c = c0 + first;
-                        if (NW % kCopyWarps == 0 || c < NW)
-                            slice_copy_rows<N, D>(base + static_cast<uint32_t>(s) * m.slot + static_cast<uint32_t>((1 + j) * NW + c) * slice_bytes(N), row[j] + c * 256, lane);
-                    }
-                    row[j] += p.lut_stride;
-                    if constexpr (N == 32) {  // few slots: the next layer's rows are asked of L2
-                        constexpr int kLines = NW * 2;  // 128-byte lines of an expert's row
-                        if (l + 1 < L) {
-#pragma unroll
-                            for (int i = lane; i < N * kLines; i += 32) prefetch_l2(row[j] + (i / kLines) * (D * 2) + (i % kLines) * 128);
-                        }
-                    }
+                for (int c0 = 0; c0 < NW; c0 += kCopyWarps) {
+                    const int c = c0 + first;
+                    if (NW % kCopyWarps == 0 || c < NW)
+                        slice_copy_rows<N, D>(base + r_slot(s) + static_cast<uint32_t>(j * NW + c) * slice_bytes(N), row[j] + c * 256, lane);
                 }
-                w += p.wr_stride;
-                if (++l == L) {
-                    l = 0;
-                    g += G;
-                    w = w0;
-                    begin_group();
-                }
-                if (++s == S) s = 0;
+                row[j] += p.lut_stride;
             }
+            if (++l == L) {
+                l = 0;
+                g += G;
+                begin_group();
+            }
+            if (++s == SR) s = 0;
+        };
+        auto issue = [&]() {  // one group of copies, or two (empty ones behind the last item)
+            router();
+            if constexpr (SPLIT) cp_async_commit();
+            token_rows();
             cp_async_commit();
         };
         fetch_ids(g);
         begin_group();
+        if constexpr (SPLIT) {
+            issue();
+            issue();
+            token_rows();
+            cp_async_commit();
+            cp_async_wait<3>();
+            __syncthreads();  // the first item has landed
+            __syncthreads();  // ... and is in registers
+            issue();
+        } else {
 #pragma unroll 1
-        for (int i = 0; i < S; ++i) issue();
-        cp_async_wait<S - AHEAD>();
-        __syncthreads();  // the first item has landed (the first two)
+            for (int i = 0; i < S; ++i) issue();
+            cp_async_wait<S - AHEAD>();
+            __syncthreads();  // the first item has landed (the first two)
+        }
         Layer y;
         if constexpr (CS > 1) {
             y.init(base, m);
@@ -389,7 +407,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
         uint32_t buf = 0;
         for (long long gg = g0; gg < groups; gg += G)
             for (int i = 0; i < L; ++i) {
-                cp_async_wait<S - 1 - AHEAD>();
+                cp_async_wait<SPLIT ? 1 : S - 1 - AHEAD>();
                 if constexpr (CS == 1) {
                     named_bar_sync(Layer::kBarLogits, Layer::COUNT);
                 } else {
@@ -426,12 +444,14 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
     wf.init(lane);
     const uint32_t w_lane = static_cast<uint32_t>(warp) * slice_bytes(N), r_lane = w_lane + RowsA<N>::lane_offset(lane);
     RowsA<N> rows[T];
-    uint32_t slot = base, buf = 0;
-    auto load_rows = [&](RowsA<N> &r, int j) { r.load(slot + static_cast<uint32_t>((1 + j) * NW) * slice_bytes(N) + r_lane); };
+    uint32_t buf = 0;
+    int ws = 0, rs = 0;
+    auto load_rows = [&](RowsA<N> &r, int j) { r.load(base + r_slot(rs) + static_cast<uint32_t>(j * NW) * slice_bytes(N) + r_lane); };
     __syncthreads();
     wf.load(base + w_lane);
 #pragma unroll
     for (int j = 0; j < T; ++j) load_rows(rows[j], j);
+    if constexpr (SPLIT) __syncthreads();
     if constexpr (CS > 1) cluster_wait();
 
     pdl_wait();
@@ -454,15 +474,16 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
                 load_norm(l + 1 < L ? l + 1 : 0);
             }
             y.logits(wf, buf);
-            slot = slot == base + static_cast<uint32_t>(S - 1) * m.slot ? base : slot + m.slot;
+            if (++ws == SW) ws = 0;
+            if (++rs == SR) rs = 0;
             // one token: the next rows go to registers of their own; two tokens: to those of the rows just multiplied
             RowsA<N> next;
             if constexpr (CS > 1) {  // the exchange is long enough to hide both (32 experts: to hide one, and the registers for one)
-                wf.load(slot + w_lane);
+                wf.load(base + w_slot(ws) + w_lane);
                 if constexpr (N == 16) load_rows(next, 0);
             }
             const float e = y.numerators(buf, [&]() {
-                if constexpr (CS == 1) wf.load(slot + w_lane);
+                if constexpr (CS == 1) wf.load(base + w_slot(ws) + w_lane);
             });
             y.weighted(rows, e, valid, [&](int j) {
                 if constexpr (CS == 1 || N == 32) load_rows(T == 1 && N == 16 ? next : rows[j], j);
