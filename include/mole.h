@@ -100,7 +100,9 @@ extern "C" {
                                    at most 24 KB or a token's rows are 128 KB.  [N = 32: 148 tokens at d = 512, up to 74 at    \
                                    1024 and 2048.]                                                                             \
                                 mole_variant says which. */
-#define MOLE_KERNEL_RING 1   /* persistent blocks, rows and router chunks streamed through a shared-memory ring: any shape */
+#define MOLE_KERNEL_RING 1   /* persistent blocks, rows and router chunks streamed through a shared-memory ring: any shape (bf16, N = 16,  \
+                                d = 768 or 1024 in one chunk: kernels of their own, a warp per 128 columns, on the tensor cores, with the   \
+                                same promise: a token's bits are those of any batch, in single, chained and fused launches) */
 #define MOLE_KERNEL_DECODE 2 /* one block per token (single layer: rows held in registers; fused step: rows through a ring, \
                                 router matrix through registers): bf16, N of 4, 8, 16 or 32, d a multiple of 128 up to   \
                                 2048 (single layer with N = 32: up to 1024), d_split 0.  A single layer with d = 2048 and \
@@ -529,7 +531,7 @@ MOLE_API int mole_plan(int M, int L, int N, int d, int dtype, int d_split, int *
               int *out_smem_bytes, int *out_stages, int *out_blocks_per_sm);
 
 /* Name of the kernel instantiation a launch of this shape runs, with its block size and dynamic shared memory:
- *   "step<storage,N,P,MODE,SHAPE,DIRECT,NORM>"        the ring kernel
+ *   "step<storage,N,P,MODE,SHAPE,DIRECT,NORM>"        the ring kernel; SHAPE 1 and 2: the kernels of bf16, N = 16, d = 768 and 1024
  *   "tile<N,NORM,width,PARTS>"                        the prefill kernel
  *   "mma<N,NORM,CS>"                                  the tensor-core step (a step whose layer strides are below 16 bytes or from
  *                                                     2^40 on, which a tensor map does not take, runs the ring kernel instead)
