@@ -9,7 +9,7 @@
 //     Warps exchange nothing but 16 partial logits per token: one block barrier per layer (and one for the norm).
 //   - Both products run on mma.m16n8k16, as in mole_mma.cuh.  A numerator's three bf16 parts are columns of one product
 //     (GateColumns): at 8.2 cycles an mma and quarter of an SM (measured) three products took 400 cycles of a layer, one takes 200.
-//   - Four warps do nothing but copy rows and router matrices into swizzled slots (cp.async).  They take part in the layer's barrier,
+//   - Four warps (beside a cluster's four: one) do nothing but copy rows and router matrices into swizzled slots (cp.async).  They take part in the layer's barrier,
 //     which so is the handshake, too: no mbarrier is polled.  The other warps take an item from its slot into registers while they
 //     compute the softmax and the weighted sum of the item before.
 //   - Widths, warps and slots are compile-time, so the chain has no loop or bound to evaluate.
@@ -68,7 +68,6 @@ __host__ __device__ constexpr int slice_slots(int N, int nw, int tokens, int cs 
 
 template <int PENDING>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
-__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // This warp's N x 128 slice of a token's rows (row: the first expert's row, at the warp's columns) into a slot: [64-column
 // half][expert][128 bytes], 16-byte pieces swizzled by the expert (RowsA).
