@@ -388,8 +388,12 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
             issue();
             token_rows();
             cp_async_commit();
-            cp_async_wait<3>();
-            __syncthreads();  // the first item has landed
+            // router 0, rows 0, router 1, rows 1, rows 2: the third is read ahead of item 0's barrier, so that it is the block barriers
+            // here that publish it
+            constexpr int kPending = 2;
+            static_assert(5 - kPending >= 3, "router 1 has landed");
+            cp_async_wait<kPending>();
+            __syncthreads();  // the first item and the second router matrix have landed
             __syncthreads();  // ... and is in registers
             issue();
         } else {

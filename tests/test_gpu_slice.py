@@ -1,6 +1,7 @@
 """The kernels of the two narrow widths (16 experts, d = 768 and 1024): a cluster of two blocks, a block and half a block per token, on
 both sides of each line, against the oracle's chain; a token's bits in every batch and in single, chained and fused launches; ids
-outside the table beside a valid one; bounded waits."""
+outside the table beside a valid one; bounded waits; and the fused step of the widest layer (32 x 2048): the bits of the step it
+stands beside, and slots that fill slowly."""
 import numpy as np
 import pytest
 import torch
@@ -91,3 +92,62 @@ def test_waits_of_the_cluster_that_run_out_are_reported(d, norm):
     step(out)
     torch.cuda.synchronize()
     assert int(status.item()) == 0 and torch.equal(out, want)
+
+
+def _peaked(N, d, M, L, seed, norm):
+    """Tables of standard deviation 1 and routers that favour other experts in every layer: a router matrix of another layer, or parts of
+    one, shows far above a rounding."""
+    g = torch.Generator().manual_seed(seed)
+    luts = torch.empty(L, V, N, d).normal_(0, 1, generator=g).to(torch.bfloat16)
+    wrs = torch.empty(L, d, N).normal_(0, 3.0 / d ** 0.5, generator=g).to(torch.bfloat16)
+    hidden = torch.empty(M, d).normal_(0, 1, generator=g).to(torch.bfloat16)
+    ids = torch.randint(0, V, (M,), generator=g, dtype=torch.int32)
+    gammas = (1.0 + 0.2 * torch.empty(L, d).normal_(0, 1, generator=g)).to(torch.bfloat16) if norm else None
+    return luts, wrs, hidden, ids, gammas
+
+
+def _fused(h, i, lu, w, gam):
+    return mole.decode_step_args(h, i, lu, w, torch.empty_like(h), None, mode=mole.STEP_FUSED, norm_weights=gam, norm_eps=1e-5)
+
+
+@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("L", [2, 3, 16])
+def test_widest_step_has_the_same_bits_on_both_sides_of_its_line(L, norm):
+    """32 x 2048: up to 37 tokens a kernel with the sizes compiled in, beyond it the general tensor-core step."""
+    few, many = SMS // 4, SMS // 4 + 27
+    luts, wrs, hidden, ids, gammas = _peaked(32, 2048, many, L, 7 * L + norm, norm)
+    h, i, lu, gam = hidden.to(DEV), ids.to(DEV), luts.to(DEV), None if gammas is None else gammas.to(DEV)
+    want = _fused(h, i, lu, wrs.to(DEV), gam)
+    for M in (1, few - 1, few, few + 1):
+        for _ in range(3):  # routers in memory that no launch has read yet
+            assert torch.equal(_fused(h[:M].contiguous(), i[:M].contiguous(), lu, wrs.to(DEV), gam), want[:M]), M
+
+
+@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("L", [2, 7])
+def test_widest_step_against_the_oracles_chain(L, norm):
+    """Entries of standard deviation 1, so that the routed term is what is compared: a bf16 rounding per layer, carried into the
+    layers after it by gates whose logits have a standard deviation of 3 and more."""
+    M = 6
+    luts, wrs, hidden, ids, gammas = _peaked(32, 2048, M, L, 31 + L, norm)
+    ref, _, _ = _oracle_chain(hidden, ids, luts, wrs, gammas, 1e-5)
+    out = _fused(hidden.to(DEV), ids.to(DEV), luts.to(DEV), wrs.to(DEV), None if gammas is None else gammas.to(DEV))
+    rel = np.linalg.norm(as_f64(out) - ref, axis=1) / np.linalg.norm(ref, axis=1)
+    assert rel.max() <= L * 2.0 ** -7, rel
+
+
+@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("N,d,M", [(32, 2048, 1), (32, 2048, SMS // 4), (16, 1024, 5), (16, 768, 100), (16, 1024, SMS + 3)])
+def test_slots_that_fill_slowly(N, d, M, norm):
+    """Routers, then tables too, in pinned host memory, which the kernel reads across the link: copies that take many layers' time, of
+    which none may be used before it has landed or overwritten before it is read."""
+    L = 9
+    luts, wrs, hidden, ids, gammas = _peaked(N, d, M, L, M + d, norm)
+    h, i, lu, gam = hidden.to(DEV), ids.to(DEV), luts.to(DEV), None if gammas is None else gammas.to(DEV)
+    want = _fused(h, i, lu, wrs.to(DEV), gam)
+    slow_w = wrs.pin_memory()
+    for table in (lu, luts.pin_memory()):
+        for _ in range(3):
+            out = _fused(h, i, table, slow_w, gam)
+            torch.cuda.synchronize()
+            assert torch.equal(out, want)
