@@ -22,7 +22,7 @@
 // the norm 44.7 / 40.3; 1000 tokens 173 / 129.  Chained, 256 tokens: 12 of 768 35.8 / 31.4, 24 of 1024 73.6 / 72.0 (up to 148 tokens
 // the host's launches are what is left: 2.2 us each).  Of a layer's 1 300 cycles at 64 tokens of d = 1024: router product 125, exchange and loads 370, logits
 // and exp 200, parts of the numerators 95, weighted sum and output 300.
-// The widest layer, 16 layers, 16 tokens, mole_mma.cuh / here: 25.7 / 20.2, with the norm (rows in L2) 35.7 / 28.4.  Beyond one block per SM a second
+// The widest layer, 16 layers, 16 tokens, mole_mma.cuh / here: 25.2 / 18.2, with the norm 35.7 / 27.7.  Beyond one block per SM a second
 // round of clusters is no faster than two blocks per SM there (64 tokens 43.7 against 36.5, with the norm 54.9 against 45.7).
 // Tried: rows straight from L2 to registers, packed with byte permutes (no slots, half the port's bytes, but one layer of lead is too
 // little for L2's latency: 256 tokens 14.5 -> 25.8 us); slots freed by a barrier of their own, half a layer earlier (14.5 -> 15.8).
@@ -286,26 +286,31 @@ __device__ __forceinline__ long long slice_id(const StepParams &p, long long t)
 }
 
 // The fused step: a block walks its groups of T tokens (group b, b + G, ..) through the L layers; (group, layer) is an item.  Slot
-// i % S holds item i's rows and router matrix.  The copying warp arrives at item i's barrier when the rows of item i + 1 and the
-// router matrix of item i + 2 have landed; ahead of it the compute warps have taken item i's rows and router matrix into registers,
-// behind it they take item i + 1's.  So it frees the slot of item i for item i + S.
+// i % S holds item i's rows and router matrix, copied as one group or, of 32 experts, as two: they are large, it is the rows that come from
+// DRAM, and so they need not have landed as early as the matrix (16 layers, 16 tokens: 18.2 us).
+// Which wait covers which read (i: an item; its barrier is the one its partial logits are counted in at):
+//   - Landed.  What a compute warp reads behind barrier i has landed before the copying warps arrive at it; what it reads ahead of
+//     barrier i -- a cluster's warps, under the exchange -- has landed before barrier i - 1.  One block: item i + 1 behind barrier i.  Clusters:
+//     the matrix of item i + 1 ahead of barrier i, and its rows there, too (16 experts) or behind it (32).
+//   - Overwritten.  Behind barrier i the copying warps fill the slot of item i with item i + S.  A compute warp asks for item i's rows and
+//     matrix ahead of or just behind barrier i - 1, and later gives its partial logits of item i to barrier i.  One block: barrier i is
+//     a block barrier.  Clusters: those logits are computed from the matrix itself and from a state that was read from shared memory
+//     after the rows, and a warp's shared-memory requests are served in order.
 template <int N, int D, int T, int NORM, int CS>
 __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS + slice_copy_warps(N)) * 32, 1) mole_slice_step_kernel(const StepParams p)
 {
     constexpr int NW = D / kMmaCols / CS, S = slice_slots(N, NW, T, CS), kCopyWarps = slice_copy_warps(N);  // warps of this block
-    constexpr int AHEAD = CS > 1 ? 2 : 1;  // items landed before an item's barrier, beside its own
-    static_assert(S > AHEAD, "slots");
+    // groups of copies per item; how many may be on their way when the first item is read, and at a barrier
+    constexpr int GROUPS = N == 32 ? 2 : 1, FIRST_PENDING = S * GROUPS - (CS == 1 ? 1 : GROUPS == 2 ? 3 : 2),
+                  PENDING = GROUPS == 2 ? 1 : S - (CS == 1 ? 2 : 3);
+    static_assert(FIRST_PENDING >= 0 && PENDING >= 0, "slots");
+    static_assert(CS == 1 ? 2 <= S - PENDING                           // behind barrier i: item i + 1, of the S + i copied by then
+                          : GROUPS == 1 ? 3 <= S - PENDING             // ahead of it: item i + 1, of the S + i - 1 behind barrier i - 1
+                                        : 5 <= 2 * S - PENDING,            // its matrix; one group less for its rows, behind barrier i
+                  "copies that are read have landed");
     using Layer = SliceLayer<N, D, T, NORM, (NW + kCopyWarps) * 32, CS>;
     constexpr SliceSmem m = slice_smem(N, NW, T, S, NORM, CS);
-    // Slots of 32 experts are large: two of router matrices and four of rows, copied in groups of their own, since it is the rows that come
-    // from DRAM and need the lead.  Behind item i's barrier the router matrix of item i + 3 is issued and the rows of item i + 4; ahead
-    // of it the router matrix of item i + 2 has landed and, issued before that, the rows of item i + 2.  (16 tokens, rows not in L2: 23.2 -> 20.2 us.)
-    constexpr bool SPLIT = N == 32;
-    constexpr int SW = SPLIT ? 2 : S, SR = SPLIT ? 4 : S;
-    constexpr uint32_t kStep = SPLIT ? NW * slice_bytes(N) : m.slot, kRows = NW * slice_bytes(N) * (SPLIT ? SW : 1);
-    auto w_slot = [](int i) { return static_cast<uint32_t>(i) * kStep; };
-    auto r_slot = [](int i) { return kRows + static_cast<uint32_t>(i) * kStep; };
-    static_assert(!SPLIT || (T == 1 && SW + SR == 2 * S), "the slots' bytes");
+    constexpr uint32_t kRows = NW * slice_bytes(N);  // of a slot: the router matrix, then the rows
     extern __shared__ __align__(1024) unsigned char smem[];
 
     pdl_enter(p.flags);
@@ -350,11 +355,11 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
 #pragma unroll
             for (int c0 = 0; c0 < NW; c0 += kCopyWarps) {
                 const int c = c0 + first;
-                if (NW % kCopyWarps == 0 || c < NW) slice_copy_router<N>(base + w_slot(sw) + static_cast<uint32_t>(c) * slice_bytes(N), w + c * slice_bytes(N), lane);
+                if (NW % kCopyWarps == 0 || c < NW) slice_copy_router<N>(base + static_cast<uint32_t>(sw) * m.slot + static_cast<uint32_t>(c) * slice_bytes(N), w + c * slice_bytes(N), lane);
             }
             w += p.wr_stride;
             if (++lw == L) lw = 0, gw += G, w = w0;
-            if (++sw == SW) sw = 0;
+            if (++sw == S) sw = 0;
         };
         auto token_rows = [&]() {  // the next item's rows
             if (g >= groups) return;
@@ -364,7 +369,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
                 for (int c0 = 0; c0 < NW; c0 += kCopyWarps) {
                     const int c = c0 + first;
                     if (NW % kCopyWarps == 0 || c < NW)
-                        slice_copy_rows<N, D>(base + r_slot(s) + static_cast<uint32_t>(j * NW + c) * slice_bytes(N), row[j] + c * 256, lane);
+                        slice_copy_rows<N, D>(base + static_cast<uint32_t>(s) * m.slot + kRows + static_cast<uint32_t>(j * NW + c) * slice_bytes(N), row[j] + c * 256, lane);
                 }
                 row[j] += p.lut_stride;
             }
@@ -373,35 +378,20 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
                 g += G;
                 begin_group();
             }
-            if (++s == SR) s = 0;
+            if (++s == S) s = 0;
         };
-        auto issue = [&]() {  // one group of copies, or two (empty ones behind the last item)
+        auto issue = [&]() {  // the next item's groups of copies (empty ones behind the last item)
             router();
-            if constexpr (SPLIT) cp_async_commit();
+            if constexpr (GROUPS == 2) cp_async_commit();
             token_rows();
             cp_async_commit();
         };
         fetch_ids(g);
         begin_group();
-        if constexpr (SPLIT) {
-            issue();
-            issue();
-            token_rows();
-            cp_async_commit();
-            // router 0, rows 0, router 1, rows 1, rows 2: the third is read ahead of item 0's barrier, so that it is the block barriers
-            // here that publish it
-            constexpr int kPending = 2;
-            static_assert(5 - kPending >= 3, "router 1 has landed");
-            cp_async_wait<kPending>();
-            __syncthreads();  // the first item and the second router matrix have landed
-            __syncthreads();  // ... and is in registers
-            issue();
-        } else {
 #pragma unroll 1
-            for (int i = 0; i < S; ++i) issue();
-            cp_async_wait<S - AHEAD>();
-            __syncthreads();  // the first item has landed (the first two)
-        }
+        for (int i = 0; i < S; ++i) issue();
+        cp_async_wait<FIRST_PENDING>();
+        __syncthreads();  // what is read ahead of item 0's barrier has landed
         Layer y;
         if constexpr (CS > 1) {
             y.init(base, m);
@@ -410,7 +400,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
         uint32_t buf = 0;
         for (long long gg = g0; gg < groups; gg += G)
             for (int i = 0; i < L; ++i) {
-                cp_async_wait<SPLIT ? 1 : S - 1 - AHEAD>();
+                cp_async_wait<PENDING>();
                 if constexpr (CS == 1) {
                     named_bar_sync(Layer::kBarLogits, Layer::COUNT);
                 } else {
@@ -448,13 +438,12 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
     const uint32_t w_lane = static_cast<uint32_t>(warp) * slice_bytes(N), r_lane = w_lane + RowsA<N>::lane_offset(lane);
     RowsA<N> rows[T];
     uint32_t buf = 0;
-    int ws = 0, rs = 0;
-    auto load_rows = [&](RowsA<N> &r, int j) { r.load(base + r_slot(rs) + static_cast<uint32_t>(j * NW) * slice_bytes(N) + r_lane); };
+    int s = 0;
+    auto load_rows = [&](RowsA<N> &r, int j) { r.load(base + static_cast<uint32_t>(s) * m.slot + kRows + static_cast<uint32_t>(j * NW) * slice_bytes(N) + r_lane); };
     __syncthreads();
     wf.load(base + w_lane);
 #pragma unroll
     for (int j = 0; j < T; ++j) load_rows(rows[j], j);
-    if constexpr (SPLIT) __syncthreads();
     if constexpr (CS > 1) cluster_wait();
 
     pdl_wait();
@@ -477,16 +466,15 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
                 load_norm(l + 1 < L ? l + 1 : 0);
             }
             y.logits(wf, buf);
-            if (++ws == SW) ws = 0;
-            if (++rs == SR) rs = 0;
+            if (++s == S) s = 0;
             // one token: the next rows go to registers of their own; two tokens: to those of the rows just multiplied
             RowsA<N> next;
             if constexpr (CS > 1) {  // the exchange is long enough to hide both (32 experts: to hide one, and the registers for one)
-                wf.load(base + w_slot(ws) + w_lane);
+                wf.load(base + static_cast<uint32_t>(s) * m.slot + w_lane);
                 if constexpr (N == 16) load_rows(next, 0);
             }
             const float e = y.numerators(buf, [&]() {
-                if constexpr (CS == 1) wf.load(base + w_slot(ws) + w_lane);
+                if constexpr (CS == 1) wf.load(base + static_cast<uint32_t>(s) * m.slot + w_lane);
             });
             y.weighted(rows, e, valid, [&](int j) {
                 if constexpr (CS == 1 || N == 32) load_rows(T == 1 && N == 16 ? next : rows[j], j);
