@@ -81,9 +81,10 @@ extern "C" {
 #define MOLE_FLAG_IDS_INT64 1u /* ids are int64_t instead of int32_t */
 #define MOLE_FLAG_CHAIN 2u     /* launch with programmatic dependent launch: the kernel may start, \
                                   and may read ids / lut / w_router, before the previous kernel    \
-                                  on the stream has finished; it reads hidden / residual only      \
-                                  after it has.  Only valid if ids, lut and w_router are not       \
-                                  written by that previous kernel. */
+                                  on the stream has finished; it reads hidden, residual and        \
+                                  norm_weight only after it has.  Only valid if ids, lut and       \
+                                  w_router are not written by that previous kernel.  (A step's:    \
+                                  see mole_step_args.) */
 
 /* which kernel family runs a single-layer launch (mole_args.kernel, mole_step_args.kernel) */
 #define MOLE_KERNEL_AUTO 0   /* the library's choice, by shape and number of tokens (limits for 148 SMs in brackets).             \

@@ -123,24 +123,19 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kClusterThreads) mo
 #pragma unroll
         for (int j = 0; j < N; ++j) rv[j] = ldg_stream_v2(row + static_cast<size_t>(j) * d * 2);
     }
-    float nw[NORM ? R : 1];
-    if constexpr (NORM) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int col = static_cast<int>(q) * kClusterSlice + (tid + r * T) / QL;
-            nw[r] = bf16_bits_to_float(__ldg(static_cast<const unsigned short *>(p.norm_weight) + col));
-        }
-    }
     __syncthreads();  // the barriers are initialised before anybody in this block polls them
 
-    // ---- the previous kernel's output: this block's slice of the token's hidden state (and residual) ----
+    // ---- the previous kernel's output: this block's slice of the token's hidden state (and residual); the norm's scale, which it may
+    // have written, too ----
     pdl_wait();
     const unsigned char *hrow = static_cast<const unsigned char *>(p.hidden) + static_cast<size_t>(t) * d * 2;
     unsigned short hs[R];
+    uint32_t nw[NORM ? R : 1];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int col = static_cast<int>(q) * kClusterSlice + (tid + r * T) / QL;  // sweep vector tid + r T covers one column of the slice
         hs[r] = ldcg_u16(hrow + 2 * col);
+        if constexpr (NORM) nw[r] = ld_scale_u16(static_cast<const unsigned short *>(p.norm_weight) + col);
     }
     uint2 res = ldcg_v2((p.residual ? static_cast<const unsigned char *>(p.residual) + static_cast<size_t>(t) * d * 2 : hrow) + own);
 
@@ -167,7 +162,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kClusterThreads) mo
         for (int w = 0; w < kClusterWarps; ++w) total += scratch[w];
         const float rinv = 1.0f / sqrtf(total / static_cast<float>(d) + p.norm_eps);
 #pragma unroll
-        for (int r = 0; r < R; ++r) hs[r] = float_to_bf16_bits((bf16_bits_to_float(hs[r]) * rinv) * nw[r]);
+        for (int r = 0; r < R; ++r) hs[r] = float_to_bf16_bits((bf16_bits_to_float(hs[r]) * rinv) * bf16_bits_to_float(nw[r]));
     }
 
     // ---- router slice in shared memory? (bounded; after a failure the block goes on with whatever is there) ----

@@ -152,25 +152,15 @@ __global__ void __launch_bounds__(decode_max_threads(N)) mole_decode_kernel(cons
 #pragma unroll
         for (int j = 0; j < N; ++j) rv[j] = ldg_stream_v2(row + static_cast<size_t>(j) * d * 2);
     }
-    // column(s) of sweep vector r of this thread: vector u = tid + r * T covers column u / QL (N >= 8)
-    // or columns u * CPV .. (N < 8)
-    float nw[NORM ? R * CPV : 1];
-    if constexpr (NORM) {
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int cc = 0; cc < CPV; ++cc) {
-                const int u = tid + r * T;
-                const int col = N >= VEC ? u / QL : u * CPV + cc;
-                nw[r * CPV + cc] = bf16_bits_to_float(__ldg(static_cast<const unsigned short *>(p.norm_weight) + col));
-            }
-    }
     __syncthreads();  // the barrier is initialised before anybody polls it
 
-    // ---- the previous kernel's output: hidden state (and residual) of this token ----
+    // ---- the previous kernel's output: hidden state (and residual) of this token; the norm's scale, which it may have written, too ----
     pdl_wait();
     const unsigned char *hrow = static_cast<const unsigned char *>(p.hidden) + static_cast<size_t>(t) * d * 2;
+    // column(s) of sweep vector r of this thread: vector u = tid + r * T covers column u / QL (N >= 8)
+    // or columns u * CPV .. (N < 8)
     unsigned short hs[R * CPV];
+    uint32_t nw[NORM ? R * CPV : 1];
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
@@ -178,6 +168,7 @@ __global__ void __launch_bounds__(decode_max_threads(N)) mole_decode_kernel(cons
             const int u = tid + r * T;
             const int col = N >= VEC ? u / QL : u * CPV + cc;
             hs[r * CPV + cc] = ldcg_u16(hrow + 2 * col);
+            if constexpr (NORM) nw[r * CPV + cc] = ld_scale_u16(static_cast<const unsigned short *>(p.norm_weight) + col);
         }
     const uint2 hown = ldcg_v2(hrow + static_cast<size_t>(tid) * 8);  // columns 4 tid .. 4 tid + 3
     uint2 res = hown;
@@ -195,7 +186,7 @@ __global__ void __launch_bounds__(decode_max_threads(N)) mole_decode_kernel(cons
         for (int w = 0; w < nwarps; ++w) total += scratch[w];  // the same order in every thread
         const float rinv = 1.0f / sqrtf(total / static_cast<float>(d) + p.norm_eps);
 #pragma unroll
-        for (int i = 0; i < R * CPV; ++i) hs[i] = float_to_bf16_bits((bf16_bits_to_float(hs[i]) * rinv) * nw[i]);
+        for (int i = 0; i < R * CPV; ++i) hs[i] = float_to_bf16_bits((bf16_bits_to_float(hs[i]) * rinv) * bf16_bits_to_float(nw[i]));
     }
 
     // ---- router matrix in shared memory? (bounded wait; after a failure the block computes on

@@ -483,9 +483,10 @@ __device__ __forceinline__ void rmsnorm_to_shared(uint32_t src, uint32_t dst, co
     constexpr int VEC = E::VEC;
     const int ngrp = d / VEC;
     const uint4 *wg = static_cast<const uint4 *>(weight_g);
-    // this thread's first vector of the scale comes from L2: asked for before the sum of squares, not after it
+    // this thread's first vector of the scale comes from L2: asked for before the sum of squares, not after it (plain loads: the kernel
+    // before a chained launch may have written it)
     uint4 w_first = make_uint4(0u, 0u, 0u, 0u);
-    if (tid < ngrp) w_first = __ldg(wg + tid);
+    if (tid < ngrp) w_first = ld_scale_v4(wg + tid);
     float ss = 0.f;
     for (int g = tid; g < ngrp; g += nc) {
         float x[VEC];
@@ -502,7 +503,7 @@ __device__ __forceinline__ void rmsnorm_to_shared(uint32_t src, uint32_t dst, co
     for (int g = tid; g < ngrp; g += nc) {
         float x[VEC], w[VEC];
         E::unpack(lds128(src + 16u * g), x);
-        E::unpack(g == tid ? w_first : __ldg(wg + g), w);
+        E::unpack(g == tid ? w_first : ld_scale_v4(wg + g), w);
         uint32_t o[4];
         if constexpr (VEC == 8) {
 #pragma unroll

@@ -509,22 +509,12 @@ __global__ void __launch_bounds__(kDecodeMaxThreads) mole_qdecode_kernel(const Q
         bulk_g2s(rec, static_cast<const unsigned char *>(p.lut) + static_cast<size_t>(valid ? id : 0) * rec_bytes, rec_bytes, bar + 1);
     }
     if (tid < 16) cbs[tid] = p.cb[tid];
-    float nw[NORM ? R * CPV : 1];
-    if constexpr (NORM) {
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int cc = 0; cc < CPV; ++cc) {
-                const int u = tid + r * T;
-                const int col = N >= VEC ? u / QL : u * CPV + cc;
-                nw[r * CPV + cc] = bf16_bits_to_float(__ldg(static_cast<const unsigned short *>(p.norm_weight) + col));
-            }
-    }
     __syncthreads();
 
-    pdl_wait();
+    pdl_wait();  // the kernel before may have written the norm's scale, too
     const unsigned char *hrow = static_cast<const unsigned char *>(p.hidden) + static_cast<size_t>(t) * d * 2;
     unsigned short hs[R * CPV];
+    uint32_t nw[NORM ? R * CPV : 1];
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
@@ -532,6 +522,7 @@ __global__ void __launch_bounds__(kDecodeMaxThreads) mole_qdecode_kernel(const Q
             const int u = tid + r * T;
             const int col = N >= VEC ? u / QL : u * CPV + cc;
             hs[r * CPV + cc] = ldcg_u16(hrow + 2 * col);
+            if constexpr (NORM) nw[r * CPV + cc] = ld_scale_u16(static_cast<const unsigned short *>(p.norm_weight) + col);
         }
     const uint2 hown = ldcg_v2(hrow + static_cast<size_t>(tid) * 8);
     uint2 res = hown;
@@ -548,7 +539,7 @@ __global__ void __launch_bounds__(kDecodeMaxThreads) mole_qdecode_kernel(const Q
         for (int w = 0; w < nwarps; ++w) total += scratch[w];
         const float rinv = 1.0f / sqrtf(total / static_cast<float>(d) + p.norm_eps);
 #pragma unroll
-        for (int i = 0; i < R * CPV; ++i) hs[i] = float_to_bf16_bits((bf16_bits_to_float(hs[i]) * rinv) * nw[i]);
+        for (int i = 0; i < R * CPV; ++i) hs[i] = float_to_bf16_bits((bf16_bits_to_float(hs[i]) * rinv) * bf16_bits_to_float(nw[i]));
     }
 
     // bounded waits for the two bulk copies; after a failure the block computes on whatever its shared

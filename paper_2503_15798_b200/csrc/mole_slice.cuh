@@ -152,12 +152,16 @@ struct SliceLayer {
             }
         }
     }
-    // 16 lanes fetch a token's 128 columns (token: lane / 16 of two); out of range: nothing
-    __device__ __forceinline__ void load_hidden(const unsigned char *hidden, long long t0, long long M)
+    // 16 lanes fetch a token's 128 columns (token: lane / 16 of two); out of range: nothing.  `under` is done while they are on their way
+    template <typename F>
+    __device__ __forceinline__ void load_hidden(const unsigned char *hidden, long long t0, long long M, F &&under)
     {
         const long long t = t0 + (T == 2 ? lane >> 4 : 0);
-        if ((T == 2 || lane < 16) && t < M)
-            sts128(hid + static_cast<uint32_t>(lane) * 16u, __ldcg(reinterpret_cast<const uint4 *>(hidden + static_cast<size_t>(t) * (D * 2) + slice * 256 + (lane & 15) * 16)));
+        const bool mine = (T == 2 || lane < 16) && t < M;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (mine) v = __ldcg(reinterpret_cast<const uint4 *>(hidden + static_cast<size_t>(t) * (D * 2) + slice * 256 + (lane & 15) * 16));
+        under();
+        if (mine) sts128(hid + static_cast<uint32_t>(lane) * 16u, v);
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < T; ++j)
@@ -172,7 +176,8 @@ struct SliceLayer {
             *reinterpret_cast<uint4 *>(out + static_cast<size_t>(t) * (D * 2) + slice * 256 + (lane & 15) * 16) = lds128(hid + static_cast<uint32_t>(lane) * 16u);
     }
     // y = (x / sqrt(mean(x^2) + eps)) * w, rounded once to bf16, into the normalised slices
-    __device__ __forceinline__ void normalise(const unsigned short (&w)[4], float eps, uint32_t buf)
+    template <typename W>  // bf16 bits
+    __device__ __forceinline__ void normalise(const W (&w)[4], float eps, uint32_t buf)
     {
         const uint32_t sq = ssq + buf * static_cast<uint32_t>(NW * T * 16);
 #pragma unroll
@@ -457,7 +462,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
             valid[j] = id >= 0 && id < p.rows;
             if (!valid[j] && g * T + j < p.M && threadIdx.x == 0 && rank == 0 && p.status) atomicOr(p.status, MOLE_STATUS_BAD_ID);
         }
-        y.load_hidden(static_cast<const unsigned char *>(p.hidden), g * T, p.M);
+        y.load_hidden(static_cast<const unsigned char *>(p.hidden), g * T, p.M, []() {});
 #pragma unroll(T == 1 && N == 16 ? 2 : 1)
         for (int l = 0; l < L; ++l) {
             y.arm(buf);
@@ -534,12 +539,6 @@ __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(
         if (!valid[j] && t0 + j < p.M && threadIdx.x == 0 && p.status) atomicOr(p.status, MOLE_STATUS_BAD_ID);
     }
     cp_async_commit();
-    unsigned short wgt[4] = {0, 0, 0, 0};
-    if constexpr (NORM) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            wgt[i] = __ldg(reinterpret_cast<const unsigned short *>(static_cast<const unsigned char *>(p.norm_weight) + warp * 256 + y.own_off + Layer::col(i)));
-    }
     __syncthreads();  // the barrier is initialised
     if (!wait_or_give_up(bar, 0, dead, p.wait_polls)) {  // nothing waits any more: what is there is computed on, and the status says so
         if (lane == 0) report_timeout(dead, p.status);
@@ -561,6 +560,7 @@ __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(
 
     pdl_wait();
 
+    uint32_t wgt[4] = {0u, 0u, 0u, 0u};
     unsigned short res[T][4] = {};
     if (p.residual) {
         const unsigned char *src = static_cast<const unsigned char *>(p.residual) + warp * 256 + y.own_off;
@@ -570,7 +570,12 @@ __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(
             for (int i = 0; i < 4; ++i)
                 if (t0 + j < p.M) res[j][i] = __ldcg(reinterpret_cast<const unsigned short *>(src + static_cast<size_t>(t0 + j) * (D * 2) + Layer::col(i)));
     }
-    y.load_hidden(static_cast<const unsigned char *>(p.hidden), t0, p.M);
+    y.load_hidden(static_cast<const unsigned char *>(p.hidden), t0, p.M, [&]() {
+        if constexpr (NORM) {  // MOLE_FLAG_CHAIN does not forbid the kernel before to write the scale
+#pragma unroll
+            for (int i = 0; i < 4; ++i) wgt[i] = ld_scale_u16(static_cast<const unsigned char *>(p.norm_weight) + warp * 256 + y.own_off + Layer::col(i));
+        }
+    });
     if constexpr (NORM) y.normalise(wgt, p.norm_eps, 0);
     y.logits(wf, 0);
     if (p.residual) {  // it takes the hidden state's place in what follows

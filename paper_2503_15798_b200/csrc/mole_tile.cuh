@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(tile_narrow(D) ? 256 : kTileMaxWarps * 32, til
                 lane_reduce_scatter<8, 8, 16, 1>(s, lane, first);
                 if ((lane & 3) == 0 && k0 + first < TB) ssq[(k0 + first) * nw + warp] = s[0];
             }
-            const uint2 wv = __ldg(reinterpret_cast<const uint2 *>(static_cast<const unsigned char *>(p.norm_weight) + static_cast<size_t>(warp) * (kSliceCols * 2) + lane * 8));
+            const uint2 wv = ld_scale_v2(static_cast<const unsigned char *>(p.norm_weight) + static_cast<size_t>(warp) * (kSliceCols * 2) + lane * 8);
             __syncthreads();
             const float w0 = bf16_bits_to_float(wv.x & 0xffffu), w1 = __uint_as_float(wv.x & 0xffff0000u);
             const float w2 = bf16_bits_to_float(wv.y & 0xffffu), w3 = __uint_as_float(wv.y & 0xffff0000u);

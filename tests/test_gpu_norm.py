@@ -134,3 +134,33 @@ def test_cluster_kernel_with_a_separate_residual(norm):
         assert np.abs(as_f64(gates) - gref).max() <= 1e-5
         err = np.abs(as_f64(out) - ref)
         assert (err <= 2.0 ** -8 * np.abs(ref) + 2e-5).all(), float(err.max())
+
+
+@pytest.mark.parametrize("M,N,d,kernel,quant", [(1, 16, 768, mole.KERNEL_AUTO, None), (300, 16, 1024, mole.KERNEL_AUTO, None), (2000, 16, 768, mole.KERNEL_AUTO, None),
+                                                (60, 32, 2048, mole.KERNEL_AUTO, None), (200, 32, 2048, mole.KERNEL_AUTO, None), (40, 16, 1536, mole.KERNEL_RING, None),
+                                                (40, 16, 768, mole.KERNEL_DECODE, None), (40, 4, 512, mole.KERNEL_DECODE, None), (40, 16, 768, mole.KERNEL_AUTO, mole.LUT_NF4)])
+def test_a_chained_layer_reads_the_scale_that_the_kernel_before_wrote(M, N, d, kernel, quant):
+    """A chained launch may start early, but of what the kernel before it may write -- the scale among it -- it reads nothing early.  The
+    kernel before is a layer, so that it lets the next one start, and its last token's output is the scale."""
+    hidden, ids, lut, wr = (t.to(DEV) for t in rand_case(M, N, d, 64, seed=M + d))
+    wr = wr * 8
+    table = lut if quant is None else mole.QuantTable.quantize(lut, quant, d)
+    for before in (1, 100, 300, 3000):
+        h0, i0, l0, w0 = (t.to(DEV) for t in rand_case(before, 16, 768 if d == 768 else 1024, 64, seed=before))
+        out0 = torch.zeros(max(h0.numel(), d), dtype=torch.bfloat16, device=DEV)
+        gamma = out0[h0.numel() - d:h0.numel()] if h0.numel() >= d else out0[:d]
+        if gamma.data_ptr() % 16:
+            pytest.skip("the scale must be aligned")
+
+        def pair(chain):
+            out0.zero_()
+            out = torch.empty_like(hidden)
+            mole.layer_forward(h0, i0, l0, w0, out=out0[:h0.numel()].view_as(h0))
+            mole.layer_forward(hidden, ids, table, wr, out=out, norm_weight=gamma, norm_eps=1e-5, kernel=kernel, chain=chain)
+            torch.cuda.synchronize()
+            return out
+
+        want = pair(False)
+        assert float(gamma.float().abs().max()) > 0 and not torch.equal(want, mole.layer_forward(hidden, ids, table, wr, norm_weight=torch.zeros_like(gamma), norm_eps=1e-5, kernel=kernel))
+        for _ in range(5):
+            assert torch.equal(pair(True), want), before
