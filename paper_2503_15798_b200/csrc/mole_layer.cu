@@ -346,7 +346,13 @@ static SlicePlan slice_plan(long long M, int L, int sms)
 {
     constexpr int NW = D / kMmaCols;
     const long long groups = (M + T - 1) / T;
-    if (L == 1) return {mole_slice_layer_kernel<D, T, NORM>, NW * 32, static_cast<int>(slice_smem(16, NW, T, 1, NORM).total), groups};
+    if (L == 1) {
+        const int smem = static_cast<int>(slice_smem(16, NW, T, 1, NORM).total);
+        const long long resident = 2LL * sms;  // blocks at once, by their registers
+        if constexpr (T == 2)
+            if (groups > resident) return {mole_slice_layer_kernel<D, T, NORM, 1>, NW * 32, smem, resident};
+        return {mole_slice_layer_kernel<D, T, NORM, 0>, NW * 32, smem, groups};
+    }
     constexpr int NB = NW / CS;
     return {mole_slice_step_kernel<16, D, T, NORM, CS>, (NB + slice_copy_warps(16)) * 32, static_cast<int>(slice_smem(16, NB, T, slice_slots(16, NB, T, CS), NORM, CS).total),
             (groups < sms / CS ? groups : sms / CS) * CS};

@@ -500,8 +500,19 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
 }
 
 // One layer, a block per group of T tokens.  What does not depend on the kernel before -- router matrix (one bulk copy for the
-// block), rows -- is requested before it is waited for.
-template <int D, int T, int NORM>
+// block), rows -- is requested before it is waited for.  LOOP: a launch of more groups than are resident at once; a block then walks every
+// gridDim.x-th, and copies the rows of the next into the slots as soon as it has those of this one in registers: where 300 groups met
+// 296 places the last four cost a wave of their own (chained layers, us each, a block per group / here: 16 x 1024, 600 tokens 6.1 / 4.7, with the
+// norm 7.1 / 6.0; 888 tokens 6.9 / 5.7, 8.0 / 6.8; 16 x 768, 600 tokens 5.0 / 3.7, 5.8 / 4.4).
+template <int LOOP>
+struct SliceIndex {
+    using type = int;
+};
+template <>
+struct SliceIndex<0> {
+    using type = long long;
+};
+template <int D, int T, int NORM, int LOOP>
 __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(const StepParams p)
 {
     constexpr int N = 16, NW = D / kMmaCols;
@@ -516,7 +527,10 @@ __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(
     Layer y;
     y.init(base, m);
     const int lane = y.lane, warp = y.warp;
-    const long long t0 = static_cast<long long>(blockIdx.x) * T;
+    // (a launch has fewer than 2^30 tokens; without the loop 64 bits measured 1 - 2 % faster, with it they are spilled)
+    using Index = typename SliceIndex<LOOP>::type;
+    const Index M = static_cast<Index>(p.M);
+    Index t0 = static_cast<Index>(blockIdx.x) * T;
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + m.off_bar);
     volatile int *dead = reinterpret_cast<volatile int *>(bar + 1);
     if (threadIdx.x == 0) {
@@ -527,18 +541,22 @@ __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(
         mbar_expect_tx(bar, kRouterBytes);
         bulk_g2s(smem, p.w_router, kRouterBytes, bar);
     }
-    long long id[T];
-    bool valid[T];
+    bool valid[T], valid_next[T];  // of the tokens at hand; of those whose rows are on their way
+    const uint32_t slots = base + static_cast<uint32_t>(NW + warp) * slice_bytes(N);  // this warp's slices, one per token
+    auto copy_rows = [&](Index t1) {
+        long long id[T];
 #pragma unroll
-    for (int j = 0; j < T; ++j) id[j] = t0 + j < p.M ? slice_id(p, t0 + j) : -1;
+        for (int j = 0; j < T; ++j) id[j] = t1 + j < M ? slice_id(p, t1 + j) : -1;
 #pragma unroll
-    for (int j = 0; j < T; ++j) {
-        valid[j] = id[j] >= 0 && id[j] < p.rows;  // otherwise row 0 is fetched and its term dropped
-        const unsigned char *row = static_cast<const unsigned char *>(p.lut) + static_cast<size_t>(valid[j] ? id[j] : 0) * (N * D * 2) + warp * 256;
-        slice_copy_rows<N, D>(base + static_cast<uint32_t>(1 + j) * (NW * slice_bytes(N)) + static_cast<uint32_t>(warp) * slice_bytes(N), row, lane);
-        if (!valid[j] && t0 + j < p.M && threadIdx.x == 0 && p.status) atomicOr(p.status, MOLE_STATUS_BAD_ID);
-    }
-    cp_async_commit();
+        for (int j = 0; j < T; ++j) {
+            valid_next[j] = id[j] >= 0 && id[j] < p.rows;  // otherwise row 0 is fetched and its term dropped
+            const unsigned char *row = static_cast<const unsigned char *>(p.lut) + static_cast<size_t>(valid_next[j] ? id[j] : 0) * (N * D * 2) + warp * 256;
+            slice_copy_rows<N, D>(slots + static_cast<uint32_t>(j) * (NW * slice_bytes(N)), row, lane);
+            if (!valid_next[j] && t1 + j < M && threadIdx.x == 0 && p.status) atomicOr(p.status, MOLE_STATUS_BAD_ID);
+        }
+        cp_async_commit();
+    };
+    copy_rows(t0);
     __syncthreads();  // the barrier is initialised
     if (!wait_or_give_up(bar, 0, dead, p.wait_polls)) {  // nothing waits any more: what is there is computed on, and the status says so
         if (lane == 0) report_timeout(dead, p.status);
@@ -551,49 +569,70 @@ __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(
 #pragma unroll
         for (int k = 0; k < 8; ++k) ldsm_x4_trans(wf.a[k][0], w + static_cast<uint32_t>(k) * 512u);
     }
-
-    cp_async_wait<0>();
-    __syncwarp();
-    RowsA<N> rows[T];
+    uint32_t buf = 0;
+#pragma unroll 1
+    for (bool first = true;; first = false) {
+        cp_async_wait<0>();
+        __syncwarp();
+        RowsA<N> rows[T];
 #pragma unroll
-    for (int j = 0; j < T; ++j) rows[j].load(base + static_cast<uint32_t>(1 + j) * (NW * slice_bytes(N)) + static_cast<uint32_t>(warp) * slice_bytes(N) + RowsA<N>::lane_offset(lane));
-
-    pdl_wait();
-
-    uint32_t wgt[4] = {0u, 0u, 0u, 0u};
-    unsigned short res[T][4] = {};
-    if (p.residual) {
-        const unsigned char *src = static_cast<const unsigned char *>(p.residual) + warp * 256 + y.own_off;
+        for (int j = 0; j < T; ++j) rows[j].load(slots + static_cast<uint32_t>(j) * (NW * slice_bytes(N)) + RowsA<N>::lane_offset(lane));
 #pragma unroll
-        for (int j = 0; j < T; ++j)
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (t0 + j < p.M) res[j][i] = __ldcg(reinterpret_cast<const unsigned short *>(src + static_cast<size_t>(t0 + j) * (D * 2) + Layer::col(i)));
-    }
-    y.load_hidden(static_cast<const unsigned char *>(p.hidden), t0, p.M, [&]() {
-        if constexpr (NORM) {  // MOLE_FLAG_CHAIN does not forbid the kernel before to write the scale
-#pragma unroll
-            for (int i = 0; i < 4; ++i) wgt[i] = ld_scale_u16(static_cast<const unsigned char *>(p.norm_weight) + warp * 256 + y.own_off + Layer::col(i));
+        for (int j = 0; j < T; ++j) valid[j] = valid_next[j];
+        const Index t1 = t0 + static_cast<Index>(gridDim.x) * T;
+        const bool more = LOOP != 0 && t1 < M;
+        if (LOOP) {
+            __syncwarp();
+            if (more) copy_rows(t1);
         }
-    });
-    if constexpr (NORM) y.normalise(wgt, p.norm_eps, 0);
-    y.logits(wf, 0);
-    if (p.residual) {  // it takes the hidden state's place in what follows
+
+        if (first) pdl_wait();
+
+        uint32_t wgt[4] = {0u, 0u, 0u, 0u};
+        unsigned short res[T][4] = {};
+        auto load_residual = [&]() {
+            if (!p.residual) return;
+            const unsigned char *src = static_cast<const unsigned char *>(p.residual) + warp * 256 + y.own_off;
 #pragma unroll
-        for (int j = 0; j < T; ++j)
+            for (int j = 0; j < T; ++j)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) y.h[j][i] = bf16_bits_to_float(res[j][i]);
+                for (int i = 0; i < 4; ++i)
+                    if (t0 + j < M) res[j][i] = __ldcg(reinterpret_cast<const unsigned short *>(src + static_cast<size_t>(t0 + j) * (D * 2) + Layer::col(i)));
+        };
+        if (!LOOP) load_residual();
+        y.load_hidden(static_cast<const unsigned char *>(p.hidden), t0, M, [&]() {
+            if constexpr (NORM) {  // MOLE_FLAG_CHAIN does not forbid the kernel before to write the scale
+#pragma unroll
+                for (int i = 0; i < 4; ++i) wgt[i] = ld_scale_u16(static_cast<const unsigned char *>(p.norm_weight) + warp * 256 + y.own_off + Layer::col(i));
+            }
+        });
+        if constexpr (NORM) y.normalise(wgt, p.norm_eps, buf);
+        y.logits(wf, buf);
+        auto use_residual = [&]() {  // it takes the hidden state's place in what follows
+            if (!p.residual) return;
+#pragma unroll
+            for (int j = 0; j < T; ++j)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) y.h[j][i] = bf16_bits_to_float(res[j][i]);
+        };
+        if (LOOP) load_residual();  // (late, for want of registers)
+        else use_residual();
+        const float e = y.numerators(buf, []() {});
+        if (LOOP) use_residual();
+        if (p.gates_out && warp == 0) {
+            float sum = e;
+#pragma unroll
+            for (int o = 8; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            const Index t = t0 + (T == 2 ? lane >> 4 : 0);
+            if ((T == 2 || lane < 16) && t < M) p.gates_out[static_cast<size_t>(t) * N + (lane & 15)] = e / sum;
+        }
+        y.weighted(rows, e, valid, [](int) {});
+        y.store_out(static_cast<unsigned char *>(p.out), t0, M);
+        if (!more) break;
+        t0 = t1;
+        buf ^= 1u;
+        __syncwarp();  // the state has been stored: its slices are free
     }
-    const float e = y.numerators(0, []() {});
-    if (p.gates_out && warp == 0) {
-        float sum = e;
-#pragma unroll
-        for (int o = 8; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        const long long t = t0 + (T == 2 ? lane >> 4 : 0);
-        if ((T == 2 || lane < 16) && t < p.M) p.gates_out[t * N + (lane & 15)] = e / sum;
-    }
-    y.weighted(rows, e, valid, [](int) {});
-    y.store_out(static_cast<unsigned char *>(p.out), t0, p.M);
 }
 
 #endif  // __CUDACC__

@@ -13,7 +13,7 @@ from test_gpu_variants import _oracle_chain
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
 N, V, SMS = 16, 61, 148
-COUNTS = [1, SMS // 2, SMS // 2 + 1, SMS, SMS + 1, 2 * SMS + 1, 4 * SMS + 3]
+COUNTS = [1, SMS // 2, SMS // 2 + 1, SMS, SMS + 1, 2 * SMS + 1, 4 * SMS, 4 * SMS + 3]
 
 
 def _case(d, M, L, norm):
@@ -54,16 +54,43 @@ def test_steps_against_the_oracles_chain_and_bits_in_every_batch(d, norm):
         assert torch.equal(last[t], h[t])
 
 
-@pytest.mark.parametrize("M", [1, SMS, SMS + 2, 301])
+@pytest.mark.parametrize("M", [1, SMS, SMS + 2, 301, 4 * SMS + 1, 6 * SMS, 1501])
 @pytest.mark.parametrize("d", [768, 1024])
 def test_single_layer_with_gates_residual_and_wide_ids(d, M):
+    """One token or two per block, and blocks that walk several pairs."""
     luts, wrs, hidden, ids, _ = _case(d, M, 1, False)
     res = torch.empty(M, d).normal_(0, 1, generator=torch.Generator().manual_seed(M)).to(torch.bfloat16)
     ref, gref, _ = oracle_layer(hidden, ids, luts[0], wrs[0], residual=res)
     gates = torch.zeros(M, N, dtype=torch.float32, device=DEV)
-    out = mole.layer_forward(hidden.to(DEV), ids.long().to(DEV), luts[0].to(DEV), wrs[0].to(DEV), residual=res.to(DEV), gates_out=gates)
+    out = mole.layer_forward(hidden.to(DEV), ids.long().to(DEV), luts[0].to(DEV), wrs[0].to(DEV), residual=res.to(DEV), gates_out=gates, kernel=mole.KERNEL_RING)
     check_out(out, ref)
     check_gates(gates, gref)
+
+
+@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("d", [768, 1024])
+def test_layers_of_blocks_that_walk_several_pairs(d, norm):
+    """1501 tokens, up to three pairs per block and one token left over: chained, in place, with residual, ids outside the table anywhere;
+    every token has the bits it has among few."""
+    M = 1501
+    luts, wrs, hidden, ids, gammas = _case(d, M, 2, norm)
+    bad = [0, 2 * 2 * SMS + 1, 700, 1199, M - 1]
+    ids[bad] = torch.tensor([-1, V, V + 7, -5, V], dtype=torch.int32)
+    h, i, lu, w = hidden.to(DEV), ids.to(DEV), luts.to(DEV), wrs.to(DEV)
+    res = torch.empty(M, d, device=DEV).normal_(0, 1, generator=torch.Generator(device=DEV).manual_seed(2)).to(torch.bfloat16)
+    gam = [None, None] if gammas is None else list(gammas.to(DEV))
+
+    def layers(s, status):
+        x = h[s].clone()
+        mole.layer_forward(x, i[s], lu[0], w[0], out=x, norm_weight=gam[0], norm_eps=1e-5, kernel=mole.KERNEL_RING, status=status)
+        return mole.layer_forward(x, i[s], lu[1], w[1], residual=res[s], norm_weight=gam[1], norm_eps=1e-5, kernel=mole.KERNEL_RING, status=status, chain=True)
+
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    out = layers(slice(0, M), status)
+    assert int(status.item()) == mole.STATUS_BAD_ID
+    for a, n in ((0, 1), (5, 40), (593, 300), (1301, 200)):
+        assert torch.equal(layers(slice(a, a + n), None), out[a:a + n]), (a, n)
+    assert torch.equal(out[bad], res[bad])
 
 
 @pytest.mark.parametrize("norm", [False, True])
