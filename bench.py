@@ -499,7 +499,7 @@ def config_rows(torch, mole, inputs, sh, L, luts, wrs, batches, steps, warmup, p
         modes = [("chained", mole.STEP_CHAINED, mole.KERNEL_AUTO, None)]
         if decode_family_covers(m, sh, 1):
             modes.append(("chained_one_block_per_token", mole.STEP_CHAINED, mole.KERNEL_DECODE, None))
-        if not mole.variant(m, sh.N, sh.d)[0].startswith("step"):  # the library's own choice is not the ring kernel: time that too
+        if mole.variant(m, sh.N, sh.d)[0] != mole.variant(m, sh.N, sh.d, kernel=mole.KERNEL_RING)[0]:  # MOLE_KERNEL_RING is another: time that too
             modes.append(("chained_ring", mole.STEP_CHAINED, mole.KERNEL_RING, None))
         if m <= 4096:
             modes.append(("fused", mole.STEP_FUSED, mole.KERNEL_AUTO, None))

@@ -94,12 +94,14 @@ extern "C" {
                                    than 2, 6 or 8 tokens per SM [296, 888, 1184] for rows N*d*2 above 32 KB, above 16 KB, or   \
                                    smaller.                                                                                    \
                                 Fused steps: the ring kernel, except                                                           \
+                                 - the step of bf16, N = 32, d = 2048, d_split 0, up to a token per four SMs [37], which has its   \
+                                   sizes compiled in and gives the bits of the next;                                          \
                                  - the tensor-core step: bf16, N of 8, 16 or 32, d a multiple of 128 up to 2048 but not 768 or \
                                    1024 with N = 16, d_split 0, layer strides a tensor map takes (16 bytes to 2^40).  A token  \
                                    has 1, 2 or 4 blocks, the fewest with at most 1024 columns and 32 KB of its rows each; up   \
                                    to as many blocks as SMs, or twice as many (while all are resident) where a block's part is \
                                    at most 24 KB or a token's rows are 128 KB.  [N = 32: 148 tokens at d = 512, up to 74 at    \
-                                   1024 and 2048.]                                                                             \
+                                   1024 and 2048.]  (Strides out of range: the ring kernel.)                                   \
                                 mole_variant says which. */
 #define MOLE_KERNEL_RING 1   /* persistent blocks, rows and router chunks streamed through a shared-memory ring: any shape (bf16, N = 16,  \
                                 d = 768 or 1024 in one chunk: kernels of their own, a warp per 128 columns, on the tensor cores, with the   \
@@ -517,6 +519,8 @@ MOLE_API int mole_version(void);
  *   group in the combine), MOLE_FORCE_COLUMN_CHUNKS (1: cut the rows by columns even where the expert
  *   cut exists), MOLE_FORCE_KERNEL (1, 2: MOLE_KERNEL_* for launches that leave the choice open),
  *   MOLE_FORCE_BUILDER_TILES (1: the table builder's single blocks, 2: its pairs of blocks).
+ * STAGES, TARGET_BLOCKS and BLOCKS_PER_SM are about the ring kernel and the fused step of MOLE_KERNEL_DECODE; the other kernels
+ * have no such choice.  LANES takes N = 16, d = 768 and 1024 from the kernels of these widths to the ring kernel.
  * One of them shortens the bounded waits inside the kernels, to let a test see a wait run out:
  *   MOLE_DEBUG_WAIT_LIMIT (n >= 1: a wait gives up after n polls; negative: after none -- any wait that
  *   is not satisfied at once gives up).  The launch then returns normally with MOLE_STATUS_TIMEOUT in
@@ -532,10 +536,13 @@ MOLE_API int mole_plan(int M, int L, int N, int d, int dtype, int d_split, int *
               int *out_smem_bytes, int *out_stages, int *out_blocks_per_sm);
 
 /* Name of the kernel instantiation a launch of this shape runs, with its block size and dynamic shared memory:
- *   "step<storage,N,P,MODE,SHAPE,DIRECT,NORM>"        the ring kernel; SHAPE 1 and 2: the kernels of bf16, N = 16, d = 768 and 1024
+ *   "step<storage,N,P,MODE,SHAPE,NORM>"               the ring kernel
+ *   "slice_layer<d,T,NORM,LOOP>"                      a layer of bf16, N = 16, d = 768 or 1024: T tokens per block, LOOP 1 more than
+ *                                                     are resident at once
+ *   "slice_step<N,d,T,NORM,CS>"                       the fused steps of these widths, and of N = 32, d = 2048: CS blocks per token
  *   "tile<N,NORM,width,PARTS>"                        the prefill kernel
- *   "mma<N,NORM,CS>"                                  the tensor-core step (a step whose layer strides are below 16 bytes or from
- *                                                     2^40 on, which a tensor map does not take, runs the ring kernel instead)
+ *   "mma<N,NORM,CS>"                                  the general tensor-core step (where this is named, a step whose layer strides are
+ *                                                     below 16 bytes or from 2^40 on, which a tensor map does not take, runs the ring kernel)
  *   "decode<N,NORM>" "cdecode<N,CS,NORM>" "fstep<N,DB,NORM>"  the kernels of MOLE_KERNEL_DECODE
  *   "qdecode<N,nfB,NORM>" "qstep<N,nfB,NORM>"         quantised layers and steps
  * L == 1: a single layer, or a layer of a CHAINED step; L > 1: a FUSED step, over quantised tables what MOLE_STEP_AUTO runs.

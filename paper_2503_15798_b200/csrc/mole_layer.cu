@@ -2,6 +2,7 @@
 // for a single layer and for a chained L-layer decode step (Eq. 4 and Eq. 8 of arXiv
 // 2503.15798).  The kernel itself is in mole_kernel.cuh.
 #include <atomic>
+#include <initializer_list>
 #include <mutex>
 #include <stdio.h>
 #include <stdlib.h>
@@ -217,22 +218,17 @@ int plan_step(long long M, int L, int N, int d, int dtype, int d_split, StepPlan
     return MOLE_OK;
 }
 
-// A kernel instantiation and its name ("step<storage,NFAST,P,MODE,SHAPE,DIRECT,NORM>" for the ring
-// kernel -- SHAPE 1 and 2: the kernels of mole_slice.cuh, MODE 2 a single layer and MODE 1 a fused step, DIRECT 1 from 128 tokens up to
-// four per SM, which once was a kernel of its own and is a part of the name only -- "decode<N,NORM>" for the one-block-per-token kernel): what mole_variant() reports, so that a
+// A kernel instantiation and its name ("step<storage,NFAST,P,MODE,SHAPE,NORM>" for the ring kernel,
+// "decode<N,NORM>" for the one-block-per-token kernel, ..): what mole_variant() reports, so that a
 // test can tell which instantiations a workload reaches.
 typedef void (*StepKernel)(const StepParams);
 typedef void (*DecodeKernel)(const DecodeParams);
 struct Variant {
     StepKernel fn;
     const char *name;
-    bool slice = false;  // the kernels of mole_slice.cuh, chosen by slice_kernel()
 };
-// N = 16, d = 768 and 1024 (SHAPE 1 and 2): mole_slice.cuh
-#define MOLE_VS(MODE, SHAPE, DIRECT, NORM) \
-    Variant { nullptr, "step<bf16,16,1," #MODE "," #SHAPE "," #DIRECT "," #NORM ">", true }
 #define MOLE_V(T, TN, NF, P, MODE, SHAPE, NORM) \
-    Variant { mole_step_kernel<T, NF, P, MODE, SHAPE, NORM>, "step<" TN "," #NF "," #P "," #MODE "," #SHAPE ",0," #NORM ">" }
+    Variant { mole_step_kernel<T, NF, P, MODE, SHAPE, NORM>, "step<" TN "," #NF "," #P "," #MODE "," #SHAPE "," #NORM ">" }
 #define MOLE_VB(NF, P, MODE, SHAPE, NORM) MOLE_V(__nv_bfloat16, "bf16", NF, P, MODE, SHAPE, NORM)
 #define MOLE_VF(NF, P, MODE, SHAPE, NORM) MOLE_V(float, "f32", NF, P, MODE, SHAPE, NORM)
 static const Variant kNoVariant = {nullptr, "none"};
@@ -277,14 +273,10 @@ static Variant pick_f32(int n_fast, int lanes)
 // The generic-N router and the fp32 storage type exist only with run-time flags (MODE 0); bf16 with
 // a compiled-in N also in the specialised shapes.
 static Variant pick_kernel(int dtype, int n_fast, int lanes, int chunks, int in_ring, int d, int dcc, int consumers,
-                           int by_expert, bool direct)
+                           int by_expert)
 {
-    // the layer widths of the paper's Table 2 (160M, 410M and 1B models) with their sizes compiled in
+    // the widest layer of the paper's Table 2 with its sizes compiled in (the others: slice_shape_ok)
     if (dtype == MOLE_DTYPE_BF16) {
-        if (n_fast == 16 && lanes == 1 && chunks == 1 && d == 768 && consumers == 96)
-            return in_ring ? MOLE_VS(1, 1, 0, 0) : (direct ? MOLE_VS(2, 1, 1, 0) : MOLE_VS(2, 1, 0, 0));
-        if (n_fast == 16 && lanes == 1 && chunks == 1 && d == 1024 && consumers == 128)
-            return in_ring ? MOLE_VS(1, 2, 0, 0) : (direct ? MOLE_VS(2, 2, 1, 0) : MOLE_VS(2, 2, 0, 0));
         if (n_fast == 32 && lanes == 2 && chunks == 4 && d == 2048 && dcc == 512 && consumers == 128 && by_expert)
             return MOLE_VB(32, 2, 3, 3, 0);
         if (n_fast == 32 && lanes == 2 && chunks == 2 && d == 2048 && dcc == 1024 && consumers == 128 && by_expert)
@@ -316,18 +308,9 @@ static Variant pick_norm_kernel(int dtype, int n_fast, int lanes)
     MOLE_PICK_N_F32(1, 0, 1)
 }
 // ... and, for the paper's three layer widths, with the sizes compiled in (single layers and fused steps)
-static Variant pick_norm_shape_kernel(const StepPlan &plan, int dtype, int d, bool direct)
+static Variant pick_norm_shape_kernel(const StepPlan &plan, int dtype, int d)
 {
     if (dtype != MOLE_DTYPE_BF16) return kNoVariant;
-    if (plan.n_fast == 16 && plan.lanes == 1 && plan.d_split == 1) {
-        if (!plan.wr_in_ring) {
-            if (d == 768 && plan.consumers == 96) return direct ? MOLE_VS(2, 1, 1, 1) : MOLE_VS(2, 1, 0, 1);
-            if (d == 1024 && plan.consumers == 128) return direct ? MOLE_VS(2, 2, 1, 1) : MOLE_VS(2, 2, 0, 1);
-        } else {
-            if (d == 768 && plan.consumers == 96) return MOLE_VS(1, 1, 0, 1);
-            if (d == 1024 && plan.consumers == 128) return MOLE_VS(1, 2, 0, 1);
-        }
-    }
     if (plan.n_fast == 32 && plan.lanes == 2 && d == 2048 && plan.consumers == 128 && plan.rows_by_expert) {
         if (plan.d_split == 4 && plan.dc == 512) return MOLE_VB(32, 2, 3, 3, 1);
         if (plan.d_split == 2 && plan.dc == 1024) return MOLE_VB(32, 2, 3, 4, 1);
@@ -335,12 +318,38 @@ static Variant pick_norm_shape_kernel(const StepPlan &plan, int dtype, int d, bo
     return kNoVariant;
 }
 
-// The kernels of mole_slice.cuh: T tokens per block.  One up to one token per SM, two beyond.
+// The kernels of mole_slice.cuh for the two narrow widths of the paper's Table 2, in one chunk (MOLE_FORCE_LANES asks for the ring
+// kernel).  T tokens per block.  One up to one token per SM, two beyond.
+static bool slice_shape_ok(const StepPlan &plan, int dtype, int d)
+{
+    return dtype == MOLE_DTYPE_BF16 && plan.n_fast == 16 && plan.lanes == 1 && plan.d_split == 1 && (d == 768 || d == 1024);
+}
 struct SlicePlan {
     StepKernel fn;
+    const char *name;
     int threads, smem;
     long long grid;
 };
+// "family<V, ..>", made once per instantiation
+template <int... V>
+static const char *slice_name(const char *family)
+{
+    struct Name {
+        char text[48];
+        explicit Name(const char *f)
+        {
+            int at = snprintf(text, sizeof text, "%s", f);
+            char before = '<';
+            for (const int v : {V...}) {
+                at += snprintf(text + at, sizeof text - at, "%c%d", before, v);
+                before = ',';
+            }
+            snprintf(text + at, sizeof text - at, ">");
+        }
+    };
+    static const Name name(family);
+    return name.text;
+}
 template <int D, int T, int NORM, int CS>
 static SlicePlan slice_plan(long long M, int L, int sms)
 {
@@ -350,12 +359,12 @@ static SlicePlan slice_plan(long long M, int L, int sms)
         const int smem = static_cast<int>(slice_smem(16, NW, T, 1, NORM).total);
         const long long resident = 2LL * sms;  // blocks at once, by their registers
         if constexpr (T == 2)
-            if (groups > resident) return {mole_slice_layer_kernel<D, T, NORM, 1>, NW * 32, smem, resident};
-        return {mole_slice_layer_kernel<D, T, NORM, 0>, NW * 32, smem, groups};
+            if (groups > resident) return {mole_slice_layer_kernel<D, T, NORM, 1>, slice_name<D, T, NORM, 1>("slice_layer"), NW * 32, smem, resident};
+        return {mole_slice_layer_kernel<D, T, NORM, 0>, slice_name<D, T, NORM, 0>("slice_layer"), NW * 32, smem, groups};
     }
     constexpr int NB = NW / CS;
-    return {mole_slice_step_kernel<16, D, T, NORM, CS>, (NB + slice_copy_warps(16)) * 32, static_cast<int>(slice_smem(16, NB, T, slice_slots(16, NB, T, CS), NORM, CS).total),
-            (groups < sms / CS ? groups : sms / CS) * CS};
+    return {mole_slice_step_kernel<16, D, T, NORM, CS>, slice_name<16, D, T, NORM, CS>("slice_step"), (NB + slice_copy_warps(16)) * 32,
+            static_cast<int>(slice_smem(16, NB, T, slice_slots(16, NB, T, CS), NORM, CS).total), (groups < sms / CS ? groups : sms / CS) * CS};
 }
 template <int D>
 static SlicePlan slice_plan_d(long long M, int L, bool norm, int sms)
@@ -370,7 +379,8 @@ template <int NORM>
 static int slice_plan_1b(long long M, int sms, bool prepare, SlicePlan *sp)
 {
     constexpr int CS = 4, NB = 2048 / kMmaCols / CS;
-    *sp = {mole_slice_step_kernel<32, 2048, 1, NORM, CS>, (NB + slice_copy_warps(32)) * 32, static_cast<int>(slice_smem(32, NB, 1, slice_slots(32, NB, 1, CS), NORM, CS).total), 0};
+    *sp = {mole_slice_step_kernel<32, 2048, 1, NORM, CS>, slice_name<32, 2048, 1, NORM, CS>("slice_step"), (NB + slice_copy_warps(32)) * 32,
+           static_cast<int>(slice_smem(32, NB, 1, slice_slots(32, NB, 1, CS), NORM, CS).total), 0};
     int clusters = sms / CS;
     if (prepare) {
         int rc = ensure_smem_opt_in(reinterpret_cast<const void *>(sp->fn), sp->smem);
@@ -688,7 +698,7 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
             c->plan = plan;
             c->step_fn = sp.fn;
             c->decode_fn = nullptr;
-            c->name = c->mplan.name;
+            c->name = sp.name;
             c->threads = sp.threads;
             c->smem = sp.smem;
             c->grid = sp.grid;
@@ -723,20 +733,21 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
         if (prepare) return ensure_smem_opt_in(reinterpret_cast<const void *>(v.fn), c->smem);
         return MOLE_OK;
     }
-    const bool direct = M >= 128 && M <= 4LL * sms;  // see pick_kernel
+    const bool slice = slice_shape_ok(plan, dtype, d);
     Variant v = kNoVariant;
-    if (norm) {
-        v = pick_norm_shape_kernel(plan, dtype, d, direct && L == 1);
-        if (!v.fn && !v.slice) {
+    if (slice) {
+        // below, where a prefill launch has been sorted out
+    } else if (norm) {
+        v = pick_norm_shape_kernel(plan, dtype, d);
+        if (!v.fn) {
             rc = plan_step(M, L, N, d, dtype, d_split, &plan, true, sms, true);  // the general kernels cut the rows by columns
             if (rc != MOLE_OK) return rc;
             v = pick_norm_kernel(dtype, plan.n_fast, plan.lanes);
         }
     } else {
-        v = pick_kernel(dtype, plan.n_fast, plan.lanes, plan.d_split, plan.wr_in_ring, d, plan.dc, plan.consumers, plan.rows_by_expert,
-                        direct);
+        v = pick_kernel(dtype, plan.n_fast, plan.lanes, plan.d_split, plan.wr_in_ring, d, plan.dc, plan.consumers, plan.rows_by_expert);
     }
-    if (!v.fn && !v.slice) return MOLE_ERR_UNSUPPORTED_SHAPE;
+    if (!v.fn && !slice) return MOLE_ERR_UNSUPPORTED_SHAPE;
     if (L == 1 && kernel == MOLE_KERNEL_AUTO && d_split == 0 && tile_shape_ok(dtype, N, d) && M > tile_from(N, d, sms)) {
         c->tile = true;
         rc = plan_tile(M, N, d, norm, sms, prepare, &c->tplan);
@@ -750,9 +761,10 @@ static int choose_launch(long long M, int L, int N, int d, int dtype, int d_spli
     c->name = v.name;
     c->threads = plan.threads;
     c->smem = plan.smem;
-    if (v.slice) {
+    if (slice) {
         const SlicePlan sp = d == 768 ? slice_plan_d<768>(M, L, norm, sms) : slice_plan_d<1024>(M, L, norm, sms);
         c->step_fn = sp.fn;
+        c->name = sp.name;
         c->threads = sp.threads;
         c->smem = sp.smem;
         c->grid = sp.grid;

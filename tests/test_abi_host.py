@@ -43,14 +43,16 @@ def test_version_and_status_strings(lib):
 def test_variant_names_and_kernel_choice(lib):
     V = binding.variant
     D, R = binding.KERNEL_DECODE, binding.KERNEL_RING
-    # the library's own choice: the ring kernel, but the prefill kernel for one layer of many tokens and the tensor-core step for
+    # the library's own choice: the kernels of the paper's widths, otherwise the ring kernel, but the prefill kernel for one layer of many tokens and the tensor-core step for
     # fused steps of the shapes where it is ahead
-    assert V(256, 16, 768)[0] == "step<bf16,16,1,2,1,1,0>" == V(256, 16, 768, kernel=R)[0]
-    assert V(16384, 16, 1024)[:2] == ("tile<16,0,1024,1>", 256) and V(16384, 16, 1024, kernel=R)[0] == "step<bf16,16,1,2,2,0,0>"
-    assert V(3000, 32, 2048, norm=True)[:2] == ("tile<32,1,2048,2>", 512) and V(3000, 16, 768, d_split=1)[0] == "step<bf16,16,1,2,1,0,0>"
-    assert V(256, 16, 768, L=12)[0] == "step<bf16,16,1,1,1,0,0>" and V(256, 32, 2048)[0] == "step<bf16,32,2,3,3,0,0>"
-    assert V(16, 32, 2048, L=16)[:2] == ("mma<32,0,4>", 160) and V(64, 32, 2048, L=16, kernel=R)[0] == "step<bf16,32,2,3,4,0,0>"
-    assert V(148, 32, 2048, L=16)[0] == "step<bf16,32,2,3,4,0,0>" and V(20, 32, 1024, L=2, norm=True)[:2] == ("mma<32,1,2>", 160)
+    assert V(256, 16, 768)[:2] == ("slice_layer<768,2,0,0>", 192) == V(256, 16, 768, kernel=R)[:2] and V(148, 16, 768, norm=True)[0] == "slice_layer<768,1,1,0>"
+    assert V(592, 16, 1024)[0] == "slice_layer<1024,2,0,0>" and V(593, 16, 1024)[0] == "slice_layer<1024,2,0,1>"
+    assert V(16384, 16, 1024)[:2] == ("tile<16,0,1024,1>", 256) and V(16384, 16, 1024, kernel=R)[0] == "slice_layer<1024,2,0,1>"
+    assert V(3000, 32, 2048, norm=True)[:2] == ("tile<32,1,2048,2>", 512) and V(3000, 16, 768, d_split=1)[0] == "slice_layer<768,2,0,1>"
+    assert V(256, 16, 768, L=12)[:2] == ("slice_step<16,768,2,0,1>", 320) and V(148, 16, 768, L=12)[0] == "slice_step<16,768,1,0,1>" and V(74, 16, 1024, L=2, norm=True)[0] == "slice_step<16,1024,1,1,2>"
+    assert V(256, 16, 768, d_split=2)[0].startswith("step<") and V(256, 32, 2048)[0] == "step<bf16,32,2,3,3,0>"
+    assert V(37, 32, 2048, L=16)[:2] == ("slice_step<32,2048,1,0,4>", 160) and V(38, 32, 2048, L=16)[:2] == ("mma<32,0,4>", 160) and V(64, 32, 2048, L=16, kernel=R)[0] == "step<bf16,32,2,3,4,0>"
+    assert V(148, 32, 2048, L=16)[0] == "step<bf16,32,2,3,4,0>" and V(20, 32, 1024, L=2, norm=True)[:2] == ("mma<32,1,2>", 160)
     # on request: one block per token (d / 4 threads), and the fused step built on it
     assert V(256, 16, 768, kernel=D) == ("decode<16,0>", 192, V(256, 16, 768, kernel=D)[2]) and V(64, 16, 1024, kernel=D)[:2] == ("decode<16,0>", 256)
     assert V(256, 16, 768, norm=True, kernel=D)[0] == "decode<16,1>" and V(64, 32, 1024, kernel=D)[0] == "decode<32,0>"
@@ -63,7 +65,7 @@ def test_variant_names_and_kernel_choice(lib):
         with pytest.raises(binding.MoleError) as e:  # shapes the family does not cover
             V(*args, kernel=D, **kw)
         assert e.value.code == binding.ERR_UNSUPPORTED_SHAPE
-    assert V(700, 32, 512)[0] == "step<bf16,32,2,2,0,0,0>" and V(700, 32, 640, L=2)[0] == "step<bf16,32,1,3,0,0,0>"
+    assert V(700, 32, 512)[0] == "step<bf16,32,2,2,0,0>" and V(700, 32, 640, L=2)[0] == "step<bf16,32,1,3,0,0>"
     assert V(64, 5, 768)[0].startswith("step<bf16,0,") and V(64, 4, 64, binding.DTYPE_F32)[0].startswith("step<f32,4,")
     # quantised tables
     assert V(256, 16, 768, lut_format=binding.LUT_NF4, lut_block=768)[:2] == ("qdecode<16,nf4,0>", 192)

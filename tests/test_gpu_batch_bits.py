@@ -9,11 +9,12 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 # N, d, L, norm, d_split, token counts with a line between every two of them, the families of MOLE_KERNEL_AUTO there
-CASES = [(16, 768, 1, False, 1, (40, 888, 889), ("step", "step", "tile")), (16, 1024, 1, True, 1, (40, 888, 889), ("step", "step", "tile")),
+CASES = [(16, 768, 1, False, 1, (40, 888, 889), ("slice_layer", "slice_layer", "tile")),
+         (16, 1024, 1, True, 1, (40, 888, 889), ("slice_layer", "slice_layer", "tile")),
          (8, 256, 1, False, 1, (3, 1184, 1185), ("step", "step", "tile")), (32, 640, 1, True, 2, (20, 296, 297), ("step", "step", "tile")),
          (32, 2048, 1, False, 4, (128, 140, 296, 297), ("cdecode", "step", "step", "tile")), (32, 1920, 1, True, 4, (148, 296, 297), ("step", "step", "tile")),
-         (32, 2048, 3, False, 4, (20, 64, 75), ("mma", "mma", "step")), (8, 1024, 2, True, 1, (148, 296, 297), ("mma", "mma", "step")),
-         (32, 512, 2, False, 1, (100, 148, 149), ("mma", "mma", "step")), (16, 768, 3, False, 1, (64, 300), ("step", "step"))]
+         (32, 2048, 3, False, 4, (20, 64, 75), ("slice_step", "mma", "step")), (8, 1024, 2, True, 1, (148, 296, 297), ("mma", "mma", "step")),
+         (32, 512, 2, False, 1, (100, 148, 149), ("mma", "mma", "step")), (16, 768, 3, False, 1, (64, 300), ("slice_step", "slice_step"))]
 
 
 @pytest.mark.parametrize("N,d,L,norm,split,counts,families", CASES)

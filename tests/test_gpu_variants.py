@@ -33,14 +33,21 @@ CASES = {
     "cdecode<32,4,1>": [(256, 32, 2048, 1, True, DEC), (16, 32, 2048, 1, True, AUTO), (1, 32, 2048, 1, True, DEC)],
     "cdecode<16,4,0>": [(40, 16, 2048, 1, False, DEC)],
     "cdecode<16,4,1>": [(40, 16, 2048, 1, True, DEC)],
-    "step<bf16,16,1,2,1,1,0>": [(256, 16, 768, 1, False, AUTO), (500, 16, 768, 1, False, AUTO)],  # the second: a one-slot ring
-    "step<bf16,16,1,2,1,0,0>": [(64, 16, 768, 1, False, AUTO), (3000, 16, 768, 1, False, RING)],
-    "step<bf16,16,1,2,2,1,0>": [(256, 16, 1024, 1, False, AUTO), (400, 16, 1024, 1, False, AUTO)],
-    "step<bf16,16,1,2,2,0,0>": [(64, 16, 1024, 1, False, AUTO), (2500, 16, 1024, 1, False, RING)],
-    "step<bf16,16,1,2,1,1,1>": [(256, 16, 768, 1, True, AUTO), (400, 16, 768, 1, True, AUTO)],  # the second: a one-slot ring
-    "step<bf16,16,1,2,1,0,1>": [(700, 16, 768, 1, True, AUTO)],
-    "step<bf16,16,1,2,2,1,1>": [(256, 16, 1024, 1, True, AUTO)],
-    "step<bf16,16,1,2,2,0,1>": [(2500, 16, 1024, 1, True, RING)],
+    # the widths of 768 and 1024: a token per block, two, blocks that walk several pairs (more cases: test_gpu_slice.py)
+    "slice_layer<768,1,0,0>": [(64, 16, 768, 1, False, AUTO), (1, 16, 768, 1, False, AUTO)],
+    "slice_layer<768,2,0,0>": [(256, 16, 768, 1, False, AUTO), (500, 16, 768, 1, False, AUTO)],
+    "slice_layer<768,2,0,1>": [(3000, 16, 768, 1, False, RING)],
+    "slice_layer<1024,1,0,0>": [(64, 16, 1024, 1, False, AUTO)],
+    "slice_layer<1024,2,0,0>": [(256, 16, 1024, 1, False, AUTO), (400, 16, 1024, 1, False, AUTO)],
+    "slice_layer<1024,2,0,1>": [(2500, 16, 1024, 1, False, RING)],
+    "slice_layer<768,1,1,0>": [(100, 16, 768, 1, True, AUTO)],
+    "slice_layer<768,2,1,0>": [(256, 16, 768, 1, True, AUTO), (400, 16, 768, 1, True, AUTO)],
+    "slice_layer<768,2,1,1>": [(700, 16, 768, 1, True, AUTO)],
+    "slice_layer<1024,1,1,0>": [(148, 16, 1024, 1, True, AUTO)],
+    "slice_layer<1024,2,1,0>": [(256, 16, 1024, 1, True, AUTO)],
+    "slice_layer<1024,2,1,1>": [(2500, 16, 1024, 1, True, RING)],
+    "step<bf16,16,1,2,0,0>": [(500, 16, 640, 1, False, AUTO), (700, 16, 640, 1, False, AUTO)],  # a one-slot ring
+    "step<bf16,16,1,0,0,1>": [(500, 16, 640, 1, True, AUTO), (256, 16, 1536, 3, True, AUTO), (64, 16, 1536, 2, True, RING)],  # the first: a one-slot ring
     # fused steps: the decode arithmetic with a ring (default) ...
     "fstep<16,1,0>": [(256, 16, 768, 3, False, DEC), (64, 16, 768, 12, False, DEC), (256, 16, 1024, 3, False, DEC),
                       (8, 16, 1024, 8, False, DEC), (1, 16, 768, 12, False, DEC), (700, 16, 768, 2, False, DEC)],
@@ -53,17 +60,27 @@ CASES = {
     "fstep<8,0,0>": [(33, 8, 256, 5, False, DEC)],
     "fstep<4,0,1>": [(33, 4, 128, 3, True, DEC)],
     # ... and the ring kernel's own fused form (on request; the offload step's groups)
-    "step<bf16,16,1,1,1,0,0>": [(256, 16, 768, 3, False, AUTO), (64, 16, 768, 12, False, AUTO)],
-    "step<bf16,16,1,1,2,0,0>": [(256, 16, 1024, 3, False, AUTO), (64, 16, 1024, 4, False, AUTO), (8, 16, 1024, 8, False, AUTO)],
-    "step<bf16,16,1,1,1,0,1>": [(256, 16, 768, 3, True, AUTO), (8, 16, 768, 12, True, AUTO)],
-    "step<bf16,16,1,1,2,0,1>": [(256, 16, 1024, 3, True, AUTO), (64, 16, 1024, 2, True, AUTO)],
-    "step<bf16,16,1,0,0,0,1>": [(256, 16, 1536, 3, True, AUTO), (64, 16, 1536, 2, True, RING)],
-    "step<bf16,32,2,3,3,0,0>": [(256, 32, 2048, 1, False, AUTO), (256, 32, 2048, 3, False, AUTO)],
-    "step<bf16,32,2,3,4,0,0>": [(64, 32, 2048, 1, False, RING), (140, 32, 2048, 1, False, AUTO), (64, 32, 2048, 3, False, RING), (148, 32, 2048, 2, False, AUTO)],
-    "step<bf16,32,2,3,3,0,1>": [(256, 32, 2048, 1, True, AUTO), (256, 32, 2048, 2, True, AUTO)],
-    "step<bf16,32,2,3,4,0,1>": [(16, 32, 2048, 1, True, RING), (64, 32, 2048, 2, True, RING)],
-    "step<bf16,32,1,0,0,0,1>": [(16, 32, 1024, 2, True, RING)],
-    "step<bf16,32,2,0,0,0,1>": [(256, 32, 4096, 2, True, AUTO)],
+    # (the widths of 768 and 1024: two blocks per token, a token per block, two)
+    "slice_step<16,768,1,0,2>": [(64, 16, 768, 12, False, AUTO)],
+    "slice_step<16,768,1,0,1>": [(120, 16, 768, 3, False, AUTO)],
+    "slice_step<16,768,2,0,1>": [(256, 16, 768, 3, False, AUTO)],
+    "slice_step<16,1024,1,0,2>": [(64, 16, 1024, 4, False, AUTO), (8, 16, 1024, 8, False, AUTO)],
+    "slice_step<16,1024,1,0,1>": [(148, 16, 1024, 2, False, AUTO)],
+    "slice_step<16,1024,2,0,1>": [(256, 16, 1024, 3, False, AUTO)],
+    "slice_step<16,768,1,1,2>": [(8, 16, 768, 12, True, AUTO)],
+    "slice_step<16,768,1,1,1>": [(75, 16, 768, 3, True, AUTO)],
+    "slice_step<16,768,2,1,1>": [(256, 16, 768, 3, True, AUTO)],
+    "slice_step<16,1024,1,1,2>": [(64, 16, 1024, 2, True, AUTO)],
+    "slice_step<16,1024,1,1,1>": [(148, 16, 1024, 2, True, AUTO)],
+    "slice_step<16,1024,2,1,1>": [(256, 16, 1024, 3, True, AUTO)],
+    "slice_step<32,2048,1,0,4>": [(16, 32, 2048, 16, False, AUTO), (1, 32, 2048, 16, False, AUTO), (37, 32, 2048, 3, False, AUTO)],
+    "slice_step<32,2048,1,1,4>": [(16, 32, 2048, 3, True, AUTO)],
+    "step<bf16,32,2,3,3,0>": [(256, 32, 2048, 1, False, AUTO), (256, 32, 2048, 3, False, AUTO)],
+    "step<bf16,32,2,3,4,0>": [(64, 32, 2048, 1, False, RING), (140, 32, 2048, 1, False, AUTO), (64, 32, 2048, 3, False, RING), (148, 32, 2048, 2, False, AUTO)],
+    "step<bf16,32,2,3,3,1>": [(256, 32, 2048, 1, True, AUTO), (256, 32, 2048, 2, True, AUTO)],
+    "step<bf16,32,2,3,4,1>": [(16, 32, 2048, 1, True, RING), (64, 32, 2048, 2, True, RING)],
+    "step<bf16,32,1,0,0,1>": [(16, 32, 1024, 2, True, RING)],
+    "step<bf16,32,2,0,0,1>": [(256, 32, 4096, 2, True, AUTO)],
     # the prefill kernel: one layer of many tokens, a warp or several per token (more cases: test_gpu_prefill.py)
     "tile<16,0,768,1>": [(3000, 16, 768, 1, False, AUTO)],
     "tile<16,1,768,1>": [(3000, 16, 768, 1, True, AUTO)],
@@ -76,8 +93,8 @@ CASES = {
     "tile<32,1,2048,2>": [(1500, 32, 2048, 1, True, AUTO)],
     "tile<32,1,2048,4>": [(500, 32, 2048, 1, True, AUTO)],
     # the tensor-core step: a token per block or per cluster (more cases: test_gpu_step_mma.py)
-    "mma<32,0,4>": [(16, 32, 2048, 16, False, AUTO), (64, 32, 2048, 3, False, AUTO), (1, 32, 2048, 16, False, AUTO)],
-    "mma<32,1,4>": [(16, 32, 2048, 3, True, AUTO), (64, 32, 2048, 2, True, AUTO)],
+    "mma<32,0,4>": [(64, 32, 2048, 3, False, AUTO), (38, 32, 2048, 16, False, AUTO)],
+    "mma<32,1,4>": [(64, 32, 2048, 2, True, AUTO)],
     "mma<32,1,2>": [(16, 32, 1024, 2, True, AUTO)],
     "mma<16,1,2>": [(64, 16, 1536, 2, True, AUTO)],
 }
@@ -205,7 +222,7 @@ def test_cluster_kernel_chained_step(M, N, norm):
 @pytest.mark.gpu
 @pytest.mark.parametrize("with_tmp", [True, False])
 def test_step_auto_on_the_widest_layers_at_few_tokens(with_tmp):
-    """mole_decode_step's own choice (MOLE_STEP_AUTO) for d = 2048 at up to 16 tokens, the fused tensor-core step, with a second
+    """mole_decode_step's own choice (MOLE_STEP_AUTO) for d = 2048 at up to 16 tokens, one fused launch, with a second
     buffer (which it does not touch) and without; against the oracle."""
     M, N, d, L, V = 8, 32, 2048, 3, 41
     g = torch.Generator().manual_seed(5)
@@ -216,7 +233,7 @@ def test_step_auto_on_the_widest_layers_at_few_tokens(with_tmp):
     ref, _, _ = _oracle_chain(hidden, ids, luts, wrs, None, 0.0)
     status = torch.zeros(1, dtype=torch.int32, device=DEV)
     hd = hidden.to(DEV)
-    assert mole.variant(M, N, d, L=L)[0] == "mma<32,0,4>"
+    assert mole.variant(M, N, d, L=L)[0] == "slice_step<32,2048,1,0,4>"
     tmp = torch.full_like(hd, 3.0) if with_tmp else None
     out = mole.decode_step_args(hd, ids.to(DEV), luts.to(DEV), wrs.to(DEV), torch.empty_like(hd), tmp, status=status, mode=mole.STEP_AUTO)
     torch.cuda.synchronize()
