@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(FStepCut<N, DB>::dmax / 4 + 32) mole_fstep_ker
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = T >> 5;
     const long long G = gridDim.x, b0 = blockIdx.x;
     const int ntok = b0 < p.M ? static_cast<int>((p.M - b0 + G - 1) / G) : 0;
-    constexpr int kr = KR, rexp = REXP, cpi = KWR + KR;  // chunks per item
+    constexpr int rexp = REXP, cpi = KWR + KR;  // experts per rows chunk; chunks per item
     const FStepSmem m = fstep_smem(N, d, stages, NORM);
     const uint32_t wchunk_bytes = static_cast<uint32_t>(d) * N * 2 / KW, rchunk_bytes = static_cast<uint32_t>(rexp) * d * 2;
 

@@ -286,7 +286,8 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 3
     mole_mma_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap r_map, const MmaParams p)
 {
     constexpr int ET = RouterA<N>::ET;
-    extern __shared__ __align__(1024) unsigned char smem[];
+    extern __shared__ __align__(1024) unsigned char smem_1k[];
+    unsigned char *const smem = smem_1k;
 
     pdl_enter(p.flags);
 

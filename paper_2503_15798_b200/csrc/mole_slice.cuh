@@ -316,7 +316,8 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__((D / kMmaCols / CS 
     using Layer = SliceLayer<N, D, T, NORM, (NW + kCopyWarps) * 32, CS>;
     constexpr SliceSmem m = slice_smem(N, NW, T, S, NORM, CS);
     constexpr uint32_t kRows = NW * slice_bytes(N);  // of a slot: the router matrix, then the rows
-    extern __shared__ __align__(1024) unsigned char smem[];
+    extern __shared__ __align__(1024) unsigned char smem_1k[];
+    unsigned char *const smem = smem_1k;
 
     pdl_enter(p.flags);
 
@@ -519,7 +520,8 @@ __global__ void __launch_bounds__(D / kMmaCols * 32, 2) mole_slice_layer_kernel(
     using Layer = SliceLayer<N, D, T, NORM, NW * 32>;
     constexpr SliceSmem m = slice_smem(N, NW, T, 1, NORM);
     constexpr uint32_t kRouterBytes = D * N * 2;
-    extern __shared__ __align__(1024) unsigned char smem[];
+    extern __shared__ __align__(1024) unsigned char smem_1k[];
+    unsigned char *const smem = smem_1k;
 
     pdl_enter(p.flags);
 
