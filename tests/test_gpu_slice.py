@@ -178,3 +178,65 @@ def test_slots_that_fill_slowly(N, d, M, norm):
             out = _fused(h, i, table, slow_w, gam)
             torch.cuda.synchronize()
             assert torch.equal(out, want)
+
+
+# a cluster of two blocks per token, a block, half a block (the neighbour of an extreme token is an ordinary one), blocks that walk pairs
+@pytest.mark.parametrize("M", [11, 100, 301, 4 * SMS + 2])
+@pytest.mark.parametrize("d", [768, 1024])
+def test_extreme_tokens_beside_ordinary_ones(d, M):
+    """Every second token has infinite table entries, or logits far beyond +-60, or (with the norm) a sum of squares that overflows: what
+    it gives is what such values mean, and the token beside it has the bits it has in a launch without them."""
+    L = 2
+    luts, wrs, hidden, _, gammas = _case(d, M, L, True)
+    ids = torch.arange(M, dtype=torch.int32) % 20
+    odd = torch.arange(M) % 2 == 1
+    ids[odd] = 20 + ids[odd]
+    i, w, gam = ids.to(DEV), wrs.to(DEV), gammas.to(DEV)
+    modes = (mole.STEP_FUSED, mole.STEP_CHAINED)
+
+    def step(lu, h, routers, g, mode):
+        return mole.decode_step_args(h, i, lu, routers, torch.empty_like(h), torch.empty_like(h), mode=mode, norm_weights=g, norm_eps=1e-6, kernel=mole.KERNEL_RING).cpu()
+
+    plain, h = luts.to(DEV), hidden.to(DEV)
+    # infinite entries, under a router of zeros (numerators of exactly 1, two of whose three parts are zero) and under an ordinary one
+    inf = luts.clone()
+    want = torch.zeros(M, d)
+    for row in range(20, 40):
+        for col, sign in ((row, 1.0), (d - 1 - 7 * row, -1.0), (d // 2 + row, 1.0)):
+            inf[L - 1, row, row % N, col] = sign * float("inf")
+            want[ids == row, col] = sign * float("inf")
+    for routers in (torch.zeros_like(w), w):
+        for mode in modes:
+            out, ordinary = step(inf.to(DEV), h, routers, None, mode), step(plain, h, routers, None, mode)
+            assert torch.equal(torch.isinf(out), torch.isinf(want)) and not torch.isnan(out).any()
+            assert torch.equal(out[torch.isinf(want)].float(), want[torch.isinf(want)])
+            assert torch.equal(out[~odd], ordinary[~odd])
+            assert torch.equal(out[~torch.isinf(want)], ordinary[~torch.isinf(want)])
+    # logits of hundreds: the gates are those of the largest, and the neighbour's bits do not move
+    big = hidden.clone()
+    big[odd] *= 300.0
+    ref, gref, _ = oracle_layer(big, ids, luts[0], wrs[0])
+    assert gref[odd.numpy()].max() > 0.999
+    gates = torch.zeros(M, N, dtype=torch.float32, device=DEV)
+    one = mole.layer_forward(big.to(DEV), i, plain[0], w[0], gates_out=gates, kernel=mole.KERNEL_RING)
+    # a logit of z carries |z| 2^-22 of fp32 rounding, and so does a gate relative to itself
+    slack = 2.0 ** -20 * np.abs(as_f64(big) @ as_f64(wrs[0])).max(axis=1, keepdims=True)
+    assert (np.abs(as_f64(gates) - gref) <= 1e-5 + slack).all()
+    assert (np.abs(as_f64(one) - ref) <= 2.0 ** -8 * np.abs(ref) + 2e-5 + slack * N * float(luts.abs().max())).all()
+    for mode in modes:
+        assert torch.equal(step(plain, big.to(DEV), w, None, mode)[~odd], step(plain, h, w, None, mode)[~odd])
+    # an overflowing sum of squares: the normalised state is zero and the gates are 1 / N
+    over = hidden.clone()
+    over[odd, 7], over[odd, d - 1] = 2e19, -3e38
+    gates.zero_()
+    mole.layer_forward(over.to(DEV), i, plain[0], w[0], gates_out=gates, norm_weight=gam[0], norm_eps=1e-6, kernel=mole.KERNEL_RING)
+    assert (gates[odd.to(DEV)] == 1.0 / N).all()
+    for mode in modes:
+        out, ordinary = step(plain, over.to(DEV), w, gam, mode), step(plain, h, w, gam, mode)
+        assert torch.equal(out[~odd], ordinary[~odd])
+        for t in torch.nonzero(odd).flatten().tolist()[:6]:
+            r = as_f64(over[t])
+            for l in range(L):  # each layer's output is rounded once
+                r = as_f64(torch.from_numpy(r + as_f64(luts[l, int(ids[t])]).mean(axis=0)).to(torch.bfloat16))
+            # a rounding tie of a layer may fall the other way: an ulp of bf16 per layer
+            assert (np.abs(as_f64(out[t]) - r) <= L * 2.0 ** -7 * np.maximum(1.0, np.abs(r))).all(), (mode, t)
