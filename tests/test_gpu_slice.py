@@ -240,3 +240,22 @@ def test_extreme_tokens_beside_ordinary_ones(d, M):
                 r = as_f64(torch.from_numpy(r + as_f64(luts[l, int(ids[t])]).mean(axis=0)).to(torch.bfloat16))
             # a rounding tie of a layer may fall the other way: an ulp of bf16 per layer
             assert (np.abs(as_f64(out[t]) - r) <= L * 2.0 ** -7 * np.maximum(1.0, np.abs(r))).all(), (mode, t)
+
+
+@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("n,d,M", [(16, 768, 9), (16, 1024, 100), (16, 768, 4 * SMS + 3), (32, 2048, 20)])
+def test_layers_that_share_a_table_or_lie_apart(n, d, M, norm):
+    """Strides of zero (one table, router and scale for all layers) and layers with other memory between them."""
+    L = 4
+    luts, wrs, hidden, ids, gammas = _peaked(n, d, M, 2 * L, d + M, norm)
+    h, i, lu, w, gam = hidden.to(DEV), ids.to(DEV), luts.to(DEV), wrs.to(DEV), None if gammas is None else gammas.to(DEV)
+    strided = (lu[::2], w[::2], None)
+    shared = (lu[1:2].expand(L, -1, -1, -1), w[1:2].expand(L, -1, -1), None if gam is None else gam[1:2].repeat(L, 1))
+    for a, b, g in (strided, shared):
+        if gam is not None and g is None:
+            g = gam[::2].contiguous()
+        for mode in (mole.STEP_FUSED, mole.STEP_CHAINED):
+            def step(x, y):
+                return mole.decode_step_args(h, i, x, y, torch.empty_like(h), torch.empty_like(h), mode=mode, norm_weights=g, norm_eps=1e-5)
+
+            assert torch.equal(step(a, b), step(a.contiguous(), b.contiguous()))
