@@ -60,12 +60,12 @@ QUANT_BLOCKS = {"160m": {"nf4": 768, "nf3": 128}, "410m": {"nf4": 1024, "nf3": 1
 # capture summarised under profiles/ ((config, batch, layers) -> bytes); None until one is taken
 # of the kernel as it stands
 TRAFFIC = {
-    # profiles/mole_step_kernel_single_layer_160m_batch256.md: mean of three captured launches (one layer each)
-    ("160m", 256, 12): 4.29e6,
+    # profiles/mole_slice_kernels.md: three captured launches (one layer each)
+    ("160m", 256, 12): 4.17e6,
 }
 FUSED_TRAFFIC = {
-    # profiles/mole_step_kernel_fused_160m_batch256.md: 8.1 MB per 2-layer launch, x6 for the 12 layers of a full launch
-    ("160m", 256, 12): 48.6e6,
+    # profiles/mole_slice_kernels.md: 7.94 MB per 2-layer launch, x6 for the 12 layers of a full launch
+    ("160m", 256, 12): 47.6e6,
 }
 
 

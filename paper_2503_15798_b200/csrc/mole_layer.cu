@@ -448,7 +448,9 @@ static DecodeVariant pick_cdecode(int N, bool norm)
 // Tokens from which a single layer runs on the prefill kernel (mole_tile.cuh).  Measured against the ring kernel, us per layer:
 // rows of more than 32 KB, which the ring cuts into chunks, from two tokens per SM on (1B shape: 11.3 against 10.4 at 200 tokens,
 // 12.1 against 14.7 at 300); rows of up to 32 KB from six (410M shape: 8.3 / 8.3 at 600, 8.4 / 10.4 at 900; 160M: 8.7 / 10.3 at
-// 900); small rows, of which the ring kernel keeps more blocks resident, from eight (N = 16, d = 384: even at 1 200).
+// 900); small rows, of which the ring kernel keeps more blocks resident, from eight (N = 16, d = 384: even at 1 200).  (At N = 16,
+// d = 768 and 1024 the kernels of mole_slice.cuh have taken the ring kernel's place below the line and are ahead beyond it, too: prefill /
+// there, 768: 8.2 / 5.8 at 1 184 tokens, 8.1 / 7.4 at 1 600, 9.8 / 13.0 at 3 000; 1024: 7.6 / 7.0 at 1 184, 7.5 / 8.0 at 1 300.)
 static long long tile_from(int N, int d, int sms)
 {
     const long long row = static_cast<long long>(N) * d * 2;

@@ -44,7 +44,7 @@ static int mma_blocks(int N, int d)
 // Whether a fused step of M tokens runs here.  Up to one block per SM: every shape but d = 768 and 1024 with N = 16, which have
 // kernels with the sizes compiled in (mole_slice.cuh: 10.5 against 17.6 us for 12 layers of 768, 64 tokens).  Up to two blocks per SM: where a block's part
 // is small (N = 8, d = 1024, 250 tokens, 10 layers: 15.4 against 19.1 us; not N = 32, d = 512: 27.3 against 22.2) or the rows are so
-// wide that the ring kernel cuts them finely (1B shape, 64 tokens: 39.8 against 53.2).  Beyond that a second wave starts where
+// wide that the ring kernel cuts them finely (1B shape, 64 tokens: 36.5 against 53.2).  Beyond that a second wave starts where
 // the ring kernel has the next token's rows in flight already.
 bool mma_preferred(long long M, int dtype, int N, int d, int sms)
 {

@@ -278,8 +278,8 @@ __device__ __forceinline__ float softmax_part(float z, int group)
 }
 
 // N: experts.  NORM: the router reads RMSNorm(hidden).  CS: blocks per token.
-// Registers: for two blocks per SM (112), but where that spills on the critical path or two large blocks rarely meet: N = 32, and
-// N = 16 in pairs (140 or 148; 12 layers of 16 x 2048 with the norm, 64 tokens 33.5 -> 24.0 us, of 16 x 1280 29.5 -> 21.5).
+// Registers: for two blocks per SM (at most 96; N = 16 without pairs spills 16 bytes, with the norm 32), but where that spills on the
+// critical path or two large blocks rarely meet: N = 32 (168), and N = 16 in pairs (119, with the norm 134; 12 layers of 16 x 2048 with the norm, 64 tokens 33.5 -> 24.0 us, of 16 x 1280 29.5 -> 21.5).
 // Launch: d / CS / 4 + 32 threads, mma_smem(..).total bytes, CS blocks per token.
 template <int N, int NORM, int CS>
 __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(8 * 32 + 32, N == 32 || (N == 16 && CS == 2) ? 1 : 2)

@@ -193,7 +193,8 @@ __global__ void __launch_bounds__(kQuantThreads) mole_quantize_wide_kernel(const
 // searched by bisection with packed bf16 compares.  A lane owns chunks of 16 consecutive elements (one 32-byte load; 8
 // bytes of NF4 codes, 4 + 2 of NF3) and keeps them in registers between the maximum and the coding.
 // One layer of the 160M shape (618 M elements) to NF3, block 128: 369 us before the bounds below, 345 with them (1486 us with two passes and a division
-// and 7 float32 compares per element); what is left is the integer pipe (compares and selects), 65 % busy.
+// and 7 float32 compares per element); what is left is the integer pipe (compares and selects): 78 % busy, and 84 % to NF4 in blocks of 1024,
+// at 63 % of the issue slots.
 __device__ __forceinline__ uint32_t bf162_bits(__nv_bfloat162 v) { return *reinterpret_cast<const uint32_t *>(&v); }
 __device__ __forceinline__ __nv_bfloat162 bits_bf162(uint32_t v) { return *reinterpret_cast<const __nv_bfloat162 *>(&v); }
 // 0xffff in each half where x > t
@@ -243,7 +244,8 @@ struct QuantGrid {
 };
 
 // Six blocks of 128 threads per SM (80 registers; left to itself the compiler takes 93 to 98 and four blocks' worth fit): 24 warps hide
-// more of the loads than 16, though a few values of the dividing branch are spilled.  20 000 ids, us: NF3 16 x 768 in blocks of 128 151.0 -> 126.6,
+// more of the loads than 16, though values of the dividing branch are spilled (none up to two chunks a lane of NF3 and one of NF4; of four chunks NF3 reloads
+// 72 bytes a thread and NF4 236: local memory is 3 % and 7 % of the instructions).  20 000 ids, us: NF3 16 x 768 in blocks of 128 151.0 -> 126.6,
 // NF4 16 x 768 in blocks of 768 236.8 -> 196.2, 16 x 2048 in blocks of 1024 564.6 -> 501.0; seven blocks 128.5, 196.4, 499.2, three of 256
 // threads 128.6, 202.2, 510.
 constexpr int kQuantTileThreads = 128;

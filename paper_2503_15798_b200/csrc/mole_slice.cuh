@@ -1,6 +1,10 @@
 // The layer and the fused L-layer step of the two narrow widths of the paper's Table 2 (N = 16 experts, d = 768 and 1024, bf16) for
-// sm_100a -- what mole_variant calls the step kernels of SHAPE 1 and 2 -- and the fused step of its widest (N = 32, d = 2048) while every
-// token has four SMs to itself, the bits of mma<32,..,4>.  (Eq. 4 and Eq. 8 of arXiv 2503.15798.)
+// sm_100a (slice_layer<d,T,NORM,LOOP> and slice_step<N,d,T,NORM,CS> to mole_variant), and the fused step of its widest (N = 32, d = 2048)
+// while every token has four SMs to itself, the bits of mma<32,..,4>.  (Eq. 4 and Eq. 8 of arXiv 2503.15798.)
+// Which widths: the paper's, each of which had a ring kernel with its sizes compiled in before, and costs a dozen instantiations.  Nothing
+// here is about them: the kernels take an even number of warps (d a multiple of 256), as far as slots and registers reach.  A neighbour run
+// through them, 12 fused layers of 16 x 512, us, mole_mma.cuh / here: 64 tokens 10.6 / 9.8, 140 tokens 10.7 / 8.9, 256 tokens 12.9 / 11.1, with
+// the norm 15.4 / 13.9, 15.6 / 12.1, 18.5 / 14.3.
 //
 // What bounds them.  A token's layer is a dependent chain -- router product, a sum over the block, a softmax, a weighted sum -- and a
 // decode batch has one or two tokens per SM, so a layer costs the length of the chain, and what it shares the chip's queues with: the
@@ -152,16 +156,22 @@ struct SliceLayer {
             }
         }
     }
-    // 16 lanes fetch a token's 128 columns (token: lane / 16 of two); out of range: nothing.  `under` is done while they are on their way
+    // 16 lanes fetch a token's 128 columns (token: lane / 16 of two); out of range: nothing.  With the norm,
+    // `under` is done while they are on their way
     template <typename F>
     __device__ __forceinline__ void load_hidden(const unsigned char *hidden, long long t0, long long M, F &&under)
     {
         const long long t = t0 + (T == 2 ? lane >> 4 : 0);
-        const bool mine = (T == 2 || lane < 16) && t < M;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (mine) v = __ldcg(reinterpret_cast<const uint4 *>(hidden + static_cast<size_t>(t) * (D * 2) + slice * 256 + (lane & 15) * 16));
-        under();
-        if (mine) sts128(hid + static_cast<uint32_t>(lane) * 16u, v);
+        auto load = [&]() { return __ldcg(reinterpret_cast<const uint4 *>(hidden + static_cast<size_t>(t) * (D * 2) + slice * 256 + (lane & 15) * 16)); };
+        if constexpr (NORM) {
+            const bool mine = (T == 2 || lane < 16) && t < M;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (mine) v = load();
+            under();
+            if (mine) sts128(hid + static_cast<uint32_t>(lane) * 16u, v);
+        } else {
+            if ((T == 2 || lane < 16) && t < M) sts128(hid + static_cast<uint32_t>(lane) * 16u, load());
+        }
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < T; ++j)
